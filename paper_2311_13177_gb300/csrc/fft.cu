@@ -118,6 +118,16 @@ struct Shape {
   static constexpr size_t SMEM = (size_t)NFFT * kFftCols * sizeof(float2) + (size_t)TW * sizeof(float2);
 };
 
+// The thread's place in its line (16 lines side by side); the mask tells the
+// compiler its range, so that what depends on a position's block or on the
+// crop is decided at compile time where TPL divides it.
+template <int NFFT, int EV>
+__device__ __forceinline__ int line_thread(int tid) {
+  constexpr int TPL = Shape<NFFT, EV>::TPL;
+  static_assert((TPL & (TPL - 1)) == 0, "threads a line: a power of two");
+  return (tid / kFftCols) & (TPL - 1);
+}
+
 // Fill the per-pass twiddle tables from the length-NFFT table exp(-2 pi i m / NFFT).
 template <int NFFT, int EV>
 __device__ void build_twiddles(float2* tws, const float2* __restrict__ base) {
@@ -424,8 +434,7 @@ __device__ __forceinline__ void fft_pass(float2* X, const float2* tws, int col, 
   } else {
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
-      const int j = tl + TPL * q;
-      const int d = (j / NS) * NS * R + (j % NS);  // = j: NS R = NFFT in the last pass
+      const int d = tl + TPL * q;  // NS R = NFFT in the last pass, so (j / NS) NS R + j % NS = j
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         if constexpr (PRUNE_OUT) {
@@ -441,13 +450,28 @@ __device__ __forceinline__ void fft_pass(float2* X, const float2* tws, int col, 
   }
 }
 
-// Position p of a length-n line holds image index i = x + N/2 for
+// Position p of a line of length n = 2N holds image index i = x + N/2 for
 // x = p (p < N/2) or x = p - n (p >= n - N/2); other positions are padding.
-__device__ __forceinline__ int image_index(int p, int N, int n) {
-  const int h = N >> 1;
+template <int n>
+__device__ __forceinline__ int image_index(int p) {
+  constexpr int h = n / 4;
   if (p < h) return p + h;
   if (p >= n - h) return p - (n - h);
   return -1;
+}
+
+// The value `off` bytes past `base`.  The passes address global memory as a
+// base that is the same for the whole CTA plus a 32-bit byte offset (an image
+// row of V or of the row intermediate, one frame's grid: all below 4 GB), and
+// the lengths n and N are compile-time, so that an access costs one multiply-add
+// and the crop is decided at compile time where a thread's positions allow:
+// the adjoint column pass at 2N = 384 issued 58 instructions a value with
+// run-time lengths and 64-bit indices.
+__device__ __forceinline__ float2 load_at(const void* base, uint32_t off) {
+  return __ldg(reinterpret_cast<const float2*>(static_cast<const char*>(base) + off));
+}
+__device__ __forceinline__ void store_at(void* base, uint32_t off, float2 v) {
+  *reinterpret_cast<float2*>(static_cast<char*>(base) + off) = v;
 }
 
 struct FftArgs {
@@ -460,129 +484,140 @@ struct FftArgs {
   int Cv;  // valid bins in this chunk (<= C)
   int f0;
   float scale;
+  const uint64_t* used;  // column passes: grid blocks in use [frame][u1 / 2], or null
+  int ushift;            // log2 of the 16-line tiles in two grid columns
 };
+
+// Blocks in use of the grid column that 16-line tile qt of frame t lies in
+// (bin strides 8 to 64: two adjacent columns hold a whole number of tiles).
+__device__ __forceinline__ uint64_t used_blocks(const uint64_t* used, int ushift, int n, size_t t, int qt) {
+  return used ? __ldg(&used[t * (n >> 1) + (qt >> ushift)]) : ~0ull;
+}
 
 enum Kind { kFwdRows = 0, kFwdCols = 1, kAdjCols = 2, kAdjRows = 3 };
 
 // Forward rows: V[t][i2][i1][f0 + f] * c(i1) c(i2), padded -> rows[t][i2][u1][f].
 struct InFwdRows {
-  const float2* V;
+  const float2* V;  // voxel (t, i2, 0, f0 + fbase)
   const float* dp;
-  int N, n, Nf, Cv, f0, fbase;
-  size_t row;  // (t*N + i2)
+  uint32_t step;    // bytes from one voxel of the row to the next
+  int live;         // valid bins from fbase on
   float c2;
   __device__ float2 at(int i1, int col) const {  // i1: image index
-    const int f = fbase + col;
-    if (f >= Cv) return make_float2(0.f, 0.f);
-    return cscale_rn(__ldg(&V[(row * N + i1) * Nf + f0 + f]), dp[i1] * c2);
+    if (col >= live) return make_float2(0.f, 0.f);
+    return cscale_rn(load_at(V, (uint32_t)i1 * step + (uint32_t)col * 8u), dp[i1] * c2);
   }
 };
 struct OutFwdRows {
-  float2* rows;
-  int n, C, fbase;
-  size_t row;
+  float2* rows;   // position (row, 0, fbase)
+  uint32_t step;  // bytes from one position to the next
+  int live;       // bins of the stride from fbase on
   __device__ void operator()(int pos, int col, float2 val) const {
-    const int f = fbase + col;
-    if (f < C) rows[(row * n + pos) * C + f] = val;
+    if (col < live) store_at(rows, (uint32_t)pos * step + (uint32_t)col * 8u, val);
   }
 };
 // Forward columns: rows[t][i2][q], padded along i2 -> grid[t][u2][q], q = u1*C + f.
 struct InFwdCols {
-  const float2* rows;
-  int N, n;
-  size_t nq, q, t;
-  __device__ float2 at(int i2, int col) const { return __ldg(&rows[(t * N + i2) * nq + q + col]); }
+  const float2* rows;  // (t, 0, q)
+  uint32_t step;       // bytes from one row to the next
+  __device__ float2 at(int i2, int col) const { return load_at(rows, (uint32_t)i2 * step + (uint32_t)col * 8u); }
 };
 struct OutFwdCols {
-  float2* grid;
-  int n;
-  size_t nq, q, t;
+  float2* grid;   // (t, 0, q)
+  uint32_t step;  // bytes from one row to the next
+  uint64_t used;  // blocks of the column that some sample reads
   __device__ void operator()(int pos, int col, float2 val) const {
-    grid[(t * n + pos) * nq + q + col] = val;
+    if (used >> (pos / kGridBlock) & 1) store_at(grid, (uint32_t)pos * step + (uint32_t)col * 8u, val);
   }
 };
 // Adjoint columns: grid[t][u2][q] -> inverse FFT along u2, crop -> rows[t][i2][q].
 struct InAdjCols {
   const float2* grid;
-  int n;
-  size_t nq, q, t;
+  uint32_t step;
+  uint64_t used;  // blocks of the column that the spread filled; the others are zero
   __device__ float2 operator()(int pos, int col) const {
-    return __ldg(&grid[(t * n + pos) * nq + q + col]);
+    if (!(used >> (pos / kGridBlock) & 1)) return make_float2(0.f, 0.f);
+    return load_at(grid, (uint32_t)pos * step + (uint32_t)col * 8u);
   }
 };
+template <int n>
 struct OutAdjCols {
   float2* rows;
-  int N, n;
-  size_t nq, q, t;
+  uint32_t step;
   __device__ void operator()(int pos, int col, float2 val) const {
-    const int i2 = image_index(pos, N, n);
-    if (i2 >= 0) rows[(t * N + i2) * nq + q + col] = val;
+    const int i2 = image_index<n>(pos);
+    if (i2 >= 0) at(i2, col, val);
   }
-  __device__ void at(int i2, int col, float2 val) const { rows[(t * N + i2) * nq + q + col] = val; }
+  __device__ void at(int i2, int col, float2 val) const {
+    store_at(rows, (uint32_t)i2 * step + (uint32_t)col * 8u, val);
+  }
 };
 // Adjoint rows: rows[t][i2][u1][f] -> inverse FFT along u1, crop,
 // * scale c(i1) c(i2) -> out[t][i2][i1][f0 + f].
 struct InAdjRows {
-  const float2* rows;
-  int n, C, Cv, fbase;
-  size_t row;
+  const float2* rows;  // position (row, 0, fbase)
+  uint32_t step;
+  int live;            // valid bins from fbase on
   __device__ float2 operator()(int pos, int col) const {
-    const int f = fbase + col;
-    if (f >= Cv) return make_float2(0.f, 0.f);
-    return __ldg(&rows[(row * n + pos) * C + f]);
+    if (col >= live) return make_float2(0.f, 0.f);
+    return load_at(rows, (uint32_t)pos * step + (uint32_t)col * 8u);
   }
 };
+template <int n>
 struct OutAdjRows {
-  float2* out;
+  float2* out;  // voxel (t, i2, 0, f0 + fbase)
   const float* dp;
-  int N, n, Nf, Cv, f0, fbase;
-  size_t row;
+  uint32_t step;
+  int live;
   float c2;
   __device__ void operator()(int pos, int col, float2 val) const {
-    const int f = fbase + col;
-    const int i1 = image_index(pos, N, n);
-    if (f < Cv && i1 >= 0) out[(row * N + i1) * Nf + f0 + f] = cscale(val, dp[i1] * c2);
+    const int i1 = image_index<n>(pos);
+    if (i1 >= 0) at(i1, col, val);
   }
   __device__ void at(int i1, int col, float2 val) const {
-    const int f = fbase + col;
-    if (f < Cv) out[(row * N + i1) * Nf + f0 + f] = cscale(val, dp[i1] * c2);
+    if (col < live) store_at(out, (uint32_t)i1 * step + (uint32_t)col * 8u, cscale(val, dp[i1] * c2));
   }
 };
 
 template <int NFFT, int KIND>
 __global__ void __launch_bounds__(Shape<NFFT, kValsPlain<NFFT>>::THREADS) fft_kernel(FftArgs a) {
   constexpr int EV = kValsPlain<NFFT>;
+  constexpr int N = NFFT / 2;
   extern __shared__ float2 smem[];
   float2* X = smem;
   float2* tw = smem + NFFT * kFftCols;
   build_twiddles<NFFT, EV>(tw, a.twiddle);
   __syncthreads();
   const int col = threadIdx.x % kFftCols;
-  const int tl = threadIdx.x / kFftCols;
-  if constexpr (KIND == kFwdRows) {
+  const int tl = line_thread<NFFT, EV>(threadIdx.x);
+  if constexpr (KIND == kFwdRows || KIND == kAdjRows) {
     const size_t row = blockIdx.y;  // t*N + i2
-    const int i2 = (int)(row % a.N);
+    const int i2 = (int)(row % N);
     const int fbase = blockIdx.x * kFftCols;
-    InFwdRows in{a.src, a.deapod, a.N, a.n, a.Nf, a.Cv, a.f0, fbase, row, a.deapod[i2]};
-    OutFwdRows out{a.dst, a.n, a.C, fbase, row};
-    fft_pass<NFFT, EV, -1, 0, 1, true, false>(X, tw, col, tl, in, out);
-  } else if constexpr (KIND == kFwdCols) {
-    const size_t nq = (size_t)a.n * a.C;
-    InFwdCols in{a.src, a.N, a.n, nq, (size_t)blockIdx.x * kFftCols, blockIdx.y};
-    OutFwdCols out{a.dst, a.n, nq, (size_t)blockIdx.x * kFftCols, blockIdx.y};
-    fft_pass<NFFT, EV, -1, 0, 1, true, false>(X, tw, col, tl, in, out);
-  } else if constexpr (KIND == kAdjCols) {
-    const size_t nq = (size_t)a.n * a.C;
-    InAdjCols in{a.src, a.n, nq, (size_t)blockIdx.x * kFftCols, blockIdx.y};
-    OutAdjCols out{a.dst, a.N, a.n, nq, (size_t)blockIdx.x * kFftCols, blockIdx.y};
-    fft_pass<NFFT, EV, +1, 0, 1, false, true>(X, tw, col, tl, in, out);
+    const size_t wpos = row * NFFT * a.C + fbase, vox = row * N * a.Nf + a.f0 + fbase;
+    const uint32_t wstep = (uint32_t)a.C * 8u, vstep = (uint32_t)a.Nf * 8u;
+    if constexpr (KIND == kFwdRows) {
+      InFwdRows in{a.src + vox, a.deapod, vstep, a.Cv - fbase, a.deapod[i2]};
+      OutFwdRows out{a.dst + wpos, wstep, a.C - fbase};
+      fft_pass<NFFT, EV, -1, 0, 1, true, false>(X, tw, col, tl, in, out);
+    } else {
+      InAdjRows in{a.src + wpos, wstep, a.Cv - fbase};
+      OutAdjRows<NFFT> out{a.dst + vox, a.deapod, vstep, a.Cv - fbase, a.deapod[i2] * a.scale};
+      fft_pass<NFFT, EV, +1, 0, 1, false, true>(X, tw, col, tl, in, out);
+    }
   } else {
-    const size_t row = blockIdx.y;
-    const int i2 = (int)(row % a.N);
-    const int fbase = blockIdx.x * kFftCols;
-    InAdjRows in{a.src, a.n, a.C, a.Cv, fbase, row};
-    OutAdjRows out{a.dst, a.deapod, a.N, a.n, a.Nf, a.Cv, a.f0, fbase, row, a.deapod[i2] * a.scale};
-    fft_pass<NFFT, EV, +1, 0, 1, false, true>(X, tw, col, tl, in, out);
+    const size_t nq = (size_t)NFFT * a.C, q = (size_t)blockIdx.x * kFftCols, t = blockIdx.y;
+    const uint32_t step = (uint32_t)(nq * sizeof(float2));
+    const uint64_t used = used_blocks(a.used, a.ushift, NFFT, t, blockIdx.x);
+    if constexpr (KIND == kFwdCols) {
+      InFwdCols in{a.src + t * N * nq + q, step};
+      OutFwdCols out{a.dst + t * NFFT * nq + q, step, used};
+      fft_pass<NFFT, EV, -1, 0, 1, true, false>(X, tw, col, tl, in, out);
+    } else {
+      InAdjCols in{a.src + t * NFFT * nq + q, step, used};
+      OutAdjCols<NFFT> out{a.dst + t * N * nq + q, step};
+      fft_pass<NFFT, EV, +1, 0, 1, false, true>(X, tw, col, tl, in, out);
+    }
   }
 }
 
@@ -627,13 +662,13 @@ struct MultiFused {
 };
 
 // Adjoint output into the CTA's gradient buffer gb[i1][col].
+template <int n>
 struct OutGrad {
   float2* gb;
   const float* dp;
-  int N, n;
   float c2;
   __device__ void operator()(int pos, int col, float2 val) const {
-    const int i1 = image_index(pos, N, n);
+    const int i1 = image_index<n>(pos);
     if (i1 >= 0) gb[i1 * kFftCols + col] = cscale(val, dp[i1] * c2);
   }
   __device__ void at(int i1, int col, float2 val) const { gb[i1 * kFftCols + col] = cscale(val, dp[i1] * c2); }
@@ -642,7 +677,6 @@ struct OutGrad {
 struct InNewRow {
   const float2* vb;
   const float* dp;
-  int N, n;
   float c2;
   __device__ float2 at(int i1, int col) const { return cscale_rn(vb[i1 * kFftCols + col], dp[i1] * c2); }
 };
@@ -777,19 +811,21 @@ __device__ __forceinline__ void fused_rows_body(const FusedArgs& a, int bx, size
   if (threadIdx.x == 0) prefetch_update_rows(a, row, i2, t);
   __syncthreads();
   const int col = threadIdx.x % kFftCols;
-  const int tl = threadIdx.x / kFftCols;
+  const int tl = line_thread<NFFT, EV>(threadIdx.x);
   const int fbase = bx * kFftCols;
+  float2* wpos = a.rows + row * NFFT * a.C + fbase;
+  const uint32_t wstep = (uint32_t)a.C * 8u;
   {
-    InAdjRows in{a.rows, a.n, a.C, a.Nf, fbase, row};
-    OutGrad out{gb, a.deapod, a.N, a.n, a.deapod[i2] * a.scale};
+    InAdjRows in{wpos, wstep, a.Nf - fbase};
+    OutGrad<NFFT> out{gb, a.deapod, a.deapod[i2] * a.scale};
     fft_pass<NFFT, EV, +1, 0, 1, false, true>(X, tw, col, tl, in, out);
   }
   __syncthreads();
   const float local = update_row_any(a, gb, row, i2, t, fbase, threadIdx.x, blockDim.x, 0.f);
   if constexpr (FWD_TAIL) {
     __syncthreads();
-    InNewRow in{gb, a.deapod, a.N, a.n, a.deapod[i2]};
-    OutFwdRows out{a.rows, a.n, a.C, fbase, row};
+    InNewRow in{gb, a.deapod, a.deapod[i2]};
+    OutFwdRows out{wpos, wstep, a.C - fbase};
     fft_pass<NFFT, EV, -1, 0, 1, true, false>(X, tw, col, tl, in, out);
   }
   finish_loss_v(local, a.partials, a.counter, a.data_loss, a.loss_out, vb, nblk);
@@ -932,7 +968,7 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsFused<NFFT>>::THREADS + kUpdT
   float local = 0.f;
   if (threadIdx.x < FT) {
     const int col = threadIdx.x % kFftCols;
-    const int tl = threadIdx.x / kFftCols;
+    const int tl = line_thread<NFFT, EV>(threadIdx.x);
     for (int i = 0; i <= nu; ++i) {
       if (i < nu) {
         if (!mbar_wait_bounded(full, (uint32_t)(i & 1)))
@@ -952,7 +988,7 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsFused<NFFT>>::THREADS + kUpdT
           }
         };
         InTile in{S};
-        OutGrad out{gbuf + (size_t)(i & 1) * gsz, a.deapod, a.N, a.n, a.deapod[i2] * a.scale};
+        OutGrad<NFFT> out{gbuf + (size_t)(i & 1) * gsz, a.deapod, a.deapod[i2] * a.scale};
         fft_pass<NFFT, EV, +1, 0, 1, false, true, FSync>(X, tw, col, tl, in, out, hook);
         mbar_arrive(&ready[i & 1]);
       }
@@ -966,8 +1002,8 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsFused<NFFT>>::THREADS + kUpdT
           const size_t row = (size_t)(u / a.nfb);
           const int fbase = (u - (u / a.nfb) * a.nfb) * kFftCols;
           const int i2 = (int)(row % a.N);
-          InNewRow in{gbuf + (size_t)(j & 1) * gsz, a.deapod, a.N, a.n, a.deapod[i2]};
-          OutFwdRows out{a.rows, a.n, a.C, fbase, row};
+          InNewRow in{gbuf + (size_t)(j & 1) * gsz, a.deapod, a.deapod[i2]};
+          OutFwdRows out{a.rows + row * NFFT * a.C + fbase, (uint32_t)a.C * 8u, a.C - fbase};
           fft_pass<NFFT, EV, -1, 0, 1, true, false, FSync>(X, tw, col, tl, in, out);
         }
       }
@@ -1021,13 +1057,19 @@ cudaError_t launch_fused_ws(const CUtensorMap& tm, const FusedArgs& a, bool fwd_
 // the first pass of the tile in it has read it, so the input of the next
 // tiles streams in while this one is transformed.
 // Forward: the staged input is the N image rows of the row intermediate
-// (padding is never stored); adjoint: the 2N grid rows.
+// (padding is never stored); adjoint: the 2N grid rows.  Of the grid only the
+// blocks that samples reach (Plan::grid_used) are written (forward) or copied
+// in (adjoint: a box without such a block is requested outside the tensor, so
+// that the copy fills it with zeros and reads nothing).
 struct ColArgs {
   float2* dst;
   const float2* twiddle;
   int* err;
   size_t nq;
   int N, n, qtiles, ntiles, bh, nbox;
+  const uint64_t* used;  // grid blocks in use [frame][u1 / 2], or null
+  int ushift;            // log2 of the 16-line tiles in two grid columns
+  uint64_t box_mask;     // adjoint: the grid blocks in one box, at bit 0
 };
 
 // Kernel parameter of a column pass over a batch of problems.
@@ -1077,12 +1119,35 @@ __device__ __forceinline__ void cols_body(const CUtensorMap* tin, const ColArgs&
   uint64_t* full = reinterpret_cast<uint64_t*>(tw + Shape<NFFT, EV>::TW);
   __shared__ volatile int s_abort;
   const uint32_t tile_bytes = (uint32_t)(H * kFftCols * sizeof(float2));
-  auto issue = [&](int tile, int b) {
-    const int t = tile / a.qtiles, qt = tile - (tile / a.qtiles) * a.qtiles;
-    mbar_expect_tx(&full[b], tile_bytes);
-    for (int i = 0; i < a.nbox; ++i)
-      tma_load_3d(tiles + ((size_t)b * H + (size_t)i * a.bh) * kFftCols, tin, qt * 2 * kFftCols, i * a.bh, t,
-                  &full[b]);
+  // A tile of this CTA: frame, 16-line tile of it, its column's blocks in use.
+  struct Tile {
+    int t, qt;
+    uint64_t used;
+  };
+  // The CTA's tiles are vg apart: (frame, tile) steps by (step_t, step_q) with
+  // one carry instead of a division by every thread for every tile.
+  const int step_t = vg / a.qtiles, step_q = vg - step_t * a.qtiles;
+  auto advance = [&](int& t, int& qt) {
+    t += step_t;
+    qt += step_q;
+    if (qt >= a.qtiles) {
+      qt -= a.qtiles;
+      ++t;
+    }
+  };
+  // Whole CTA: request the copy of a tile into buffer b, the boxes dealt out
+  // over the warps (a warp issues its boxes one after the other, and the other
+  // warps would wait for it at the next barrier).  A box that lands before
+  // thread 0 has stated the bytes is made up for by it: the phase cannot end
+  // before that arrival.
+  constexpr int WARPS = Shape<NFFT, EV>::THREADS >= 32 ? Shape<NFFT, EV>::THREADS / 32 : 1;
+  auto issue = [&](const Tile& x, int b) {
+    if (threadIdx.x == 0) mbar_expect_tx(&full[b], tile_bytes);
+    for (int i = (threadIdx.x % 32) * WARPS + threadIdx.x / 32; i < a.nbox; i += 32 * WARPS) {
+      const bool want = KIND == kFwdCols || (x.used >> (i * a.bh / kGridBlock) & a.box_mask) != 0;
+      tma_load_3d(tiles + ((size_t)b * H + (size_t)i * a.bh) * kFftCols, tin, x.qt * 2 * kFftCols,
+                  want ? i * a.bh : NFFT, x.t, &full[b]);
+    }
   };
   if (threadIdx.x == 0) {
     for (int b = 0; b < NB; ++b) mbar_init(&full[b], 1);
@@ -1090,37 +1155,49 @@ __device__ __forceinline__ void cols_body(const CUtensorMap* tin, const ColArgs&
     s_abort = 0;
   }
   build_twiddles<NFFT, EV>(tw, a.twiddle);
+  int nt = vb / a.qtiles, nq = vb - nt * a.qtiles;  // the next tile to request
+  Tile tile_of[NB];                                 // of the tiles in the buffers, the current one's first
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    tile_of[b] = Tile{nt, nq, vb + b * vg < a.ntiles ? used_blocks(a.used, a.ushift, NFFT, nt, nq) : 0};
+    advance(nt, nq);
+  }
   grid_dep_wait();
   grid_dep_release();
-  if (threadIdx.x == 0)
-    for (int b = 0; b < NB; ++b)
-      if (vb + b * vg < a.ntiles) issue(vb + b * vg, b);
-  __syncthreads();
+  __syncthreads();  // the barriers are initialised before any warp issues on them
+#pragma unroll
+  for (int b = 0; b < NB; ++b)
+    if (vb + b * vg < a.ntiles) issue(tile_of[b], b);
   const int col = threadIdx.x % kFftCols;
-  const int tl = threadIdx.x / kFftCols;
+  const int tl = line_thread<NFFT, EV>(threadIdx.x);
+  const uint32_t step = (uint32_t)(a.nq * sizeof(float2));
   int k = 0;
   for (int tile = vb; tile < a.ntiles; tile += vg, ++k) {
     const int b = k % NB;
     if (!mbar_wait_bounded(&full[b], (uint32_t)((k / NB) & 1))) s_abort = 1;
     __syncthreads();  // the previous tile's last pass is done with X; all threads see s_abort
     if (s_abort) break;
-    const size_t t = (size_t)(tile / a.qtiles);
-    const size_t q = (size_t)(tile - (tile / a.qtiles) * a.qtiles) * kFftCols;
-    const int next = tile + NB * vg;
+    const size_t t = (size_t)tile_of[0].t, q = (size_t)tile_of[0].qt * kFftCols;
+    const bool more = tile + NB * vg < a.ntiles;
+    const Tile next{nt, nq, more ? used_blocks(a.used, a.ushift, NFFT, nt, nq) : 0};
     auto hook = [&]() {
-      if (threadIdx.x == 0 && next < a.ntiles) {
+      if (more) {
         fence_proxy_async_smem();
         issue(next, b);
       }
     };
     InTile in{tiles + (size_t)b * H * kFftCols};
     if constexpr (KIND == kFwdCols) {
-      OutFwdCols out{a.dst, a.n, a.nq, q, t};
+      OutFwdCols out{a.dst + t * NFFT * a.nq + q, step, tile_of[0].used};
       fft_pass<NFFT, EV, -1, 0, 1, true, false>(X, tw, col, tl, in, out, hook);
     } else {
-      OutAdjCols out{a.dst, a.N, a.n, a.nq, q, t};
+      OutAdjCols<NFFT> out{a.dst + t * (NFFT / 2) * a.nq + q, step};
       fft_pass<NFFT, EV, +1, 0, 1, false, true>(X, tw, col, tl, in, out, hook);
     }
+#pragma unroll
+    for (int i = 0; i + 1 < NB; ++i) tile_of[i] = tile_of[i + 1];
+    tile_of[NB - 1] = next;
+    advance(nt, nq);
   }
   if (s_abort && threadIdx.x == 0) {
     atomicExch(a.err, 1);
@@ -1296,6 +1373,24 @@ int box_rows(int h) {
   return b;
 }
 
+// Box height of a column pass's input copies: where the adjoint skips unused
+// blocks about a sixteenth of the column, a whole number of blocks (lower
+// boxes skip more and cost more requests).
+int col_box_rows(const Plan& p, int kind) {
+  if (kind == kFwdCols) return box_rows(p.N);
+  if (!p.grid_used || !p.grid_sparse) return box_rows(p.n);
+  int bh = kGridBlock;
+  while (bh * 16 < p.n) bh *= 2;
+  return p.n % bh == 0 ? bh : kGridBlock;
+}
+
+// log2 of the 16-line tiles in two grid columns (bin strides 8, 16, 32, 64).
+int used_shift(const Plan& p) {
+  int s = 0;
+  while ((kFftCols << s) < 2 * p.cs) ++s;
+  return s;
+}
+
 ColArgs col_args(const Plan& p, int kind) {
   ColArgs a{};
   a.dst = kind == kFwdCols ? p.grid : p.rows;
@@ -1306,8 +1401,11 @@ ColArgs col_args(const Plan& p, int kind) {
   a.n = p.n;
   a.qtiles = (int)(a.nq / kFftCols);
   a.ntiles = a.qtiles * p.T;
-  a.bh = box_rows(kind == kFwdCols ? p.N : p.n);
+  a.bh = col_box_rows(p, kind);
   a.nbox = (kind == kFwdCols ? p.N : p.n) / a.bh;
+  a.used = p.grid_used;
+  a.ushift = used_shift(p);
+  a.box_mask = a.bh >= 64 * kGridBlock ? ~0ull : (1ull << std::max(1, a.bh / kGridBlock)) - 1;
   return a;
 }
 
@@ -1522,6 +1620,8 @@ FftArgs base_args(const Plan& p) {
   a.Cv = p.chunk;
   a.f0 = 0;
   a.scale = 1.f;
+  a.used = p.grid_used;
+  a.ushift = used_shift(p);
   return a;
 }
 
@@ -1566,18 +1666,18 @@ void fft_make_maps(Plan& p) {
   }
   if (p.cs % 2 != 0 || p.T > 65536) return;
   const size_t nq = (size_t)p.n * p.cs;
-  auto make = [&](CUtensorMap* tm, float2* base, int h) {
+  auto make = [&](CUtensorMap* tm, float2* base, int h, int bh) {
     const cuuint64_t dims[3] = {(cuuint64_t)(2 * nq), (cuuint64_t)h, (cuuint64_t)p.T};
     const cuuint64_t strides[2] = {(cuuint64_t)(2 * nq * sizeof(float)), (cuuint64_t)(2 * nq * h * sizeof(float))};
-    const cuuint32_t box[3] = {(cuuint32_t)(2 * kFftCols), (cuuint32_t)box_rows(h), 1};
+    const cuuint32_t box[3] = {(cuuint32_t)(2 * kFftCols), (cuuint32_t)bh, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     return encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   };
   const size_t room = (size_t)p.smem_optin - 1024;
-  p.cols_tma_fwd = cols_smem(p.n, kFwdCols) <= room && make(&p.tm_rows, p.rows, p.N);
-  p.cols_tma_adj = cols_smem(p.n, kAdjCols) <= room && make(&p.tm_grid, p.grid, p.n);
+  p.cols_tma_fwd = cols_smem(p.n, kFwdCols) <= room && make(&p.tm_rows, p.rows, p.N, col_box_rows(p, kFwdCols));
+  p.cols_tma_adj = cols_smem(p.n, kAdjCols) <= room && make(&p.tm_grid, p.grid, p.n, col_box_rows(p, kAdjCols));
   // fused row kernel input: [T N][n][2 cs] floats, box = 16 bins x box_rows(n) positions of one row.
   // Automatic choice: the warp-specialised kernel pipelines the units of a
   // CTA, which pays off once every SM has several (at 3.4 units per SM the

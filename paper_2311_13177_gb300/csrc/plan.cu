@@ -58,7 +58,8 @@ bool fft_size_supported(int n) {
 // same order as a per-cell list would.  Every list is padded to a multiple
 // of four entries with (row M, zero weights), row M of the phased residual
 // being kept zero.  Groups are taken in frame, 4 x 4-group patch, row-major
-// order and cut into items of about equal work, each item one blob of int2
+// order, those in grid blocks that no sample reaches (grid_used_h) left out,
+// and cut into items of about equal work, each item one blob of int2
 // words staged by a single bulk copy:
 //   groups[ngp]      (first cell index, end of its list), ngp = ngroups rounded up to even
 //   offs[nent / 2]   nent int32 offsets (nent a multiple of 4)
@@ -92,20 +93,26 @@ bool build_group_lists(const Plan& p, const std::vector<int>& first_tap, const s
   for (size_t g = 0; g < ngroup; ++g) glen[g] = (gcnt[g] + kSpreadListPad - 1) / kSpreadListPad * kSpreadListPad;
   std::vector<int> gorder;
   gorder.reserve(ngroup);
+  static_assert(kGridBlock % kSpreadGroup == 0, "a group lies in one grid block");
+  auto in_use = [&](int t, int gr, int gc) {
+    return p.grid_used_h.empty() || (p.grid_used_h[(size_t)t * gps + gc] >> (gr * G / kGridBlock) & 1);
+  };
   for (int t = 0; t < p.T; ++t)
     for (int pr = 0; pr < gps / PG; ++pr)
       for (int pc = 0; pc < gps / PG; ++pc)
         for (int r = 0; r < PG; ++r)
-          for (int c = 0; c < PG; ++c) gorder.push_back((t * gps + pr * PG + r) * gps + pc * PG + c);
+          for (int c = 0; c < PG; ++c)
+            if (in_use(t, pr * PG + r, pc * PG + c)) gorder.push_back((t * gps + pr * PG + r) * gps + pc * PG + c);
+  const size_t nlisted = gorder.size();
   std::vector<int> item_of(ngroup), first(ngroup);
   struct ItemSec { size_t offs, wts; };
   std::vector<ItemSec> secs;
   auto words = [](long ng, long ne) { return ((ng + 1) & ~1L) + ne / 2 + 2 * ne; };
   size_t i = 0;
-  while (i < ngroup) {
+  while (i < nlisted) {
     size_t j = i;
     long cost = 0, nent = 0;
-    while (j < ngroup) {
+    while (j < nlisted) {
       const int c = glen[gorder[j]];
       if (words((long)(j + 1 - i), nent + c) > kSpreadStageInt2) {
         if (j == i) return false;  // one group exceeds a stage
@@ -161,6 +168,24 @@ bool build_group_lists(const Plan& p, const std::vector<int>& first_tap, const s
   return true;
 }
 
+// Grid blocks (kGridBlock rows of two adjacent columns) that some sample's
+// W x W footprint meets.
+void mark_used_blocks(Plan& p, const std::vector<int>& first_tap) {
+  const int n = p.n, W = p.W;
+  static_assert(kGridBlock >= 8, "a footprint's rows meet at most two blocks");
+  p.grid_used_h.assign((size_t)p.T * (n / 2), 0);
+  const size_t LR = (size_t)p.L * p.R;
+  for (size_t m = 0; m < (size_t)p.M; ++m) {
+    uint64_t* used = &p.grid_used_h[(size_t)p.blade_frame[m / LR] * (n / 2)];
+    const int r0 = first_tap[2 * m + 1], c0 = first_tap[2 * m];
+    const uint64_t rows = 1ull << (r0 / kGridBlock) | 1ull << ((r0 + W - 1) % n / kGridBlock);
+    for (int b = 0; b < W; ++b) used[(c0 + b) % n / 2] |= rows;
+  }
+  size_t count = 0;
+  for (uint64_t u : p.grid_used_h) count += (size_t)__builtin_popcountll(u);
+  p.grid_sparse = 2 * count < p.grid_used_h.size() * (size_t)(n / kGridBlock);
+}
+
 struct DevAlloc {
   Plan* p;
   size_t* counter;
@@ -203,7 +228,7 @@ void plan_dev_free(Plan* p, void* ptr) {
 void plan_free(Plan* p) {
   if (!p) return;
   void* ptrs[] = {p->kb_idx, p->kb_w, p->phase, p->deapod, p->twiddle, p->blade_frame_d,
-                  p->order, p->items, p->item_cta_off, p->sitems, p->sitem_cta_off, p->spread_claim, p->sblob, p->contrib, p->grid, p->rows,
+                  p->order, p->items, p->item_cta_off, p->grid_used, p->sitems, p->sitem_cta_off, p->spread_claim, p->sblob, p->contrib, p->grid, p->rows,
                   p->resid, p->grad, p->status_dev,
                   p->vol2, p->adam_m, p->adam_v, p->loss_dev, p->scalars,
                   p->red_interp.partials, p->red_interp.counter, p->red_tv.partials,
@@ -468,9 +493,11 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
   std::vector<int4> sitems;
   std::vector<int2> blob;
   const int2 pad_entry = make_int2((int)((size_t)p->M * p->cs), 0);
-  p->spread_grouped = (p->cs == 8 || p->cs == 16 || p->cs == 32 || p->cs == 64) &&
-                      build_group_lists(*p, first_tap, wd, sitems, blob);
+  const bool stride_ok = p->cs == 8 || p->cs == 16 || p->cs == 32 || p->cs == 64;
+  if (stride_ok) mark_used_blocks(*p, first_tap);
+  p->spread_grouped = stride_ok && build_group_lists(*p, first_tap, wd, sitems, blob);
   if (!p->spread_grouped) {
+  p->grid_used_h.clear();  // the cell lists fill the whole grid
   sitems.clear();
   blob.clear();
   const size_t ncell = (size_t)p->T * n * n;
@@ -630,9 +657,17 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
   TRY(tab(&p->sitems, std::max<size_t>(sitems.size(), 1), "spread items"));
   TRY(tab(&p->sitem_cta_off, scta_off.size(), "spread item ranges"));
   TRY(tab(&p->sblob, blob.size(), "spread lists"));
+  if (!p->grid_used_h.empty()) TRY(tab(&p->grid_used, p->grid_used_h.size(), "grid block use"));
   TRY(wrk(&p->grid, (size_t)p->T * n * n * p->cs, "grid workspace"));
   TRY(wrk(&p->rows, (size_t)p->T * N * n * p->cs, "row workspace"));
   TRY(wrk(&p->contrib, (size_t)(p->M + 1) * p->cs, "phased residual"));
+  // The blocks of the grid that no sample reaches are never written again and
+  // hold the zeros that the adjoint columns take them for.  (Before the
+  // uploads: those synchronise with it.)
+  if (cudaError_t e = cudaMemset(p->grid, 0, (size_t)p->T * n * n * p->cs * sizeof(float2))) {
+    plan_free(p);
+    return cuda_fail(e, "grid workspace");
+  }
   TRY(upload(p->kb_idx, kb_idx));
   TRY(upload(p->kb_w, kb_w));
   TRY(upload(p->phase, phase));
@@ -643,6 +678,7 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
   if (!sitems.empty()) TRY(upload(p->sitems, sitems));
   TRY(upload(p->sitem_cta_off, scta_off));
   TRY(upload(p->sblob, blob));
+  if (p->grid_used) TRY(upload(p->grid_used, p->grid_used_h));
   if (!items.empty()) TRY(upload(p->items, items));
   TRY(upload(p->item_cta_off, cta_off));
   p->row_kernel = d->row_kernel;
@@ -738,6 +774,7 @@ size_t plan_estimate_bytes(const prop_plan_desc* d, int iters) {
   const size_t cell_lists = 8 * (ncell + spread_items) + 8 * (M * W * W + (kSpreadListPad - 1) * std::min(ncell, M * W * W));
   const size_t group_lists = 8 * (ncell / 4) + 8 + (4 + 16) * 2 * 16 * M + 16 * (ncell / 4);  // items <= groups
   b += 16 * interp_items + 16 * spread_items + std::max(cell_lists, group_lists) + 4 * 1024;  // lists
+  b += 8 * T * (n / 2);                                                                             // grid block use
   b += 8 * T * n * n * cs + 8 * T * N * n * cs + 8 * (M + 1) * cs;                                  // workspace
   b += 8 * M + 4 * 8 * vol + 64 + 2 * 8 * std::max<size_t>(std::max<size_t>(32768, interp_items), (Nf + 15) / 16 * T * N) + 8 +
        8 * std::max<size_t>((size_t)std::max(iters, 1), 64);                                           // optimiser

@@ -48,6 +48,11 @@ constexpr int kCartCols = 4;
 constexpr int interp_tile_rows(int cs, int W) { return cs > 32 ? 8 : (W == 8 && cs == 32 ? 12 : 16); }
 constexpr int interp_tile_cols(int cs, int W) { return (void)W, cs > 32 ? 8 : 16; }
 
+// Rows of a grid block whose use by the samples is tracked (the unit in which
+// the column passes and the spread skip the grid): a thread of the column
+// passes at 2N = 192 to 512 then finds its rows' bits at compile-time places,
+// and 2N = 1024 still has one 64-bit word of blocks a column.
+constexpr int kGridBlock = 16;
 constexpr int kMaxChunk = 64;      // most bins in one grid pass
 constexpr int kMaxBatch = 8;       // most problems in one multi-problem launch
 
@@ -165,6 +170,16 @@ struct Plan {
   size_t spread_entries = 0;
   bool spread_staged = true;     // cell lists: every item fits a shared-memory stage
   bool spread_grouped = false;   // sblob/sitems hold grouped lists (2 x 2-cell groups), else cell lists
+  // Which parts of the grid any sample's taps reach: bit (u2 / kGridBlock) of
+  // entry (t, u1 / 2).  The forward column pass writes only these blocks, the
+  // spread fills only them and the adjoint column pass takes the others as
+  // zero without reading them.  Empty / null: the whole grid is in use (bin
+  // strides without grouped spread lists).
+  std::vector<uint64_t> grid_used_h;  // [T][n / 2]
+  uint64_t* grid_used = nullptr;      // the same on the device
+  // Under half of the blocks are in use: the adjoint column pass copies its
+  // input block by block and leaves the unused ones out.
+  bool grid_sparse = false;
 
   // TMA tensor maps of the column passes' inputs (row workspace, grid), and
   // whether the staged column kernels run for this plan's size
