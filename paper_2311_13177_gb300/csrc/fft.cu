@@ -688,13 +688,15 @@ struct InNewRow {
 // next one is loaded per step.  The adjoint gradient comes from gb[i1][col],
 // the new value goes to Vout and back into gb (zero for bins >= Nf, the
 // padding of the next forward row transform).  Adds this thread's TV shares
-// to `local` in walk order and returns it.  Every load is unconditional
-// (missing neighbours and bins >= Nf read a valid voxel whose value is then
-// not used), so the loads of several steps are in flight together; TT: the
-// volume has time neighbours (T > 1 and tv_t != 0).
-template <bool TT>
-__device__ __forceinline__ float update_row(const FusedArgs& a, float2* gb, size_t row, int i2, int t, int fbase,
-                                            int tid, int nthreads, float local) {
+// to `local` in walk order and returns it.  The walk goes U voxels at a time:
+// all their loads are issued before the first is used (left to the compiler,
+// the stores of one voxel held back the loads of the next, and a voxel cost
+// 3000 clocks of load latency).  Every load is unconditional (missing
+// neighbours and bins >= Nf read a valid voxel whose value is then not used).
+// TT: the volume has time neighbours (T > 1 and tv_t != 0).
+template <bool TT, int U>
+__device__ __forceinline__ float update_row(const FusedArgs& a, float2* gb, int i2, int t, int fbase, int tid,
+                                            int nthreads, float local) {
   const float eps2 = a.ad.tv_eps * a.ad.tv_eps;
   // The volumes and moments never alias: loads of later voxels may be issued
   // ahead of the stores of earlier ones.
@@ -708,80 +710,114 @@ __device__ __forceinline__ float update_row(const FusedArgs& a, float2* gb, size
   const int lo = (tid / kFftCols) * len;
   const int hi = min(a.N, lo + len);
   if (lo >= hi) return local;
-  const size_t sx = (size_t)a.Nf, sy = (size_t)a.N * a.Nf, st = (size_t)a.N * a.N * a.Nf;
+  const size_t sy = (size_t)a.N * a.Nf, st = (size_t)a.N * a.N * a.Nf;
   const bool xy = a.ad.tv_xy != 0.f;
   const bool h2p = xy && i2 + 1 < a.N, h2m = xy && i2 > 0;
   const bool htp = TT && t + 1 < a.T, htm = TT && t > 0;
   const int f = fbase + col;
   const bool fv = f < a.Nf;
-  const size_t base = row * a.N * a.Nf + (size_t)(fv ? f : a.Nf - 1);  // voxel (t, i2, 0, f)
-  float2 xm = Vin[lo > 0 ? base + (size_t)(lo - 1) * sx : base];
-  float2 x = Vin[base + (size_t)lo * sx];
-#pragma unroll 4
-  for (int i1 = lo; i1 < hi; ++i1) {
-    const size_t idx = base + (size_t)i1 * sx;
-    const bool more = i1 + 1 < a.N;
-    const float2 xp = Vin[more ? idx + sx : idx];
-    TvNbrs nb;
-    nb.h1p = xy && more;
-    nb.h1m = xy && i1 > 0;
-    nb.h2p = h2p;
-    nb.h2m = h2m;
-    nb.htp = htp;
-    nb.htm = htm;
-    nb.x1p = xp;
-    nb.x1m = xm;
-    nb.x2p = Vin[h2p ? idx + sy : idx];
-    nb.x2m = Vin[h2m ? idx - sy : idx];
-    if constexpr (TT) {
-      nb.tp = Vin[htp ? idx + st : idx];
-      nb.tm = Vin[htm ? idx - st : idx];
-    } else {
-      nb.tp = nb.tm = x;
+  // A voxel is one 32-bit byte offset into each array, from the frame before
+  // the unit's (its own when t = 0); the neighbouring rows and frames are
+  // fixed distances from it, 0 for a missing one (this voxel is read).
+  const size_t first = (size_t)(t > 0 ? t - 1 : 0) * st;
+  const float2* rx = Vin + first;
+  float2* rm = mom1 + first;
+  float2* rv = mom2 + first;
+  float2* ro = Vout + first;
+  const uint32_t sx = (uint32_t)a.Nf * 8u;
+  const uint32_t d2 = (uint32_t)sy * 8u, dt = (uint32_t)st * 8u;
+  const uint32_t d2p = h2p ? d2 : 0u, d2m = h2m ? d2 : 0u, dtp = htp ? dt : 0u, dtm = htm ? dt : 0u;
+  uint32_t off = (t > 0 ? dt : 0u) + (uint32_t)i2 * d2 + (uint32_t)lo * sx + (uint32_t)(fv ? f : a.Nf - 1) * 8u;
+  auto at = [](const float2* b, uint32_t o) {
+    return load_at(b, o);  // (Vin is not written by this kernel)
+  };
+  const float tv_xy = a.ad.tv_xy, tv_t = TT ? a.ad.tv_t : 0.f;
+  float2 x = at(rx, off);
+  // The TV term of the difference from the voxel before: it is that voxel's
+  // own term towards this one, computed once and handed on along the walk.
+  float mag;
+  float2 g1m = make_float2(0.f, 0.f);
+  if (xy && lo > 0) g1m = tv_term(csub_rn(x, at(rx, off - sx)), eps2, &mag);
+  for (int i0 = lo; i0 < hi; i0 += U, off += U * sx) {
+    // every load of U voxels before the first use of one
+    float2 xp[U], x2p[U], x2m[U], xtp[U], xtm[U], mm[U], vv[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t o = off + (uint32_t)min(u, hi - 1 - i0) * sx;
+      xp[u] = at(rx, min(i0 + u, hi - 1) + 1 < a.N ? o + sx : o);
+      x2p[u] = at(rx, o + d2p);
+      x2m[u] = at(rx, o - d2m);
+      if constexpr (TT) {
+        xtp[u] = at(rx, o + dtp);
+        xtm[u] = at(rx, o - dtm);
+      }
+      mm[u] = *reinterpret_cast<const float2*>(reinterpret_cast<const char*>(rm) + o);
+      vv[u] = *reinterpret_cast<const float2*>(reinterpret_cast<const char*>(rv) + o);
     }
-    float2 mm = mom1[idx], vv = mom2[idx];
-    float2* gp = gb + i1 * kFftCols + col;
-    const float2 gd = *gp;
-    float2 gxy, gt;
-    const float tv = voxel_tv_nb(x, nb, a.ad.tv_xy, TT ? a.ad.tv_t : 0.f, eps2, &gxy, &gt);
-    float2 nx = make_float2(0.f, 0.f);
-    if (fv) {
-      local = __fadd_rn(local, tv);
-      const float2 g = total_grad(gd, gxy, gt, a.ad);
-      nx = adam_voxel(x, g, mm, vv, a.ad);
-      mom1[idx] = mm;
-      mom2[idx] = vv;
-      Vout[idx] = nx;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i1 = i0 + u;
+      if (i1 >= hi) break;
+      const uint32_t o = off + (uint32_t)u * sx;
+      float2* gp = gb + i1 * kFftCols + col;
+      const float2 gd = *gp;
+      // voxel_tv_nb's terms in its order
+      float2 gxy = make_float2(0.f, 0.f), gt = make_float2(0.f, 0.f), g1p = make_float2(0.f, 0.f);
+      float sxy = 0.f, stt = 0.f;
+      if (xy) {
+        if (i1 + 1 < a.N) {
+          g1p = tv_term(csub_rn(xp[u], x), eps2, &mag);
+          gxy = csub_rn(gxy, g1p);
+          sxy = __fadd_rn(sxy, mag);
+        }
+        if (i1 > 0) gxy = cadd_rn(gxy, g1m);
+        if (h2p) {
+          gxy = csub_rn(gxy, tv_term(csub_rn(x2p[u], x), eps2, &mag));
+          sxy = __fadd_rn(sxy, mag);
+        }
+        if (h2m) gxy = cadd_rn(gxy, tv_term(csub_rn(x, x2m[u]), eps2, &mag));
+      }
+      if constexpr (TT) {
+        if (htp) {
+          gt = csub_rn(gt, tv_term(csub_rn(xtp[u], x), eps2, &mag));
+          stt = __fadd_rn(stt, mag);
+        }
+        if (htm) gt = cadd_rn(gt, tv_term(csub_rn(x, xtm[u]), eps2, &mag));
+      }
+      float2 nx = make_float2(0.f, 0.f);
+      if (fv) {
+        local = __fadd_rn(local, fmaf(tv_xy, sxy, __fmul_rn(tv_t, stt)));
+        const float2 g = total_grad(gd, gxy, gt, a.ad);
+        nx = adam_voxel(x, g, mm[u], vv[u], a.ad);
+        store_at(rm, o, mm[u]);
+        store_at(rv, o, vv[u]);
+        store_at(ro, o, nx);
+      }
+      *gp = nx;
+      g1m = g1p;
+      x = xp[u];
     }
-    *gp = nx;
-    xm = x;
-    x = xp;
   }
   return local;
 }
 
-__device__ __forceinline__ float update_row_any(const FusedArgs& a, float2* gb, size_t row, int i2, int t,
-                                                int fbase, int tid, int nthreads, float local) {
-  if (a.T > 1 && a.ad.tv_t != 0.f) return update_row<true>(a, gb, row, i2, t, fbase, tid, nthreads, local);
-  return update_row<false>(a, gb, row, i2, t, fbase, tid, nthreads, local);
+// UT, UP: voxels whose loads are issued together with and without time
+// neighbours, as many as the caller's registers hold.
+template <int UT, int UP>
+__device__ __forceinline__ float update_row_any(const FusedArgs& a, float2* gb, int i2, int t, int fbase, int tid,
+                                                int nthreads, float local) {
+  if (a.T > 1 && a.ad.tv_t != 0.f) return update_row<true, UT>(a, gb, i2, t, fbase, tid, nthreads, local);
+  return update_row<false, UP>(a, gb, i2, t, fbase, tid, nthreads, local);
 }
 
-// L2 prefetch of the update's operands for image row `row`: this row of V,
-// m and v, and the neighbouring rows the TV terms read.
-__device__ __forceinline__ void prefetch_update_rows(const FusedArgs& a, size_t row, int i2, int t) {
+// L2 prefetch of the update's Adam moments for image row `row`.  (The rows of
+// V are read by their neighbours' updates at about the same time; prefetching
+// them too cost more L2 requests than it hid: dynamic 375 against 369 us.)
+__device__ __forceinline__ void prefetch_update_rows(const FusedArgs& a, size_t row) {
   const size_t rl = (size_t)a.N * a.Nf;
   const uint32_t rb = (uint32_t)(rl * sizeof(float2));
-  prefetch_l2(a.Vin + row * rl, rb);
   prefetch_l2(a.m + row * rl, rb);
   prefetch_l2(a.v + row * rl, rb);
-  if (a.ad.tv_xy != 0.f) {
-    if (i2 + 1 < a.N) prefetch_l2(a.Vin + (row + 1) * rl, rb);
-    if (i2 > 0) prefetch_l2(a.Vin + (row - 1) * rl, rb);
-  }
-  if (a.ad.tv_t != 0.f) {
-    if (t + 1 < a.T) prefetch_l2(a.Vin + (row + a.N) * rl, rb);
-    if (t > 0) prefetch_l2(a.Vin + (row - a.N) * rl, rb);
-  }
 }
 
 // Register cap: 64 a thread (two CTAs of 512 threads per SM).
@@ -808,7 +844,7 @@ __device__ __forceinline__ void fused_rows_body(const FusedArgs& a, int bx, size
   grid_dep_wait();
   grid_dep_release();
   // the update's operands stream into L2 while the inverse FFT runs
-  if (threadIdx.x == 0) prefetch_update_rows(a, row, i2, t);
+  if (threadIdx.x == 0) prefetch_update_rows(a, row);
   __syncthreads();
   const int col = threadIdx.x % kFftCols;
   const int tl = line_thread<NFFT, EV>(threadIdx.x);
@@ -821,7 +857,7 @@ __device__ __forceinline__ void fused_rows_body(const FusedArgs& a, int bx, size
     fft_pass<NFFT, EV, +1, 0, 1, false, true>(X, tw, col, tl, in, out);
   }
   __syncthreads();
-  const float local = update_row_any(a, gb, row, i2, t, fbase, threadIdx.x, blockDim.x, 0.f);
+  const float local = update_row_any<2, 2>(a, gb, i2, t, fbase, threadIdx.x, blockDim.x, 0.f);
   if constexpr (FWD_TAIL) {
     __syncthreads();
     InNewRow in{gb, a.deapod, a.deapod[i2]};
@@ -966,7 +1002,15 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsFused<NFFT>>::THREADS + kUpdT
   }
   __syncthreads();
   float local = 0.f;
+  // The update's loads in flight are what its registers hold, so it takes
+  // part of the transform group's (whole warpgroups; the shares of both
+  // groups add up to the launch's 64 a thread): 80 a thread hold three
+  // voxels' loads with time neighbours where 64 spilled at two.  Together
+  // with those loads issued at once: dynamic 445 -> 370 us.
+  constexpr bool SPLIT = FT == kUpdThreads;
+  constexpr int FREG = EV == 12 ? 48 : 56;  // configure_n checks the launch's registers
   if (threadIdx.x < FT) {
+    if constexpr (SPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(FREG));
     const int col = threadIdx.x % kFftCols;
     const int tl = line_thread<NFFT, EV>(threadIdx.x);
     for (int i = 0; i <= nu; ++i) {
@@ -1009,10 +1053,10 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsFused<NFFT>>::THREADS + kUpdT
       }
     }
   } else {
+    if constexpr (SPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(128 - FREG));
     const int ut = threadIdx.x - FT;
     if (ut == 0 && nu > 0) {
-      const size_t row = (size_t)(blockIdx.x / a.nfb);
-      prefetch_update_rows(a, row, (int)(row % a.N), (int)(row / a.N));
+      prefetch_update_rows(a, (size_t)(blockIdx.x / a.nfb));
     }
     for (int i = 0; i < nu; ++i) {
       const int u = (int)blockIdx.x + i * (int)gridDim.x;
@@ -1021,12 +1065,12 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsFused<NFFT>>::THREADS + kUpdT
       const int i2 = (int)(row % a.N), t = (int)(row / a.N);
       if (ut == 0 && i + 1 < nu) {
         const size_t nrow = (size_t)((u + (int)gridDim.x) / a.nfb);
-        if (nrow != row) prefetch_update_rows(a, nrow, (int)(nrow % a.N), (int)(nrow / a.N));
+        if (nrow != row) prefetch_update_rows(a, nrow);
       }
       if (!mbar_wait_bounded(&ready[i & 1], (uint32_t)((i >> 1) & 1))) s_abort_u = 1;
       USync::sync();
       if (s_abort_u) break;
-      local = update_row_any(a, gbuf + (size_t)(i & 1) * gsz, row, i2, t, fbase, ut, kUpdThreads, local);
+      local = update_row_any<3, 2>(a, gbuf + (size_t)(i & 1) * gsz, i2, t, fbase, ut, kUpdThreads, local);
       mbar_arrive(&done[i & 1]);
     }
   }
@@ -1274,6 +1318,14 @@ cudaError_t configure_n() {
     return e;
   if constexpr (fused_ws_fits<NFFT>()) {
     if (fused_ws_smem<NFFT>() <= (size_t)optin - 1024) {
+      if (Shape<NFFT, kValsFused<NFFT>>::THREADS == kUpdThreads) {
+        // the register split of the two groups takes 64 a thread of the launch
+        // and would wait forever for registers that it does not have
+        cudaFuncAttributes fa, fb;
+        if ((e = cudaFuncGetAttributes(&fa, fused_rows_ws_kernel<NFFT, true>))) return e;
+        if ((e = cudaFuncGetAttributes(&fb, fused_rows_ws_kernel<NFFT, false>))) return e;
+        if (fa.numRegs < 64 || fb.numRegs < 64) return cudaErrorInvalidConfiguration;
+      }
       const int wsm = (int)fused_ws_smem<NFFT>();
       if ((e = cudaFuncSetAttribute(fused_rows_ws_kernel<NFFT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     wsm)))
