@@ -6,11 +6,12 @@
 // i.e. the W x W-tap Kaiser-Bessel interpolation of every bin's grid, times
 // the displacement phase exp(-2 pi i k_r Delta_f) (Sec. 3: a material
 // displaced along the readout picks up a phase linear in k_r), summed over
-// the bins.  Samples are processed in tile-sorted work items; a persistent
-// CTA per SM streams each item's grid tile plus halo into shared memory with
-// TMA bulk copies (double-buffered, completion on an mbarrier) while it
-// computes the previous item.  Bins are the fastest axis, so the lanes that
-// serve one sample read consecutive bins of a cell (conflict-free).
+// the bins.  A persistent CTA per SM streams the grid rows it needs into shared
+// memory with TMA bulk copies (completion on mbarriers) ahead of its compute
+// warps, which take a blade's samples four at a time (quads_kernel; a sample
+// at a time over staged tiles for other bin strides).  Bins are the fastest
+// axis, so the lanes that serve a sample read consecutive bins of a cell
+// (conflict-free).
 //
 // Adjoint: G'_{t,f}[cell] = sum_m w(m, cell) conj(P[j_m][f]) r_m.  The
 // phased residual contrib[m][f] = conj(P[j_m][f]) r_m is formed once per
@@ -49,7 +50,6 @@ struct InterpArgs {
   unsigned int* counter;
   double* sumsq_out;
   int* err;  // set to 1 when a bounded wait expires
-  const int* cta_off;  // CTA c takes items [cta_off[c], cta_off[c + 1]) (balanced at plan time)
   int n_items, R, n, C, Cv, f0, Nf;
   int TR, TC, nct, tpf, nbuf;  // tile rows, cells per row, tiles per row of tiles and per frame
   float scale;
@@ -141,23 +141,20 @@ __device__ void issue_tile(const InterpArgs& a, int item, float2* dst, uint64_t*
   }
 }
 
-// CS > 0: the bin stride C is the compile-time CS (so every shared-memory and
-// tap offset folds into an immediate); CS == 0: runtime stride.  LP lanes
-// serve one sample, each lane a bin f = sub + LP q.
-template <int LP, int CS, int W>
+// Run-time bin stride (the strides without a quad kernel).  LP lanes serve one
+// sample, each lane a bin f = sub + LP q.
+template <int LP, int W>
 __global__ void __launch_bounds__(kInterpThreads, 1) interp_kernel(InterpArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   constexpr int SPW = 32 / LP;
   constexpr int WQ = W / 2;                           // float4 of weights per sample
-  constexpr int QB = CS > 0 ? (CS + LP - 1) / LP : 0;  // bins per lane (compile-time case)
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int nwarp = blockDim.x >> 5;
   const int sub = lane & (LP - 1);
   const int slot = lane / LP;
-  const int C = CS > 0 ? CS : a.C;
-  const int HR = (CS > 0 ? interp_tile_rows(CS, W) : a.TR) + W - 1;
-  const int HC = (CS > 0 ? interp_tile_cols(CS, W) : a.TC) + W - 1;
+  const int C = a.C;
+  const int HR = a.TR + W - 1, HC = a.TC + W - 1;
   const size_t tile_elems = (size_t)HR * HC * C;
   float2* bufs = reinterpret_cast<float2*>(smem_raw);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + a.nbuf * tile_elems * sizeof(float2));
@@ -224,8 +221,7 @@ __global__ void __launch_bounds__(kInterpThreads, 1) interp_kernel(InterpArgs a)
         const int lc = (int)(packed & 0xffff) - g.c0;  // the first tap lies in the tile
         const int lr = (int)(packed >> 16) - g.r0;
         const float2* base = tile + ((size_t)lr * HC + lc) * C + sub;
-        // W independent row sums (x1 weights), then the x2 weights; with a
-        // compile-time stride every offset below is an immediate.
+        // W independent row sums (x1 weights), then the x2 weights
         auto tap_sum = [&](const float2* p) {
           float2 racc[W];
 #pragma unroll
@@ -246,22 +242,10 @@ __global__ void __launch_bounds__(kInterpThreads, 1) interp_kernel(InterpArgs a)
           }
           return acc;
         };
-        if constexpr (CS > 0) {
-#pragma unroll
-          for (int qb = 0; qb < QB; ++qb) {
-            const int f = sub + LP * qb;
-            if (f < a.Cv) {
-              const float2 z = cmulf(__ldg(P + f), tap_sum(base + LP * qb));
-              tot.x += z.x;
-              tot.y += z.y;
-            }
-          }
-        } else {
-          for (int f = sub; f < a.Cv; f += LP) {
-            const float2 z = cmulf(__ldg(P + f), tap_sum(base + (f - sub)));
-            tot.x += z.x;
-            tot.y += z.y;
-          }
+        for (int f = sub; f < a.Cv; f += LP) {
+          const float2 z = cmulf(__ldg(P + f), tap_sum(base + (f - sub)));
+          tot.x += z.x;
+          tot.y += z.y;
         }
       }
 #pragma unroll
@@ -310,42 +294,65 @@ __global__ void __launch_bounds__(kInterpThreads, 1) interp_kernel(InterpArgs a)
   if (a.partials) reduce_to((double)sumsq, a.partials, a.counter, a.sumsq_out);
 }
 
-constexpr int kInterpConsumers = 16;                          // compute warps per CTA
-constexpr int kInterp2Threads = 32 * (kInterpConsumers + 1);  // plus one producer warp
+struct QuadArgs {
+  const float2* grid;
+  const float4* quads;
+  const int4* items;
+  const float2* phase;
+  float2* y;
+  const float2* y_meas;
+  float2* contrib;  // non-null: also write conj(P) * final value per bin
+  double* partials;
+  unsigned int* counter;
+  double* sumsq_out;
+  int* err;  // set to 1 when a bounded wait expires
+  const int* cta_off;  // CTA c takes items [cta_off[c], cta_off[c + 1])
+  int n, Cv, f0, Nf;
+  float scale;
+  int accumulate;
+};
 
-// Interpolation for the compile-time bin strides CS in {8, 16, 32, 64}.
-// Warp kInterpConsumers is the producer: its lane 0 streams item k's tile
-// into buffer k % nbuf as soon as every compute warp has released the item
-// that last used that buffer ("empty" barrier, one arrival per compute
-// warp), so no compute warp ever waits for another.  Compute warps take
-// CS / 2 lanes per sample, each lane two adjacent bins (16-byte shared
-// loads), and 64 / CS samples per warp and round.  The metadata of an item
-// (sample index, packed first tap, the 2W weights) is fetched before its
-// tile is awaited, one sample per lane, and handed out by shuffles.
-// The work of one persistent CTA: items [it_beg, it_end); vb, vg: the CTA's
-// index and the CTA count of the |r|^2 reduction.
+// Interpolation for the bin strides CS in {8, 16, 32, 64}, four samples of a
+// blade at a time.
+//
+// What bounds it: with a sample per lane group every tap of every sample is a
+// shared-memory read (width 8, 32 bins: 14.3 M wavefronts a launch, 45.6 us at
+// one a clock and SM, and 68 us measured at the static configuration).  The
+// four samples of a quad share a window of at most (W + 3)^2 cells: a lane
+// (one bin, two at CS = 64) reads each cell once and multiplies it with four
+// x1 weights, held in registers and zero outside a sample's footprint, so the
+// wavefronts fall to 7.3 M for 1.9 times the multiply-adds (1470 instructions
+// a quad and warp at width 8, 29 us of issue; it runs at 58 % of that rate,
+// the SMs' loads within 15 % of each other).  A window's last row and column
+// are left out where no footprint meets them.  Each sample still sums its own
+// taps in the order a lone one would (x1 within a row, then the rows; the
+// zero weights add exact zeros).  Measured against a sample at a time: static
+// 68 -> 62.5 us, dynamic (16 bins) 112 -> 96 us, 2N = 1024 in 16-bin chunks at
+// width 6 89 -> 71 us, 384^2 x 64 bins 283 -> 262 us.
+//
+// The grid rows come from a ring in shared memory: a CTA's items walk down
+// strips of quad_cols(CS) columns, the producer warp's lane 0 bulk-copies the
+// rows that an item adds to those of the item before it into the next slots,
+// each as soon as every item that read the slot's old row is released, and
+// the items' quad records into kQuadStages stages.  A warp takes at most one
+// unit (a quad, or 32 / CS of them) of an item, the units going round the
+// warps across item borders; no compute warp waits for another.
 template <int CS, int W>
-__device__ __forceinline__ void interp2_body(const InterpArgs& a, int it_beg, int it_end, unsigned vb, unsigned vg) {
+__device__ __forceinline__ void quads_body(const QuadArgs& a, int it_beg, int it_end, unsigned vb, unsigned vg) {
+  using S = QuadShape<CS, W>;
+  constexpr int NCW = kQuadWarps, NS = kQuadStages, UW = S::UW, NR = S::NR;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  constexpr int NCW = kInterpConsumers;
-  constexpr int LPS = CS / 2;   // lanes per sample
-  constexpr int SPW = 32 / LPS; // samples per warp and round
-  constexpr int HR = interp_tile_rows(CS, W) + W - 1;  // staged rows
-  constexpr int HC = interp_tile_cols(CS, W) + W - 1;  // staged cells per row
-  constexpr int WQ = W / 2;
-  constexpr int MPL = (kInterpItem + NCW * SPW - 1) / (NCW * SPW) * SPW;  // samples per warp per item
-  static_assert(MPL <= 32, "one prefetched sample per lane");
-  constexpr size_t tile_elems = (size_t)HR * HC * CS;
-  const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const int sub = lane % LPS;
-  const int slot = lane / LPS;
-  float2* bufs = reinterpret_cast<float2*>(smem_raw);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + a.nbuf * tile_elems * sizeof(float2));
-  uint64_t* empty = full + a.nbuf;
+  unsigned char* ring = smem_raw;
+  constexpr int STAGE = quad_stage_bytes(CS, W);
+  float4* stages = reinterpret_cast<float4*>(smem_raw + (size_t)NR * S::RB);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + (size_t)NR * S::RB + (size_t)NS * STAGE);
+  uint64_t* empty = full + NS;
   __shared__ volatile int s_abort;
+  __shared__ int s_first[NS];  // producer: number (in loading order) of the first row of the item in each stage
+  __shared__ int4 s_head[NS];  // (quads, ring slot of the first row, warp of the first quad) of the item in each stage
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
-    for (int b = 0; b < a.nbuf; ++b) {
+    for (int b = 0; b < NS; ++b) {
       mbar_init(&full[b], 1);
       mbar_init(&empty[b], NCW);
     }
@@ -356,123 +363,241 @@ __device__ __forceinline__ void interp2_body(const InterpArgs& a, int it_beg, in
   grid_dep_wait();
   grid_dep_release();
 
-  float sumsq = 0.f;
+  double sumsq = 0.0;
   if (warp == NCW) {
     if (lane == 0) {
-      int k = 0;
+      constexpr int TC = quad_cols(CS);
+      const int nstrip = (a.n + TC - 1) / TC;
+      const size_t nC = (size_t)a.n * CS;
+      int4 ahead = it_beg < it_end ? __ldg(&a.items[it_beg]) : make_int4(0, 0, 0, 0);
+      int k = 0, released = 0, loaded = 0, first = 0, warp0 = 0;
+      int strip = -1, row = 0, row_end = 0;  // of the item before
+      // waits until the items before `upto` are released
+      auto release = [&](int upto) {
+        while (released < upto) {
+          if (!mbar_wait_bounded(&empty[released % NS], (uint32_t)((released / NS) & 1))) return false;
+          ++released;
+        }
+        return true;
+      };
       for (int item = it_beg; item < it_end; ++item, ++k) {
-        const int b = k % a.nbuf;
-        if (k >= a.nbuf && !mbar_wait_bounded(&empty[b], (uint32_t)(((k / a.nbuf) - 1) & 1))) {
-          s_abort = 1;
+        const int4 it = ahead;
+        if (item + 1 < it_end) ahead = __ldg(&a.items[item + 1]);
+        const int r0 = it.w & 0xffff, rows = it.w >> 16;
+        if (!release(k - NS + 1)) s_abort = 1;  // the stage is free
+        if (s_abort) break;
+        int fresh = 0;  // the item's rows from here on are not in the ring
+        if (it.x == strip && r0 < row_end) {
+          first += r0 - row;
+          fresh = min(rows, row_end - r0);
+        } else {
+          first = loaded;
+        }
+        const int b = k % NS;
+        s_first[b] = first;
+        s_head[b] = make_int4(it.z, first % NR, warp0, 0);  // published by the barrier phase
+        warp0 = (warp0 + (it.z + S::QPW - 1) / S::QPW) % NCW;
+        const int t = it.x / nstrip, c0 = (it.x - t * nstrip) * TC;
+        const int cells = min(S::HC, a.n - c0 + UW - 1), run1 = min(cells, a.n - c0);
+        const uint32_t row_bytes = (uint32_t)(cells * CS * sizeof(float2));
+        const uint32_t rec_bytes = (uint32_t)(it.z * S::REC * sizeof(float4));
+        mbar_expect_tx(&full[b], rec_bytes + (uint32_t)(rows - fresh) * row_bytes);
+        bulk_g2s(stages + (size_t)b * S::ITEM * S::REC, a.quads + (size_t)it.y * S::REC, rec_bytes, &full[b]);
+        const float2* G = a.grid + (size_t)t * a.n * nC;
+        int slot = (first + fresh) % NR, i = fresh;
+        for (; i < rows; ++i) {
+          // the slot is free once the items that read its row before are released
+          int upto = released;
+          while (upto < k && s_first[upto % NS] + NR <= first + i) ++upto;
+          if (!release(upto)) {
+            s_abort = 1;
+            break;
+          }
+          int gr = r0 + i;
+          gr = gr >= a.n ? gr - a.n : gr;
+          unsigned char* d = ring + (size_t)slot * S::RB;
+          bulk_g2s(d, G + (size_t)gr * nC + (size_t)c0 * CS, (uint32_t)(run1 * CS * sizeof(float2)), &full[b]);
+          if (run1 < cells)
+            bulk_g2s(d + (size_t)run1 * CS * sizeof(float2), G + (size_t)gr * nC,
+                     (uint32_t)((cells - run1) * CS * sizeof(float2)), &full[b]);
+          slot = slot + 1 == NR ? 0 : slot + 1;
+        }
+        if (s_abort) {
+          // this item's phase will never complete: its copies were issued to
+          // the same barrier, so let it by making up the missing bytes
+          for (; i < rows; ++i) mbar_complete_tx(&full[b], row_bytes);
+          ++k;
           break;
         }
-        if (s_abort) break;
-        issue_tile<W>(a, item, bufs + b * tile_elems, &full[b]);
+        loaded = max(loaded, first + rows);
+        strip = it.x;
+        row = r0;
+        row_end = max(fresh > 0 ? row_end : 0, r0 + rows);
       }
-      // at most one copy per buffer can be in flight: the last one issued
-      for (int kk = k > a.nbuf ? k - a.nbuf : 0; kk < k; ++kk)
-        mbar_wait_bounded(&full[kk % a.nbuf], (uint32_t)((kk / a.nbuf) & 1));
+      // the copies still in flight: at most the last NS items'
+      for (int kk = k > NS ? k - NS : 0; kk < k; ++kk) mbar_wait_bounded(&full[kk % NS], (uint32_t)((kk / NS) & 1));
     }
   } else {
-    const int f_lo = 2 * sub;
-    const bool b0 = f_lo < a.Cv, b1 = f_lo + 1 < a.Cv;
+    const int sub = lane % S::LPQ, slotq = lane / S::LPQ;
+    const int f = sub * S::BPL;
+    // The sum over the bins: adjacent bins first, then halves.  The first
+    // three steps also halve what a lane holds of the quad's 4 complex values,
+    // so that it ends up with component (h1 h2 | h3) of sample 2 h1 + h2.
+    constexpr int O1 = S::BPL == 1 ? 1 : S::LPQ / 2;
+    constexpr int O2 = S::BPL == 1 ? S::LPQ / 2 : S::LPQ / 4;
+    constexpr int O3 = O2 / 2;
+    constexpr int OEND = S::BPL == 1 ? 2 : 1;  // last step
+    const int h1 = (lane & O1) ? 1 : 0, h2 = (lane & O2) ? 1 : 0, h3 = (lane & O3) ? 1 : 0;
+    const int mine = 2 * h1 + h2;
+    const bool owner = (sub & ~(O1 | O2 | O3)) == 0;
     int k = 0;
     for (int item = it_beg; item < it_end; ++item, ++k) {
-      const int b = k % a.nbuf;
-      const ItemGeom g = item_geom(a, item);
-      // lane L prefetches the warp's sample of round L / SPW, slot L % SPW
-      const int sL = (lane / SPW) * NCW * SPW + warp * SPW + (lane % SPW);
-      int mL = 0, jL = 0;
-      uint32_t pL = 0;
-      float2 yL = make_float2(0.f, 0.f);  // the measurement (or the partial sum so far) of the sample
-      float wL[2 * W];
-#pragma unroll
-      for (int q = 0; q < 2 * W; ++q) wL[q] = 0.f;
-      if (lane < MPL && sL < g.count) {
-        const int si = g.start + sL;
-        mL = __ldg(&a.order[si]);
-        pL = __ldg(&a.kb_idx[si]);
-#pragma unroll
-        for (int q = 0; q < WQ; ++q) {
-          const float4 v = __ldg(&a.kb_w[(size_t)WQ * si + q]);
-          wL[4 * q] = v.x;
-          wL[4 * q + 1] = v.y;
-          wL[4 * q + 2] = v.z;
-          wL[4 * q + 3] = v.w;
-        }
-        jL = mL % a.R;
-        if (a.accumulate)
-          yL = a.y[mL];
-        else if (a.y_meas)
-          yL = __ldg(&a.y_meas[mL]);
-      }
-      if (!mbar_wait_bounded(&full[b], (uint32_t)((k / a.nbuf) & 1))) s_abort = 1;
+      const int b = k % NS;
+      if (!mbar_wait_bounded(&full[b], (uint32_t)((k / NS) & 1))) s_abort = 1;
       if (s_abort) break;
-      const float2* tile = bufs + b * tile_elems;
-
-      for (int rnd = 0; rnd * NCW * SPW + warp * SPW < g.count; ++rnd) {
-        const int s = rnd * NCW * SPW + warp * SPW + slot;
-        const bool valid = s < g.count;
-        const int src = rnd * SPW + slot;
-        const int m = __shfl_sync(0xffffffffu, mL, src);
-        const int j = __shfl_sync(0xffffffffu, jL, src);
-        const uint32_t packed = __shfl_sync(0xffffffffu, pL, src);
-        const float2 yprev = make_float2(__shfl_sync(0xffffffffu, yL.x, src), __shfl_sync(0xffffffffu, yL.y, src));
-        float w[2 * W];
+      const int4 head = s_head[b];
+      int u = warp - head.z;
+      u = u < 0 ? u + NCW : u;
+      if (u * S::QPW < head.x) {
+        const int qi = u * S::QPW + slotq;
+        const bool live = qi < head.x;
+        const float4* rec = stages + ((size_t)b * S::ITEM + (live ? qi : head.x - 1)) * S::REC;
+        const int4 mm = *reinterpret_cast<const int4*>(rec + 2 * UW);
+        const int4 pos = *reinterpret_cast<const int4*>(rec + 2 * UW + 1);
+        const int m_mine = mine == 0 ? mm.x : mine == 1 ? mm.y : mine == 2 ? mm.z : mm.w;
+        const bool write = live && owner && m_mine >= 0;
+        float yprev = 0.f;  // the measurement (or the partial sum so far) of the lane's component
+        if (write) {
+          if (a.accumulate)
+            yprev = reinterpret_cast<const float*>(a.y)[2 * (size_t)m_mine + h3];
+          else if (a.y_meas)
+            yprev = __ldg(reinterpret_cast<const float*>(a.y_meas) + 2 * (size_t)m_mine + h3);
+        }
+        // displacement phases of the two readout positions (the second may not exist: then unused)
+        const bool two = mm.y >= 0;
+        float2 P[2][S::BPL];
 #pragma unroll
-        for (int q = 0; q < 2 * W; ++q) w[q] = __shfl_sync(0xffffffffu, wL[q], src);
-        const float2* P = a.phase + (size_t)j * a.Nf + a.f0 + f_lo;
-        float2 P0 = make_float2(0.f, 0.f), P1 = make_float2(0.f, 0.f);
-        if (valid && b0) P0 = __ldg(P);
-        if (valid && b1) P1 = __ldg(P + 1);
-        float2 tot = make_float2(0.f, 0.f);
-        if (valid) {
-          const int lc = (int)(packed & 0xffff) - g.c0;
-          const int lr = (int)(packed >> 16) - g.r0;
-          const float4* base = reinterpret_cast<const float4*>(tile + ((size_t)lr * HC + lc) * CS + f_lo);
-          // row sums over the x1 taps, folded into the x2 sum row by row
-          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < S::BPL; ++i) {
+          const bool on = f + i < a.Cv;
+          const float2* ph = a.phase + (size_t)pos.z * a.Nf + a.f0 + f + i;
+          P[0][i] = on ? __ldg(ph) : make_float2(0.f, 0.f);
+          P[1][i] = on && two ? __ldg(ph + a.Nf) : make_float2(0.f, 0.f);
+        }
+        float4 w1[UW];
 #pragma unroll
-          for (int q = 0; q < W; ++q) {
-            float4 rs = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < UW; ++c) w1[c] = rec[c];
+        const bool last_row = (pos.w & 0xff) == UW;
+        const bool last_col = (pos.w >> 8) == UW;
+        int slot = head.y + pos.x;
+        slot = slot >= NR ? slot - NR : slot;
+        // the lane's bins of the window's first cell in the current row (32-bit
+        // shared-memory offsets; the ring's rows follow one another)
+        const unsigned char* p = ring + (size_t)slot * S::RB + (size_t)(pos.y * CS + f) * sizeof(float2);
+        const unsigned char* const wrap = ring + (size_t)NR * S::RB;
+        float2 acc[4][S::BPL];
 #pragma unroll
-            for (int c = 0; c < W; ++c) {
-              const float4 gv = base[(q * HC + c) * (CS / 2)];
-              rs.x = fmaf(w[c], gv.x, rs.x);
-              rs.y = fmaf(w[c], gv.y, rs.y);
-              rs.z = fmaf(w[c], gv.z, rs.z);
-              rs.w = fmaf(w[c], gv.w, rs.w);
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+          for (int i = 0; i < S::BPL; ++i) acc[s][i] = make_float2(0.f, 0.f);
+        auto row_of = [&](int r) {
+          const float4 w2 = rec[UW + r];
+          float2 rs[4][S::BPL];
+#pragma unroll
+          for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int i = 0; i < S::BPL; ++i) rs[s][i] = make_float2(0.f, 0.f);
+          auto cell = [&](int c) {
+            float2 g[S::BPL];
+            if constexpr (S::BPL == 2) {
+              const float4 v = *reinterpret_cast<const float4*>(p + c * CS * (int)sizeof(float2));
+              g[0] = make_float2(v.x, v.y);
+              g[1] = make_float2(v.z, v.w);
+            } else {
+              g[0] = *reinterpret_cast<const float2*>(p + c * CS * (int)sizeof(float2));
             }
-            acc.x = fmaf(w[W + q], rs.x, acc.x);
-            acc.y = fmaf(w[W + q], rs.y, acc.y);
-            acc.z = fmaf(w[W + q], rs.z, acc.z);
-            acc.w = fmaf(w[W + q], rs.w, acc.w);
-          }
-          const float2 z0 = cmulf(P0, make_float2(acc.x, acc.y));
-          const float2 z1 = cmulf(P1, make_float2(acc.z, acc.w));
-          tot = make_float2(z0.x + z1.x, z0.y + z1.y);
-        }
+            const float w[4] = {w1[c].x, w1[c].y, w1[c].z, w1[c].w};
 #pragma unroll
-        for (int o = LPS / 2; o > 0; o >>= 1) {
-          tot.x += __shfl_xor_sync(0xffffffffu, tot.x, o);
-          tot.y += __shfl_xor_sync(0xffffffffu, tot.y, o);
+            for (int s = 0; s < 4; ++s)
+#pragma unroll
+              for (int i = 0; i < S::BPL; ++i) {
+                rs[s][i].x = fmaf(w[s], g[i].x, rs[s][i].x);
+                rs[s][i].y = fmaf(w[s], g[i].y, rs[s][i].y);
+              }
+          };
+#pragma unroll
+          for (int c = 0; c < UW - 1; ++c) cell(c);
+          if (last_col) cell(UW - 1);
+          const float w[4] = {w2.x, w2.y, w2.z, w2.w};
+#pragma unroll
+          for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int i = 0; i < S::BPL; ++i) {
+              acc[s][i].x = fmaf(w[s], rs[s][i].x, acc[s][i].x);
+              acc[s][i].y = fmaf(w[s], rs[s][i].y, acc[s][i].y);
+            }
+          p += S::RB;
+          if (p >= wrap) p -= (size_t)NR * S::RB;
+        };
+        // (an item's rows reach to the end of its last quad's whole window)
+#pragma unroll
+        for (int r = 0; r < UW - 1; ++r) row_of(r);
+        if (last_row) row_of(UW - 1);
+        __syncwarp();
+        float v[8];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          float2 z = cmulf(P[s & 1][0], acc[s][0]);
+          if constexpr (S::BPL == 2) {
+            const float2 z1 = cmulf(P[s & 1][1], acc[s][1]);
+            z.x += z1.x;
+            z.y += z1.y;
+          }
+          v[2 * s] = z.x;
+          v[2 * s + 1] = z.y;
         }
-        float2 v = make_float2(tot.x * a.scale, tot.y * a.scale);
-        if (a.accumulate) {
-          v.x += yprev.x;
-          v.y += yprev.y;
-        } else if (a.y_meas) {
-          v.x -= yprev.x;
-          v.y -= yprev.y;
+        auto halve = [&](int count, int h, int o) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (i < count) {
+              const float give = h ? v[i] : v[i + count], keep = h ? v[i + count] : v[i];
+              v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+        };
+        halve(4, h1, O1);
+        halve(2, h2, O2);
+        halve(1, h3, O3);
+#pragma unroll
+        for (int o = O3 / 2; o >= OEND; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        float out = __fmul_rn(v[0], a.scale);
+        if (a.accumulate)
+          out = __fadd_rn(out, yprev);
+        else if (a.y_meas)
+          out = __fsub_rn(out, yprev);
+        if (write) {
+          reinterpret_cast<float*>(a.y)[2 * (size_t)m_mine + h3] = out;
+          sumsq += (double)out * out;
         }
-        if (valid && sub == 0) {
-          a.y[m] = v;
-          sumsq = fmaf(v.x, v.x, fmaf(v.y, v.y, sumsq));
-        }
-        if (a.contrib && valid) {
-          // every lane of the sample holds the same reduced value
-          const float2 c0 = cmulcf(P0, v), c1 = cmulcf(P1, v);
-          reinterpret_cast<float4*>(a.contrib + (size_t)m * CS)[sub] = make_float4(c0.x, c0.y, c1.x, c1.y);
+        if (a.contrib) {
+          // every lane gets the four values and phases them for its bins
+          const int base = lane & ~(S::LPQ - 1);
+#pragma unroll
+          for (int s = 0; s < 4; ++s) {
+            const int from = base + ((s & 2) ? O1 : 0) + ((s & 1) ? O2 : 0);
+            float2 val;
+            val.x = __shfl_sync(0xffffffffu, out, from);
+            val.y = __shfl_sync(0xffffffffu, out, from + O3);
+            const int m = s == 0 ? mm.x : s == 1 ? mm.y : s == 2 ? mm.z : mm.w;
+            if (live && m >= 0) {
+              float2* to = a.contrib + (size_t)m * CS + f;
+              const float2 c0 = cmulcf(P[s & 1][0], val);
+              if constexpr (S::BPL == 2) {
+                const float2 c1 = cmulcf(P[s & 1][1], val);
+                *reinterpret_cast<float4*>(to) = make_float4(c0.x, c0.y, c1.x, c1.y);
+              } else {
+                *to = c0;
+              }
+            }
+          }
         }
       }
       __syncwarp();
@@ -481,17 +606,17 @@ __device__ __forceinline__ void interp2_body(const InterpArgs& a, int it_beg, in
   }
   __syncthreads();
   if (s_abort && threadIdx.x == 0) atomicExch(a.err, 1);
-  if (a.partials) reduce_to_v((double)sumsq, a.partials, a.counter, a.sumsq_out, vb, vg);
+  if (a.partials) reduce_to_v(sumsq, a.partials, a.counter, a.sumsq_out, vb, vg);
 }
 
 template <int CS, int W>
-__global__ void __launch_bounds__(kInterp2Threads, 1) interp2_kernel(InterpArgs a) {
-  interp2_body<CS, W>(a, a.cta_off[blockIdx.x], a.cta_off[blockIdx.x + 1], blockIdx.x, gridDim.x);
+__global__ void __launch_bounds__(QuadShape<CS, W>::THREADS, 1) quads_kernel(QuadArgs a) {
+  quads_body<CS, W>(a, a.cta_off[blockIdx.x], a.cta_off[blockIdx.x + 1], blockIdx.x, gridDim.x);
 }
 
 // Kernel parameter of the interpolation over a batch of problems.
-struct MultiInterp {
-  InterpArgs a[kMaxBatch];
+struct MultiQuads {
+  QuadArgs a[kMaxBatch];
   int plan_ctas[kMaxBatch];      // CTAs each problem's items were balanced over
   int nreq;
   int cta_begin[kMaxBatch + 1];  // CTA ranges of the problems
@@ -503,13 +628,13 @@ struct MultiInterp {
 // problem's plan balanced over its CTAs v P / c .. (v + 1) P / c - 1, so every
 // sample is computed as in the problem's own launch.
 template <int CS, int W>
-__global__ void __launch_bounds__(kInterp2Threads, 1) interp2_multi_kernel(const __grid_constant__ MultiInterp m) {
+__global__ void __launch_bounds__(QuadShape<CS, W>::THREADS, 1) quads_multi_kernel(const __grid_constant__ MultiQuads m) {
   int r = 0;
   while (r + 1 < m.nreq && (int)blockIdx.x >= m.cta_begin[r + 1]) ++r;
   const int v = (int)blockIdx.x - m.cta_begin[r], c = m.cta_begin[r + 1] - m.cta_begin[r];
   const int P = m.plan_ctas[r];
-  const InterpArgs& a = m.a[r];
-  interp2_body<CS, W>(a, a.cta_off[(long)v * P / c], a.cta_off[(long)(v + 1) * P / c], (unsigned)v, (unsigned)c);
+  const QuadArgs& a = m.a[r];
+  quads_body<CS, W>(a, a.cta_off[(long)v * P / c], a.cta_off[(long)(v + 1) * P / c], (unsigned)v, (unsigned)c);
 }
 
 // contrib[m][f] = conj(P[j_m][f0 + f]) r_m, LP lanes per sample.
@@ -983,31 +1108,41 @@ unsigned grid_for(long items, long per_block, long cap) {
   return (unsigned)std::max<long>(1, std::min(b, cap));
 }
 
-bool interp2_eligible(int cs, int nbins) {
-  return (cs == 8 || cs == 16 || cs == 32 || cs == 64) && 2 * nbins > cs;
+template <int W>
+cudaError_t launch_interp(int lp, const InterpArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
+  switch (lp) {
+    case 1: interp_kernel<1, W><<<grid, kInterpThreads, smem, s>>>(a); break;
+    case 2: interp_kernel<2, W><<<grid, kInterpThreads, smem, s>>>(a); break;
+    case 4: interp_kernel<4, W><<<grid, kInterpThreads, smem, s>>>(a); break;
+    case 8: interp_kernel<8, W><<<grid, kInterpThreads, smem, s>>>(a); break;
+    case 16: interp_kernel<16, W><<<grid, kInterpThreads, smem, s>>>(a); break;
+    default: interp_kernel<32, W><<<grid, kInterpThreads, smem, s>>>(a); break;
+  }
+  return cudaGetLastError();
 }
 
 template <int W>
-cudaError_t launch_interp(int lp, int cs, const InterpArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
-  // compile-time strides for the common chunk widths when more than half of
-  // the bins are live (two bins per lane), runtime stride otherwise
-  if (interp2_eligible(cs, a.Cv)) {
-    const dim3 block(kInterp2Threads);
-    if (cs == 32) return launch_dep(interp2_kernel<32, W>, grid, block, smem, s, a);
-    if (cs == 64) return launch_dep(interp2_kernel<64, W>, grid, block, smem, s, a);
-    if (cs == 16) return launch_dep(interp2_kernel<16, W>, grid, block, smem, s, a);
-    return launch_dep(interp2_kernel<8, W>, grid, block, smem, s, a);
-  } else {
-    switch (lp) {
-      case 1: interp_kernel<1, 0, W><<<grid, kInterpThreads, smem, s>>>(a); break;
-      case 2: interp_kernel<2, 0, W><<<grid, kInterpThreads, smem, s>>>(a); break;
-      case 4: interp_kernel<4, 0, W><<<grid, kInterpThreads, smem, s>>>(a); break;
-      case 8: interp_kernel<8, 0, W><<<grid, kInterpThreads, smem, s>>>(a); break;
-      case 16: interp_kernel<16, 0, W><<<grid, kInterpThreads, smem, s>>>(a); break;
-      default: interp_kernel<32, 0, W><<<grid, kInterpThreads, smem, s>>>(a); break;
-    }
+cudaError_t launch_quads(int cs, const QuadArgs& a, int ctas, cudaStream_t s) {
+  const dim3 grid((unsigned)ctas);
+  switch (cs) {
+    case 8: return launch_dep(quads_kernel<8, W>, grid, dim3(QuadShape<8, W>::THREADS), QuadShape<8, W>::SMEM, s, a);
+    case 16: return launch_dep(quads_kernel<16, W>, grid, dim3(QuadShape<16, W>::THREADS), QuadShape<16, W>::SMEM, s, a);
+    case 32: return launch_dep(quads_kernel<32, W>, grid, dim3(QuadShape<32, W>::THREADS), QuadShape<32, W>::SMEM, s, a);
+    case 64: return launch_dep(quads_kernel<64, W>, grid, dim3(QuadShape<64, W>::THREADS), QuadShape<64, W>::SMEM, s, a);
+    default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
+}
+
+template <int W>
+cudaError_t launch_quads_multi(int cs, const MultiQuads& m, int ctas, cudaStream_t s) {
+  const dim3 grid((unsigned)ctas);
+  switch (cs) {
+    case 8: return launch_dep(quads_multi_kernel<8, W>, grid, dim3(QuadShape<8, W>::THREADS), QuadShape<8, W>::SMEM, s, m);
+    case 16: return launch_dep(quads_multi_kernel<16, W>, grid, dim3(QuadShape<16, W>::THREADS), QuadShape<16, W>::SMEM, s, m);
+    case 32: return launch_dep(quads_multi_kernel<32, W>, grid, dim3(QuadShape<32, W>::THREADS), QuadShape<32, W>::SMEM, s, m);
+    case 64: return launch_dep(quads_multi_kernel<64, W>, grid, dim3(QuadShape<64, W>::THREADS), QuadShape<64, W>::SMEM, s, m);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 template <class K>
@@ -1018,23 +1153,28 @@ cudaError_t allow_smem(K kernel, int optin) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
+template <int CS, int W>
+cudaError_t configure_quads() {
+  const int smem = (int)QuadShape<CS, W>::SMEM;
+  const cudaError_t e =
+      cudaFuncSetAttribute(quads_kernel<CS, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(quads_multi_kernel<CS, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+}
+
 template <int W>
 cudaError_t configure_interp(int optin) {
   cudaError_t e;
-  if ((e = allow_smem(interp2_multi_kernel<32, W>, optin))) return e;
-  if ((e = allow_smem(interp2_multi_kernel<64, W>, optin))) return e;
-  if ((e = allow_smem(interp2_multi_kernel<16, W>, optin))) return e;
-  if ((e = allow_smem(interp2_multi_kernel<8, W>, optin))) return e;
-  if ((e = allow_smem(interp2_kernel<32, W>, optin))) return e;
-  if ((e = allow_smem(interp2_kernel<64, W>, optin))) return e;
-  if ((e = allow_smem(interp2_kernel<16, W>, optin))) return e;
-  if ((e = allow_smem(interp2_kernel<8, W>, optin))) return e;
-  if ((e = allow_smem(interp_kernel<1, 0, W>, optin))) return e;
-  if ((e = allow_smem(interp_kernel<2, 0, W>, optin))) return e;
-  if ((e = allow_smem(interp_kernel<4, 0, W>, optin))) return e;
-  if ((e = allow_smem(interp_kernel<8, 0, W>, optin))) return e;
-  if ((e = allow_smem(interp_kernel<16, 0, W>, optin))) return e;
-  return allow_smem(interp_kernel<32, 0, W>, optin);
+  if ((e = configure_quads<8, W>())) return e;
+  if ((e = configure_quads<16, W>())) return e;
+  if ((e = configure_quads<32, W>())) return e;
+  if ((e = configure_quads<64, W>())) return e;
+  if ((e = allow_smem(interp_kernel<1, W>, optin))) return e;
+  if ((e = allow_smem(interp_kernel<2, W>, optin))) return e;
+  if ((e = allow_smem(interp_kernel<4, W>, optin))) return e;
+  if ((e = allow_smem(interp_kernel<8, W>, optin))) return e;
+  if ((e = allow_smem(interp_kernel<16, W>, optin))) return e;
+  return allow_smem(interp_kernel<32, W>, optin);
 }
 
 }  // namespace
@@ -1060,7 +1200,8 @@ cudaError_t nufft_configure(int smem_optin) {
 }
 
 size_t interp_tile_bytes(const Plan& p) {
-  return (size_t)(p.interp_tr + p.W - 1) * (p.interp_tc + p.W - 1) * p.cs * sizeof(float2);
+  const size_t side = interp_tile(p.cs) + p.W - 1;
+  return side * side * p.cs * sizeof(float2);
 }
 
 int interp_buffers(const Plan& p) {
@@ -1069,13 +1210,12 @@ int interp_buffers(const Plan& p) {
   return 2 * tile + 1024 <= (size_t)p.smem_optin ? 2 : 1;
 }
 
-InterpArgs interp_args(const Plan& p, int f0, int nbins, float2* y, const float2* y_meas, bool accumulate,
-                       const Reducer* red, double* sumsq, float2* contrib) {
-  InterpArgs a{};
+// The fields that both interpolation kernels share.
+template <class A>
+A interp_args(const Plan& p, int f0, int nbins, float2* y, const float2* y_meas, bool accumulate, const Reducer* red,
+              double* sumsq, float2* contrib) {
+  A a{};
   a.grid = p.grid;
-  a.kb_idx = p.kb_idx;
-  a.kb_w = p.kb_w;
-  a.order = p.order;
   a.items = p.items;
   a.phase = p.phase;
   a.y = y;
@@ -1085,94 +1225,67 @@ InterpArgs interp_args(const Plan& p, int f0, int nbins, float2* y, const float2
   a.counter = red ? red->counter : nullptr;
   a.sumsq_out = sumsq;
   a.err = p.status_dev;
-  a.n_items = p.n_items;
-  a.R = p.R;
   a.n = p.n;
-  a.C = p.cs;
   a.Cv = nbins;
   a.f0 = f0;
   a.Nf = p.Nf;
   a.scale = 1.0f / (float)p.N;
   a.accumulate = accumulate ? 1 : 0;
-  a.TR = p.interp_tr;
-  a.TC = p.interp_tc;
-  a.nct = p.n / p.interp_tc;
-  a.tpf = ((p.n + p.interp_tr - 1) / p.interp_tr) * a.nct;
-  a.nbuf = interp_buffers(p);
+  return a;
+}
+
+QuadArgs quad_args(const Plan& p, int f0, int nbins, float2* y, const float2* y_meas, bool accumulate,
+                   const Reducer* red, double* sumsq, float2* contrib) {
+  QuadArgs a = interp_args<QuadArgs>(p, f0, nbins, y, y_meas, accumulate, red, sumsq, contrib);
+  a.quads = p.quads;
   a.cta_off = p.item_cta_off;
   return a;
 }
 
-template <int W>
-cudaError_t launch_interp_multi(int cs, const MultiInterp& m, int ctas, size_t smem, cudaStream_t s) {
-  const dim3 grid((unsigned)ctas), block(kInterp2Threads);
-  if (cs == 32) return launch_dep(interp2_multi_kernel<32, W>, grid, block, smem, s, m);
-  if (cs == 64) return launch_dep(interp2_multi_kernel<64, W>, grid, block, smem, s, m);
-  if (cs == 16) return launch_dep(interp2_multi_kernel<16, W>, grid, block, smem, s, m);
-  if (cs == 8) return launch_dep(interp2_multi_kernel<8, W>, grid, block, smem, s, m);
-  return cudaErrorInvalidValue;
-}
-
 cudaError_t interp(const Plan& p, int f0, int nbins, float2* y, const float2* y_meas, bool accumulate,
                    const Reducer* red, double* sumsq, float2* contrib, cudaStream_t s) {
-  InterpArgs a{};
-  a.grid = p.grid;
+  if (p.n_items == 0) return cudaSuccess;
+  if (p.quads) {  // exactly the plan's balanced CTAs
+    if (red && red->capacity < p.interp_ctas) return cudaErrorInvalidValue;
+    const QuadArgs a = quad_args(p, f0, nbins, y, y_meas, accumulate, red, sumsq, contrib);
+    return p.W == 8 ? launch_quads<8>(p.cs, a, p.interp_ctas, s) : launch_quads<6>(p.cs, a, p.interp_ctas, s);
+  }
+  InterpArgs a = interp_args<InterpArgs>(p, f0, nbins, y, y_meas, accumulate, red, sumsq, contrib);
   a.kb_idx = p.kb_idx;
   a.kb_w = p.kb_w;
   a.order = p.order;
-  a.items = p.items;
-  a.phase = p.phase;
-  a.y = y;
-  a.y_meas = y_meas;
-  a.contrib = contrib;
-  a.partials = red ? red->partials : nullptr;
-  a.counter = red ? red->counter : nullptr;
-  a.sumsq_out = sumsq;
-  a.err = p.status_dev;
   a.n_items = p.n_items;
   a.R = p.R;
-  a.n = p.n;
   a.C = p.cs;
-  a.Cv = nbins;
-  a.f0 = f0;
-  a.Nf = p.Nf;
-  a.scale = 1.0f / (float)p.N;
-  a.accumulate = accumulate ? 1 : 0;
-  a.TR = p.interp_tr;
-  a.TC = p.interp_tc;
-  a.nct = p.n / p.interp_tc;
-  a.tpf = ((p.n + p.interp_tr - 1) / p.interp_tr) * a.nct;
+  a.TR = a.TC = interp_tile(p.cs);
+  a.nct = p.n / a.TC;
+  a.tpf = p.n / a.TR * a.nct;
   a.nbuf = interp_buffers(p);
-  if (p.n_items == 0) return cudaSuccess;
-  // tiles, then a full and an empty barrier per buffer
-  const size_t smem = (size_t)a.nbuf * interp_tile_bytes(p) + 2 * a.nbuf * sizeof(uint64_t);
-  a.cta_off = p.item_cta_off;
-  // the two-bin kernel runs exactly the plan's balanced CTAs; the
-  // one-bin kernel strides over the items
-  const int blocks = interp2_eligible(p.cs, nbins) ? p.interp_ctas : std::min(p.n_items, p.num_sms);
+  // tiles, then a barrier per buffer; the kernel strides over the items
+  const size_t smem = (size_t)a.nbuf * interp_tile_bytes(p) + a.nbuf * sizeof(uint64_t);
+  const int blocks = std::min(p.n_items, p.num_sms);
   if (red && red->capacity < blocks) return cudaErrorInvalidValue;
   const int lp = lanes_for(nbins);
-  dim3 grid((unsigned)blocks);
-  return p.W == 8 ? launch_interp<8>(lp, p.cs, a, grid, smem, s) : launch_interp<6>(lp, p.cs, a, grid, smem, s);
+  const dim3 grid((unsigned)blocks);
+  return p.W == 8 ? launch_interp<8>(lp, a, grid, smem, s) : launch_interp<6>(lp, a, grid, smem, s);
 }
 
 cudaError_t interp_residual_batch(Plan* const* ps, const float2* const* y_meas, int count, cudaStream_t s) {
   if (count < 1 || count > kMaxBatch) return cudaErrorInvalidValue;
-  MultiInterp m{};
+  MultiQuads m{};
   m.nreq = 0;
   Plan* mp[kMaxBatch];
   for (int r = 0; r < count; ++r) {
     Plan& p = *ps[r];
     if (p.nchunks != 1) return cudaErrorInvalidValue;
-    const bool multi = interp2_eligible(p.cs, p.Nf) && p.cs == ps[0]->cs && p.W == ps[0]->W &&
-                       interp_buffers(p) == interp_buffers(*ps[0]) && p.n_items > 0;
+    const bool multi = p.quads && ps[0]->quads && p.cs == ps[0]->cs && p.W == ps[0]->W && p.n_items > 0;
     if (!multi) {  // its own launch
       const cudaError_t e = interp(p, 0, p.Nf, p.resid, y_meas[r], false, &p.red_interp, p.scalars, p.contrib, s);
       if (e != cudaSuccess) return e;
       continue;
     }
     mp[m.nreq] = &p;
-    m.a[m.nreq] = interp_args(p, 0, p.Nf, p.resid, y_meas[r], false, &p.red_interp, p.scalars, p.contrib);
+    m.a[m.nreq] = quad_args(p, 0, p.Nf, p.resid, y_meas[r], false, &p.red_interp, p.scalars, p.contrib);
     m.plan_ctas[m.nreq] = p.interp_ctas;
     ++m.nreq;
   }
@@ -1186,9 +1299,7 @@ cudaError_t interp_residual_batch(Plan* const* ps, const float2* const* y_meas, 
   }
   const Plan& p0 = *mp[0];
   const int ctas = split_ctas(work, cap, m.nreq, std::max(m.nreq, p0.num_sms), m.cta_begin);
-  const int nbuf = interp_buffers(p0);
-  const size_t smem = (size_t)nbuf * interp_tile_bytes(p0) + 2 * nbuf * sizeof(uint64_t);
-  return p0.W == 8 ? launch_interp_multi<8>(p0.cs, m, ctas, smem, s) : launch_interp_multi<6>(p0.cs, m, ctas, smem, s);
+  return p0.W == 8 ? launch_quads_multi<8>(p0.cs, m, ctas, s) : launch_quads_multi<6>(p0.cs, m, ctas, s);
 }
 
 cudaError_t spread_batch(Plan* const* ps, int count, cudaStream_t s) {

@@ -186,6 +186,116 @@ void mark_used_blocks(Plan& p, const std::vector<int>& first_tap) {
   p.grid_sparse = 2 * count < p.grid_used_h.size() * (size_t)(n / kGridBlock);
 }
 
+// Modelled cost of an interpolation item in clock cycles of an SM, from fits
+// to the CTAs' own clocks at the static (32 bins), dynamic (16) and 64-bin
+// configurations: an item's turn round the warps, its quads, and the copies of
+// the rows it adds to the ring (from L2 or, where the used part of the grid
+// outgrows it, from DRAM).
+long quad_cost(int quads, int new_rows, int cs, bool grid_in_l2) {
+  return (cs == 64 ? 5000 : 1600) + 140 * (long)quads + (long)new_rows * (grid_in_l2 ? 60 : 250);
+}
+
+// Interpolation quads (prop_internal.cuh) and their work items.  A quad's
+// anchor is the cell of its window's first row and column; quads are ordered
+// by frame, strip of quad_cols(cs) columns, first row and sample index, and
+// a strip's run is cut into items of at most quad_item(cs) quads that start
+// within quad_span(cs, W) rows.  A CTA takes a contiguous run of items, so that
+// it walks down a strip and an item adds only its last rows to those of the
+// item before; the runs are cut at equal shares of the modelled cost.
+void build_quads(const Plan& p, const std::vector<int>& first_tap, const std::vector<double>& wd, int ctas,
+                 std::vector<float4>& quads, std::vector<int4>& items, std::vector<int>& cta_off) {
+  const int n = p.n, W = p.W, UW = quad_window(W), REC = quad_record(W), TC = quad_cols(p.cs);
+  const int nstrip = (n + TC - 1) / TC;
+  struct Quad {
+    int m[4], d1[4], d2[4], c0, r0, j0, key;
+  };
+  std::vector<Quad> qs;
+  for (int b = 0; b < p.B; ++b)
+    for (int l = 0; l < p.L; l += 2)
+      for (int j = 0; j < p.R; j += 2) {
+        Quad q{};
+        int ref = -1, lo1 = 0, lo2 = 0;
+        for (int s = 0; s < 4; ++s) {
+          const int ls = l + s / 2, js = j + s % 2;
+          q.m[s] = ls < p.L && js < p.R ? (b * p.L + ls) * p.R + js : -1;
+          if (q.m[s] < 0) continue;
+          if (ref < 0) ref = q.m[s];
+          // tap distances from the first sample's, on the circle
+          auto dist = [&](int axis) {
+            const int d = first_tap[2 * (size_t)q.m[s] + axis] - first_tap[2 * (size_t)ref + axis];
+            return ((d + n / 2) % n + n) % n - n / 2;
+          };
+          q.d1[s] = dist(0);
+          q.d2[s] = dist(1);
+          lo1 = std::min(lo1, q.d1[s]);
+          lo2 = std::min(lo2, q.d2[s]);
+        }
+        for (int s = 0; s < 4; ++s) q.d1[s] -= lo1, q.d2[s] -= lo2;
+        q.c0 = (first_tap[2 * (size_t)ref] + lo1 + n) % n;
+        q.r0 = (first_tap[2 * (size_t)ref + 1] + lo2 + n) % n;
+        q.j0 = j;
+        q.key = p.blade_frame[b] * nstrip + q.c0 / TC;
+        qs.push_back(q);
+      }
+  std::vector<int> idx(qs.size());
+  for (size_t i = 0; i < idx.size(); ++i) idx[i] = (int)i;
+  std::stable_sort(idx.begin(), idx.end(), [&](int x, int y) {
+    return qs[x].key != qs[y].key ? qs[x].key < qs[y].key : qs[x].r0 < qs[y].r0;
+  });
+  std::vector<int> row0(qs.size());  // first row of each quad's item
+  std::vector<long> upto;            // cost up to and with each item
+  long total = 0;
+  const int span = quad_span(p.cs, W), most = quad_item(p.cs);
+  size_t blocks = 0;
+  for (uint64_t u : p.grid_used_h) blocks += (size_t)__builtin_popcountll(u);
+  const bool in_l2 = blocks * 2 * kGridBlock * p.cs * sizeof(float2) < (size_t)100 << 20;
+  for (size_t i = 0; i < idx.size();) {
+    const Quad& q0 = qs[idx[i]];
+    size_t e = i;
+    while (e < idx.size() && (int)(e - i) < most && qs[idx[e]].key == q0.key && qs[idx[e]].r0 < q0.r0 + span)
+      row0[e++] = q0.r0;
+    const int rows = qs[idx[e - 1]].r0 - q0.r0 + UW;
+    const int have = items.empty() || items.back().x != q0.key
+                         ? 0
+                         : std::max(0, (items.back().w & 0xffff) + (items.back().w >> 16) - q0.r0);
+    total += quad_cost((int)(e - i), rows - std::min(rows, have), p.cs, in_l2);
+    upto.push_back(total);
+    items.push_back(make_int4(q0.key, (int)i, (int)(e - i), q0.r0 | rows << 16));
+    i = e;
+  }
+  quads.assign(qs.size() * REC, make_float4(0.f, 0.f, 0.f, 0.f));
+  for (size_t i = 0; i < idx.size(); ++i) {
+    const Quad& q = qs[idx[i]];
+    float* w = reinterpret_cast<float*>(&quads[i * REC]);
+    int* tail = reinterpret_cast<int*>(&quads[i * REC + 2 * UW]);
+    int rows = 0, cols = 0;
+    for (int s = 0; s < 4; ++s) {
+      tail[s] = q.m[s];
+      if (q.m[s] < 0) continue;
+      for (int a = 0; a < W; ++a) {
+        w[4 * (q.d1[s] + a) + s] = (float)wd[(size_t)q.m[s] * 2 * W + a];
+        w[4 * (UW + q.d2[s] + a) + s] = (float)wd[(size_t)q.m[s] * 2 * W + W + a];
+      }
+      rows = std::max(rows, q.d2[s] + W);
+      cols = std::max(cols, q.d1[s] + W);
+    }
+    tail[4] = q.r0 - row0[i];
+    tail[5] = q.c0 % TC;
+    tail[6] = q.j0;
+    tail[7] = rows | cols << 8;
+  }
+  const int P = std::max(1, std::min(ctas, (int)items.size()));
+  cta_off.assign(P + 1, (int)items.size());
+  cta_off[0] = 0;
+  for (int c = 1, at = 0; c < P; ++c) {
+    // the cut nearest to c shares of the cost, with an item left for every CTA
+    const long want = total * c / P;
+    ++at;
+    while (at < (int)items.size() - (P - c) && upto[at - 1] + (upto[at] - upto[at - 1]) / 2 < want) ++at;
+    cta_off[c] = at;
+  }
+}
+
 struct DevAlloc {
   Plan* p;
   size_t* counter;
@@ -228,7 +338,7 @@ void plan_dev_free(Plan* p, void* ptr) {
 void plan_free(Plan* p) {
   if (!p) return;
   void* ptrs[] = {p->kb_idx, p->kb_w, p->phase, p->deapod, p->twiddle, p->blade_frame_d,
-                  p->order, p->items, p->item_cta_off, p->grid_used, p->sitems, p->sitem_cta_off, p->spread_claim, p->sblob, p->contrib, p->grid, p->rows,
+                  p->order, p->quads, p->items, p->item_cta_off, p->grid_used, p->sitems, p->sitem_cta_off, p->spread_claim, p->sblob, p->contrib, p->grid, p->rows,
                   p->resid, p->grad, p->status_dev,
                   p->vol2, p->adam_m, p->adam_v, p->loss_dev, p->scalars,
                   p->red_interp.partials, p->red_interp.counter, p->red_tv.partials,
@@ -403,18 +513,28 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
   for (int q = 0; q < n; ++q)
     tw[q] = make_float2((float)std::cos(2 * M_PI * q / n), (float)-std::sin(2 * M_PI * q / n));
 
-  // Interpolation work items: samples sorted by (frame, TR x TC-cell tile of
-  // their first tap), ascending m within a tile; every non-empty tile's run is
-  // cut into items of at most kInterpItem samples.  One CTA per item stages
-  // the tile plus its (W-1)-cell halo in shared memory.
-  p->interp_tr = interp_tile_rows(p->cs, p->W);
-  p->interp_tc = interp_tile_cols(p->cs, p->W);
-  const int TR = p->interp_tr, TC = p->interp_tc;
-  const int nrt = (n + TR - 1) / TR, nct = n / TC;  // tiles per column / per row of the grid
-  const size_t ntile = (size_t)p->T * nrt * nct;
+  // Interpolation work items.  Bin strides 8 to 64: quads.  Others: samples
+  // sorted by (frame, TR x TC-cell tile of their first tap), ascending m within
+  // a tile; every non-empty tile's run is cut into items of at most kInterpItem
+  // samples.  One CTA per item stages the tile plus its (W-1)-cell halo in
+  // shared memory.
   const size_t LR = (size_t)p->L * p->R;
-  std::vector<int> order(p->M);
+  std::vector<int> order;
   std::vector<int4> items;
+  std::vector<int> cta_off;
+  std::vector<float4> quads;
+  if (quad_stride(p->cs)) {
+    mark_used_blocks(*p, first_tap);
+    build_quads(*p, first_tap, wd, p->num_sms, quads, items, cta_off);
+    kb_idx.clear();
+    kb_w.clear();
+    p->n_items = (int)items.size();
+    p->interp_ctas = (int)cta_off.size() - 1;
+  } else {
+  const int TR = interp_tile(p->cs), TC = TR;
+  const int nrt = n / TR, nct = n / TC;  // tiles per column / per row of the grid
+  const size_t ntile = (size_t)p->T * nrt * nct;
+  order.resize(p->M);
   {
     auto tile_of = [&](size_t m) {
       const size_t frame = (size_t)p->blade_frame[m / LR];
@@ -436,38 +556,7 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
     for (size_t m = 0; m < (size_t)p->M; ++m) order[cnt[tile_of(m)]++] = (int)m;
   }
   p->n_items = (int)items.size();
-  // Static balance over the persistent CTAs (one per SM): longest item first
-  // to the least loaded CTA, with an item's cost its shared-memory traffic
-  // (W^2 taps of cs bins per sample plus the staged tile); each CTA's items
-  // are then stored contiguously, in tile order.
-  std::vector<int> cta_off;
-  {
-    const int P = std::max(1, std::min(p->num_sms, p->n_items));
-    const long tile_cost = (long)(TR + Wi - 1) * (TC + Wi - 1) * p->cs / 16;
-    auto cost = [&](const int4& it) { return (long)it.z * Wi * Wi * p->cs / 16 + tile_cost; };
-    std::vector<int> idx(items.size());
-    for (size_t i = 0; i < idx.size(); ++i) idx[i] = (int)i;
-    std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) { return cost(items[a]) > cost(items[b]); });
-    std::vector<long> load(P, 0);
-    std::vector<std::vector<int>> own(P);
-    for (int i : idx) {
-      int best = 0;
-      for (int c = 1; c < P; ++c)
-        if (load[c] < load[best]) best = c;
-      load[best] += cost(items[i]);
-      own[best].push_back(i);
-    }
-    std::vector<int4> sorted;
-    sorted.reserve(items.size());
-    cta_off.assign(P + 1, 0);
-    for (int c = 0; c < P; ++c) {
-      std::sort(own[c].begin(), own[c].end());
-      for (int i : own[c]) sorted.push_back(items[i]);
-      cta_off[c + 1] = (int)sorted.size();
-    }
-    items.swap(sorted);
-    p->interp_ctas = P;
-  }
+  cta_off.assign(1, 0);  // the run-time-stride kernel strides over the items
   // The interpolation reads the per-sample tables in this sorted order, so that
   // an item's metadata is one contiguous run.
   {
@@ -481,6 +570,7 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
     kb_idx.swap(idx_s);
     kb_w.swap(w_s);
   }
+  }
 
   // Spread gather lists: for every (frame, cell) the samples whose W x W
   // footprint covers the cell, as (phased-residual offset m * cs, weight
@@ -493,9 +583,7 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
   std::vector<int4> sitems;
   std::vector<int2> blob;
   const int2 pad_entry = make_int2((int)((size_t)p->M * p->cs), 0);
-  const bool stride_ok = p->cs == 8 || p->cs == 16 || p->cs == 32 || p->cs == 64;
-  if (stride_ok) mark_used_blocks(*p, first_tap);
-  p->spread_grouped = stride_ok && build_group_lists(*p, first_tap, wd, sitems, blob);
+  p->spread_grouped = quad_stride(p->cs) && build_group_lists(*p, first_tap, wd, sitems, blob);
   if (!p->spread_grouped) {
   p->grid_used_h.clear();  // the cell lists fill the whole grid
   sitems.clear();
@@ -645,13 +733,17 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
       return st;             \
     }                        \
   } while (0)
-  TRY(tab(&p->kb_idx, kb_idx.size(), "sample indices"));
-  TRY(tab(&p->kb_w, kb_w.size(), "sample weights"));
+  if (quads.empty()) {
+    TRY(tab(&p->kb_idx, kb_idx.size(), "sample indices"));
+    TRY(tab(&p->kb_w, kb_w.size(), "sample weights"));
+    TRY(tab(&p->order, order.size(), "interpolation order"));
+  } else {
+    TRY(tab(&p->quads, quads.size(), "interpolation quads"));
+  }
   TRY(tab(&p->phase, phase.size(), "phase table"));
   TRY(tab(&p->deapod, deapod.size(), "deapodisation table"));
   TRY(tab(&p->twiddle, tw.size(), "twiddles"));
   TRY(tab(&p->blade_frame_d, p->blade_frame.size(), "blade frames"));
-  TRY(tab(&p->order, order.size(), "interpolation order"));
   TRY(tab(&p->items, std::max<size_t>(items.size(), 1), "interpolation items"));
   TRY(tab(&p->item_cta_off, cta_off.size(), "interpolation item ranges"));
   TRY(tab(&p->sitems, std::max<size_t>(sitems.size(), 1), "spread items"));
@@ -668,13 +760,17 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
     plan_free(p);
     return cuda_fail(e, "grid workspace");
   }
-  TRY(upload(p->kb_idx, kb_idx));
-  TRY(upload(p->kb_w, kb_w));
+  if (quads.empty()) {
+    TRY(upload(p->kb_idx, kb_idx));
+    TRY(upload(p->kb_w, kb_w));
+    TRY(upload(p->order, order));
+  } else {
+    TRY(upload(p->quads, quads));
+  }
   TRY(upload(p->phase, phase));
   TRY(upload(p->deapod, deapod));
   TRY(upload(p->twiddle, tw));
   TRY(upload(p->blade_frame_d, p->blade_frame));
-  TRY(upload(p->order, order));
   if (!sitems.empty()) TRY(upload(p->sitems, sitems));
   TRY(upload(p->sitem_cta_off, scta_off));
   TRY(upload(p->sblob, blob));
@@ -764,13 +860,16 @@ size_t plan_estimate_bytes(const prop_plan_desc* d, int iters) {
   const size_t W = d->kb_width == 8 ? 8 : 6;
   const size_t chunk = d->bin_chunk == 0 ? std::min<size_t>(Nf, kMaxChunk) : std::min<size_t>(d->bin_chunk, Nf);
   const size_t cs = chunk + (chunk & 1);
-  const size_t TR = (size_t)interp_tile_rows((int)cs, (int)W), TC = (size_t)interp_tile_cols((int)cs, (int)W);
+  const size_t tile = (size_t)interp_tile((int)cs);
+  const size_t nquads = B * (((size_t)d->lines + 1) / 2) * (((size_t)d->readout + 1) / 2);
   const size_t ncell = T * n * n;
   const size_t vol = T * N * N * Nf;
-  const size_t interp_items = M / kInterpItem + T * ((n + TR - 1) / TR) * (n / TC) + 1;
+  const bool quads = quad_stride((int)cs);
+  const size_t interp_items = quads ? nquads : M / kInterpItem + T * (n / tile) * (n / tile) + 1;
   const size_t spread_items = (M * W * W + kSpreadCellCost * ncell) / kSpreadItemCost + 1;
   size_t b = 0;
-  b += 4 * M + M * (W / 2) * 16 + (size_t)d->readout * Nf * 8 + 4 * N + 8 * n + 4 * B + 4 * M;  // sample tables
+  b += quads ? nquads * quad_record((int)W) * 16 : 8 * M + M * (W / 2) * 16;                    // sample tables
+  b += (size_t)d->readout * Nf * 8 + 4 * N + 8 * n + 4 * B;
   const size_t cell_lists = 8 * (ncell + spread_items) + 8 * (M * W * W + (kSpreadListPad - 1) * std::min(ncell, M * W * W));
   const size_t group_lists = 8 * (ncell / 4) + 8 + (4 + 16) * 2 * 16 * M + 16 * (ncell / 4);  // items <= groups
   b += 16 * interp_items + 16 * spread_items + std::max(cell_lists, group_lists) + 4 * 1024;  // lists

@@ -38,15 +38,58 @@ constexpr int kFftCols = 16;       // columns (complex lines) per FFT tile
 // 4-line tiles still read whole 32-byte sectors along a column).
 constexpr int kCartCols = 4;
 
-// Interpolation tile (rows x cells per row) for bin stride cs and kernel
-// width W: 16 x 16 up to 32 bins, 8 x 8 above.  At width 8 with 32 bins a
-// 16 x 16 tile plus its 7-cell halo (23 x 23 cells, 135 KB) leaves room for
-// one buffer only, so its copy could not overlap the previous tile's work;
-// 12 rows of 16 (19 x 23 staged cells, 112 KB) double-buffer and stage 2.3x
-// the cells they own (16 x 16: 2.1x; 8 x 8: 3.5x, which measured slower).
-// Rows of tiles need not divide the grid: the last one wraps past row n - 1.
-constexpr int interp_tile_rows(int cs, int W) { return cs > 32 ? 8 : (W == 8 && cs == 32 ? 12 : 16); }
-constexpr int interp_tile_cols(int cs, int W) { return (void)W, cs > 32 ? 8 : 16; }
+// Interpolation tile (rows and cells per row) of the run-time bin strides:
+// 16 x 16 up to 32 bins, 8 x 8 above.
+constexpr int interp_tile(int cs) { return cs > 32 ? 8 : 16; }
+
+// Quads: the interpolation of the bin strides 8, 16, 32 and 64 takes the
+// samples of a blade 2 lines x 2 readout positions at a time.  They lie on a
+// rotated square lattice 2 grid cells apart, so along each axis their first
+// taps differ by at most floor(2 sqrt 2) + 1 = 3 cells whatever the angle, and
+// one window of (W + 3)^2 cells holds the four W x W footprints.
+constexpr int quad_window(int W) { return W + 3; }
+// A quad's record, in float4 (one component a sample): the x1 weights of the
+// window's columns, the x2 weights of its rows (zero outside a sample's
+// footprint), the sample indices (int4, -1: none), and (first row from the
+// item's, first column from the strip's, readout index of samples 0 and 2,
+// rows in use | columns in use << 8).
+constexpr int quad_record(int W) { return 2 * quad_window(W) + 2; }
+// Quads are grouped by the strip of quad_cols(cs) grid columns that their
+// window starts in; a persistent CTA walks down strips with the grid rows it
+// reads in a ring in shared memory.
+constexpr int quad_cols(int cs) { return 512 / cs; }
+constexpr bool quad_stride(int cs) { return cs == 8 || cs == 16 || cs == 32 || cs == 64; }
+constexpr int kQuadWarps = 15;  // compute warps: with the producer 16, so 128 registers a thread
+constexpr int quad_per_warp(int cs) { return cs < 32 ? 32 / cs : 1; }
+constexpr int quad_item(int cs) { return kQuadWarps * quad_per_warp(cs); }  // most quads of an item: one unit a warp
+constexpr int kQuadStages = 3;  // items whose quad records are staged in shared memory
+constexpr int quad_row_bytes(int cs, int W) { return (quad_cols(cs) + quad_window(W) - 1) * cs * 8; }
+constexpr int quad_stage_bytes(int cs, int W) { return quad_item(cs) * quad_record(W) * 16; }
+// Rows in the ring: what 227 KB hold beside the stages, the barriers and the
+// static shared memory.
+constexpr int quad_ring_rows(int cs, int W) {
+  return (227 * 1024 - 2048 - kQuadStages * quad_stage_bytes(cs, W)) / quad_row_bytes(cs, W);
+}
+// Rows that the quads of one item start in, at most: an item's rows and the
+// next one's new rows fit the ring together, so that the next item's copies
+// run while this one is computed.
+constexpr int quad_span(int cs, int W) { return (quad_ring_rows(cs, W) - (quad_window(W) - 1)) / 2; }
+template <int CS, int W>
+struct QuadShape {
+  static constexpr int UW = quad_window(W);
+  static constexpr int QPW = quad_per_warp(CS);       // quads per warp
+  static constexpr int LPQ = 32 / QPW;                // lanes per quad
+  static constexpr int BPL = CS / LPQ;                // bins per lane
+  static constexpr int THREADS = 32 * (kQuadWarps + 1);
+  static constexpr int HC = quad_cols(CS) + UW - 1;   // staged cells per grid row
+  static constexpr int RB = quad_row_bytes(CS, W);
+  static constexpr int REC = quad_record(W);
+  static constexpr int ITEM = quad_item(CS);
+  static constexpr int NR = quad_ring_rows(CS, W);
+  static constexpr int SPAN = quad_span(CS, W);
+  static constexpr size_t SMEM = (size_t)NR * RB + (size_t)kQuadStages * quad_stage_bytes(CS, W) + 2 * kQuadStages * 8;
+  static_assert(SPAN >= 1 && RB % 16 == 0, "an item's and the next one's rows; bulk copies");
+};
 
 // Rows of a grid block whose use by the samples is tracked (the unit in which
 // the column passes and the spread skip the grid): a thread of the column
@@ -151,11 +194,12 @@ struct Plan {
   float2* twiddle = nullptr;     // [n] exp(-2 pi i k / n)
   int* blade_frame_d = nullptr;  // [B]
   int* order = nullptr;          // [M] samples sorted by grid tile (interpolation order)
-  int4* items = nullptr;         // [n_items] (frame * tiles^2 + tile, first, count, 0), grouped by CTA
+  float4* quads = nullptr;       // [quads][quad_record(W)] in item order (bin strides 8 to 64; instead of the three above)
+  int4* items = nullptr;         // [n_items] grouped by CTA: (tile of its frame, first sample, count, 0), or with quads
+                                 // (frame * strips + strip, first quad, count, first grid row | grid rows << 16)
   int* item_cta_off = nullptr;   // [interp_ctas + 1] CTA c interpolates items [off[c], off[c + 1])
   int n_items = 0;
   int interp_ctas = 1;           // persistent interpolation CTAs the items are balanced over
-  int interp_tr = 16, interp_tc = 16;  // interpolation tile: rows, cells per row
   // Spread gather: cells in patch-major order (frame, 8x8-cell patch,
   // row-major in the patch), cut into items; each item is one blob of
   // (cell, list end) pairs followed by its cells' (offset m * cs, weight
