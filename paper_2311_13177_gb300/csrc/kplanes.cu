@@ -91,6 +91,33 @@ __device__ __forceinline__ float2 kcmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.x, b.y, -a.y * b.x));
 }
 __device__ __forceinline__ float2 kadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+// c + a b and c + conj(a) b, four multiply-adds each
+__device__ __forceinline__ float2 kfma(float2 a, float2 b, float2 c) {
+  return make_float2(fmaf(a.x, b.x, fmaf(-a.y, b.y, c.x)), fmaf(a.x, b.y, fmaf(a.y, b.x, c.y)));
+}
+__device__ __forceinline__ float2 kcfma(float2 a, float2 b, float2 c) {
+  return make_float2(fmaf(a.x, b.x, fmaf(a.y, b.y, c.x)), fmaf(a.x, b.y, fmaf(-a.y, b.x, c.y)));
+}
+
+// Asynchronous 8-byte copies global -> shared (zeros where !live).
+__device__ __forceinline__ void copy8_async(float2* dst, const float2* src, bool live) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(live ? 8 : 0)
+               : "memory");
+}
+// Two values; wide: both addresses are 16-byte aligned.
+__device__ __forceinline__ void copy16_async(float2* dst, const float2* src, bool live, bool wide) {
+  if (wide) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(live ? 16 : 0)
+                 : "memory");
+  } else {
+    copy8_async(dst, src, live);
+    copy8_async(dst + 1, src + (live ? 1 : 0), live);
+  }
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // Plane c's voxel-resolution axes: (extent of the first expanded index, of the second).
 __host__ __device__ inline void exp_axes(const KpArgs& a, int c, int* e0, int* e1) {
@@ -219,22 +246,25 @@ __global__ void __launch_bounds__(kKpThreads) kp_contract_kernel(const float2* _
 
 // --- render ------------------------------------------------------------------
 
-// CTA = (column strip of XS image columns, image row y); thread = (column x,
-// bin w) with w fastest; the CTA walks the frames TB at a time: the
-// frames' Eyt Ewt (laid out [frame][q][w]) and Ext ([frame][q][x]) are staged
-// in shared memory with one barrier per batch (double-buffered), so each
-// thread has TB independent loads in flight per fill; conflict-free reads.
-template <int QM>
-__global__ void __launch_bounds__(kKpThreads) kp_render_kernel(const float2* __restrict__ E, KpArgs a, int XS,
-                                                               int TB, float2* __restrict__ V) {
-  extern __shared__ float2 kp_sm[];
+// CTA = (strip of XS image columns, image row y); thread = (bin w fastest, PX
+// columns x apart by XS / PX), with its R in registers; the CTA walks the
+// frames TB at a time: their Eyt Ewt ([frame][w][q], rows of QM + 2 values so
+// that the bins of a warp hit different banks) and Ext ([frame][x][q]), both
+// read two q a load at compile-time offsets, are staged in shared memory with
+// one barrier per batch (double-buffered).  Two complex products a voxel and q
+// are the least this factorisation takes (62 us of multiply-adds at 192^2 x 16
+// bins x 32 frames, Q = 16); with one column a thread the two shared-memory
+// loads for them were the bound (78 % of the LSU pipe), two columns share the
+// Eyt Ewt load.
+template <int QM, int PX>
+__global__ void __launch_bounds__(kKpThreads, 2) kp_render_kernel(const float2* __restrict__ E, KpArgs a, int XS,
+                                                                  int TB, float2* __restrict__ V) {
+  extern __shared__ __align__(16) float2 kp_sm[];
   grid_dep_wait();
   grid_dep_release();
   const int Q = a.Q, Nf = a.Nf, N = a.N;
-  const int y = blockIdx.y;
-  const int xl = threadIdx.x / Nf, w = threadIdx.x - xl * Nf;
-  const int x = blockIdx.x * XS + xl;
-  const bool valid = xl < XS && x < N;
+  const int y = blockIdx.y, x0 = blockIdx.x * XS;
+  const int xl = threadIdx.x / Nf, w = threadIdx.x - xl * Nf, XH = XS / PX;
   const float2* Exy = E + a.e_off[kXY];
   const float2* Exw = E + a.e_off[kXW];
   const float2* Ext = E + a.e_off[kXT];
@@ -242,37 +272,62 @@ __global__ void __launch_bounds__(kKpThreads) kp_render_kernel(const float2* __r
   const float2* Eyt = E + a.e_off[kYT];
   const float2* Ewt = E + a.e_off[kWT];
   const float2* A = E + a.e_off[kKpPlanes];
-  float2 R[QM];
+  float2 R[PX][QM];
 #pragma unroll
-  for (int q = 0; q < QM; ++q) {
-    R[q] = make_float2(0.f, 0.f);
-    if (valid && q < Q)
-      R[q] = kmul(kmul(A[q], Exy[((size_t)y * N + x) * Q + q]),
-                  kmul(Exw[((size_t)x * Nf + w) * Q + q], Eyw[((size_t)y * Nf + w) * Q + q]));
+  for (int i = 0; i < PX; ++i) {
+    const int x = x0 + xl + i * XH;
+#pragma unroll
+    for (int q = 0; q < QM; ++q) {
+      R[i][q] = make_float2(0.f, 0.f);
+      if (xl < XH && x < N && q < Q)
+        R[i][q] = kmul(kmul(A[q], Exy[((size_t)y * N + x) * Q + q]),
+                       kmul(Exw[((size_t)x * Nf + w) * Q + q], Eyw[((size_t)y * Nf + w) * Q + q]));
+    }
   }
-  const int hsz = Nf * Q, usz = XS * Q, bsz = TB * (hsz + usz);
+  // q >= Q: zero factors (R is zero there, the staged values must be finite)
+  constexpr int HS = QM + 2;
+  const int hsz = Nf * HS, usz = XS * QM, bsz = TB * (hsz + usz);
   for (int t0 = 0, buf = 0; t0 < a.T; t0 += TB, buf ^= 1) {
     const int nt = min(TB, a.T - t0);
-    float2* H = kp_sm + buf * bsz;       // [frame][q][w]
-    float2* U = H + TB * hsz;            // [frame][q][x]
-    for (int e = threadIdx.x; e < hsz; e += blockDim.x) {
-      const int ww = e % Nf, q = e / Nf;
+    float2* H = kp_sm + buf * bsz;       // [frame][w][q]
+    float2* U = H + TB * hsz;            // [frame][x][q]
+    for (int e = threadIdx.x; e < Nf * QM; e += blockDim.x) {
+      const int ww = e / QM, q = e - ww * QM;
       for (int tb = 0; tb < nt; ++tb)
-        H[tb * hsz + e] = kmul(Eyt[((size_t)(t0 + tb) * N + y) * Q + q], Ewt[((size_t)(t0 + tb) * Nf + ww) * Q + q]);
+        H[tb * hsz + ww * HS + q] = q < Q ? kmul(Eyt[((size_t)(t0 + tb) * N + y) * Q + q],
+                                                 Ewt[((size_t)(t0 + tb) * Nf + ww) * Q + q])
+                                          : make_float2(0.f, 0.f);
     }
     for (int e = threadIdx.x; e < usz; e += blockDim.x) {
-      const int xx = blockIdx.x * XS + e % XS, q = e / XS;
+      const int xx = e / QM, q = e - xx * QM;
       for (int tb = 0; tb < nt; ++tb)
-        U[tb * usz + e] = xx < N ? Ext[((size_t)(t0 + tb) * N + xx) * Q + q] : make_float2(0.f, 0.f);
+        U[tb * usz + e] = x0 + xx < N && q < Q ? Ext[((size_t)(t0 + tb) * N + x0 + xx) * Q + q] : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    if (valid)
+    if (xl < XH)
       for (int tb = 0; tb < nt; ++tb) {
-        float2 acc = make_float2(0.f, 0.f);
+        float2 acc[PX];
 #pragma unroll
-        for (int q = 0; q < QM; ++q)
-          if (q < Q) acc = kadd(acc, kmul(R[q], kmul(U[tb * usz + q * XS + xl], H[tb * hsz + q * Nf + w])));
-        V[((((size_t)t0 + tb) * N + y) * N + x) * Nf + w] = acc;
+        for (int i = 0; i < PX; ++i) acc[i] = make_float2(0.f, 0.f);
+        const float4* Hq = reinterpret_cast<const float4*>(H + tb * hsz + w * HS);
+        const float4* Ux[PX];
+#pragma unroll
+        for (int i = 0; i < PX; ++i) Ux[i] = reinterpret_cast<const float4*>(U + tb * usz + (xl + i * XH) * QM);
+#pragma unroll
+        for (int q = 0; q < QM; q += 2) {
+          const float4 h = Hq[q / 2];
+#pragma unroll
+          for (int i = 0; i < PX; ++i) {
+            const float4 u = Ux[i][q / 2];
+            acc[i] = kfma(R[i][q], kmul(make_float2(u.x, u.y), make_float2(h.x, h.y)), acc[i]);
+            acc[i] = kfma(R[i][q + 1], kmul(make_float2(u.z, u.w), make_float2(h.z, h.w)), acc[i]);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < PX; ++i) {
+          const int x = x0 + xl + i * XH;
+          if (x < N) V[((((size_t)t0 + tb) * N + y) * N + x) * Nf + w] = acc[i];
+        }
       }
   }
 }
@@ -381,6 +436,248 @@ __global__ void __launch_bounds__(kKpThreads) kp_wgrad_kernel(const float2* __re
     for (int yi = 0; yi < ny; ++yi) dE[a.e_off[kXY] + ((size_t)(y0 + yi) * N + x) * Q + q] = dxy[yi];
 }
 
+// The W kernel for Nf = WR bins, few enough that a thread (x, q) keeps its Exw
+// for every bin in registers.  The bound is the two complex products a voxel
+// and q (62 us of multiply-adds at 192^2 x 16 x 32 frames, Q = 16); the general
+// kernel above spends three loads on them, two from shared memory and one of
+// grad V from global memory whose latency nothing hides.  Here one load of
+// A Eyw Ewt (shared by the columns of a warp) and half a load of grad V (two
+// bins at once, the same for all q) remain, both from shared memory; grad V of
+// the next frame is copied in asynchronously meanwhile.  QM >= Q is the row
+// length of the staged products, so that their offsets are compile-time.
+template <int WR, int QM>
+__global__ void __launch_bounds__(kKpThreads, 2) kp_wgrad_reg_kernel(const float2* __restrict__ E, KpArgs a, int XS,
+                                                                     const float2* __restrict__ gV,
+                                                                     float2* __restrict__ dE, KpPart part) {
+  extern __shared__ __align__(16) float2 kp_sm[];
+  grid_dep_wait();
+  grid_dep_release();
+  constexpr int Y = kKpYChunk;
+  const int Q = a.Q, N = a.N;
+  const int xl = threadIdx.x / Q, q = threadIdx.x - xl * Q;
+  const int x0 = blockIdx.x * XS, x = x0 + xl;
+  const bool valid = x < N;
+  const int y0 = blockIdx.y * Y, ny = min(Y, N - y0);
+  const float2* Exy = E + a.e_off[kXY];
+  const float2* Exw = E + a.e_off[kXW];
+  const float2* Ext = E + a.e_off[kXT];
+  const float2* Eyw = E + a.e_off[kYW];
+  const float2* Eyt = E + a.e_off[kYT];
+  const float2* Ewt = E + a.e_off[kWT];
+  const float2* A = E + a.e_off[kKpPlanes];
+  const int gsz = Y * XS * WR;
+  constexpr int csz = Y * WR * QM;
+  float2* sG = kp_sm;              // [2][row][xl][w] grad V
+  float2* sC = sG + 2 * gsz;       // [row][w][q] A Eyw Ewt of the current frame
+  float2* sR = sC + csz;           // [row][xl][q] dEyt terms of the current frame
+  // grad V of a frame: Y rows of PR 16-byte chunks; a thread's chunks are
+  // blockDim apart, (row, chunk) stepped with one carry
+  const int PR = XS * WR / 2, row0 = threadIdx.x / PR, c0 = threadIdx.x - row0 * PR;
+  const int drow = blockDim.x / PR, dc = blockDim.x - drow * PR, cmax = (N - x0) * WR / 2;
+  const bool wide = ((uintptr_t)gV & 15) == 0;
+  auto fetch = [&](int t, int buf) {
+    const float2* src = gV + (((size_t)t * N + y0) * N + x0) * WR;
+    float2* dst = sG + buf * gsz;
+    for (int row = row0, c = c0; row < Y;) {
+      const bool live = row < ny && c < cmax;
+      copy16_async(dst + 2 * (row * PR + c), src + (live ? row * (N * WR) + 2 * c : 0), live, wide);
+      row += drow;
+      c += dc;
+      if (c >= PR) {
+        c -= PR;
+        ++row;
+      }
+    }
+    copies_commit();
+  };
+  fetch(0, 0);
+  float2 ew[WR];
+#pragma unroll
+  for (int w = 0; w < WR; ++w) ew[w] = valid ? Exw[((size_t)x * WR + w) * Q + q] : make_float2(0.f, 0.f);
+  float2 dxy[Y], exy[Y];
+#pragma unroll
+  for (int i = 0; i < Y; ++i) {
+    dxy[i] = make_float2(0.f, 0.f);
+    exy[i] = (valid && i < ny) ? Exy[((size_t)(y0 + i) * N + x) * Q + q] : make_float2(0.f, 0.f);
+  }
+  const float2 Aq = A[q];
+  const float2* Eyw0 = Eyw + (size_t)y0 * WR * Q + q;
+  const int xq = x * Q + q, yq = y0 * Q + q, NQ = N * Q;
+  for (int t = 0; t < a.T; ++t) {
+    for (int w = xl; w < WR; w += XS) {
+      const float2 aw = kmul(Aq, Ewt[(t * WR + w) * Q + q]);
+#pragma unroll
+      for (int i = 0; i < Y; ++i) {
+        if (i >= ny) break;
+        sC[i * WR * QM + w * QM + q] = kmul(aw, Eyw0[(i * WR + w) * Q]);
+      }
+    }
+    const float2 ext = valid ? Ext[t * NQ + xq] : make_float2(0.f, 0.f);
+    const float2* eyt_row = Eyt + (size_t)t * NQ + yq;
+    copies_wait();
+    __syncthreads();
+    if (t + 1 < a.T) fetch(t + 1, (t + 1) & 1);
+    const float2* G = sG + (t & 1) * gsz + xl * WR;
+    float2 dxt = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < Y; ++i) {
+      if (i >= ny) break;
+      const float2* C = sC + i * WR * QM + q;
+      const float4* g = reinterpret_cast<const float4*>(G + i * XS * WR);
+      float2 ws0 = make_float2(0.f, 0.f), ws1 = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int w = 0; w < WR; w += 2) {
+        const float4 gg = g[w / 2];
+        ws0 = kcfma(C[w * QM], kcmul(ew[w], make_float2(gg.x, gg.y)), ws0);
+        ws1 = kcfma(C[(w + 1) * QM], kcmul(ew[w + 1], make_float2(gg.z, gg.w)), ws1);
+      }
+      const float2 ws = kadd(ws0, ws1);
+      const float2 eyt = eyt_row[i * Q];
+      dxy[i] = kcfma(kmul(ext, eyt), ws, dxy[i]);
+      dxt = kcfma(kmul(exy[i], eyt), ws, dxt);
+      sR[i * XS * Q + threadIdx.x] = kcmul(kmul(exy[i], ext), ws);
+    }
+    if (valid) part.xt[(((size_t)blockIdx.y * a.T + t) * N + x) * Q + q] = dxt;
+    __syncthreads();
+    // dEyt partial of this strip: sum the columns' terms in column order
+    for (int e = threadIdx.x; e < ny * Q; e += blockDim.x) {
+      const int yi = e / Q, qq = e - yi * Q;
+      float2 s = make_float2(0.f, 0.f);
+      for (int xx = 0; xx < XS; ++xx) s = kadd(s, sR[(yi * XS + xx) * Q + qq]);
+      part.yt[(((size_t)blockIdx.x * a.T + t) * N + y0 + yi) * Q + qq] = s;
+    }
+    // (the next frame's barrier comes before sR is rewritten; sC is not read after this one)
+  }
+  if (valid)
+    for (int yi = 0; yi < ny; ++yi) dE[a.e_off[kXY] + ((size_t)(y0 + yi) * N + x) * Q + q] = dxy[yi];
+}
+
+// The T kernel for runs of WR bins (grid z), thread (x, q): Tsum of the WR bins
+// in registers, so that a bin costs one load of Ewt (shared by the columns of
+// a warp) and half a load of grad V for its two complex products; with a
+// thread per (x, w) (below) each product pair took two loads and the staging
+// of Exy Ext Eyt.  Ewt of up to TH frames stays in shared memory, grad V comes
+// in asynchronously a batch of kKpTG frames ahead.
+constexpr int kKpTG = 4;
+template <int WR, int QM>
+__global__ void __launch_bounds__(kKpThreads, 2) kp_tgrad_reg_kernel(const float2* __restrict__ E, KpArgs a, int XS,
+                                                                     int TH, const float2* __restrict__ gV,
+                                                                     KpPart part) {
+  extern __shared__ __align__(16) float2 kp_sm[];
+  grid_dep_wait();
+  grid_dep_release();
+  constexpr int TG = kKpTG;
+  const int Q = a.Q, Nf = a.Nf, N = a.N, T = a.T;
+  const int xl = threadIdx.x / Q, q = threadIdx.x - xl * Q;
+  const int x0 = blockIdx.x * XS, x = x0 + xl, w0 = blockIdx.z * WR;
+  const bool valid = x < N;
+  const int y0 = blockIdx.y * kKpYChunk, ny = min(kKpYChunk, N - y0);
+  const float2* Exy = E + a.e_off[kXY];
+  const float2* Exw = E + a.e_off[kXW];
+  const float2* Ext = E + a.e_off[kXT];
+  const float2* Eyw = E + a.e_off[kYW];
+  const float2* Eyt = E + a.e_off[kYT];
+  const float2* Ewt = E + a.e_off[kWT];
+  const float2* A = E + a.e_off[kKpPlanes];
+  const int gsz = TG * XS * WR;
+  float2* sG = kp_sm;                          // [2][frame][xl][w] grad V
+  float2* sR = sG + 2 * gsz;                   // [w][xl][q] dEyw terms of the current row
+  float2* sH = sR + (size_t)WR * XS * Q;       // [frame][w][q] Ewt of the current TH frames
+  const int nb = (T + TG - 1) / TG, nstep = ny * nb;  // batches of frames, row by row
+  // grad V of a batch: TG frames of PR 16-byte chunks, stepped as in the W kernel
+  const int PR = XS * WR / 2, f0 = threadIdx.x / PR, c0 = threadIdx.x - f0 * PR;
+  const int df = blockDim.x / PR, dc = blockDim.x - df * PR, cmax = (N - x0) * WR / 2;
+  const bool wide = ((uintptr_t)gV & 15) == 0;
+  auto fetch = [&](int y, int t0, int buf) {
+    const float2* src = gV + (((size_t)t0 * N + y) * N + x0) * Nf + w0;
+    float2* dst = sG + buf * gsz;
+    for (int tb = f0, c = c0; tb < TG;) {
+      const bool live = t0 + tb < T && c < cmax;
+      const int xx = 2 * c / WR;
+      copy16_async(dst + 2 * (tb * PR + c), src + (live ? (size_t)tb * N * N * Nf + xx * Nf + 2 * c % WR : 0), live, wide);
+      tb += df;
+      c += dc;
+      if (c >= PR) {
+        c -= PR;
+        ++tb;
+      }
+    }
+    copies_commit();
+  };
+  fetch(y0, 0, 0);
+  const float2 Aq = A[q];
+  float2 dxw[WR], acc[WR];
+#pragma unroll
+  for (int w = 0; w < WR; ++w) dxw[w] = acc[w] = make_float2(0.f, 0.f);
+  const int xq = x * Q + q, NQ = N * Q;
+  int y = y0, t0 = 0, th = 0;  // the batch: row, first frame, that frame's place among the staged ones
+  for (int step = 0; step < nstep; ++step) {
+    const int nt = min(TG, T - t0);
+    // conj(Exy Ext Eyt)'s factors of the batch
+    const float2 exy = valid ? Exy[y * NQ + xq] : make_float2(0.f, 0.f);
+    const float2* ext_t = Ext + (size_t)t0 * NQ + xq;
+    const float2* eyt_t = Eyt + (size_t)t0 * NQ + y * Q + q;
+    float2 u[TG];
+#pragma unroll
+    for (int tb = 0; tb < TG; ++tb) {
+      const int at = min(tb, nt - 1) * NQ;
+      u[tb] = valid ? kmul(ext_t[at], eyt_t[at]) : make_float2(0.f, 0.f);
+    }
+    if (th == 0 && (step == 0 || TH < T)) {
+      __syncthreads();  // the previous frames' Ewt have been read
+      const int nh = min(TH, T - t0);
+      for (int w = xl; w < WR; w += XS)
+        for (int tt = 0; tt < nh; ++tt) sH[(tt * WR + w) * QM + q] = Ewt[((size_t)(t0 + tt) * Nf + w0 + w) * Q + q];
+    }
+    copies_wait();
+    __syncthreads();
+    const int cy = y, ch = th;
+    t0 += TG;
+    th = th + TG == TH ? 0 : th + TG;
+    const bool row_end = t0 >= T;
+    if (row_end) {
+      t0 = th = 0;
+      ++y;
+    }
+    if (step + 1 < nstep) fetch(y, t0, (step + 1) & 1);
+    const float2* G = sG + (step & 1) * gsz + xl * WR;
+#pragma unroll
+    for (int tb = 0; tb < TG; ++tb) {
+      if (tb >= nt) break;
+      const float2 ua = kmul(exy, u[tb]);
+      const float4* g = reinterpret_cast<const float4*>(G + tb * XS * WR);
+      const float2* H = sH + (ch + tb) * (WR * QM) + q;
+#pragma unroll
+      for (int w = 0; w < WR; w += 2) {
+        const float4 gg = g[w / 2];
+        acc[w] = kcfma(H[w * QM], kcmul(ua, make_float2(gg.x, gg.y)), acc[w]);
+        acc[w + 1] = kcfma(H[(w + 1) * QM], kcmul(ua, make_float2(gg.z, gg.w)), acc[w + 1]);
+      }
+    }
+    if (!row_end) continue;
+    // the row's Tsum is in acc: fold it into the dExw chunk partial and sum
+    // the dEyw terms over the columns, in column order
+#pragma unroll
+    for (int w = 0; w < WR; ++w) {
+      const float2 ex = valid ? Exw[(x * Nf + w0 + w) * Q + q] : make_float2(0.f, 0.f);
+      dxw[w] = kcfma(kmul(Aq, Eyw[(cy * Nf + w0 + w) * Q + q]), acc[w], dxw[w]);
+      sR[w * XS * Q + threadIdx.x] = kcmul(kmul(Aq, ex), acc[w]);
+      acc[w] = make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < WR * Q; e += blockDim.x) {
+      const int w = e / Q, qq = e - w * Q;
+      float2 s = make_float2(0.f, 0.f);
+      for (int xx = 0; xx < XS; ++xx) s = kadd(s, sR[(w * XS + xx) * Q + qq]);
+      part.yw[(((size_t)blockIdx.x * N + cy) * Nf + w0 + w) * Q + qq] = s;
+    }
+    // (the next batch's barrier comes before sR is rewritten)
+  }
+  if (valid)
+#pragma unroll
+    for (int w = 0; w < WR; ++w) part.xw[(((size_t)blockIdx.y * N + x) * Nf + w0 + w) * Q + q] = dxw[w];
+}
+
 template <int QM>
 __global__ void __launch_bounds__(kKpThreads) kp_tgrad_kernel(const float2* __restrict__ E, KpArgs a, int XS, int TB,
                                                               const float2* __restrict__ gV, KpPart part) {
@@ -466,60 +763,91 @@ __global__ void __launch_bounds__(kKpThreads) kp_tgrad_kernel(const float2* __re
   }
 }
 
-__global__ void __launch_bounds__(kKpThreads) kp_xgrad_kernel(const float2* __restrict__ E, KpArgs a, int XS, int YB,
-                                                              const float2* __restrict__ gV, KpPart part) {
-  extern __shared__ float2 kp_sm[];
+// Thread (w, q), q fastest; strips of kKpXR columns whose Exw the thread keeps
+// in registers.  Per staged image row: U [xl][q] = Exy Ext Eyt, G [w][xl] =
+// grad V (two columns a load, rows kKpXR + 2 apart), Y [w][q] = Eyw.  A voxel
+// and q costs one load of U (shared by the bins of a warp) and half a load of
+// G for its two complex products.
+constexpr int kKpXR = 16;
+template <int QM>
+__global__ void __launch_bounds__(kKpThreads, 2) kp_xgrad_kernel(const float2* __restrict__ E, KpArgs a, int YB,
+                                                                 const float2* __restrict__ gV, KpPart part) {
+  extern __shared__ __align__(16) float2 kp_sm[];
   grid_dep_wait();
   grid_dep_release();
+  constexpr int XR = kKpXR, GS = XR + 2;
   const int Q = a.Q, Nf = a.Nf, N = a.N;
   const int t = blockIdx.y;
-  const int x0 = blockIdx.x * XS, nx = min(XS, N - x0);
+  const int x0 = blockIdx.x * XR;
   const float2* Exy = E + a.e_off[kXY];
   const float2* Exw = E + a.e_off[kXW];
   const float2* Ext = E + a.e_off[kXT];
   const float2* Eyw = E + a.e_off[kYW];
   const float2* Eyt = E + a.e_off[kYT];
-  // per staged row: U [xl][q] = Exy Ext Eyt, G [xl][w] = grad V, Y [w][q] = Eyw
-  const int usz = XS * Q, gsz = XS * Nf, ysz = Nf * Q, rsz = usz + gsz + ysz;
-  float2* sEw = kp_sm;                          // [xl][w][q] Exw of the strip
-  float2* sB = sEw + (size_t)XS * Nf * Q;       // 2 x YB staged rows
-  for (int e = threadIdx.x; e < nx * Nf * Q; e += blockDim.x) sEw[e] = Exw[(size_t)x0 * Nf * Q + e];
   const int npair = Nf * Q;
+  constexpr int usz = XR * QM;
+  const int gsz = Nf * GS, ysz = (npair + 1) & ~1, rsz = gsz + usz + ysz;
   for (int pb = 0; pb < npair; pb += blockDim.x) {  // (w, q) pairs of this pass
     const int e = pb + threadIdx.x;
     const bool own = e < npair;
     const int w = own ? e / Q : 0, q = own ? e - w * Q : 0;
+    float2 ew[XR];
+#pragma unroll
+    for (int xx = 0; xx < XR; ++xx)
+      ew[xx] = own && x0 + xx < N ? Exw[((size_t)(x0 + xx) * Nf + w) * Q + q] : make_float2(0.f, 0.f);
     float2 acc = make_float2(0.f, 0.f);
+    // grad V and Eyw of a batch of rows by asynchronous copies, U by products
+    auto fetch = [&](int yb, int buf) {
+      const int nyb = min(YB, N - yb);
+      float2* B = kp_sm + (size_t)buf * YB * rsz;
+      for (int c = threadIdx.x; c < XR * Nf; c += blockDim.x) {
+        const int xx = c / Nf, ww = c - xx * Nf;
+        const bool live = x0 + xx < N;
+        const float2* src = gV + (((size_t)t * N + yb) * N + (live ? x0 + xx : 0)) * Nf + ww;
+        float2* dst = B + ww * GS + xx;
+        for (int r = 0; r < nyb; ++r, src += N * Nf, dst += rsz) copy8_async(dst, src, live);
+      }
+      for (int c = threadIdx.x; c < npair; c += blockDim.x) {
+        const float2* src = Eyw + (size_t)yb * npair + c;
+        float2* dst = B + gsz + usz + c;
+        for (int r = 0; r < nyb; ++r, src += npair, dst += rsz) copy8_async(dst, src, true);
+      }
+      copies_commit();
+      for (int u = threadIdx.x; u < XR * Q; u += blockDim.x) {
+        const int xl = u / Q, xx = x0 + xl, qq = u - xl * Q;
+        const bool live = xx < N;
+        const float2 ext = live ? Ext[((size_t)t * N + xx) * Q + qq] : make_float2(0.f, 0.f);
+        const float2* exy = Exy + ((size_t)yb * N + (live ? xx : 0)) * Q + qq;
+        const float2* eyt = Eyt + ((size_t)t * N + yb) * Q + qq;
+        float2* dst = B + gsz + xl * QM + qq;
+#pragma unroll 4
+        for (int r = 0; r < nyb; ++r) dst[r * rsz] = kmul(kmul(exy[r * N * Q], ext), eyt[r * Q]);
+      }
+    };
+    fetch(0, 0);
     int buf = 0;
     for (int yb = 0; yb < N; yb += YB, buf ^= 1) {
       const int nyb = min(YB, N - yb);
-      float2* Bf = sB + (size_t)buf * YB * rsz;
-      for (int u = threadIdx.x; u < nx * Q; u += blockDim.x) {
-        const int xx = x0 + u / Q, qq = u % Q;
-        const float2 ext = Ext[((size_t)t * N + xx) * Q + qq];
-        for (int r = 0; r < nyb; ++r) {
-          const int y = yb + r;
-          Bf[(size_t)r * rsz + u] = kmul(kmul(Exy[((size_t)y * N + xx) * Q + qq], ext), Eyt[((size_t)t * N + y) * Q + qq]);
-        }
-      }
-      for (int u = threadIdx.x; u < nx * Nf; u += blockDim.x)
-        for (int r = 0; r < nyb; ++r)
-          Bf[(size_t)r * rsz + usz + u] = gV[(((size_t)t * N + yb + r) * N + x0) * Nf + u];
-      for (int u = threadIdx.x; u < ysz; u += blockDim.x)
-        for (int r = 0; r < nyb; ++r) Bf[(size_t)r * rsz + usz + gsz + u] = Eyw[(size_t)(yb + r) * Nf * Q + u];
-      __syncthreads();
+      copies_wait();
+      __syncthreads();  // this batch has arrived; the other buffer has been read
+      if (yb + YB < N) fetch(yb + YB, buf ^ 1);
       if (own)
         for (int r = 0; r < nyb; ++r) {
-          const float2* Ur = Bf + (size_t)r * rsz;
-          const float2* Gr = Ur + usz;
-          float2 sx = make_float2(0.f, 0.f);
-          for (int xx = 0; xx < nx; ++xx)
-            sx = kadd(sx, kcmul(kmul(sEw[((size_t)xx * Nf + w) * Q + q], Ur[xx * Q + q]), Gr[xx * Nf + w]));
-          acc = kadd(acc, kcmul(Gr[gsz + w * Q + q], sx));
+          const float2* B = kp_sm + (size_t)(buf * YB + r) * rsz;
+          const float4* g = reinterpret_cast<const float4*>(B + w * GS);
+          const float2* U = B + gsz + q;
+          float2 s0 = make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int xx = 0; xx < XR; xx += 2) {
+            const float4 gg = g[xx / 2];
+            s0 = kcfma(U[xx * QM], kcmul(ew[xx], make_float2(gg.x, gg.y)), s0);
+            s1 = kcfma(U[(xx + 1) * QM], kcmul(ew[xx + 1], make_float2(gg.z, gg.w)), s1);
+          }
+          acc = kcfma(B[gsz + usz + w * Q + q], kadd(s0, s1), acc);
         }
     }
     if (own) part.wt[(((size_t)blockIdx.x * a.T + t) * Nf + w) * Q + q] = acc;
-    __syncthreads();
+    __syncthreads();  // the buffers are refilled for the next pass
   }
 }
 
@@ -632,43 +960,59 @@ unsigned kp_blocks(size_t count, const Plan& p) {
 // Tile widths (image columns per CTA) and batch depths (frames or rows
 // staged per barrier) of the frame-walking kernels.
 struct KpTiles {
-  int xs_r, xs_w, xs_t, xs_x;  // render (thread per (x, w)), W (x, q), T (x, w), X (strip in shared memory)
+  int xs_r, xs_w, xs_t;             // columns per CTA: render, W, T
   int ns_r, ns_w, ns_t, ns_x, nch;  // strips of the render, W, T and X kernels; row chunks
-  int tb_r, tb_t, yb_x, yb_w;   // frames per barrier (render, T), rows per barrier (X, W)
+  int tb_r, tb_t, yb_x, yb_w;       // frames per barrier (render, T), rows per barrier (X, W)
+  int px, qm;                       // render: columns a thread, q of its registers
+  int wr_w, wr_t;                   // bins in registers: W kernel, T kernel (0: the general kernels)
+  int th;                           // T kernel with bins in registers: frames whose Ewt is staged at once
 };
 KpTiles kp_tiles(const Plan& p, int Q) {
   KpTiles k;
-  const int c8 = (int)sizeof(float2);
-  k.xs_r = std::max(1, std::min(std::min(p.N, 64), kKpThreads / p.Nf));
-  k.xs_t = k.xs_r;
-  k.xs_w = std::max(1, std::min(std::min(p.N, kKpThreads / Q), 8192 / (p.Nf * Q)));
-  k.xs_x = std::max(1, std::min(8, (96 * 1024) / ((p.Nf + 2) * Q * c8)));
+  const int c8 = (int)sizeof(float2), Nf = p.Nf;
+  // Bins in registers: exactly 8 or 16 for the W kernel (its sum runs over all
+  // of them), multiples of them for the T kernel, at least one whole warp.
+  k.wr_w = Nf == 16 || Nf == 8 ? Nf : 0;
+  k.wr_t = Nf % 16 == 0 ? 16 : Nf % 8 == 0 ? 8 : 0;
+  k.qm = Q <= 8 ? 8 : Q <= 16 ? 16 : 32;
+  k.px = Q <= 16 ? 2 : 1;
+  const int xh = std::max(1, std::min(std::min((p.N + k.px - 1) / k.px, 64), kKpThreads / Nf));
+  k.xs_r = k.px * xh;
+  const int xs_reg = std::max(1, std::min(std::min(p.N, kKpThreads / Q), 32));
+  k.xs_t = k.wr_t ? xs_reg : std::max(1, std::min(std::min(p.N, 64), kKpThreads / Nf));
+  k.xs_w = k.wr_w ? xs_reg : std::max(1, std::min(std::min(p.N, kKpThreads / Q), 8192 / (Nf * Q)));
   k.ns_r = (p.N + k.xs_r - 1) / k.xs_r;
   k.ns_w = (p.N + k.xs_w - 1) / k.xs_w;
   k.ns_t = (p.N + k.xs_t - 1) / k.xs_t;
-  k.ns_x = (p.N + k.xs_x - 1) / k.xs_x;
+  k.ns_x = (p.N + kKpXR - 1) / kKpXR;
   k.nch = (p.N + kKpYChunk - 1) / kKpYChunk;
-  const int per_frame = 2 * (p.Nf + k.xs_r) * Q * c8;  // double-buffered staging of one frame
-  k.tb_r = std::max(1, std::min(kKpTB, (96 * 1024) / per_frame));
-  k.tb_t = k.tb_r;
-  const int xrow = k.xs_x * Q + k.xs_x * p.Nf + p.Nf * Q;  // one staged row of the X kernel
-  k.yb_x = std::max(1, std::min(kKpTB, (64 * 1024) / (2 * xrow * c8)));
-  k.yb_w = std::max(1, std::min(kKpYChunk, 4096 / (p.Nf * Q)));
+  const int render_frame = 2 * (Nf * (k.qm + 2) + k.xs_r * k.qm) * c8;  // double-buffered staging of one frame
+  k.tb_r = std::max(1, std::min(kKpTB, (96 * 1024) / render_frame));
+  const int t_frame = 2 * (Nf + k.xs_t) * Q * c8;
+  k.tb_t = std::max(1, std::min(kKpTB, (96 * 1024) / t_frame));
+  k.th = k.wr_t ? std::max(1, 64 * 1024 / (k.wr_t * k.qm * c8) / kKpTG) * kKpTG : 1;
+  const int xrow = Nf * (kKpXR + 2) + kKpXR * k.qm + ((Nf * Q + 1) & ~1);  // one staged row of the X kernel
+  k.yb_x = std::max(1, std::min(kKpTB, (96 * 1024) / (2 * xrow * c8)));
+  k.yb_w = std::max(1, std::min(kKpYChunk, 4096 / (Nf * Q)));
   return k;
 }
-size_t smem_render(const Plan& p, const KpArgs& a, const KpTiles& k) {
-  return 2 * (size_t)k.tb_r * (p.Nf + k.xs_r) * a.Q * sizeof(float2);
+size_t smem_render(const Plan& p, const KpArgs&, const KpTiles& k) {
+  return 2 * (size_t)k.tb_r * (p.Nf * (k.qm + 2) + k.xs_r * k.qm) * sizeof(float2);
 }
 size_t smem_w(const Plan& p, const KpArgs& a, const KpTiles& k) {
-  return ((size_t)p.Nf * k.xs_w * a.Q + (size_t)k.yb_w * p.Nf * a.Q + (size_t)kKpYChunk * k.xs_w * a.Q) *
-         sizeof(float2);
+  const size_t xq = (size_t)k.xs_w * a.Q;
+  if (k.wr_w) return ((size_t)2 * kKpYChunk * k.xs_w * p.Nf + (size_t)kKpYChunk * p.Nf * k.qm + kKpYChunk * xq) * sizeof(float2);
+  return (p.Nf * xq + (size_t)k.yb_w * p.Nf * a.Q + kKpYChunk * xq) * sizeof(float2);
 }
 size_t smem_t(const Plan& p, const KpArgs& a, const KpTiles& k) {
+  if (k.wr_t)
+    return ((size_t)2 * kKpTG * k.xs_t * k.wr_t + (size_t)k.wr_t * k.xs_t * a.Q +
+            (size_t)std::min(k.th, (p.T + kKpTG - 1) / kKpTG * kKpTG) * k.wr_t * k.qm) * sizeof(float2);
   return (2 * (size_t)k.tb_t * (p.Nf * a.Q + k.xs_t * a.Q) + (size_t)a.Q * k.xs_t * p.Nf) * sizeof(float2);
 }
 size_t smem_x(const Plan& p, const KpArgs& a, const KpTiles& k) {
-  const size_t row = (size_t)k.xs_x * a.Q + (size_t)k.xs_x * p.Nf + (size_t)p.Nf * a.Q;
-  return ((size_t)k.xs_x * p.Nf * a.Q + 2 * (size_t)k.yb_x * row) * sizeof(float2);
+  const size_t row = (size_t)p.Nf * (kKpXR + 2) + kKpXR * k.qm + ((p.Nf * a.Q + 1) & ~1);
+  return 2 * (size_t)k.yb_x * row * sizeof(float2);
 }
 
 // Device workspace of the model (the expanded planes, their gradients and
@@ -739,14 +1083,35 @@ cudaError_t kp_configure(const Plan& p, const KpArgs& a) {
       e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
   const size_t sr = smem_render(p, a, k), st = smem_t(p, a, k);
-  opt((const void*)kp_render_kernel<8>, sr);
-  opt((const void*)kp_render_kernel<16>, sr);
-  opt((const void*)kp_render_kernel<32>, sr);
-  opt((const void*)kp_tgrad_kernel<8>, st);
-  opt((const void*)kp_tgrad_kernel<16>, st);
-  opt((const void*)kp_tgrad_kernel<32>, st);
-  opt((const void*)kp_wgrad_kernel, smem_w(p, a, k));
-  opt((const void*)kp_xgrad_kernel, smem_x(p, a, k));
+  opt((const void*)kp_render_kernel<8, 2>, sr);
+  opt((const void*)kp_render_kernel<16, 2>, sr);
+  opt((const void*)kp_render_kernel<32, 1>, sr);
+  if (k.wr_t) {
+    opt((const void*)kp_tgrad_reg_kernel<8, 8>, st);
+    opt((const void*)kp_tgrad_reg_kernel<8, 16>, st);
+    opt((const void*)kp_tgrad_reg_kernel<8, 32>, st);
+    opt((const void*)kp_tgrad_reg_kernel<16, 8>, st);
+    opt((const void*)kp_tgrad_reg_kernel<16, 16>, st);
+    opt((const void*)kp_tgrad_reg_kernel<16, 32>, st);
+  } else {
+    opt((const void*)kp_tgrad_kernel<8>, st);
+    opt((const void*)kp_tgrad_kernel<16>, st);
+    opt((const void*)kp_tgrad_kernel<32>, st);
+  }
+  if (k.wr_w) {
+    const size_t sw = smem_w(p, a, k);
+    opt((const void*)kp_wgrad_reg_kernel<8, 8>, sw);
+    opt((const void*)kp_wgrad_reg_kernel<8, 16>, sw);
+    opt((const void*)kp_wgrad_reg_kernel<8, 32>, sw);
+    opt((const void*)kp_wgrad_reg_kernel<16, 8>, sw);
+    opt((const void*)kp_wgrad_reg_kernel<16, 16>, sw);
+    opt((const void*)kp_wgrad_reg_kernel<16, 32>, sw);
+  } else {
+    opt((const void*)kp_wgrad_kernel, smem_w(p, a, k));
+  }
+  opt((const void*)kp_xgrad_kernel<8>, smem_x(p, a, k));
+  opt((const void*)kp_xgrad_kernel<16>, smem_x(p, a, k));
+  opt((const void*)kp_xgrad_kernel<32>, smem_x(p, a, k));
   return e;
 }
 
@@ -755,25 +1120,45 @@ cudaError_t kp_expand(Plan& p, const KpArgs& a, const KpWork& w, const float2* P
   return launch_dep(kp_expand_kernel, dim3(kp_blocks(a.e_count, p)), dim3(kKpThreads), 0, s, P, a, w.E);
 }
 
-template <int QM>
+template <int QM, int PX>
 cudaError_t launch_render_q(const Plan& p, const KpArgs& a, const KpWork& w, float2* V, cudaStream_t s) {
   const KpTiles k = kp_tiles(p, a.Q);
-  return launch_dep(kp_render_kernel<QM>, dim3(k.ns_r, p.N), dim3(k.xs_r * p.Nf), smem_render(p, a, k), s,
+  return launch_dep(kp_render_kernel<QM, PX>, dim3(k.ns_r, p.N), dim3(k.xs_r / PX * p.Nf), smem_render(p, a, k), s,
                     (const float2*)w.E, a, k.xs_r, k.tb_r, V);
 }
 
 cudaError_t kp_render(Plan& p, const KpArgs& a, const KpWork& w, float2* V, cudaStream_t s) {
   StageScope sc(p, kStKpRender, s);
-  if (a.Q <= 8) return launch_render_q<8>(p, a, w, V, s);
-  if (a.Q <= 16) return launch_render_q<16>(p, a, w, V, s);
-  return launch_render_q<32>(p, a, w, V, s);
+  if (a.Q <= 8) return launch_render_q<8, 2>(p, a, w, V, s);
+  if (a.Q <= 16) return launch_render_q<16, 2>(p, a, w, V, s);
+  return launch_render_q<32, 1>(p, a, w, V, s);
 }
 
+// The W, T and X kernels for Q <= QM.
 template <int QM>
-cudaError_t launch_tgrad_q(const Plan& p, const KpArgs& a, const KpWork& w, const float2* gV, cudaStream_t s) {
+cudaError_t launch_grads_q(const Plan& p, const KpArgs& a, const KpWork& w, const float2* gV, cudaStream_t s) {
   const KpTiles k = kp_tiles(p, a.Q);
-  return launch_dep(kp_tgrad_kernel<QM>, dim3(k.ns_t, k.nch), dim3(k.xs_t * p.Nf), smem_t(p, a, k), s,
-                    (const float2*)w.E, a, k.xs_t, k.tb_t, gV, w.part);
+  const float2* E = w.E;
+  const dim3 gw(k.ns_w, k.nch), bw(k.xs_w * a.Q);
+  const size_t mw = smem_w(p, a, k), mt = smem_t(p, a, k);
+  cudaError_t e;
+  if (k.wr_w == 16)
+    e = launch_dep(kp_wgrad_reg_kernel<16, QM>, gw, bw, mw, s, E, a, k.xs_w, gV, w.dE, w.part);
+  else if (k.wr_w == 8)
+    e = launch_dep(kp_wgrad_reg_kernel<8, QM>, gw, bw, mw, s, E, a, k.xs_w, gV, w.dE, w.part);
+  else
+    e = launch_dep(kp_wgrad_kernel, gw, bw, mw, s, E, a, k.xs_w, k.yb_w, gV, w.dE, w.part);
+  if (e != cudaSuccess) return e;
+  const dim3 gt(k.ns_t, k.nch, k.wr_t ? p.Nf / k.wr_t : 1);
+  if (k.wr_t == 16)
+    e = launch_dep(kp_tgrad_reg_kernel<16, QM>, gt, dim3(k.xs_t * a.Q), mt, s, E, a, k.xs_t, k.th, gV, w.part);
+  else if (k.wr_t == 8)
+    e = launch_dep(kp_tgrad_reg_kernel<8, QM>, gt, dim3(k.xs_t * a.Q), mt, s, E, a, k.xs_t, k.th, gV, w.part);
+  else
+    e = launch_dep(kp_tgrad_kernel<QM>, gt, dim3(k.xs_t * p.Nf), mt, s, E, a, k.xs_t, k.tb_t, gV, w.part);
+  if (e != cudaSuccess) return e;
+  return launch_dep(kp_xgrad_kernel<QM>, dim3(k.ns_x, p.T), dim3(kKpThreads), smem_x(p, a, k), s, E, a, k.yb_x, gV,
+                    w.part);
 }
 
 // Parameter gradients G from grad V, with w.E holding the expanded planes.
@@ -783,14 +1168,12 @@ cudaError_t kp_vjp(Plan& p, const KpArgs& a, const KpWork& w, const float2* gV, 
   const KpTiles k = kp_tiles(p, a.Q);
   const float2* A = w.E + a.e_off[kKpPlanes];
   cudaError_t e;
-  e = launch_dep(kp_wgrad_kernel, dim3(k.ns_w, k.nch), dim3(k.xs_w * a.Q), smem_w(p, a, k), s, (const float2*)w.E,
-                 a, k.xs_w, k.yb_w, gV, w.dE, w.part);
-  if (e != cudaSuccess) return e;
-  e = a.Q <= 8 ? launch_tgrad_q<8>(p, a, w, gV, s)
-               : a.Q <= 16 ? launch_tgrad_q<16>(p, a, w, gV, s) : launch_tgrad_q<32>(p, a, w, gV, s);
-  if (e != cudaSuccess) return e;
-  e = launch_dep(kp_xgrad_kernel, dim3(k.ns_x, p.T), dim3(kKpThreads), smem_x(p, a, k), s, (const float2*)w.E, a,
-                 k.xs_x, k.yb_x, gV, w.part);
+  if (a.Q <= 8)
+    e = launch_grads_q<8>(p, a, w, gV, s);
+  else if (a.Q <= 16)
+    e = launch_grads_q<16>(p, a, w, gV, s);
+  else
+    e = launch_grads_q<32>(p, a, w, gV, s);
   if (e != cudaSuccess) return e;
   const size_t lxt = (size_t)p.T * p.N * a.Q, lxw = (size_t)p.N * p.Nf * a.Q;
   e = launch_dep(kp_sum_kernel, dim3(kp_blocks(lxt, p)), dim3(kKpThreads), 0, s, (const float2*)w.part.xt, k.nch,
