@@ -5,6 +5,7 @@
 #include "prop_internal.cuh"
 
 #include <cmath>
+#include <cstring>
 #include <algorithm>
 
 namespace prop {
@@ -73,6 +74,24 @@ prop_status check_device_status(Plan& p) {
     return fail(PROP_ERR_TIMEOUT, "a bounded device-side wait expired (grid tile staging did not complete)");
   }
   return PROP_OK;
+}
+
+// Copies `count` doubles of a call's result to the host, synchronises and
+// reports an expired bounded wait.  A single value and the status word go
+// through the plan's pinned words, so that the call waits for the device once.
+prop_status finish_call(Plan& p, double* host, const double* dev, int count, cudaStream_t s) {
+  if (count == 1 && p.host_words) {
+    PROP_CUDA(cudaMemcpyAsync(p.host_words, dev, sizeof(double), cudaMemcpyDeviceToHost, s));
+    PROP_CUDA(cudaMemcpyAsync(p.host_words + 1, p.status_dev, sizeof(int), cudaMemcpyDeviceToHost, s));
+    PROP_CUDA(cudaStreamSynchronize(s));
+    int st = 0;
+    std::memcpy(&st, p.host_words + 1, sizeof(int));
+    *host = p.host_words[0];
+    return st ? check_device_status(p) : PROP_OK;
+  }
+  PROP_CUDA(cudaMemcpyAsync(host, dev, sizeof(double) * count, cudaMemcpyDeviceToHost, s));
+  PROP_CUDA(cudaStreamSynchronize(s));
+  return check_device_status(p);
 }
 
 // y = A V, or r = A V - y_meas with |r|^2 reduced into *sumsq.  rows_ready:
@@ -256,6 +275,20 @@ prop_status loss_grad_device(Plan& p, const float2* y, const AdamArgs& a, const 
                              double* loss_out, cudaStream_t s) {
   prop_status st;
   if ((st = forward_impl(p, V, p.resid, y, &p.red_interp, p.scalars, s)) != PROP_OK) return st;
+  if (p.nchunks == 1) {  // the last adjoint pass and the TV gradient as one kernel
+    p.rows_of = nullptr;  // the adjoint passes overwrite the row workspace
+    {
+      StageScope sc(p, kStSpread, s);
+      PROP_LAUNCH(spread(p, 0, p.Nf, p.resid, true, s));
+    }
+    {
+      StageScope sc(p, kStAdjCols, s);
+      PROP_LAUNCH(fft_adjoint_cols(p, s));
+    }
+    StageScope sc(p, kStFused, s);
+    PROP_LAUNCH(fused_rows_grad(p, V, grad, a, &p.red_tv, p.scalars, loss_out, s));
+    return PROP_OK;
+  }
   if ((st = adjoint_impl(p, p.resid, p.grad, true, s)) != PROP_OK) return st;
   StageScope sc(p, kStOpt, s);
   PROP_LAUNCH(tv_grad(p, V, p.grad, grad, a, &p.red_tv, p.scalars, loss_out, s));
@@ -531,23 +564,15 @@ prop_status prop_loss_grad(prop_plan plan, const void* y_dev, const prop_recon_p
   cudaStream_t s = (cudaStream_t)stream;
   prop_status st = plan_ensure_recon(&p, 1);
   if (st != PROP_OK) return st;
-  if ((st = forward_impl(p, (const float2*)V_dev, p.resid, (const float2*)y_dev, &p.red_interp, p.scalars, s)) != PROP_OK)
-    return st;
-  if ((st = adjoint_impl(p, p.resid, p.grad, true, s)) != PROP_OK) return st;
   AdamArgs a{};
   a.tv_xy = params->tv_xy;
   a.tv_t = params->tv_t;
   a.tv_eps = params->tv_eps;
   a.gscale = 2.f;
   float2* out = grad_dev ? (float2*)grad_dev : p.grad;
-  {
-    StageScope sc(p, kStOpt, s);
-    PROP_LAUNCH(tv_grad(p, (const float2*)V_dev, p.grad, out, a, &p.red_tv, p.scalars, p.scalars + 1, s));
-  }
-  PROP_CUDA(cudaMemcpyAsync(loss_host, p.scalars + 1, sizeof(double), cudaMemcpyDeviceToHost, s));
-  PROP_CUDA(cudaStreamSynchronize(s));
-  if ((st = check_device_status(p)) != PROP_OK) return st;
-  return PROP_OK;
+  if ((st = loss_grad_device(p, (const float2*)y_dev, a, (const float2*)V_dev, out, p.scalars + 1, s)) != PROP_OK)
+    return st;
+  return finish_call(p, loss_host, p.scalars + 1, 1, s);
 }
 
 prop_status prop_render(prop_plan plan, const void* V_dev, int f_lo, int f_hi, void* image_dev, void* stream) {

@@ -165,6 +165,8 @@ __global__ void __launch_bounds__(kInterpThreads, 1) interp_kernel(InterpArgs a)
     s_abort = 0;
   }
   __syncthreads();
+  grid_dep_wait();
+  grid_dep_release();
   if (threadIdx.x == 0)
     for (int b = 0; b < a.nbuf; ++b) {
       const int item = blockIdx.x + b * gridDim.x;
@@ -641,6 +643,8 @@ __global__ void __launch_bounds__(QuadShape<CS, W>::THREADS, 1) quads_multi_kern
 template <int LP>
 __global__ void __launch_bounds__(256) phase_expand_kernel(const float2* r, const float2* phase, float2* contrib,
                                                             int M, int R, int Nf, int C, int Cv, int f0) {
+  grid_dep_wait();
+  grid_dep_release();
   constexpr int SPW = 32 / LP;
   const int lane = threadIdx.x & 31;
   const int sub = lane & (LP - 1);
@@ -664,6 +668,8 @@ __global__ void __launch_bounds__(256) resid_expand_kernel(const float2* y_sum, 
                                                             const float2* phase, float2* contrib, int M, int R,
                                                             int Nf, int C, int Cv, int f0, double* partials,
                                                             unsigned int* counter, double* sumsq_out) {
+  grid_dep_wait();
+  grid_dep_release();
   constexpr int SPW = 32 / LP;
   const int lane = threadIdx.x & 31;
   const int sub = lane & (LP - 1);
@@ -1048,6 +1054,8 @@ __global__ void __launch_bounds__(kSpreadThreads, kSpreadCtasPerSm)
 template <int LP>
 __global__ void __launch_bounds__(256) spread_global_kernel(float2* grid, const float2* contrib, const int4* sitems,
                                                             const int2* blob, int n_items, int C, int Cv) {
+  grid_dep_wait();
+  grid_dep_release();
   constexpr int CPW = 32 / LP;
   const int lane = threadIdx.x & 31;
   const int sub = lane & (LP - 1);
@@ -1110,15 +1118,15 @@ unsigned grid_for(long items, long per_block, long cap) {
 
 template <int W>
 cudaError_t launch_interp(int lp, const InterpArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
+  const dim3 block(kInterpThreads);
   switch (lp) {
-    case 1: interp_kernel<1, W><<<grid, kInterpThreads, smem, s>>>(a); break;
-    case 2: interp_kernel<2, W><<<grid, kInterpThreads, smem, s>>>(a); break;
-    case 4: interp_kernel<4, W><<<grid, kInterpThreads, smem, s>>>(a); break;
-    case 8: interp_kernel<8, W><<<grid, kInterpThreads, smem, s>>>(a); break;
-    case 16: interp_kernel<16, W><<<grid, kInterpThreads, smem, s>>>(a); break;
-    default: interp_kernel<32, W><<<grid, kInterpThreads, smem, s>>>(a); break;
+    case 1: return launch_dep(interp_kernel<1, W>, grid, block, smem, s, a);
+    case 2: return launch_dep(interp_kernel<2, W>, grid, block, smem, s, a);
+    case 4: return launch_dep(interp_kernel<4, W>, grid, block, smem, s, a);
+    case 8: return launch_dep(interp_kernel<8, W>, grid, block, smem, s, a);
+    case 16: return launch_dep(interp_kernel<16, W>, grid, block, smem, s, a);
+    default: return launch_dep(interp_kernel<32, W>, grid, block, smem, s, a);
   }
-  return cudaGetLastError();
 }
 
 template <int W>
@@ -1364,33 +1372,37 @@ cudaError_t residual(const Plan& p, const float2* y_sum, const float2* y_meas, f
   const int lp = lanes_for(nbins);
   dim3 g(grid_for(p.M, 8L * (32 / lp), std::min(red.capacity, 16384)));
   float2* contrib = with_contrib ? p.contrib : nullptr;
-  switch (lp) {
 #define RE(L)                                                                                              \
-  case L:                                                                                                  \
-    resid_expand_kernel<L><<<g, 256, 0, s>>>(y_sum, y_meas, r, p.phase, contrib, p.M, p.R, p.Nf, p.cs, nbins, \
-                                             0, red.partials, red.counter, sumsq);                          \
-    break;
-    RE(1) RE(2) RE(4) RE(8) RE(16)
-    default:
-      resid_expand_kernel<32><<<g, 256, 0, s>>>(y_sum, y_meas, r, p.phase, contrib, p.M, p.R, p.Nf, p.cs, nbins, 0,
-                                                red.partials, red.counter, sumsq);
-#undef RE
+  return launch_dep(resid_expand_kernel<L>, g, dim3(256), 0, s, y_sum, y_meas, r, (const float2*)p.phase, contrib, p.M, \
+                    p.R, p.Nf, p.cs, nbins, 0, red.partials, red.counter, sumsq)
+  switch (lp) {
+    case 1: RE(1);
+    case 2: RE(2);
+    case 4: RE(4);
+    case 8: RE(8);
+    case 16: RE(16);
+    default: RE(32);
   }
-  return cudaGetLastError();
+#undef RE
 }
 
 cudaError_t spread(const Plan& p, int f0, int nbins, const float2* r, bool contrib_ready, cudaStream_t s) {
   const int lp = lanes_for(nbins);
   if (!contrib_ready) {
     dim3 g(grid_for(p.M, 8L * (32 / lp), 16384));
+    cudaError_t e;
+#define PE(L)                                                                                              \
+  e = launch_dep(phase_expand_kernel<L>, g, dim3(256), 0, s, r, (const float2*)p.phase, p.contrib, p.M, p.R, p.Nf, p.cs, \
+                 nbins, f0)
     switch (lp) {
-#define PE(L) \
-  case L: phase_expand_kernel<L><<<g, 256, 0, s>>>(r, p.phase, p.contrib, p.M, p.R, p.Nf, p.cs, nbins, f0); break;
-      PE(1) PE(2) PE(4) PE(8) PE(16)
-      default: phase_expand_kernel<32><<<g, 256, 0, s>>>(r, p.phase, p.contrib, p.M, p.R, p.Nf, p.cs, nbins, f0);
-#undef PE
+      case 1: PE(1); break;
+      case 2: PE(2); break;
+      case 4: PE(4); break;
+      case 8: PE(8); break;
+      case 16: PE(16); break;
+      default: PE(32);
     }
-    cudaError_t e = cudaGetLastError();
+#undef PE
     if (e != cudaSuccess) return e;
   }
   if (p.n_sitems == 0) return cudaSuccess;
@@ -1426,18 +1438,19 @@ cudaError_t spread(const Plan& p, int f0, int nbins, const float2* r, bool contr
 #undef SS
   } else {
     dim3 g((unsigned)std::max(1, std::min(p.n_sitems, 65535)));
-#define SG(L) spread_global_kernel<L><<<g, 256, 0, s>>>(p.grid, p.contrib, p.sitems, p.sblob, p.n_sitems, p.cs, nbins)
+#define SG(L)                                                                                              \
+  return launch_dep(spread_global_kernel<L>, g, dim3(256), 0, s, p.grid, (const float2*)p.contrib, (const int4*)p.sitems, \
+                    (const int2*)p.sblob, p.n_sitems, p.cs, nbins)
     switch (lanes_for((p.cs + 1) / 2)) {
-      case 1: SG(1); break;
-      case 2: SG(2); break;
-      case 4: SG(4); break;
-      case 8: SG(8); break;
-      case 16: SG(16); break;
-      default: SG(32); break;
+      case 1: SG(1);
+      case 2: SG(2);
+      case 4: SG(4);
+      case 8: SG(8);
+      case 16: SG(16);
+      default: SG(32);
     }
 #undef SG
   }
-  return cudaGetLastError();
 }
 
 }  // namespace prop

@@ -57,6 +57,8 @@ template <bool ADAM>
 __global__ void __launch_bounds__(kOptThreads) opt_kernel(OptArgs a) {
   // Work unit: a segment of kSeg consecutive values of one image row (t, i2);
   // a row holds N * Nf values (i1, f).
+  grid_dep_wait();
+  grid_dep_release();
   const float eps2 = a.p.tv_eps * a.p.tv_eps;
   const int rowlen = a.N * a.Nf;
   const int segs = (rowlen + kSeg - 1) / kSeg;
@@ -181,15 +183,13 @@ cudaError_t tv_adam(const Plan& p, const float2* Vin, const float2* g, float2* m
   OptArgs a = make_args(p, Vin, g, Vout, aa, red, data_loss, loss_out);
   a.m = m;
   a.v = v;
-  opt_kernel<true><<<opt_blocks(p, red), kOptThreads, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(opt_kernel<true>, dim3(opt_blocks(p, red)), dim3(kOptThreads), 0, s, a);
 }
 
 cudaError_t tv_grad(const Plan& p, const float2* V, const float2* g, float2* grad, const AdamArgs& aa,
                     const Reducer* red, const double* data_loss, double* loss_out, cudaStream_t s) {
   OptArgs a = make_args(p, V, g, grad, aa, red, data_loss, loss_out);
-  opt_kernel<false><<<opt_blocks(p, red), kOptThreads, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(opt_kernel<false>, dim3(opt_blocks(p, red)), dim3(kOptThreads), 0, s, a);
 }
 
 cudaError_t psnr(const Plan& p, const float2* img, const float2* ref, long count, double* out, cudaStream_t s) {

@@ -347,6 +347,7 @@ void plan_free(Plan* p) {
                   p->red_proj_k.partials, p->red_proj_k.counter, p->red_proj_u.partials, p->red_proj_u.counter,
                   p->psnr_scratch, p->kp_work};
   for (void* q : ptrs) plan_dev_free(p, q);
+  if (p->host_words) cudaFreeHost(p->host_words);
   for (cudaEvent_t e : p->ev_pool) cudaEventDestroy(e);
   for (auto& v : p->ev_rec)
     for (auto& pr : v) {
@@ -795,6 +796,10 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
     }
   }
   TRY(tab(&p->status_dev, 1, "status word"));
+  if (!alloc && cudaHostAlloc((void**)&p->host_words, 2 * sizeof(double), cudaHostAllocDefault) != cudaSuccess) {
+    cudaGetLastError();
+    p->host_words = nullptr;  // the calls then copy into pageable memory
+  }
   if (p->spread_claimed) TRY(tab(&p->spread_claim, 2, "spread item counter"));
   {
     cudaError_t e = cudaMemset(p->status_dev, 0, sizeof(int));

@@ -179,6 +179,10 @@ struct Plan {
   int num_sms = 1;               // streaming multiprocessors of the device
   int smem_optin = 48 * 1024;    // largest opt-in shared memory per block (bytes)
   int* status_dev = nullptr;     // device status word: 1 = a bounded device wait expired
+  // Pinned host words that a call's loss and the status word are copied into
+  // before its one synchronisation (null with a request server's allocator:
+  // pinning memory may wait for the device)
+  double* host_words = nullptr;
   int chunk = 0;                 // bins per grid pass
   int cs = 0;                    // bin stride of the grid workspaces (chunk rounded up to even)
   int nchunks = 0;
@@ -484,6 +488,10 @@ prop_status batch_step(BatchMember* mb, int count, cudaStream_t s);
 cudaError_t fused_rows_update(const Plan& p, const float2* Vin, float2* m, float2* v, float2* Vout,
                               const AdamArgs& aa, const Reducer* red, const double* data_loss, double* loss_out,
                               bool fwd_tail, cudaStream_t s);
+// The same inverse row FFT fused with the TV gradient: grad = gscale (adjoint) + TV grads at V,
+// loss as in tv_adam.
+cudaError_t fused_rows_grad(const Plan& p, const float2* V, float2* grad, const AdamArgs& aa, const Reducer* red,
+                            const double* data_loss, double* loss_out, cudaStream_t s);
 
 }  // namespace prop
 
