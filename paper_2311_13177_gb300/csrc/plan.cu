@@ -245,7 +245,11 @@ void build_quads(const Plan& p, const std::vector<int>& first_tap, const std::ve
   std::vector<int> row0(qs.size());  // first row of each quad's item
   std::vector<long> upto;            // cost up to and with each item
   long total = 0;
-  const int span = quad_span(p.cs, W), most = quad_item(p.cs);
+  // Small problems take smaller items (of whole units), so that every CTA has
+  // one: 5 blades of 8 x 32 samples in 8 bins 12.3 -> 8.6 us, 8 blades of 16 x
+  // 64 samples 15.8 -> 13.8 us.
+  const int per = quad_per_warp(p.cs), fair = ((int)qs.size() + ctas - 1) / ctas;
+  const int span = quad_span(p.cs, W), most = std::min(quad_item(p.cs), (fair + per - 1) / per * per);
   size_t blocks = 0;
   for (uint64_t u : p.grid_used_h) blocks += (size_t)__builtin_popcountll(u);
   const bool in_l2 = blocks * 2 * kGridBlock * p.cs * sizeof(float2) < (size_t)100 << 20;
