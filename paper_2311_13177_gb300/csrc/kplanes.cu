@@ -769,8 +769,11 @@ __global__ void __launch_bounds__(kKpThreads) kp_tgrad_kernel(const float2* __re
 // and q costs one load of U (shared by the bins of a warp) and half a load of
 // G for its two complex products.
 constexpr int kKpXR = 16;
+// Grid z: runs of YR image rows, as many as fill the last wave of CTAs best
+// (one run a frame and strip left 37 % of the CTA slots of two waves idle at
+// 192^2 x 32 frames; all parameter gradients of that size 790 -> 724 us).
 template <int QM>
-__global__ void __launch_bounds__(kKpThreads, 2) kp_xgrad_kernel(const float2* __restrict__ E, KpArgs a, int YB,
+__global__ void __launch_bounds__(kKpThreads, 2) kp_xgrad_kernel(const float2* __restrict__ E, KpArgs a, int YB, int YR,
                                                                  const float2* __restrict__ gV, KpPart part) {
   extern __shared__ __align__(16) float2 kp_sm[];
   grid_dep_wait();
@@ -779,6 +782,7 @@ __global__ void __launch_bounds__(kKpThreads, 2) kp_xgrad_kernel(const float2* _
   const int Q = a.Q, Nf = a.Nf, N = a.N;
   const int t = blockIdx.y;
   const int x0 = blockIdx.x * XR;
+  const int y0 = blockIdx.z * YR, y1 = min(N, y0 + YR);
   const float2* Exy = E + a.e_off[kXY];
   const float2* Exw = E + a.e_off[kXW];
   const float2* Ext = E + a.e_off[kXT];
@@ -798,7 +802,7 @@ __global__ void __launch_bounds__(kKpThreads, 2) kp_xgrad_kernel(const float2* _
     float2 acc = make_float2(0.f, 0.f);
     // grad V and Eyw of a batch of rows by asynchronous copies, U by products
     auto fetch = [&](int yb, int buf) {
-      const int nyb = min(YB, N - yb);
+      const int nyb = min(YB, y1 - yb);
       float2* B = kp_sm + (size_t)buf * YB * rsz;
       for (int c = threadIdx.x; c < XR * Nf; c += blockDim.x) {
         const int xx = c / Nf, ww = c - xx * Nf;
@@ -824,13 +828,13 @@ __global__ void __launch_bounds__(kKpThreads, 2) kp_xgrad_kernel(const float2* _
         for (int r = 0; r < nyb; ++r) dst[r * rsz] = kmul(kmul(exy[r * N * Q], ext), eyt[r * Q]);
       }
     };
-    fetch(0, 0);
+    fetch(y0, 0);
     int buf = 0;
-    for (int yb = 0; yb < N; yb += YB, buf ^= 1) {
-      const int nyb = min(YB, N - yb);
+    for (int yb = y0; yb < y1; yb += YB, buf ^= 1) {
+      const int nyb = min(YB, y1 - yb);
       copies_wait();
       __syncthreads();  // this batch has arrived; the other buffer has been read
-      if (yb + YB < N) fetch(yb + YB, buf ^ 1);
+      if (yb + YB < y1) fetch(yb + YB, buf ^ 1);
       if (own)
         for (int r = 0; r < nyb; ++r) {
           const float2* B = kp_sm + (size_t)(buf * YB + r) * rsz;
@@ -846,7 +850,7 @@ __global__ void __launch_bounds__(kKpThreads, 2) kp_xgrad_kernel(const float2* _
           acc = kcfma(B[gsz + usz + w * Q + q], kadd(s0, s1), acc);
         }
     }
-    if (own) part.wt[(((size_t)blockIdx.x * a.T + t) * Nf + w) * Q + q] = acc;
+    if (own) part.wt[((((size_t)blockIdx.z * gridDim.x + blockIdx.x) * a.T + t) * Nf + w) * Q + q] = acc;
     __syncthreads();  // the buffers are refilled for the next pass
   }
 }
@@ -965,6 +969,7 @@ struct KpTiles {
   int tb_r, tb_t, yb_x, yb_w;       // frames per barrier (render, T), rows per barrier (X, W)
   int px, qm;                       // render: columns a thread, q of its registers
   int wr_w, wr_t;                   // bins in registers: W kernel, T kernel (0: the general kernels)
+  int nyr_x, yr_x;                  // X kernel: runs of image rows, rows of a run
   int th;                           // T kernel with bins in registers: frames whose Ewt is staged at once
 };
 KpTiles kp_tiles(const Plan& p, int Q) {
@@ -994,6 +999,20 @@ KpTiles kp_tiles(const Plan& p, int Q) {
   const int xrow = Nf * (kKpXR + 2) + kKpXR * k.qm + ((Nf * Q + 1) & ~1);  // one staged row of the X kernel
   k.yb_x = std::max(1, std::min(kKpTB, (96 * 1024) / (2 * xrow * c8)));
   k.yb_w = std::max(1, std::min(kKpYChunk, 4096 / (Nf * Q)));
+  // X kernel: up to four runs of rows (of at least four batches each), the
+  // count whose last wave of two CTAs per SM is the fullest
+  k.nyr_x = 1;
+  double best = 0.0;
+  for (int r = 1; r <= 4 && (r == 1 || p.N / r >= 4 * k.yb_x); ++r) {
+    const double waves = (double)k.ns_x * p.T * r / (2.0 * p.num_sms);
+    const double fill = waves / std::ceil(waves);
+    if (fill > best + 0.05) {
+      best = fill;
+      k.nyr_x = r;
+    }
+  }
+  k.yr_x = (p.N + k.nyr_x - 1) / k.nyr_x;
+  k.nyr_x = (p.N + k.yr_x - 1) / k.yr_x;
   return k;
 }
 size_t smem_render(const Plan& p, const KpArgs&, const KpTiles& k) {
@@ -1026,7 +1045,7 @@ struct KpWork {
 size_t kp_part_elems(const Plan& p, const KpArgs& a, const KpTiles& k, size_t* off) {
   const size_t Q = a.Q, N = p.N, Nf = p.Nf, T = p.T;
   const size_t sz[5] = {k.nch * T * N * Q, k.ns_w * T * N * Q, k.nch * N * Nf * Q, k.ns_t * N * Nf * Q,
-                        k.ns_x * T * Nf * Q};
+                        (size_t)k.nyr_x * k.ns_x * T * Nf * Q};
   size_t o = 0;
   for (int i = 0; i < 5; ++i) {
     if (off) off[i] = o;
@@ -1157,8 +1176,8 @@ cudaError_t launch_grads_q(const Plan& p, const KpArgs& a, const KpWork& w, cons
   else
     e = launch_dep(kp_tgrad_kernel<QM>, gt, dim3(k.xs_t * p.Nf), mt, s, E, a, k.xs_t, k.tb_t, gV, w.part);
   if (e != cudaSuccess) return e;
-  return launch_dep(kp_xgrad_kernel<QM>, dim3(k.ns_x, p.T), dim3(kKpThreads), smem_x(p, a, k), s, E, a, k.yb_x, gV,
-                    w.part);
+  return launch_dep(kp_xgrad_kernel<QM>, dim3(k.ns_x, p.T, k.nyr_x), dim3(kKpThreads), smem_x(p, a, k), s, E, a, k.yb_x,
+                    k.yr_x, gV, w.part);
 }
 
 // Parameter gradients G from grad V, with w.E holding the expanded planes.
@@ -1188,7 +1207,7 @@ cudaError_t kp_vjp(Plan& p, const KpArgs& a, const KpWork& w, const float2* gV, 
   e = launch_dep(kp_sum_kernel, dim3(kp_blocks(lxw, p)), dim3(kKpThreads), 0, s, (const float2*)w.part.yw, k.ns_t,
                  lxw, A, a.Q, 0, w.dE + a.e_off[kYW]);
   if (e != cudaSuccess) return e;
-  e = launch_dep(kp_dwt_kernel, dim3(a.Q), dim3(kKpThreads), 0, s, (const float2*)w.E, a, k.ns_x,
+  e = launch_dep(kp_dwt_kernel, dim3(a.Q), dim3(kKpThreads), 0, s, (const float2*)w.E, a, k.nyr_x * k.ns_x,
                  (const float2*)w.part.wt, w.dE);
   if (e != cudaSuccess) return e;
   return launch_dep(kp_contract_kernel, dim3(kp_blocks(count, p)), dim3(kKpThreads), 0, s, (const float2*)w.dE, a,

@@ -25,6 +25,8 @@ pytestmark = pytest.mark.gpu
     (16, 1, 1, 2, 1),     # one bin, one frame
     (16, 13, 2, 8, 2),    # general kernels
     (16, 64, 2, 16, 2),   # largest bin and feature counts
+    (96, 8, 3, 4, 1),     # X kernel: image rows in three equal runs
+    (256, 8, 6, 1, 1),    # and in runs of 86, 86 and 84
 ])
 def test_render_and_gradients(N, Nf, T, F, S):
     from paper_2311_13177_gb300 import Plan
