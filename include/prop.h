@@ -416,7 +416,7 @@ PROP_API prop_status prop_proj_adjoint(prop_plan plan, int blade, const void* z_
  *   + tv_xy TV_xy + tv_f TV_f + tv_t TV_t + l1 L1,   Z = U P_b V_t(b),
  * each TV term sum sqrt(|d|^2 + tv_eps^2) over forward differences (no wrap).
  * ycart_dev: [B][N][N] Cartesian k-space data (cells outside each mask are
- * not read); img_dev: [B][N][N] blade images, or NULL for U^H M_b ycart_b.
+ * not used); img_dev: [B][N][N] blade images, or NULL for U^H M_b ycart_b.
  * V_dev: the start in, the result out.  loss_trace_host (may be NULL):
  * [iters] loss of each iteration's blade before its update.  Synchronises
  * only when a trace is requested. */

@@ -1492,9 +1492,9 @@ cudaError_t dispatch_fused(int n, const FusedArgs& a, int mode, dim3 grid, cudaS
 // --- Centred unitary 2-D DFT of one N x N image (projection model) ----------
 //
 // Four passes of NFFT = N point transforms, kCartCols lines per CTA: forward rows,
-// forward columns (scale 1/N; optionally masked, or fused with the blade's
-// data term), inverse columns (input optionally masked), inverse rows (scale
-// 1/N).  The centring (image index i = x + N/2, k index u = N k + N/2) is
+// forward columns (scale 1/N; optionally masked), inverse columns (input
+// optionally masked), inverse rows (scale 1/N); in a reconstruction both column
+// passes and the blade's data term between them are one kernel.  The centring (image index i = x + N/2, k index u = N k + N/2) is
 // the index map position -> (position + N/2) mod N on every input and
 // output, which is where an unshifted DFT's position 0 holds x = 0 / k = 0.
 struct CartArgs {
@@ -1554,11 +1554,13 @@ struct OutCartCols {
     dst[i] = z;
   }
 };
-// Forward column output fused with the blade's data term: on the mask,
-// r_k = Z - y, r_i = Z - yimg (the image term through the unitary DFT),
-// loss += wk |r_k|^2 + wi |r_i|^2 and dst = 2 (wk r_k + wi r_i); 0 elsewhere.
+// Forward column output of the data term: on the mask, r_k = Z - y,
+// r_i = Z - yimg (the image term through the unitary DFT), loss += wk |r_k|^2 +
+// wi |r_i|^2, and the gradient 2 (wk r_k + wi r_i), 0 elsewhere, into the CTA's
+// buffer g[k position][col].  The data are loaded whether on the mask or not,
+// so that no load waits for another.
 struct OutCartLoss {
-  float2* dst;
+  float2* g;
   const uint8_t* mask;
   const float2* y;
   const float2* yimg;
@@ -1567,19 +1569,21 @@ struct OutCartLoss {
   float scale;
   float* acc;
   __device__ void operator()(int q, int col, float2 v) const {
-    const size_t i = (size_t)cshift(q, N) * N + c0 + col;
-    float2 g = make_float2(0.f, 0.f);
-    if (mask[i]) {
-      const float2 z = cscale(v, scale);
-      const float2 yy = y[i];
-      const float2 yi = yimg ? yimg[i] : yy;
-      const float2 rk = make_float2(z.x - yy.x, z.y - yy.y);
-      const float2 ri = make_float2(z.x - yi.x, z.y - yi.y);
-      *acc += wk * fmaf(rk.x, rk.x, rk.y * rk.y) + wi * fmaf(ri.x, ri.x, ri.y * ri.y);
-      g = make_float2(2.f * fmaf(wk, rk.x, wi * ri.x), 2.f * fmaf(wk, rk.y, wi * ri.y));
-    }
-    dst[i] = g;
+    const int i = cshift(q, N) * N + c0 + col;
+    const bool on = __ldg(&mask[i]) != 0;
+    const float2 yy = __ldg(&y[i]);
+    const float2 yi = yimg ? __ldg(&yimg[i]) : yy;
+    const float2 z = cscale(v, scale);
+    const float2 rk = make_float2(z.x - yy.x, z.y - yy.y);
+    const float2 ri = make_float2(z.x - yi.x, z.y - yi.y);
+    if (on) *acc += wk * fmaf(rk.x, rk.x, rk.y * rk.y) + wi * fmaf(ri.x, ri.x, ri.y * ri.y);
+    g[q * kCartCols + col] = on ? make_float2(2.f * fmaf(wk, rk.x, wi * ri.x), 2.f * fmaf(wk, rk.y, wi * ri.y))
+                                : make_float2(0.f, 0.f);
   }
+};
+struct InCartBuf {
+  const float2* g;
+  __device__ float2 operator()(int pos, int col) const { return g[pos * kCartCols + col]; }
 };
 
 template <int NFFT>
@@ -1589,6 +1593,10 @@ constexpr int cart_threads() {
 template <int NFFT>
 constexpr size_t cart_smem() {
   return (size_t)NFFT * kCartCols * sizeof(float2) + (size_t)Shape<NFFT, kValsPlain<NFFT>>::TW * sizeof(float2);
+}
+template <int NFFT>
+constexpr size_t cart_loss_smem() {  // and the gradient between the two column passes
+  return cart_smem<NFFT>() + (size_t)NFFT * kCartCols * sizeof(float2);
 }
 
 template <int NFFT, int PASS>
@@ -1611,17 +1619,19 @@ __global__ void __launch_bounds__(cart_threads<NFFT>()) cart_fft_kernel(CartArgs
     fft_pass<NFFT, EV, -1, 0, 1, false, false, CtaSync, InCartRows, OutCartRows, NoHook, CC>(X, tw, col, tl, in, out);
   } else if constexpr (PASS == kCartColsFwd) {
     InCartCols in{a.src, nullptr, NFFT, l0};
-    if (a.y) {
-      float acc = 0.f;
-      OutCartLoss out{a.dst, a.mask, a.y, a.yimg, a.wk, a.wi, NFFT, l0, a.scale, &acc};
-      fft_pass<NFFT, EV, -1, 0, 1, false, false, CtaSync, InCartCols, OutCartLoss, NoHook, CC>(X, tw, col, tl, in,
-                                                                                             out);
-      finish_loss(acc, a.partials, a.counter, a.loss_const, a.loss_out);
-    } else {
-      OutCartCols out{a.dst, a.mask, NFFT, l0, a.scale};
-      fft_pass<NFFT, EV, -1, 0, 1, false, false, CtaSync, InCartCols, OutCartCols, NoHook, CC>(X, tw, col, tl, in,
-                                                                                             out);
-    }
+    OutCartCols out{a.dst, a.mask, NFFT, l0, a.scale};
+    fft_pass<NFFT, EV, -1, 0, 1, false, false, CtaSync, InCartCols, OutCartCols, NoHook, CC>(X, tw, col, tl, in, out);
+  } else if constexpr (PASS == kCartColsLoss) {
+    float2* g = tw + Shape<NFFT, EV>::TW;
+    InCartCols in{a.src, nullptr, NFFT, l0};
+    float acc = 0.f;
+    OutCartLoss mid{g, a.mask, a.y, a.yimg, a.wk, a.wi, NFFT, l0, a.scale, &acc};
+    fft_pass<NFFT, EV, -1, 0, 1, false, false, CtaSync, InCartCols, OutCartLoss, NoHook, CC>(X, tw, col, tl, in, mid);
+    __syncthreads();
+    InCartBuf back{g};
+    OutCartCols out{a.dst, nullptr, NFFT, l0, 1.f};
+    fft_pass<NFFT, EV, +1, 0, 1, false, false, CtaSync, InCartBuf, OutCartCols, NoHook, CC>(X, tw, col, tl, back, out);
+    finish_loss(acc, a.partials, a.counter, a.loss_const, a.loss_out);
   } else if constexpr (PASS == kCartColsInv) {
     InCartCols in{a.src, a.mask, NFFT, l0};
     OutCartCols out{a.dst, nullptr, NFFT, l0, a.scale};
@@ -1641,6 +1651,7 @@ cudaError_t launch_cart(int pass, const CartArgs& a, cudaStream_t s) {
     case kCartRowsFwd: return launch_dep(cart_fft_kernel<NFFT, kCartRowsFwd>, grid, block, smem, s, a);
     case kCartColsFwd: return launch_dep(cart_fft_kernel<NFFT, kCartColsFwd>, grid, block, smem, s, a);
     case kCartColsInv: return launch_dep(cart_fft_kernel<NFFT, kCartColsInv>, grid, block, smem, s, a);
+    case kCartColsLoss: return launch_dep(cart_fft_kernel<NFFT, kCartColsLoss>, grid, block, cart_loss_smem<NFFT>(), s, a);
     default: return launch_dep(cart_fft_kernel<NFFT, kCartRowsInv>, grid, block, smem, s, a);
   }
 }
@@ -1654,6 +1665,9 @@ cudaError_t configure_cart() {
   if ((e = cudaFuncSetAttribute(cart_fft_kernel<NFFT, kCartColsFwd>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
     return e;
   if ((e = cudaFuncSetAttribute(cart_fft_kernel<NFFT, kCartColsInv>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
+    return e;
+  if ((e = cudaFuncSetAttribute(cart_fft_kernel<NFFT, kCartColsLoss>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)cart_loss_smem<NFFT>())))
     return e;
   return cudaFuncSetAttribute(cart_fft_kernel<NFFT, kCartRowsInv>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
@@ -1931,8 +1945,9 @@ cudaError_t cart_fft_pass(int N, int pass, const float2* src, float2* dst, const
   a.mask = mask;
   a.N = N;
   a.scale = scale;
+  if ((pass == kCartColsLoss) != (loss != nullptr)) return cudaErrorInvalidValue;
   if (loss) {
-    if (pass != kCartColsFwd || !loss->red || !mask || loss->red->capacity < N / kCartCols) return cudaErrorInvalidValue;
+    if (!loss->red || !mask || loss->red->capacity < N / kCartCols) return cudaErrorInvalidValue;
     a.y = loss->y;
     a.yimg = loss->yimg;
     a.wk = loss->wk;

@@ -9,10 +9,11 @@
 // one blade per iteration in turn, on w_k |M (Z - y)|^2 + w_i |U^H M Z - img|^2
 // plus smoothed TV along x1, x2, the spectral axis and time, and L1.
 //
-// One iteration is six launches: the projection (a gather, one warp per
-// pixel with the bins across the lanes), four passes of N-point transforms
-// (the forward column pass fused with the mask, the residuals, the data
-// loss and the data-term gradient 2 M (w_k r_k + w_i r_i); the image term is
+// One iteration is five launches: the projection (a gather, one warp per
+// four pixels with the bins across the lanes), three passes of N-point
+// transforms (rows; columns forward, the mask, the residuals, the data loss and
+// the data-term gradient 2 M (w_k r_k + w_i r_i), and the columns back, all in
+// one kernel since a column stays in its CTA; rows back; the image term is
 // taken through the unitary DFT, ||U^H M Z - img||^2 = ||M (Z - U img)||^2
 // + ||(1 - M) U img||^2, with the second part a per-blade constant computed
 // once), and a fused update: for every voxel the transposed projection (a
@@ -144,6 +145,7 @@ struct ProjUpdArgs {
   const float2* gimg;  // [N][N] image-space gradient of the data term (U^H of the masked k-space gradient)
   const int4* sh;      // [Nf] shifts of the iteration's blade
   int N, Nf, T, tb;
+  int len;             // voxels of an image row that a thread takes
   AdamArgs ad;         // gscale 1 (gimg already holds the factor 2 and the weights)
   float tv_f, l1;
   double* partials;
@@ -152,79 +154,149 @@ struct ProjUpdArgs {
   double* loss_out;
 };
 
+// Threads of the update along the bins and, by what is left of a block, along x1.
+__host__ __device__ inline int update_bins(int Nf) { return Nf < kProjThreads ? Nf : kProjThreads; }
+
 // Fused update: data gradient by the transposed projection, TV along x1, x2
 // and t (the same arithmetic as the non-uniform model's update), TV along
 // the spectral axis, L1, Adam, and the FP64 loss of the iterate it reads.
-// Grid: (blocks per image row, T N rows); 32-bit index math within a row.
-// Every neighbour load is unconditional (a missing neighbour reads the voxel
-// itself and is not used), so the loads of several voxels are in flight
-// together; TT: the volume has time neighbours.
-template <bool TT>
+// Grid: (x1 blocks x bin groups, T N rows).  A thread takes one bin and walks
+// `len` voxels along x1, so the x1 TV term and the two pixels that it shares
+// with the voxel before are handed on (two pixel loads instead of four), the
+// bin's shift and its weights are loaded once, and a voxel is one 32-bit byte
+// offset; the loads of U voxels are issued together.  Every neighbour load is
+// unconditional (a missing neighbour reads the voxel itself and is not used).
+// TT: the volume has time neighbours.  Off: uint32_t while three frames are
+// within 4 GB (64-bit offsets cost a CTA per SM: 98 registers instead of 80,
+// 1196 instead of 1053 us for 16 iterations at 256^2 x 32), else size_t.
+template <bool TT, typename Off>
 __global__ void __launch_bounds__(kProjThreads) proj_update_kernel(ProjUpdArgs a) {
   grid_dep_wait();
   grid_dep_release();
+  constexpr int U = 2;
   const int row = blockIdx.y;  // t N + i2
   const int i2 = row % a.N, t = row / a.N;
-  const int rl = a.N * a.Nf;
-  const size_t base = (size_t)row * rl;
-  const size_t sx = (size_t)a.Nf, sy = (size_t)rl, st = (size_t)a.N * rl;
-  const float eps2 = a.ad.tv_eps * a.ad.tv_eps;
-  const bool xy = a.ad.tv_xy != 0.f;
-  const bool h2p = xy && i2 + 1 < a.N, h2m = xy && i2 > 0;
-  const bool htp = TT && t + 1 < a.T, htm = TT && t > 0;
-  const bool data = t == a.tb;
-  const float2* __restrict__ Vin = a.Vin;
+  const int fw = update_bins(a.Nf), nfg = (a.Nf + fw - 1) / fw, runs = kProjThreads / fw;
+  const int fg = blockIdx.x % nfg, run = threadIdx.x / fw;
+  const int f = fg * fw + threadIdx.x - run * fw;
+  const int lo = ((int)(blockIdx.x / nfg) * runs + run) * a.len;
+  const int hi = run < runs && f < a.Nf ? min(a.N, lo + a.len) : 0;
   float local = 0.f;
-#pragma unroll 2
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < rl; e += gridDim.x * blockDim.x) {
-    const int i1 = e / a.Nf;
-    const int f = e - i1 * a.Nf;
-    const size_t idx = base + e;
-    const float2 x = Vin[idx];
-    TvNbrs nb;
-    nb.h1p = xy && i1 + 1 < a.N;
-    nb.h1m = xy && i1 > 0;
-    nb.h2p = h2p;
-    nb.h2m = h2m;
-    nb.htp = htp;
-    nb.htm = htm;
-    nb.x1p = Vin[nb.h1p ? idx + sx : idx];
-    nb.x1m = Vin[nb.h1m ? idx - sx : idx];
-    nb.x2p = Vin[h2p ? idx + sy : idx];
-    nb.x2m = Vin[h2m ? idx - sy : idx];
-    if constexpr (TT) {
-      nb.tp = Vin[htp ? idx + st : idx];
-      nb.tm = Vin[htm ? idx - st : idx];
-    } else {
-      nb.tp = nb.tm = x;
-    }
+  if (lo < hi) {
+    const float eps2 = a.ad.tv_eps * a.ad.tv_eps;
+    const size_t st = (size_t)a.N * a.N * a.Nf;
+    const bool xy = a.ad.tv_xy != 0.f;
+    const bool h2p = xy && i2 + 1 < a.N, h2m = xy && i2 > 0;
+    const bool htp = TT && t + 1 < a.T, htm = TT && t > 0;
     const bool hfp = a.tv_f != 0.f && f + 1 < a.Nf, hfm = a.tv_f != 0.f && f > 0;
-    const float2 xfp = Vin[hfp ? idx + 1 : idx];
-    const float2 xfm = Vin[hfm ? idx - 1 : idx];
-    float2 mm = a.m[idx], vv = a.v[idx];
-    const float2 gd = data ? proj_gather(a.gimg, __ldg(&a.sh[f]), a.N, i1, i2) : make_float2(0.f, 0.f);
-    float2 gxy, gt;
-    float tv = voxel_tv_nb(x, nb, a.ad.tv_xy, TT ? a.ad.tv_t : 0.f, eps2, &gxy, &gt);
-    float2 gf = make_float2(0.f, 0.f);
+    // offsets count from the frame before this one (from this one when t = 0)
+    const size_t first = (size_t)(t > 0 ? t - 1 : 0) * st;
+    const char* V = reinterpret_cast<const char*>(a.Vin + first);
+    char* M1 = reinterpret_cast<char*>(a.m + first);
+    char* M2 = reinterpret_cast<char*>(a.v + first);
+    char* Vo = reinterpret_cast<char*>(a.Vout + first);
+    auto at = [](const char* b, Off o) { return __ldg(reinterpret_cast<const float2*>(b + o)); };
+    auto ref = [](char* b, Off o) -> float2& { return *reinterpret_cast<float2*>(b + o); };
+    const Off sx = (Off)a.Nf * 8, d2 = (Off)a.N * sx, dt = (Off)st * 8;
+    const Off d2p = h2p ? d2 : 0, d2m = h2m ? d2 : 0, dtp = htp ? dt : 0, dtm = htm ? dt : 0;
+    const Off dfp = hfp ? 8 : 0, dfm = hfm ? 8 : 0;
+    Off off = (t > 0 ? dt : 0) + (Off)i2 * d2 + (Off)lo * sx + (Off)f * 8;
+    // pixel rows i2 - o2 and i2 - o2 - 1 of the transposed projection
+    const bool data = t == a.tb;
+    const int4 o = __ldg(&a.sh[f]);
+    const float w1 = __int_as_float(o.z), w2 = __int_as_float(o.w);
+    const int p0 = i2 - o.y, p1 = p0 - 1;
+    const bool r0 = data && p0 >= 0 && p0 < a.N, r1 = data && p1 >= 0 && p1 < a.N;
+    const float2* g0 = a.gimg + (size_t)(r0 ? p0 : 0) * a.N;
+    const float2* g1 = a.gimg + (size_t)(r1 ? p1 : 0) * a.N;
+    const float w00 = (1.f - w2) * (1.f - w1), w01 = (1.f - w2) * w1, w10 = w2 * (1.f - w1), w11 = w2 * w1;
+    auto pix = [&](const float2* g, bool row_ok, int p) {
+      const bool ok = row_ok && p >= 0 && p < a.N;
+      const float2 v = __ldg(&g[ok ? p : 0]);
+      return ok ? v : make_float2(0.f, 0.f);
+    };
+    float2 x = at(V, off);
+    float2 q0 = pix(g0, r0, lo - o.x - 1), q1 = pix(g1, r1, lo - o.x - 1);  // the pixels of the voxel before
     float mag;
-    if (hfp) {
-      gf = csub_rn(gf, tv_term(csub_rn(xfp, x), eps2, &mag));
-      tv = fmaf(a.tv_f, mag, tv);
+    float2 t1m = make_float2(0.f, 0.f);
+    if (xy && lo > 0) t1m = tv_term(csub_rn(x, at(V, off - sx)), eps2, &mag);
+    for (int i0 = lo; i0 < hi; i0 += U, off += U * sx) {
+      float2 xp[U], x2p[U], x2m[U], xtp[U], xtm[U], xfp[U], xfm[U], mm[U], vv[U], n0[U], n1[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i1 = min(i0 + u, hi - 1);
+        const Off c = off + (Off)(i1 - i0) * sx;
+        xp[u] = at(V, i1 + 1 < a.N ? c + sx : c);
+        x2p[u] = at(V, c + d2p);
+        x2m[u] = at(V, c - d2m);
+        if constexpr (TT) {
+          xtp[u] = at(V, c + dtp);
+          xtm[u] = at(V, c - dtm);
+        }
+        xfp[u] = at(V, c + dfp);
+        xfm[u] = at(V, c - dfm);
+        mm[u] = ref(M1, c);
+        vv[u] = ref(M2, c);
+        n0[u] = pix(g0, r0, i1 - o.x);
+        n1[u] = pix(g1, r1, i1 - o.x);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i1 = i0 + u;
+        if (i1 >= hi) break;
+        const Off c = off + (Off)u * sx;
+        // proj_gather's taps in its order (missing pixels are zero)
+        const float gx = fmaf(w11, q1.x, fmaf(w10, n1[u].x, fmaf(w01, q0.x, w00 * n0[u].x)));
+        const float gy = fmaf(w11, q1.y, fmaf(w10, n1[u].y, fmaf(w01, q0.y, w00 * n0[u].y)));
+        q0 = n0[u];
+        q1 = n1[u];
+        // voxel_tv_nb's terms in its order
+        float2 gxy = make_float2(0.f, 0.f), gt = make_float2(0.f, 0.f), t1p = make_float2(0.f, 0.f);
+        float sxy = 0.f, stt = 0.f;
+        if (xy) {
+          if (i1 + 1 < a.N) {
+            t1p = tv_term(csub_rn(xp[u], x), eps2, &mag);
+            gxy = csub_rn(gxy, t1p);
+            sxy = __fadd_rn(sxy, mag);
+          }
+          if (i1 > 0) gxy = cadd_rn(gxy, t1m);
+          if (h2p) {
+            gxy = csub_rn(gxy, tv_term(csub_rn(x2p[u], x), eps2, &mag));
+            sxy = __fadd_rn(sxy, mag);
+          }
+          if (h2m) gxy = cadd_rn(gxy, tv_term(csub_rn(x, x2m[u]), eps2, &mag));
+        }
+        if constexpr (TT) {
+          if (htp) {
+            gt = csub_rn(gt, tv_term(csub_rn(xtp[u], x), eps2, &mag));
+            stt = __fadd_rn(stt, mag);
+          }
+          if (htm) gt = cadd_rn(gt, tv_term(csub_rn(x, xtm[u]), eps2, &mag));
+        }
+        float tv = fmaf(a.ad.tv_xy, sxy, __fmul_rn(TT ? a.ad.tv_t : 0.f, stt));
+        float2 gf = make_float2(0.f, 0.f);
+        if (hfp) {
+          gf = csub_rn(gf, tv_term(csub_rn(xfp[u], x), eps2, &mag));
+          tv = fmaf(a.tv_f, mag, tv);
+        }
+        if (hfm) gf = cadd_rn(gf, tv_term(csub_rn(x, xfm[u]), eps2, &mag));
+        float2 gl = make_float2(0.f, 0.f);
+        if (a.l1 != 0.f) {
+          gl = tv_term(x, eps2, &mag);  // x / sqrt(|x|^2 + eps^2) and the smoothed modulus
+          tv = fmaf(a.l1, mag, tv);
+        }
+        float2 g = total_grad(make_float2(gx, gy), gxy, gt, a.ad);
+        g.x = fmaf(a.l1, gl.x, fmaf(a.tv_f, gf.x, g.x));
+        g.y = fmaf(a.l1, gl.y, fmaf(a.tv_f, gf.y, g.y));
+        local = __fadd_rn(local, tv);
+        const float2 nx = adam_voxel(x, g, mm[u], vv[u], a.ad);
+        ref(M1, c) = mm[u];
+        ref(M2, c) = vv[u];
+        ref(Vo, c) = nx;
+        t1m = t1p;
+        x = xp[u];
+      }
     }
-    if (hfm) gf = cadd_rn(gf, tv_term(csub_rn(x, xfm), eps2, &mag));
-    float2 gl = make_float2(0.f, 0.f);
-    if (a.l1 != 0.f) {
-      gl = tv_term(x, eps2, &mag);  // x / sqrt(|x|^2 + eps^2) and the smoothed modulus
-      tv = fmaf(a.l1, mag, tv);
-    }
-    float2 g = total_grad(gd, gxy, gt, a.ad);
-    g.x = fmaf(a.l1, gl.x, fmaf(a.tv_f, gf.x, g.x));
-    g.y = fmaf(a.l1, gl.y, fmaf(a.tv_f, gf.y, g.y));
-    local = __fadd_rn(local, tv);
-    const float2 nx = adam_voxel(x, g, mm, vv, a.ad);
-    a.m[idx] = mm;
-    a.v[idx] = vv;
-    a.Vout[idx] = nx;
   }
   finish_loss(local, a.partials, a.counter, a.data_loss, a.loss_out);
 }
@@ -268,10 +340,15 @@ __global__ void __launch_bounds__(kProjThreads) proj_baseline_kernel(const float
   }
 }
 
-// Blocks per image row of the update: about 8 voxels a thread, at most 4.
+// Voxels of a row that a thread of the update takes (at most 8), and the
+// update's blocks per image row.
+int update_len(const Plan& p) {
+  const int runs = kProjThreads / update_bins(p.Nf);
+  return std::min(8, (p.N + runs - 1) / runs);
+}
 int update_row_blocks(const Plan& p) {
-  const int rl = p.N * p.Nf;
-  return std::max(1, std::min(4, rl / (8 * kProjThreads)));
+  const int fw = update_bins(p.Nf), runs = kProjThreads / fw, span = runs * update_len(p);
+  return (p.Nf + fw - 1) / fw * ((p.N + span - 1) / span);
 }
 
 // Allocates *ptr unless a previous, interrupted set-up already did.
@@ -372,15 +449,31 @@ namespace {
 const int4* blade_shifts(const Plan& p, int b) { return p.proj_shift + (size_t)b * p.Nf; }
 const uint8_t* blade_mask(const Plan& p, int b) { return p.proj_mask + (size_t)b * p.N * p.N; }
 
-// Z = M_b U P_b V_t(b) into z (or, with `loss`, the data term and its k-space gradient into p.proj_kg).
-prop_status proj_forward_impl(Plan& p, int b, const float2* V, float2* z, const CartLoss* loss, cudaStream_t s) {
+// Row transforms of blade b's projected image into p.proj_k.
+prop_status proj_rows_impl(Plan& p, int b, const float2* V, cudaStream_t s) {
   const long warps = (long)p.N * p.N / kProjPix;
   const unsigned blocks = (unsigned)((warps + kProjThreads / 32 - 1) / (kProjThreads / 32));
   PROP_CUDA(launch_dep(proj_image_kernel, dim3(blocks), dim3(kProjThreads), 0, s, V, blade_shifts(p, b), p.N, p.Nf,
                       p.blade_frame[b], p.proj_img));
   PROP_CUDA(cart_fft_pass(p.N, kCartRowsFwd, p.proj_img, p.proj_k, p.proj_twiddle, nullptr, nullptr, 1.f, s));
-  PROP_CUDA(cart_fft_pass(p.N, kCartColsFwd, p.proj_k, loss ? p.proj_kg : z, p.proj_twiddle, blade_mask(p, b), loss,
+  return PROP_OK;
+}
+
+// Z = M_b U P_b V_t(b) into z.
+prop_status proj_forward_impl(Plan& p, int b, const float2* V, float2* z, cudaStream_t s) {
+  const prop_status st = proj_rows_impl(p, b, V, s);
+  if (st != PROP_OK) return st;
+  PROP_CUDA(cart_fft_pass(p.N, kCartColsFwd, p.proj_k, z, p.proj_twiddle, blade_mask(p, b), nullptr, 1.f / (float)p.N, s));
+  return PROP_OK;
+}
+
+// The blade's data term at V: its loss, and its image-space gradient into p.proj_g.
+prop_status proj_data_grad(Plan& p, int b, const float2* V, const CartLoss& loss, cudaStream_t s) {
+  const prop_status st = proj_rows_impl(p, b, V, s);
+  if (st != PROP_OK) return st;
+  PROP_CUDA(cart_fft_pass(p.N, kCartColsLoss, p.proj_k, p.proj_kg, p.proj_twiddle, blade_mask(p, b), &loss,
                          1.f / (float)p.N, s));
+  PROP_CUDA(cart_fft_pass(p.N, kCartRowsInv, p.proj_kg, p.proj_g, p.proj_twiddle, nullptr, nullptr, 1.f / (float)p.N, s));
   return PROP_OK;
 }
 
@@ -419,7 +512,7 @@ prop_status prop_proj_forward(prop_plan plan, int blade, const void* V_dev, void
   DeviceGuard g(p.device);
   prop_status st = plan_ensure_proj(p, false);
   if (st != PROP_OK) return st;
-  return proj_forward_impl(p, blade, (const float2*)V_dev, (float2*)z_dev, nullptr, (cudaStream_t)stream);
+  return proj_forward_impl(p, blade, (const float2*)V_dev, (float2*)z_dev, (cudaStream_t)stream);
 }
 
 prop_status prop_proj_adjoint(prop_plan plan, int blade, const void* z_dev, void* V_dev, void* stream) {
@@ -486,6 +579,7 @@ prop_status prop_proj_reconstruct(prop_plan plan, const void* ycart_dev, const v
   float2* cur = (float2*)V_dev;
   float2* nxt = p.vol2;
   const dim3 ugrid((unsigned)update_row_blocks(p), (unsigned)(p.T * p.N));
+  const bool small = frames_in_32_bits(p);
   if ((long)ugrid.x * ugrid.y > p.red_proj_u.capacity) return fail(PROP_ERR_INVALID_ARG, "proj_reconstruct: reduction capacity");
   for (int k = 1; k <= q.iters; ++k) {
     const int b = (k - 1) % p.B;
@@ -497,8 +591,7 @@ prop_status prop_proj_reconstruct(prop_plan plan, const void* ycart_dev, const v
     loss.red = &p.red_proj_k;
     loss.loss_const = img_dev ? p.proj_const + b : nullptr;
     loss.loss_out = p.scalars + 3;
-    if ((st = proj_forward_impl(p, b, cur, nullptr, &loss, s)) != PROP_OK) return st;
-    if ((st = proj_kadjoint_impl(p, b, p.proj_kg, s)) != PROP_OK) return st;
+    if ((st = proj_data_grad(p, b, cur, loss, s)) != PROP_OK) return st;
     ProjUpdArgs u{};
     u.Vin = cur;
     u.Vout = nxt;
@@ -509,6 +602,7 @@ prop_status prop_proj_reconstruct(prop_plan plan, const void* ycart_dev, const v
     u.N = p.N;
     u.Nf = p.Nf;
     u.T = p.T;
+    u.len = update_len(p);
     u.tb = p.blade_frame[b];
     const double bc1 = 1.0 - std::pow((double)q.beta1, k);
     const double bc2 = 1.0 - std::pow((double)q.beta2, k);
@@ -528,9 +622,11 @@ prop_status prop_proj_reconstruct(prop_plan plan, const void* ycart_dev, const v
     u.data_loss = p.scalars + 3;
     u.loss_out = p.loss_dev + (k - 1);
     if (p.T > 1 && q.tv_t != 0.f)
-      PROP_CUDA(launch_dep(proj_update_kernel<true>, ugrid, dim3(kProjThreads), 0, s, u));
+      PROP_CUDA(launch_dep(small ? proj_update_kernel<true, uint32_t> : proj_update_kernel<true, size_t>, ugrid,
+                           dim3(kProjThreads), 0, s, u));
     else
-      PROP_CUDA(launch_dep(proj_update_kernel<false>, ugrid, dim3(kProjThreads), 0, s, u));
+      PROP_CUDA(launch_dep(small ? proj_update_kernel<false, uint32_t> : proj_update_kernel<false, size_t>, ugrid,
+                           dim3(kProjThreads), 0, s, u));
     std::swap(cur, nxt);
   }
   if (cur != (float2*)V_dev) PROP_CUDA(cudaMemcpyAsync(V_dev, cur, vbytes, cudaMemcpyDeviceToDevice, s));

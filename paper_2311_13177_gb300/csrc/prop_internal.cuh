@@ -348,19 +348,21 @@ cudaError_t fft_configure(int n);
 prop_status plan_ensure_proj(Plan& p, bool images);
 // Centred unitary 2-D DFT of one N x N image, [i2][i1] <-> [u2][u1] (projection
 // model): one pass of N-point transforms over the rows or the columns.
-enum CartPass { kCartRowsFwd = 0, kCartColsFwd = 1, kCartColsInv = 2, kCartRowsInv = 3 };
-struct CartLoss {              // blade data term fused into the forward column pass
+enum CartPass { kCartRowsFwd = 0, kCartColsFwd = 1, kCartColsInv = 2, kCartRowsInv = 3, kCartColsLoss = 4 };
+struct CartLoss {              // blade data term between the forward and the inverse column pass
   const float2* y;             // [N][N] k-space data of the blade
   const float2* yimg;          // [N][N] DFT of the blade's image, or null (image term against y)
   float wk, wi;                // k-space and image-space weights
-  const Reducer* red;          // >= N/16 partials
+  const Reducer* red;          // >= N / kCartCols partials
   const double* loss_const;    // added to the data loss (image term outside the mask), or null
   double* loss_out;
 };
-// kCartColsFwd writes Z * scale masked by `mask` (when given), or with `loss`
-// the data-term gradient 2 M (wk (Z - y) + wi (Z - yimg)) and the loss;
-// kCartColsInv masks its input by `mask` (when given).  Rows passes and the
-// inverse column pass multiply by `scale`.
+// kCartColsFwd writes Z * scale masked by `mask` (when given); kCartColsInv
+// masks its input by `mask` (when given); kCartColsLoss (with `loss` and
+// `mask`) is the forward column pass, the data-term gradient
+// 2 M (wk (Z - y) + wi (Z - yimg)) of Z * scale with its loss, and the inverse
+// column pass of that gradient.  Rows passes and kCartColsInv multiply by
+// `scale`.
 cudaError_t cart_fft_pass(int N, int pass, const float2* src, float2* dst, const float2* twiddleN,
                           const uint8_t* mask, const CartLoss* loss, float scale, cudaStream_t s);
 cudaError_t cart_fft_configure(int N);
@@ -396,6 +398,10 @@ struct AdamArgs {
   float tv_xy, tv_t, tv_eps;
   float gscale;      // factor on the adjoint (2 for the squared-L2 data term)
 };
+// Three frames of a volume (what an update reads around a voxel) within 32-bit byte offsets.
+inline bool frames_in_32_bits(const Plan& p) {
+  return (size_t)3 * p.N * p.N * p.Nf * sizeof(float2) < (size_t)1 << 32;
+}
 // Fused smoothed-TV gradient + Adam: Vout = Adam(Vin, gscale*g + TV grads).
 // Writes data + tv_xy*TV_xy + tv_t*TV_t of Vin into loss_out[0] when red != null.
 cudaError_t tv_adam(const Plan& p, const float2* Vin, const float2* g, float2* m, float2* v,
