@@ -31,18 +31,24 @@ struct RadixPlan {
   int r[8];
 };
 
-// Radices for E values a thread (every radix divides E, so a thread holds
-// whole butterflies in every pass): with E = 32, radix 32 while it divides
-// and then 16; else radix 8 where E allows (E = 16 or 24), radix 4 where it
-// does not (E = 12, lengths with a factor 3: half the registers of 24,
-// twice the threads); then 4, 2 and the threes, a leftover factor 2 merged
-// with a 3 into one radix-6 pass.
+// Radices for E values a thread (a thread holds whole butterflies in every
+// pass): with E = 32, radix 32 while it divides and then 16; with E = 24,
+// radix 24 and then the rest (16 or 32) in one pass, of which some warps take
+// a butterfly more than others; else every radix divides E, radix 8 where E
+// allows (E = 16), radix 4 where it does not (E = 12, lengths with a factor 3:
+// half the registers of 24, twice the threads); then 4, 2 and the threes, a
+// leftover factor 2 merged with a 3 into one radix-6 pass.
 __host__ __device__ constexpr RadixPlan radix_plan(int n, int E) {
   RadixPlan p{0, {1, 1, 1, 1, 1, 1, 1, 1}};
   int m = n, threes = 0;
   while (m % 3 == 0) {
     m /= 3;
     ++threes;
+  }
+  if (E == 24) {
+    p.r[p.count++] = 24;
+    p.r[p.count++] = n / 24;
+    return p;
   }
   while (E % 32 == 0 && threes == 0 && m % 32 == 0) {
     p.r[p.count++] = 32;
@@ -101,13 +107,18 @@ template <int NFFT>
 constexpr int kValsPlain = (NFFT % 3 == 0) ? 12 : 16;
 template <int NFFT>
 constexpr int kValsFused = (NFFT % 3 == 0) ? 12 : 16;
-// Values per thread of the TMA-staged column passes: 32 at n = 512 (radix
-// 32 then 16: one shared-memory exchange instead of two) and 24 at n = 384
-// (radices 8, 8, 6: two instead of three), with twice the registers and
-// half the threads of a 16-value shape; 2N = 512: 23.9 -> 20.3 us forward,
-// 24.8 -> 22.3 us adjoint; 2N = 384: 184.7 -> 153.8 us and 193.4 -> 164.7 us.
+// Values per thread of the column passes, as many as make two passes of them
+// (one shared-memory exchange): 32 at n = 512 (radix 32 then 16) and 1024 (32,
+// 32), 24 at n = 384 (24, 16) and 768 (24, 32), with twice the registers and
+// half the threads of a 16- or 12-value shape.  The exchanges and the twiddle
+// products between passes are what the passes spend their issue slots and
+// shared-memory wavefronts on (60 % of both at 2N = 384).  2N = 512: 23.9 ->
+// 20.3 us forward, 24.8 -> 22.3 us adjoint; 384 (64 bins, 16 frames): 126 -> 113
+// us and 128 -> 111 us (with radices 8, 8, 6); 768: 142 -> 82 us and 146 -> 84
+// us (12 values a thread before, the forward pass spilling); 1024: 98 -> 39 us
+// and 62 -> 53 us.
 template <int NFFT>
-constexpr int kValsCols = NFFT == 512 ? 32 : NFFT == 384 ? 24 : kValsPlain<NFFT>;
+constexpr int kValsCols = NFFT == 512 || NFFT == 1024 ? 32 : NFFT == 384 || NFFT == 768 ? 24 : kValsPlain<NFFT>;
 
 template <int NFFT, int EV>
 struct Shape {
@@ -270,20 +281,36 @@ __host__ __device__ constexpr double cos32(int m) {
 }
 __host__ __device__ constexpr double sin32(int m) { return cos32(m - 8); }
 
-// z * exp(SIGN 2 pi i M / R) for R dividing 32; quarter turns exactly.
+// cos(2 pi m / 24) and sin(2 pi m / 24) likewise, for the radix-24 butterfly.
+__host__ __device__ constexpr double cos24(int m) {
+  constexpr double q[7] = {1.0,
+                           0.96592582628906828674974319972890,   // cos(pi / 12)
+                           0.86602540378443864676372317075294,   // cos(pi / 6)
+                           0.70710678118654752440084436210485,   // cos(pi / 4)
+                           0.5,
+                           0.25881904510252076234889883762405,   // cos(5 pi / 12)
+                           0.0};
+  m = (m % 24 + 24) % 24;
+  return m <= 6 ? q[m] : m <= 12 ? -q[12 - m] : m <= 18 ? -q[m - 12] : q[24 - m];
+}
+__host__ __device__ constexpr double sin24(int m) { return cos24(m - 6); }
+
+// z * exp(SIGN 2 pi i M / R) for R dividing 32 or R = 24; quarter turns exactly.
 template <int SIGN, int R, int M>
 __device__ __forceinline__ float2 rotate(float2 z) {
-  constexpr int m = (M % R) * (32 / R);  // in 32nds of a turn
+  constexpr int D = R == 24 ? 24 : 32;
+  constexpr int m = (M % R) * (D / R);  // in D-ths of a turn
   if constexpr (m == 0) {
     return z;
-  } else if constexpr (m == 8) {
+  } else if constexpr (4 * m == D) {
     return mul_si<SIGN>(z);
-  } else if constexpr (m == 16) {
+  } else if constexpr (2 * m == D) {
     return make_float2(-z.x, -z.y);
-  } else if constexpr (m == 24) {
+  } else if constexpr (4 * m == 3 * D) {
     return mul_si<-SIGN>(z);
   } else {
-    constexpr float c = (float)cos32(m), sn = (float)(SIGN * sin32(m));
+    constexpr float c = (float)(D == 24 ? cos24(m) : cos32(m));
+    constexpr float sn = (float)(SIGN * (D == 24 ? sin24(m) : sin32(m)));
     return make_float2(fmaf(z.x, c, -z.y * sn), fmaf(z.x, sn, z.y * c));
   }
 }
@@ -334,6 +361,11 @@ struct Dft<32, SIGN> {
   __device__ __forceinline__ static void run(float2* v) { dft_compose<8, 4, SIGN>(v); }
 };
 
+template <int SIGN>
+struct Dft<24, SIGN> {
+  __device__ __forceinline__ static void run(float2* v) { dft_compose<8, 3, SIGN>(v); }
+};
+
 // One Stockham pass; recurses into the next pass at compile time.
 // PIN: the input line is a zero-padded image line (image index i at
 // position i - N/2 mod n, N = n/2, zeros elsewhere); the first pass then
@@ -365,22 +397,23 @@ __device__ __forceinline__ void fft_pass(float2* X, const float2* tws, int col, 
                                          const Out& out, const Hook& hook = Hook()) {
   constexpr RadixPlan RP = radix_plan(NFFT, EV);
   constexpr int R = RP.r[PI];
-  constexpr int E = EV;
   constexpr int TPL = NFFT / EV;
-  constexpr int NB = E / R;
-  constexpr int STRIDE = NFFT / R;
+  constexpr int STRIDE = NFFT / R;                 // butterflies a line
+  constexpr int NB = (STRIDE + TPL - 1) / TPL;     // and a thread
+  constexpr bool EVEN = STRIDE % TPL == 0;         // else some warps sit the last one out
+  static_assert(EVEN || COLS == kFftCols, "whole warps");
   constexpr bool FIRST = PI == 0;
   constexpr bool LAST = PI == RP.count - 1;
   constexpr bool PRUNE_IN = FIRST && PIN && R % 4 == 0;
   constexpr bool PRUNE_OUT = LAST && POUT && R % 4 == 0;
   constexpr int Q = NFFT / 4;  // N / 2
-  static_assert(E % R == 0, "radix must divide the per-thread count");
-  static_assert(!(FIRST && PIN) || PRUNE_IN, "padded input needs a first radix of 32, 16, 8 or 4");
-  float2 v[E];
+  static_assert(!(FIRST && PIN) || PRUNE_IN, "padded input needs a first radix that 4 divides");
+  float2 v[NB * R];
 #pragma unroll
   for (int q = 0; q < NB; ++q) {
     const int j = tl + TPL * q;
-    const int k = j % NS;
+    if (!EVEN && j >= STRIDE) continue;
+    const int k = LAST ? j : j % NS;  // (NS R = NFFT in the last pass)
     float2 w[R];
     if constexpr (NS > 1) {
       const float2* T = tws + tw_offset<NFFT, EV>(PI) + k * R;
@@ -424,6 +457,7 @@ __device__ __forceinline__ void fft_pass(float2* X, const float2* tws, int col, 
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const int j = tl + TPL * q;
+      if (!EVEN && j >= STRIDE) continue;
       const int d = (j / NS) * NS * R + (j % NS);
 #pragma unroll
       for (int r = 0; r < R; ++r) X[(d + r * NS) * COLS + col] = v[q * R + r];
@@ -435,6 +469,7 @@ __device__ __forceinline__ void fft_pass(float2* X, const float2* tws, int col, 
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const int d = tl + TPL * q;  // NS R = NFFT in the last pass, so (j / NS) NS R + j % NS = j
+      if (!EVEN && d >= STRIDE) continue;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         if constexpr (PRUNE_OUT) {
@@ -580,8 +615,11 @@ struct OutAdjRows {
 };
 
 template <int NFFT, int KIND>
-__global__ void __launch_bounds__(Shape<NFFT, kValsPlain<NFFT>>::THREADS) fft_kernel(FftArgs a) {
-  constexpr int EV = kValsPlain<NFFT>;
+constexpr int kValsOf = KIND == kFwdCols || KIND == kAdjCols ? kValsCols<NFFT> : kValsPlain<NFFT>;
+
+template <int NFFT, int KIND>
+__global__ void __launch_bounds__(Shape<NFFT, kValsOf<NFFT, KIND>>::THREADS) fft_kernel(FftArgs a) {
+  constexpr int EV = kValsOf<NFFT, KIND>;
   constexpr int N = NFFT / 2;
   extern __shared__ float2 smem[];
   float2* X = smem;
@@ -1146,17 +1184,19 @@ constexpr int col_rows() {
 }
 // Tile buffers and CTAs per SM: the forward pass stages the N image rows in
 // one buffer (the next tile is requested once the first pass has read the
-// current one) with two CTAs per SM; the adjoint stages all 2N rows in one
-// buffer with two CTAs per SM where two such CTAs fit an SM's shared memory
-// (2N <= kAdjColsTwoCtaMax), else double-buffered with one CTA per SM.
-constexpr int kAdjColsTwoCtaMax = 384;
+// current one) with two CTAs per SM up to 2N = 512 and one above (two would
+// not fit the shared memory, and their bound on the registers made 1024
+// threads spill); the adjoint stages all 2N rows, in one buffer with two CTAs
+// per SM where two such CTAs fit an SM's shared memory (2N <= 384), double-
+// buffered with one CTA per SM at 512, in one buffer at 768 (at 1024 a tile
+// beside the exchange buffer does not fit: unstaged).
 template <int NFFT, int KIND>
 constexpr int col_bufs() {
-  return KIND == kFwdCols || NFFT <= kAdjColsTwoCtaMax ? 1 : 2;
+  return KIND == kAdjCols && NFFT == 512 ? 2 : 1;
 }
 template <int NFFT, int KIND>
 constexpr int col_ctas_per_sm() {
-  return KIND == kFwdCols || NFFT <= kAdjColsTwoCtaMax ? 2 : 1;
+  return NFFT <= (KIND == kFwdCols ? 512 : 384) ? 2 : 1;
 }
 template <int NFFT, int KIND>
 constexpr size_t col_smem() {
@@ -1287,23 +1327,23 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsCols<NFFT>>::THREADS, col_cta
 
 template <int NFFT>
 cudaError_t launch(int kind, const FftArgs& a, dim3 grid, cudaStream_t s) {
-  const size_t smem = Shape<NFFT, kValsPlain<NFFT>>::SMEM;
-  const dim3 block(Shape<NFFT, kValsPlain<NFFT>>::THREADS);
+  using Rows = Shape<NFFT, kValsPlain<NFFT>>;
+  using Cols = Shape<NFFT, kValsCols<NFFT>>;
   switch (kind) {
-    case kFwdRows: return launch_dep(fft_kernel<NFFT, kFwdRows>, grid, block, smem, s, a);
-    case kFwdCols: return launch_dep(fft_kernel<NFFT, kFwdCols>, grid, block, smem, s, a);
-    case kAdjCols: return launch_dep(fft_kernel<NFFT, kAdjCols>, grid, block, smem, s, a);
-    default: return launch_dep(fft_kernel<NFFT, kAdjRows>, grid, block, smem, s, a);
+    case kFwdRows: return launch_dep(fft_kernel<NFFT, kFwdRows>, grid, dim3(Rows::THREADS), Rows::SMEM, s, a);
+    case kFwdCols: return launch_dep(fft_kernel<NFFT, kFwdCols>, grid, dim3(Cols::THREADS), Cols::SMEM, s, a);
+    case kAdjCols: return launch_dep(fft_kernel<NFFT, kAdjCols>, grid, dim3(Cols::THREADS), Cols::SMEM, s, a);
+    default: return launch_dep(fft_kernel<NFFT, kAdjRows>, grid, dim3(Rows::THREADS), Rows::SMEM, s, a);
   }
 }
 
 template <int NFFT>
 cudaError_t configure_n() {
-  const int smem = (int)Shape<NFFT, kValsPlain<NFFT>>::SMEM;
+  const int smem = (int)Shape<NFFT, kValsPlain<NFFT>>::SMEM, csmem = (int)Shape<NFFT, kValsCols<NFFT>>::SMEM;
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(fft_kernel<NFFT, kFwdRows>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-  if ((e = cudaFuncSetAttribute(fft_kernel<NFFT, kFwdCols>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-  if ((e = cudaFuncSetAttribute(fft_kernel<NFFT, kAdjCols>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+  if ((e = cudaFuncSetAttribute(fft_kernel<NFFT, kFwdCols>, cudaFuncAttributeMaxDynamicSharedMemorySize, csmem))) return e;
+  if ((e = cudaFuncSetAttribute(fft_kernel<NFFT, kAdjCols>, cudaFuncAttributeMaxDynamicSharedMemorySize, csmem))) return e;
   if ((e = cudaFuncSetAttribute(fft_kernel<NFFT, kAdjRows>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
   int optin = 0, dev = 0;
   if ((e = cudaGetDevice(&dev))) return e;
