@@ -10,8 +10,8 @@
 //   per real component: m = b1 m + (1 - b1) g, v = b2 v + (1 - b2) g^2,
 //   V -= (lr / (1 - b1^k)) m / (sqrt(v) / sqrt(1 - b2^k) + eps).
 // The update reads Vin and writes Vout (ping-pong), because neighbours of a
-// voxel are read by other threads.  One thread per complex voxel, bins
-// fastest, so warps read and write contiguous runs.
+// voxel are read by other threads.  Bins are fastest, so warps read and write
+// contiguous runs; a thread walks a few voxels of one bin along x1.
 #include "prop_internal.cuh"
 #include "tv_adam.cuh"
 
@@ -19,7 +19,7 @@ namespace prop {
 namespace {
 
 constexpr int kOptThreads = 256;
-constexpr int kSeg = 1024;  // values per work unit
+constexpr int kOptLen = 8;   // most voxels that a thread walks
 
 __device__ double block_sum_d(double v, double* sh) {
 #pragma unroll
@@ -48,44 +48,116 @@ struct OptArgs {
   unsigned int* counter;
   const double* data_loss;
   double* loss_out;
-  long nvox;
   int N, Nf, T;
+  int fw, nfg, runs, len, nxb;  // a unit: fw bins (of nfg groups) x runs walks of len voxels (of nxb blocks) of a row
   AdamArgs p;
 };
 
-template <bool ADAM>
+// The TV gradient and the update of plans with several bin chunks.  Bound by
+// instruction issue, not by its bytes: a flat voxel index with a branch for
+// each neighbour took 80 us for the gradient of 512^2 x 24 voxels, whose
+// volume, data gradient and result are 151 MB (23 us).  A thread walks kOptLen
+// voxels along x1, so that the TV term towards the next voxel is handed on to
+// it, a voxel is one offset into each array, every neighbour load is
+// unconditional (a missing neighbour reads the voxel itself and is not used)
+// and the loads of U voxels are issued together: 55 us (61 us with a 64-bit
+// pointer for each row, 64 us at U = 1; U = 4 takes 54 us but 93 registers
+// and more).  TT: the volume has time neighbours.  Off: uint32_t while three
+// frames are within 4 GB, else size_t.
+template <bool ADAM, bool TT, typename Off>
 __global__ void __launch_bounds__(kOptThreads) opt_kernel(OptArgs a) {
-  // Work unit: a segment of kSeg consecutive values of one image row (t, i2);
-  // a row holds N * Nf values (i1, f).
   grid_dep_wait();
   grid_dep_release();
+  constexpr int U = 2;
   const float eps2 = a.p.tv_eps * a.p.tv_eps;
-  const int rowlen = a.N * a.Nf;
-  const int segs = (rowlen + kSeg - 1) / kSeg;
-  const long nseg = (long)a.T * a.N * segs;
+  const bool xy = a.p.tv_xy != 0.f;
+  const size_t st = (size_t)a.N * a.N * a.Nf;
+  const Off sx = (Off)a.Nf * 8, d2 = (Off)a.N * sx, dt = (Off)st * 8;
+  const int run = threadIdx.x / a.fw, fl = threadIdx.x - run * a.fw, per_row = a.nfg * a.nxb;
+  const long units = (long)a.T * a.N * per_row;
   float local = 0.f;
-  for (long sgi = blockIdx.x; sgi < nseg; sgi += gridDim.x) {
-    const long row = sgi / segs;
-    const int seg = (int)(sgi - row * segs);
-    const int i2 = (int)(row % a.N);
-    const int t = (int)(row / a.N);
-    const long rbase = row * rowlen;
-    for (int e = seg * kSeg + threadIdx.x; e < min(rowlen, (seg + 1) * kSeg); e += blockDim.x) {
-      const long idx = rbase + e;
-      const int i1 = e / a.Nf;
-      const float2 x = a.Vin[idx];
-      float2 gxy, gt;
-      local = __fadd_rn(local, voxel_tv(a.Vin, (size_t)idx, x, i1, i2, t, a.N, a.Nf, a.T, a.p.tv_xy, a.p.tv_t,
-                                        eps2, &gxy, &gt));
-      const float2 g = total_grad(a.g[idx], gxy, gt, a.p);
-      if constexpr (ADAM) {
-        float2 mm = a.m[idx], vv = a.v[idx];
-        const float2 nx = adam_voxel(x, g, mm, vv, a.p);
-        a.m[idx] = mm;
-        a.v[idx] = vv;
-        a.out[idx] = nx;
-      } else {
-        a.out[idx] = g;
+  for (long unit = blockIdx.x; unit < units; unit += gridDim.x) {
+    const int row = (int)(unit / per_row), rest = (int)(unit - (long)row * per_row);
+    const int xb = rest / a.nfg, f = (rest - xb * a.nfg) * a.fw + fl;
+    const int i2 = row % a.N, t = row / a.N;
+    const int lo = (xb * a.runs + run) * a.len, hi = min(a.N, lo + a.len);
+    if (run >= a.runs || f >= a.Nf || lo >= hi) continue;
+    const bool h2p = xy && i2 + 1 < a.N, h2m = xy && i2 > 0;
+    const bool htp = TT && t + 1 < a.T, htm = TT && t > 0;
+    // offsets count from the frame before this one (from this one when t = 0)
+    const size_t first = (size_t)(t > 0 ? t - 1 : 0) * st;
+    const char* V = reinterpret_cast<const char*>(a.Vin + first);
+    char* G = reinterpret_cast<char*>(const_cast<float2*>(a.g) + first);
+    char* M1 = reinterpret_cast<char*>(a.m + (ADAM ? first : 0));
+    char* M2 = reinterpret_cast<char*>(a.v + (ADAM ? first : 0));
+    char* O = reinterpret_cast<char*>(a.out + first);  // may be G
+    auto at = [](const char* b, Off o) { return __ldg(reinterpret_cast<const float2*>(b + o)); };
+    auto ref = [](char* b, Off o) -> float2& { return *reinterpret_cast<float2*>(b + o); };
+    const Off d2p = h2p ? d2 : 0, d2m = h2m ? d2 : 0, dtp = htp ? dt : 0, dtm = htm ? dt : 0;
+    Off off = (t > 0 ? dt : 0) + (Off)i2 * d2 + (Off)lo * sx + (Off)f * 8;
+    float2 x = at(V, off);
+    float mag;
+    float2 t1m = make_float2(0.f, 0.f);
+    if (xy && lo > 0) t1m = tv_term(csub_rn(x, at(V, off - sx)), eps2, &mag);
+    for (int i0 = lo; i0 < hi; i0 += U, off += U * sx) {
+      float2 xp[U], x2p[U], x2m[U], xtp[U], xtm[U], gd[U], mm[U], vv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i1 = min(i0 + u, hi - 1);
+        const Off c = off + (Off)(i1 - i0) * sx;
+        xp[u] = at(V, i1 + 1 < a.N ? c + sx : c);
+        x2p[u] = at(V, c + d2p);
+        x2m[u] = at(V, c - d2m);
+        if constexpr (TT) {
+          xtp[u] = at(V, c + dtp);
+          xtm[u] = at(V, c - dtm);
+        }
+        gd[u] = ref(G, c);
+        if constexpr (ADAM) {
+          mm[u] = ref(M1, c);
+          vv[u] = ref(M2, c);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i1 = i0 + u;
+        if (i1 >= hi) break;
+        const Off c = off + (Off)u * sx;
+        // voxel_tv_nb's terms in its order
+        float2 gxy = make_float2(0.f, 0.f), gt = make_float2(0.f, 0.f), t1p = make_float2(0.f, 0.f);
+        float sxy = 0.f, stt = 0.f;
+        if (xy) {
+          if (i1 + 1 < a.N) {
+            t1p = tv_term(csub_rn(xp[u], x), eps2, &mag);
+            gxy = csub_rn(gxy, t1p);
+            sxy = __fadd_rn(sxy, mag);
+          }
+          if (i1 > 0) gxy = cadd_rn(gxy, t1m);
+          if (h2p) {
+            gxy = csub_rn(gxy, tv_term(csub_rn(x2p[u], x), eps2, &mag));
+            sxy = __fadd_rn(sxy, mag);
+          }
+          if (h2m) gxy = cadd_rn(gxy, tv_term(csub_rn(x, x2m[u]), eps2, &mag));
+        }
+        if constexpr (TT) {
+          if (htp) {
+            gt = csub_rn(gt, tv_term(csub_rn(xtp[u], x), eps2, &mag));
+            stt = __fadd_rn(stt, mag);
+          }
+          if (htm) gt = cadd_rn(gt, tv_term(csub_rn(x, xtm[u]), eps2, &mag));
+        }
+        local = __fadd_rn(local, fmaf(a.p.tv_xy, sxy, __fmul_rn(TT ? a.p.tv_t : 0.f, stt)));
+        const float2 g = total_grad(gd[u], gxy, gt, a.p);
+        if constexpr (ADAM) {
+          const float2 nx = adam_voxel(x, g, mm[u], vv[u], a.p);
+          ref(M1, c) = mm[u];
+          ref(M2, c) = vv[u];
+          ref(O, c) = nx;
+        } else {
+          ref(O, c) = g;
+        }
+        t1m = t1p;
+        x = xp[u];
       }
     }
   }
@@ -150,13 +222,6 @@ __global__ void __launch_bounds__(kOptThreads) psnr_kernel(const float2* a, cons
   }
 }
 
-unsigned opt_blocks(const Plan& p, const Reducer* red) {
-  const long segs = ((long)p.N * p.Nf + kSeg - 1) / kSeg;
-  long need = (long)p.T * p.N * segs;
-  long cap = red ? std::min<long>(red->capacity, 16384) : 16384;
-  return (unsigned)std::max<long>(1, std::min(need, cap));
-}
-
 OptArgs make_args(const Plan& p, const float2* Vin, const float2* g, float2* out, const AdamArgs& aa,
                   const Reducer* red, const double* data_loss, double* loss_out) {
   OptArgs a{};
@@ -167,12 +232,27 @@ OptArgs make_args(const Plan& p, const float2* Vin, const float2* g, float2* out
   a.counter = red ? red->counter : nullptr;
   a.data_loss = data_loss;
   a.loss_out = loss_out;
-  a.nvox = (long)p.vol_elems();
   a.N = p.N;
   a.Nf = p.Nf;
   a.T = p.T;
+  a.fw = std::min(p.Nf, kOptThreads);
+  a.nfg = (p.Nf + a.fw - 1) / a.fw;
+  a.runs = kOptThreads / a.fw;
+  a.len = std::min(kOptLen, (p.N + a.runs - 1) / a.runs);
+  a.nxb = (p.N + a.runs * a.len - 1) / (a.runs * a.len);
   a.p = aa;
   return a;
+}
+
+template <bool ADAM>
+cudaError_t launch_opt(const OptArgs& a, bool small, const Reducer* red, cudaStream_t s) {
+  const long units = (long)a.T * a.N * a.nfg * a.nxb;
+  const long cap = red ? std::min<long>(red->capacity, 16384) : 16384;
+  const dim3 grid((unsigned)std::max<long>(1, std::min(units, cap)));
+  auto go = [&](auto kern) { return launch_dep(kern, grid, dim3(kOptThreads), 0, s, a); };
+  if (a.T > 1 && a.p.tv_t != 0.f)
+    return small ? go(opt_kernel<ADAM, true, uint32_t>) : go(opt_kernel<ADAM, true, size_t>);
+  return small ? go(opt_kernel<ADAM, false, uint32_t>) : go(opt_kernel<ADAM, false, size_t>);
 }
 
 }  // namespace
@@ -183,13 +263,12 @@ cudaError_t tv_adam(const Plan& p, const float2* Vin, const float2* g, float2* m
   OptArgs a = make_args(p, Vin, g, Vout, aa, red, data_loss, loss_out);
   a.m = m;
   a.v = v;
-  return launch_dep(opt_kernel<true>, dim3(opt_blocks(p, red)), dim3(kOptThreads), 0, s, a);
+  return launch_opt<true>(a, frames_in_32_bits(p), red, s);
 }
 
 cudaError_t tv_grad(const Plan& p, const float2* V, const float2* g, float2* grad, const AdamArgs& aa,
                     const Reducer* red, const double* data_loss, double* loss_out, cudaStream_t s) {
-  OptArgs a = make_args(p, V, g, grad, aa, red, data_loss, loss_out);
-  return launch_dep(opt_kernel<false>, dim3(opt_blocks(p, red)), dim3(kOptThreads), 0, s, a);
+  return launch_opt<false>(make_args(p, V, g, grad, aa, red, data_loss, loss_out), frames_in_32_bits(p), red, s);
 }
 
 cudaError_t psnr(const Plan& p, const float2* img, const float2* ref, long count, double* out, cudaStream_t s) {
