@@ -100,13 +100,20 @@ __host__ __device__ constexpr int tw_offset(int pass) {
   return off;
 }
 
-// Values per thread: 16 (two radix-8 butterflies a pass), 12 for lengths
-// with a factor 3 (radices 4, 2, 3).  (8 values a thread, twice the
-// threads, measured slower for the column passes at n = 512.)
+// Values per thread of the row passes, alone and fused (the same, so that they
+// round alike): 16 (two radix-8 butterflies a pass), 12 for lengths with a
+// factor 3 (radices 4, 2, 3); above 512 points, where one CTA of 1024 threads
+// was all that fitted an SM, 32 and 24, which make two passes as in the columns
+// (768 points, 64 bins: forward 82 -> 64 us, adjoint 72 -> 62, fused update
+// 248 -> 229; 1024 points 41 -> 36 and 36 -> 36 us; 32 at 512 points leaves the
+// fused update half its threads, 56 -> 68 us).  The image transforms of the
+// projection model, 4 lines a CTA, keep 16 and 12.
 template <int NFFT>
-constexpr int kValsPlain = (NFFT % 3 == 0) ? 12 : 16;
+constexpr int kValsPlain = NFFT == 1024 ? 32 : NFFT == 768 ? 24 : NFFT % 3 == 0 ? 12 : 16;
 template <int NFFT>
-constexpr int kValsFused = (NFFT % 3 == 0) ? 12 : 16;
+constexpr int kValsFused = kValsPlain<NFFT>;
+template <int NFFT>
+constexpr int kValsCart = NFFT % 3 == 0 ? 12 : 16;
 // Values per thread of the column passes, as many as make two passes of them
 // (one shared-memory exchange): 32 at n = 512 (radix 32 then 16) and 1024 (32,
 // 32), 24 at n = 384 (24, 16) and 768 (24, 32), with twice the registers and
@@ -129,14 +136,14 @@ struct Shape {
   static constexpr size_t SMEM = (size_t)NFFT * kFftCols * sizeof(float2) + (size_t)TW * sizeof(float2);
 };
 
-// The thread's place in its line (16 lines side by side); the mask tells the
+// The thread's place in its line (COLS lines side by side); the mask tells the
 // compiler its range, so that what depends on a position's block or on the
 // crop is decided at compile time where TPL divides it.
-template <int NFFT, int EV>
+template <int NFFT, int EV, int COLS = kFftCols>
 __device__ __forceinline__ int line_thread(int tid) {
   constexpr int TPL = Shape<NFFT, EV>::TPL;
   static_assert((TPL & (TPL - 1)) == 0, "threads a line: a power of two");
-  return (tid / kFftCols) & (TPL - 1);
+  return (tid / COLS) & (TPL - 1);
 }
 
 // Fill the per-pass twiddle tables from the length-NFFT table exp(-2 pi i m / NFFT).
@@ -401,7 +408,11 @@ __device__ __forceinline__ void fft_pass(float2* X, const float2* tws, int col, 
   constexpr int STRIDE = NFFT / R;                 // butterflies a line
   constexpr int NB = (STRIDE + TPL - 1) / TPL;     // and a thread
   constexpr bool EVEN = STRIDE % TPL == 0;         // else some warps sit the last one out
-  static_assert(EVEN || COLS == kFftCols, "whole warps");
+  static_assert((STRIDE % TPL) * COLS % 32 == 0, "whole warps");
+  // With 8 lines a tile a half-warp's two positions are in different halves of
+  // the banks when they are read, and would be in the same half when they are
+  // written (R apart): odd rows of the R0 x R1 exchange swap their neighbours.
+  constexpr bool SWAP = COLS == 8 && RP.count == 2 && RP.r[0] % 2 == 0;
   constexpr bool FIRST = PI == 0;
   constexpr bool LAST = PI == RP.count - 1;
   constexpr bool PRUNE_IN = FIRST && PIN && R % 4 == 0;
@@ -443,7 +454,7 @@ __device__ __forceinline__ void fft_pass(float2* X, const float2* tws, int col, 
       } else if constexpr (FIRST) {
         x = in(pos, col);
       } else {
-        x = X[pos * COLS + col];
+        x = X[(SWAP ? r * STRIDE + (j ^ (r & 1)) : pos) * COLS + col];
       }
       if constexpr (NS > 1) {
         if (r > 0) x = SIGN < 0 ? cmul(x, w[r]) : cmulc(x, w[r]);
@@ -460,7 +471,10 @@ __device__ __forceinline__ void fft_pass(float2* X, const float2* tws, int col, 
       if (!EVEN && j >= STRIDE) continue;
       const int d = (j / NS) * NS * R + (j % NS);
 #pragma unroll
-      for (int r = 0; r < R; ++r) X[(d + r * NS) * COLS + col] = v[q * R + r];
+      for (int r = 0; r < R; ++r) {
+        const int pos = SWAP ? d + r + (r & 1 ? -(j & 1) : j & 1) : d + r * NS;
+        X[pos * COLS + col] = v[q * R + r];
+      }
     }
     Sync::sync();
     if constexpr (FIRST) hook();
@@ -617,33 +631,48 @@ struct OutAdjRows {
 template <int NFFT, int KIND>
 constexpr int kValsOf = KIND == kFwdCols || KIND == kAdjCols ? kValsCols<NFFT> : kValsPlain<NFFT>;
 
+// Lines a CTA of these kernels.  The long rows take 8, so that two or three
+// CTAs fit an SM and one's loads overlap another's butterflies (16 lines, one
+// CTA -> 8 lines: 1024 points 36 -> 32 us forward and 36 -> 30 us adjoint, 768
+// points 64 -> 53 us forward at three CTAs, 58 at two; the 768-point adjoint
+// pass, which writes half as much as it reads, is better off with 16: 62
+// against 66 us).
 template <int NFFT, int KIND>
-__global__ void __launch_bounds__(Shape<NFFT, kValsOf<NFFT, KIND>>::THREADS) fft_kernel(FftArgs a) {
-  constexpr int EV = kValsOf<NFFT, KIND>;
+constexpr int kColsOf = (NFFT > 512 && KIND == kFwdRows) || (NFFT == 1024 && KIND == kAdjRows) ? 8 : kFftCols;
+template <int NFFT, int KIND>
+constexpr int kMinCtasOf = kColsOf<NFFT, KIND> == kFftCols ? 0 : NFFT == 768 ? 3 : 2;
+template <int NFFT, int KIND>
+constexpr int kThreadsOf = NFFT / kValsOf<NFFT, KIND> * kColsOf<NFFT, KIND>;
+template <int NFFT, int KIND>
+constexpr size_t kSmemOf = ((size_t)NFFT * kColsOf<NFFT, KIND> + Shape<NFFT, kValsOf<NFFT, KIND>>::TW) * sizeof(float2);
+
+template <int NFFT, int KIND>
+__global__ void __launch_bounds__(kThreadsOf<NFFT, KIND>, kMinCtasOf<NFFT, KIND>) fft_kernel(FftArgs a) {
+  constexpr int EV = kValsOf<NFFT, KIND>, COLS = kColsOf<NFFT, KIND>;
   constexpr int N = NFFT / 2;
   extern __shared__ float2 smem[];
   float2* X = smem;
-  float2* tw = smem + NFFT * kFftCols;
+  float2* tw = smem + NFFT * COLS;
   build_twiddles<NFFT, EV>(tw, a.twiddle);
   grid_dep_wait();
   grid_dep_release();
   __syncthreads();
-  const int col = threadIdx.x % kFftCols;
-  const int tl = line_thread<NFFT, EV>(threadIdx.x);
+  const int col = threadIdx.x % COLS;
+  const int tl = line_thread<NFFT, EV, COLS>(threadIdx.x);
   if constexpr (KIND == kFwdRows || KIND == kAdjRows) {
     const size_t row = blockIdx.y;  // t*N + i2
     const int i2 = (int)(row % N);
-    const int fbase = blockIdx.x * kFftCols;
+    const int fbase = blockIdx.x * COLS;
     const size_t wpos = row * NFFT * a.C + fbase, vox = row * N * a.Nf + a.f0 + fbase;
     const uint32_t wstep = (uint32_t)a.C * 8u, vstep = (uint32_t)a.Nf * 8u;
     if constexpr (KIND == kFwdRows) {
       InFwdRows in{a.src + vox, a.deapod, vstep, a.Cv - fbase, a.deapod[i2]};
       OutFwdRows out{a.dst + wpos, wstep, a.C - fbase};
-      fft_pass<NFFT, EV, -1, 0, 1, true, false>(X, tw, col, tl, in, out);
+      fft_pass<NFFT, EV, -1, 0, 1, true, false, CtaSync, InFwdRows, OutFwdRows, NoHook, COLS>(X, tw, col, tl, in, out);
     } else {
       InAdjRows in{a.src + wpos, wstep, a.Cv - fbase};
       OutAdjRows<NFFT> out{a.dst + vox, a.deapod, vstep, a.Cv - fbase, a.deapod[i2] * a.scale};
-      fft_pass<NFFT, EV, +1, 0, 1, false, true>(X, tw, col, tl, in, out);
+      fft_pass<NFFT, EV, +1, 0, 1, false, true, CtaSync, InAdjRows, OutAdjRows<NFFT>, NoHook, COLS>(X, tw, col, tl, in, out);
     }
   } else {
     const size_t nq = (size_t)NFFT * a.C, q = (size_t)blockIdx.x * kFftCols, t = blockIdx.y;
@@ -869,10 +898,11 @@ __device__ __forceinline__ void prefetch_update_rows(const FusedArgs& a, size_t 
   prefetch_l2(a.v + row * rl, rb);
 }
 
-// Register cap: 64 a thread (two CTAs of 512 threads per SM).
+// Register cap: 64 a thread (two CTAs of 512 threads per SM); above 512 points
+// one CTA of 512 threads fits the shared memory.
 template <int NFFT>
 constexpr int fused_min_blocks() {
-  return 65536 / (Shape<NFFT, kValsFused<NFFT>>::THREADS * 64) > 16
+  return NFFT > 512 ? 1 : 65536 / (Shape<NFFT, kValsFused<NFFT>>::THREADS * 64) > 16
              ? 16
              : 65536 / (Shape<NFFT, kValsFused<NFFT>>::THREADS * 64);
 }
@@ -1000,7 +1030,7 @@ struct InTile {
 
 template <int NFFT>
 constexpr bool fused_ws_fits() {
-  return Shape<NFFT, kValsFused<NFFT>>::THREADS % 32 == 0 && Shape<NFFT, kValsFused<NFFT>>::THREADS <= 512;
+  return NFFT <= 512 && Shape<NFFT, kValsFused<NFFT>>::THREADS % 32 == 0 && Shape<NFFT, kValsFused<NFFT>>::THREADS <= 512;
 }
 
 template <int NFFT>
@@ -1327,24 +1357,29 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsCols<NFFT>>::THREADS, col_cta
 
 template <int NFFT>
 cudaError_t launch(int kind, const FftArgs& a, dim3 grid, cudaStream_t s) {
-  using Rows = Shape<NFFT, kValsPlain<NFFT>>;
-  using Cols = Shape<NFFT, kValsCols<NFFT>>;
+  auto go = [&](auto kern, int lines, int threads, size_t smem) {
+    return launch_dep(kern, dim3((grid.x + lines - 1) / lines, grid.y), dim3(threads), smem, s, a);
+  };
+#define PROP_GO(K) go(fft_kernel<NFFT, K>, kColsOf<NFFT, K>, kThreadsOf<NFFT, K>, kSmemOf<NFFT, K>)
   switch (kind) {
-    case kFwdRows: return launch_dep(fft_kernel<NFFT, kFwdRows>, grid, dim3(Rows::THREADS), Rows::SMEM, s, a);
-    case kFwdCols: return launch_dep(fft_kernel<NFFT, kFwdCols>, grid, dim3(Cols::THREADS), Cols::SMEM, s, a);
-    case kAdjCols: return launch_dep(fft_kernel<NFFT, kAdjCols>, grid, dim3(Cols::THREADS), Cols::SMEM, s, a);
-    default: return launch_dep(fft_kernel<NFFT, kAdjRows>, grid, dim3(Rows::THREADS), Rows::SMEM, s, a);
+    case kFwdRows: return PROP_GO(kFwdRows);
+    case kFwdCols: return PROP_GO(kFwdCols);
+    case kAdjCols: return PROP_GO(kAdjCols);
+    default: return PROP_GO(kAdjRows);
   }
+#undef PROP_GO
 }
 
 template <int NFFT>
 cudaError_t configure_n() {
-  const int smem = (int)Shape<NFFT, kValsPlain<NFFT>>::SMEM, csmem = (int)Shape<NFFT, kValsCols<NFFT>>::SMEM;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(fft_kernel<NFFT, kFwdRows>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-  if ((e = cudaFuncSetAttribute(fft_kernel<NFFT, kFwdCols>, cudaFuncAttributeMaxDynamicSharedMemorySize, csmem))) return e;
-  if ((e = cudaFuncSetAttribute(fft_kernel<NFFT, kAdjCols>, cudaFuncAttributeMaxDynamicSharedMemorySize, csmem))) return e;
-  if ((e = cudaFuncSetAttribute(fft_kernel<NFFT, kAdjRows>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+  auto smem = [](auto kern, size_t bytes) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  };
+  if ((e = smem(fft_kernel<NFFT, kFwdRows>, kSmemOf<NFFT, kFwdRows>))) return e;
+  if ((e = smem(fft_kernel<NFFT, kFwdCols>, kSmemOf<NFFT, kFwdCols>))) return e;
+  if ((e = smem(fft_kernel<NFFT, kAdjCols>, kSmemOf<NFFT, kAdjCols>))) return e;
+  if ((e = smem(fft_kernel<NFFT, kAdjRows>, kSmemOf<NFFT, kAdjRows>))) return e;
   int optin = 0, dev = 0;
   if ((e = cudaGetDevice(&dev))) return e;
   if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
@@ -1628,11 +1663,11 @@ struct InCartBuf {
 
 template <int NFFT>
 constexpr int cart_threads() {
-  return NFFT / kValsPlain<NFFT> * kCartCols;
+  return NFFT / kValsCart<NFFT> * kCartCols;
 }
 template <int NFFT>
 constexpr size_t cart_smem() {
-  return (size_t)NFFT * kCartCols * sizeof(float2) + (size_t)Shape<NFFT, kValsPlain<NFFT>>::TW * sizeof(float2);
+  return (size_t)NFFT * kCartCols * sizeof(float2) + (size_t)Shape<NFFT, kValsCart<NFFT>>::TW * sizeof(float2);
 }
 template <int NFFT>
 constexpr size_t cart_loss_smem() {  // and the gradient between the two column passes
@@ -1641,7 +1676,7 @@ constexpr size_t cart_loss_smem() {  // and the gradient between the two column 
 
 template <int NFFT, int PASS>
 __global__ void __launch_bounds__(cart_threads<NFFT>()) cart_fft_kernel(CartArgs a) {
-  constexpr int EV = kValsPlain<NFFT>;
+  constexpr int EV = kValsCart<NFFT>;
   constexpr int CC = kCartCols;
   extern __shared__ float2 smem[];
   float2* X = smem;
@@ -1767,7 +1802,7 @@ cudaError_t fft_forward_rows(const Plan& p, const float2* V, int f0, cudaStream_
   a.dst = p.rows;
   a.f0 = f0;
   a.Cv = std::min(p.chunk, p.Nf - f0);
-  dim3 grid((a.C + kFftCols - 1) / kFftCols, p.T * p.N);
+  dim3 grid(a.C, p.T * p.N);  // x: lines
   return dispatch(p.n, kFwdRows, a, grid, s);
 }
 
@@ -1827,7 +1862,7 @@ cudaError_t fft_forward_cols(const Plan& p, cudaStream_t s) {
   FftArgs a = base_args(p);
   a.src = p.rows;
   a.dst = p.grid;
-  dim3 grid(p.n * p.cs / kFftCols, p.T);
+  dim3 grid(p.n * p.cs, p.T);  // x: lines
   return dispatch(p.n, kFwdCols, a, grid, s);
 }
 
@@ -1836,7 +1871,7 @@ cudaError_t fft_adjoint_cols(const Plan& p, cudaStream_t s) {
   FftArgs a = base_args(p);
   a.src = p.grid;
   a.dst = p.rows;
-  dim3 grid(p.n * p.cs / kFftCols, p.T);
+  dim3 grid(p.n * p.cs, p.T);  // x: lines
   return dispatch(p.n, kAdjCols, a, grid, s);
 }
 
@@ -1847,7 +1882,7 @@ cudaError_t fft_adjoint_rows(const Plan& p, float2* out, int f0, float scale, cu
   a.f0 = f0;
   a.scale = scale;
   a.Cv = std::min(p.chunk, p.Nf - f0);
-  dim3 grid((a.Cv + kFftCols - 1) / kFftCols, p.T * p.N);
+  dim3 grid(a.Cv, p.T * p.N);  // x: lines
   return dispatch(p.n, kAdjRows, a, grid, s);
 }
 

@@ -23,6 +23,8 @@ TOL = 5e-6
     (32, 16, 4, 5, 32, 2, 0.0),
     (96, 8, 3, 4, 64, 2, 1e-2),
     (64, 33, 3, 4, 64, 1, 1e-2),   # one frame: TV in time is zero
+    (384, 5, 2, 1, 16, 2, 1e-2),   # 24 values a thread
+    (512, 3, 2, 1, 16, 1, 0.0),    # 32 values a thread
 ])
 def test_loss_and_gradient(N, Nf, B, L, R, T, tv_t):
     from paper_2311_13177_gb300 import Plan, ReconParams
@@ -37,3 +39,20 @@ def test_loss_and_gradient(N, Nf, B, L, R, T, tv_t):
     plan.destroy()
     assert abs(loss - want) < TOL * abs(want)
     assert rel(grad.cpu().numpy(), ref) < TOL
+
+
+@pytest.mark.parametrize("N,Nf", [(384, 5), (512, 3)])
+def test_update_of_long_rows(N, Nf):
+    """Three iterations of the fused update at 24 and 32 values a thread: Adam's
+    epsilon of 100, above the gradient's components, makes a step proportional
+    to the gradient, whose 5e-6 the volume then has; 1e-5."""
+    from paper_2311_13177_gb300 import Plan, ReconParams
+    c = random_case(N, Nf, 2, 1, 16, 1, seed=N + Nf)
+    g = geometry(N, 1, 16, c["theta"], c["delta"], c["blade_frame"], 1)
+    kw = dict(iters=3, lr=1e-1, eps=1e2, tv_xy=5.0, tv_eps=1e-2)
+    Vo, tro = oracle.reconstruct(c["y"].astype(np.complex128), g, oracle.ReconParams(**kw))
+    plan = Plan(N, 1, 16, c["theta"], c["delta"], c["blade_frame"], 1, kb_width=8)
+    V, tr = plan.reconstruct(torch.from_numpy(c["y"]).cuda(), ReconParams(**kw))
+    plan.destroy()
+    assert rel(V.cpu().numpy(), Vo) < 1e-5
+    assert np.max(np.abs(tr - tro) / np.abs(tro)) < 1e-5
