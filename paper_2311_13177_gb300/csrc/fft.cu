@@ -2,13 +2,13 @@
 //
 // The 2N x 2N transform of every (frame, bin) slice is done as two passes of
 // 1-D transforms of length n = 2N along one axis, each CTA transforming a
-// tile of kFftCols = 16 lines that are adjacent in memory, so that every
-// global access of a warp covers two runs of 16 consecutive complex64
-// values (2 x 128 B, fully coalesced).  Bins are the fastest axis of every
+// tile of kFftCols = 16 lines (8 in the long row passes) that are adjacent in
+// memory, so that every global access of a warp covers two runs of 16
+// consecutive complex64 values (2 x 128 B, fully coalesced).  Bins are the fastest axis of every
 // array, so the "lines" of a pass are (u1, f) columns of the grid or the
 // bins of one image row.
 //
-// Each 1-D transform is a mixed-radix Stockham FFT (radices 8, 4, 2, 3):
+// Each 1-D transform is a mixed-radix Stockham FFT (radix_plan):
 // pass p with radix R and stride Ns (product of the previous radices)
 // reads R values at stride n/R, multiplies by exp(-+2 pi i r (j mod Ns) /
 // (Ns R)), does an R-point DFT in registers and writes the results at
@@ -16,7 +16,8 @@
 // directly (zero padding and deapodisation applied on the fly), the last
 // pass writes global memory directly (cropping and scaling applied on the
 // fly); intermediate passes exchange through shared memory in place.
-// Every thread holds E = 16 (n = 2^a) or 12 (n = 3 * 2^a) values per pass.
+// Every thread holds E = 16 (n = 2^a) or 12 (n = 3 * 2^a) values per pass,
+// 32 and 24 in the long transforms (kValsPlain, kValsCols).
 #include <type_traits>
 
 #include "prop_internal.cuh"

@@ -946,7 +946,7 @@ struct MultiSpread {
 
 // One launch for several problems with the same bin stride and list kind,
 // CTAs mapped onto each problem's balanced item ranges as in
-// interp2_multi_kernel; every cell sums its own terms in its list's order.
+// quads_multi_kernel; every cell sums its own terms in its list's order.
 template <int CS, bool GROUPED>
 __global__ void __launch_bounds__(kSpreadThreads, kSpreadCtasPerSm)
     spread_stage_multi_kernel(const __grid_constant__ MultiSpread m) {
