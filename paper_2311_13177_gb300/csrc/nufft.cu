@@ -455,8 +455,7 @@ __device__ __forceinline__ void quads_body(const QuadArgs& a, int it_beg, int it
     int k = 0;
     for (int item = it_beg; item < it_end; ++item, ++k) {
       const int b = k % NS;
-      if (!mbar_wait_bounded(&full[b], (uint32_t)((k / NS) & 1))) s_abort = 1;
-      if (s_abort) break;
+      if (!mbar_wait_warp(&full[b], (uint32_t)((k / NS) & 1), &s_abort)) break;
       const int4 head = s_head[b];
       int u = warp - head.z;
       u = u < 0 ? u + NCW : u;
@@ -906,8 +905,7 @@ __device__ __forceinline__ void spread_stage_body(float2* grid, const float2* co
       const int b = k % NBUF;
       const int4 d = __ldg(&sitems[item]);
       const int ncp = (d.y + 1) & ~1;
-      if (!mbar_wait_bounded(&full[b], (uint32_t)((k / NBUF) & 1))) s_abort = 1;
-      if (s_abort) break;
+      if (!mbar_wait_warp(&full[b], (uint32_t)((k / NBUF) & 1), &s_abort)) break;
       if constexpr (GROUPED)
         gather_groups<CS>(stage + (size_t)b * kSpreadStageInt2, d.y, d.z, lane, &s_next[b], grid, contrib, Cv, n);
       else
@@ -1029,8 +1027,7 @@ __global__ void __launch_bounds__(kSpreadThreads, kSpreadCtasPerSm)
     grid_dep_release();
     for (int k = 0;; ++k) {
       const int b = k % NBUF;
-      if (!mbar_wait_bounded(&full[b], (uint32_t)((k / NBUF) & 1))) s_abort = 1;
-      if (s_abort) break;
+      if (!mbar_wait_warp(&full[b], (uint32_t)((k / NBUF) & 1), &s_abort)) break;
       const int item = s_item[b];
       if (item < 0) break;
       const int4 d = __ldg(&sitems[item]);

@@ -69,6 +69,16 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     if (clock64() - t0 > limit) return false;
   return true;
 }
+// Bounded wait of a whole warp: true when the warp goes on.  An expired wait
+// sets *abort, and a set flag ends every warp's work.  The lanes leave the wait
+// one by one and another warp may set the flag in between, so what each lane
+// reads of it may differ: the warp goes by their vote, as lanes that went on
+// alone would wait for the others in the next shuffle for good.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                               long long limit = kWaitLimitCycles) {
+  if (!mbar_wait_bounded(bar, parity, limit)) *abort = 1;
+  return !__any_sync(0xffffffffu, *abort);
+}
 // Asynchronous prefetch of a contiguous range into L2 (16-byte aligned
 // address, size a multiple of 16); no completion to wait for.
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
