@@ -1093,7 +1093,7 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsFused<NFFT>>::THREADS + kUpdT
   // voxels' loads with time neighbours where 64 spilled at two.  Together
   // with those loads issued at once: dynamic 445 -> 370 us.
   constexpr bool SPLIT = FT == kUpdThreads;
-  constexpr int FREG = EV == 12 ? 48 : 56;  // configure_n checks the launch's registers
+  constexpr int FREG = EV == 12 ? 48 : 56;  // fused_ws_runs checks the launch's registers
   if (threadIdx.x < FT) {
     if constexpr (SPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(FREG));
     const int col = threadIdx.x % kFftCols;
@@ -1412,14 +1412,6 @@ cudaError_t configure_n() {
     return e;
   if constexpr (fused_ws_fits<NFFT>()) {
     if (fused_ws_smem<NFFT>() <= (size_t)optin - 1024) {
-      if (Shape<NFFT, kValsFused<NFFT>>::THREADS == kUpdThreads) {
-        // the register split of the two groups takes 64 a thread of the launch
-        // and would wait forever for registers that it does not have
-        cudaFuncAttributes fa, fb;
-        if ((e = cudaFuncGetAttributes(&fa, fused_rows_ws_kernel<NFFT, true>))) return e;
-        if ((e = cudaFuncGetAttributes(&fb, fused_rows_ws_kernel<NFFT, false>))) return e;
-        if (fa.numRegs < 64 || fb.numRegs < 64) return cudaErrorInvalidConfiguration;
-      }
       const int wsm = (int)fused_ws_smem<NFFT>();
       if ((e = cudaFuncSetAttribute(fused_rows_ws_kernel<NFFT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     wsm)))
@@ -1759,10 +1751,30 @@ cudaError_t dispatch_fused_ws(int n, const CUtensorMap& tm, const FusedArgs& a, 
   }
 }
 
-bool fused_ws_size_ok(int n, size_t room) {
+// Whether the warp-specialised row kernel can run: its shared memory fits, and
+// where its two groups share out the launch's registers, the launch has the 64
+// a thread that the split hands out (it would wait forever for registers that
+// it does not have).  The per-row kernel serves what it cannot.
+template <int NFFT>
+bool fused_ws_runs_n(size_t room) {
+  if constexpr (fused_ws_fits<NFFT>()) {
+    if (fused_ws_smem<NFFT>() > room) return false;
+    if (Shape<NFFT, kValsFused<NFFT>>::THREADS != kUpdThreads) return true;
+    cudaFuncAttributes fa, fb;
+    if (cudaFuncGetAttributes(&fa, fused_rows_ws_kernel<NFFT, true>) != cudaSuccess ||
+        cudaFuncGetAttributes(&fb, fused_rows_ws_kernel<NFFT, false>) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    return fa.numRegs >= 64 && fb.numRegs >= 64;
+  }
+  return false;
+}
+
+bool fused_ws_runs(int n, size_t room) {
   switch (n) {
 #define CASE(v) \
-  case v: return fused_ws_fits<v>() && fused_ws_smem<v>() <= room;
+  case v: return fused_ws_runs_n<v>(room);
     PROP_FFT_SIZES(CASE)
 #undef CASE
     default: return false;
@@ -1846,7 +1858,7 @@ void fft_make_maps(Plan& p) {
   const long units = (long)((p.Nf + kFftCols - 1) / kFftCols) * p.T * p.N;
   const bool want = p.row_kernel == 2 || (p.row_kernel == 0 && units >= 8L * p.num_sms);
   if (want && p.cs % kFftCols == 0 && p.nchunks == 1 && (size_t)p.T * p.N <= 0xffffffffu &&
-      fused_ws_size_ok(p.n, room)) {
+      fused_ws_runs(p.n, room)) {
     const cuuint64_t dims[3] = {(cuuint64_t)(2 * p.cs), (cuuint64_t)p.n, (cuuint64_t)p.T * p.N};
     const cuuint64_t strides[2] = {(cuuint64_t)(2 * p.cs * sizeof(float)),
                                    (cuuint64_t)(2 * (size_t)p.cs * p.n * sizeof(float))};
