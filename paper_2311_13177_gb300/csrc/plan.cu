@@ -591,6 +591,7 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
   p->spread_grouped = quad_stride(p->cs) && build_group_lists(*p, first_tap, wd, sitems, blob);
   if (!p->spread_grouped) {
   p->grid_used_h.clear();  // the cell lists fill the whole grid
+  p->grid_sparse = false;
   sitems.clear();
   blob.clear();
   const size_t ncell = (size_t)p->T * n * n;
