@@ -18,10 +18,10 @@ TOL = 2e-6
 
 
 @pytest.mark.parametrize("N,Nf,B,L,R", [
-    (64, 16, 130, 3, 64),     # cell lists, staged
-    (64, 16, 130, 2, 24),     # a short readout: the middle of the grid only
-    (64, 8, 1400, 1, 24),     # cell lists in global memory
-    (32, 64, 200, 2, 24),     # bin stride 64
+    (64, 16, 130, 6, 64),     # cell lists, staged
+    (64, 16, 130, 8, 24),     # a short readout: the middle of the grid only
+    (64, 8, 1400, 2, 24),     # cell lists in global memory
+    (32, 64, 200, 6, 24),     # bin stride 64
 ])
 def test_cell_lists_beside_the_stride_kernels(N, Nf, B, L, R):
     from paper_2311_13177_gb300 import Plan, ReconParams
