@@ -1235,6 +1235,22 @@ constexpr size_t col_smem() {
          Shape<NFFT, kValsCols<NFFT>>::SMEM + 2 * sizeof(uint64_t);
 }
 
+// Shared memory of a launch of `ctas` persistent CTAs over ntiles tiles.  The
+// launch may find SMs still held by the kernel before it; a CTA of a short
+// transform leaves room for many, so the free SMs would then take more than
+// their share of the CTAs and the pass would last as long as the fullest SM.
+// From two tiles a CTA on, a launch therefore asks for so much that no SM holds
+// more than its share (32 frames of 32^2 x 32 bins: forward 37.2 -> 30.6 us,
+// gradient 137 -> 123, an iteration 12.5 -> 10.7; 32 frames of 64^2 x 64 bins:
+// an iteration 79 -> 72 us).  Below that the CTAs are over before it matters and
+// early ones beside the spread's are worth more (64^2 x 64 bins: 7.1 us an
+// iteration, 7.4 with it).
+template <int NFFT, int KIND>
+size_t col_launch_smem(int ctas, int ntiles) {
+  const size_t share = (size_t)228 * 1024 / (col_ctas_per_sm<NFFT, KIND>() + 1);
+  return ntiles > 2 * ctas ? std::max(col_smem<NFFT, KIND>(), share) : col_smem<NFFT, KIND>();
+}
+
 // The column pass of one problem run by vg persistent CTAs, this being the
 // vb-th: tile vb, vb + vg, ... ; tin is the problem's input tensor map (in
 // the kernel's parameter space).
@@ -1356,10 +1372,20 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsCols<NFFT>>::THREADS, col_cta
   cols_body<NFFT, KIND>(&m.tm[r], m.a[r], (int)blockIdx.x - m.cta_begin[r], m.cta_begin[r + 1] - m.cta_begin[r]);
 }
 
+// The same for the plain passes, whose CTAs are few where a problem is small: up
+// to four an SM, a launch asks for so much shared memory that no SM takes more
+// than its share (forward passes one after the other: 64^2 x 16 bins 14.2 ->
+// 11.4 us, 8 frames of 32^2 x 32 bins 14.8 -> 12.4; adjoint of 96^2 x 64 bins
+// 38.1 -> 31.2).
+constexpr size_t kEvenShare = (size_t)228 * 1024 / 2;  // the most that is asked for: one CTA an SM
+
 template <int NFFT>
-cudaError_t launch(int kind, const FftArgs& a, dim3 grid, cudaStream_t s) {
+cudaError_t launch(int kind, const FftArgs& a, dim3 grid, int sms, cudaStream_t s) {
   auto go = [&](auto kern, int lines, int threads, size_t smem) {
-    return launch_dep(kern, dim3((grid.x + lines - 1) / lines, grid.y), dim3(threads), smem, s, a);
+    const dim3 g((grid.x + lines - 1) / lines, grid.y);
+    const size_t share = ((size_t)g.x * g.y + sms - 1) / sms;
+    if (share <= 4) smem = std::max(smem, (size_t)228 * 1024 / (share + 1));
+    return launch_dep(kern, g, dim3(threads), smem, s, a);
   };
 #define PROP_GO(K) go(fft_kernel<NFFT, K>, kColsOf<NFFT, K>, kThreadsOf<NFFT, K>, kSmemOf<NFFT, K>)
   switch (kind) {
@@ -1377,28 +1403,23 @@ cudaError_t configure_n() {
   auto smem = [](auto kern, size_t bytes) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
-  if ((e = smem(fft_kernel<NFFT, kFwdRows>, kSmemOf<NFFT, kFwdRows>))) return e;
-  if ((e = smem(fft_kernel<NFFT, kFwdCols>, kSmemOf<NFFT, kFwdCols>))) return e;
-  if ((e = smem(fft_kernel<NFFT, kAdjCols>, kSmemOf<NFFT, kAdjCols>))) return e;
-  if ((e = smem(fft_kernel<NFFT, kAdjRows>, kSmemOf<NFFT, kAdjRows>))) return e;
+  if ((e = smem(fft_kernel<NFFT, kFwdRows>, std::max(kEvenShare, kSmemOf<NFFT, kFwdRows>)))) return e;
+  if ((e = smem(fft_kernel<NFFT, kFwdCols>, std::max(kEvenShare, kSmemOf<NFFT, kFwdCols>)))) return e;
+  if ((e = smem(fft_kernel<NFFT, kAdjCols>, std::max(kEvenShare, kSmemOf<NFFT, kAdjCols>)))) return e;
+  if ((e = smem(fft_kernel<NFFT, kAdjRows>, std::max(kEvenShare, kSmemOf<NFFT, kAdjRows>)))) return e;
   int optin = 0, dev = 0;
   if ((e = cudaGetDevice(&dev))) return e;
   if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
-  if (col_smem<NFFT, kFwdCols>() <= (size_t)optin - 1024) {
-    if ((e = cudaFuncSetAttribute(fft_cols_tma_kernel<NFFT, kFwdCols>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)col_smem<NFFT, kFwdCols>())))
-      return e;
-    if ((e = cudaFuncSetAttribute(fft_cols_multi_kernel<NFFT, kFwdCols>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)col_smem<NFFT, kFwdCols>())))
-      return e;
+  const size_t room = (size_t)optin - 1024;
+  if (col_smem<NFFT, kFwdCols>() <= room) {
+    const size_t most = col_launch_smem<NFFT, kFwdCols>(0, 1);
+    if ((e = smem(fft_cols_tma_kernel<NFFT, kFwdCols>, most))) return e;
+    if ((e = smem(fft_cols_multi_kernel<NFFT, kFwdCols>, most))) return e;
   }
-  if (col_smem<NFFT, kAdjCols>() <= (size_t)optin - 1024) {
-    if ((e = cudaFuncSetAttribute(fft_cols_tma_kernel<NFFT, kAdjCols>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)col_smem<NFFT, kAdjCols>())))
-      return e;
-    if ((e = cudaFuncSetAttribute(fft_cols_multi_kernel<NFFT, kAdjCols>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)col_smem<NFFT, kAdjCols>())))
-      return e;
+  if (col_smem<NFFT, kAdjCols>() <= room) {
+    const size_t most = col_launch_smem<NFFT, kAdjCols>(0, 1);
+    if ((e = smem(fft_cols_tma_kernel<NFFT, kAdjCols>, most))) return e;
+    if ((e = smem(fft_cols_multi_kernel<NFFT, kAdjCols>, most))) return e;
   }
   const int fsm = (int)fused_smem<NFFT>(NFFT / 2);
   if ((e = cudaFuncSetAttribute(fused_rows_multi_kernel<NFFT>, cudaFuncAttributeMaxDynamicSharedMemorySize, fsm)))
@@ -1426,10 +1447,10 @@ cudaError_t configure_n() {
 
 #define PROP_FFT_SIZES(X) X(16) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512) X(768) X(1024)
 
-cudaError_t dispatch(int n, int kind, const FftArgs& a, dim3 grid, cudaStream_t s) {
+cudaError_t dispatch(int n, int kind, const FftArgs& a, dim3 grid, int sms, cudaStream_t s) {
   switch (n) {
 #define CASE(v) \
-  case v: return launch<v>(kind, a, grid, s);
+  case v: return launch<v>(kind, a, grid, sms, s);
     PROP_FFT_SIZES(CASE)
 #undef CASE
     default: return cudaErrorInvalidValue;
@@ -1439,11 +1460,13 @@ cudaError_t dispatch(int n, int kind, const FftArgs& a, dim3 grid, cudaStream_t 
 template <int NFFT>
 cudaError_t launch_cols_tma(int kind, const CUtensorMap& tm, const ColArgs& a, int sms, cudaStream_t s) {
   const int per_sm = kind == kFwdCols ? col_ctas_per_sm<NFFT, kFwdCols>() : col_ctas_per_sm<NFFT, kAdjCols>();
-  const dim3 grid((unsigned)std::max(1, std::min(a.ntiles, per_sm * sms)));
-  const dim3 block(Shape<NFFT, kValsCols<NFFT>>::THREADS);
+  const int ctas = std::max(1, std::min(a.ntiles, per_sm * sms));
+  const dim3 grid((unsigned)ctas), block(Shape<NFFT, kValsCols<NFFT>>::THREADS);
   if (kind == kFwdCols)
-    return launch_dep(fft_cols_tma_kernel<NFFT, kFwdCols>, grid, block, col_smem<NFFT, kFwdCols>(), s, tm, a);
-  return launch_dep(fft_cols_tma_kernel<NFFT, kAdjCols>, grid, block, col_smem<NFFT, kAdjCols>(), s, tm, a);
+    return launch_dep(fft_cols_tma_kernel<NFFT, kFwdCols>, grid, block, col_launch_smem<NFFT, kFwdCols>(ctas, a.ntiles), s,
+                      tm, a);
+  return launch_dep(fft_cols_tma_kernel<NFFT, kAdjCols>, grid, block, col_launch_smem<NFFT, kAdjCols>(ctas, a.ntiles), s,
+                    tm, a);
 }
 
 size_t cols_smem(int n, int kind) {
@@ -1479,9 +1502,11 @@ cudaError_t dispatch_cols_tma(int n, int kind, const CUtensorMap& tm, const ColA
 template <int NFFT>
 cudaError_t launch_cols_multi(int kind, const MultiCols& m, int ctas, cudaStream_t s) {
   const dim3 grid((unsigned)ctas), block(Shape<NFFT, kValsCols<NFFT>>::THREADS);
+  int ntiles = 0;
+  for (int r = 0; r < m.nreq; ++r) ntiles += m.a[r].ntiles;
   if (kind == kFwdCols)
-    return launch_dep(fft_cols_multi_kernel<NFFT, kFwdCols>, grid, block, col_smem<NFFT, kFwdCols>(), s, m);
-  return launch_dep(fft_cols_multi_kernel<NFFT, kAdjCols>, grid, block, col_smem<NFFT, kAdjCols>(), s, m);
+    return launch_dep(fft_cols_multi_kernel<NFFT, kFwdCols>, grid, block, col_launch_smem<NFFT, kFwdCols>(ctas, ntiles), s, m);
+  return launch_dep(fft_cols_multi_kernel<NFFT, kAdjCols>, grid, block, col_launch_smem<NFFT, kAdjCols>(ctas, ntiles), s, m);
 }
 
 cudaError_t dispatch_cols_multi(int n, int kind, const MultiCols& m, int ctas, cudaStream_t s) {
@@ -1816,7 +1841,7 @@ cudaError_t fft_forward_rows(const Plan& p, const float2* V, int f0, cudaStream_
   a.f0 = f0;
   a.Cv = std::min(p.chunk, p.Nf - f0);
   dim3 grid(a.C, p.T * p.N);  // x: lines
-  return dispatch(p.n, kFwdRows, a, grid, s);
+  return dispatch(p.n, kFwdRows, a, grid, p.num_sms, s);
 }
 
 void fft_make_maps(Plan& p) {
@@ -1876,7 +1901,7 @@ cudaError_t fft_forward_cols(const Plan& p, cudaStream_t s) {
   a.src = p.rows;
   a.dst = p.grid;
   dim3 grid(p.n * p.cs, p.T);  // x: lines
-  return dispatch(p.n, kFwdCols, a, grid, s);
+  return dispatch(p.n, kFwdCols, a, grid, p.num_sms, s);
 }
 
 cudaError_t fft_adjoint_cols(const Plan& p, cudaStream_t s) {
@@ -1885,7 +1910,7 @@ cudaError_t fft_adjoint_cols(const Plan& p, cudaStream_t s) {
   a.src = p.grid;
   a.dst = p.rows;
   dim3 grid(p.n * p.cs, p.T);  // x: lines
-  return dispatch(p.n, kAdjCols, a, grid, s);
+  return dispatch(p.n, kAdjCols, a, grid, p.num_sms, s);
 }
 
 cudaError_t fft_adjoint_rows(const Plan& p, float2* out, int f0, float scale, cudaStream_t s) {
@@ -1896,7 +1921,7 @@ cudaError_t fft_adjoint_rows(const Plan& p, float2* out, int f0, float scale, cu
   a.scale = scale;
   a.Cv = std::min(p.chunk, p.Nf - f0);
   dim3 grid(a.Cv, p.T * p.N);  // x: lines
-  return dispatch(p.n, kAdjRows, a, grid, s);
+  return dispatch(p.n, kAdjRows, a, grid, p.num_sms, s);
 }
 
 namespace {
