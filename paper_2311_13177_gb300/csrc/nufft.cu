@@ -1435,9 +1435,14 @@ cudaError_t spread(const Plan& p, int f0, int nbins, const float2* r, bool contr
 #undef SS
   } else {
     dim3 g((unsigned)std::max(1, std::min(p.n_sitems, 65535)));
+    // More than two items an SM: not beside the interpolation's tiles (its rows
+    // are re-read from L1; 61 bins at N = 128, an iteration: 362 us beside them,
+    // 331 after them; 20 bins at N = 64: 120 and 102).  Few items gain from the
+    // early launch (5 bins at N = 32: 44.4 us, 45.9 without).
+    const bool early = p.n_sitems <= 2 * p.num_sms;
 #define SG(L)                                                                                              \
-  return launch_dep(spread_global_kernel<L>, g, dim3(256), 0, s, p.grid, (const float2*)p.contrib, (const int4*)p.sitems, \
-                    (const int2*)p.sblob, p.n_sitems, p.cs, nbins)
+  return launch_when(early, spread_global_kernel<L>, g, dim3(256), 0, s, p.grid, (const float2*)p.contrib, \
+                     (const int4*)p.sitems, (const int2*)p.sblob, p.n_sitems, p.cs, nbins)
     switch (lanes_for((p.cs + 1) / 2)) {
       case 1: SG(1);
       case 2: SG(2);

@@ -139,11 +139,17 @@ struct DeviceGuard {
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+//
+// A kernel whose CTAs live on the L1 cache and come in several waves is launched
+// plainly (dependent = false): early CTAs beside a predecessor that holds most
+// of the SM's shared memory keep the L1 at what that left for as long as the
+// waves last.
 template <class... P, class... A>
-cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+cudaError_t launch_when(bool dependent, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                        A&&... args) {
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -152,6 +158,10 @@ cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);
+}
+template <class... P, class... A>
+cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  return launch_when(true, kernel, grid, block, smem, s, static_cast<A&&>(args)...);
 }
 
 // Deterministic "last block reduces" accumulator: every block writes one
