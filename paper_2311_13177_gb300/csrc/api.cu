@@ -275,7 +275,7 @@ prop_status loss_grad_device(Plan& p, const float2* y, const AdamArgs& a, const 
                              double* loss_out, cudaStream_t s) {
   prop_status st;
   if ((st = forward_impl(p, V, p.resid, y, &p.red_interp, p.scalars, s)) != PROP_OK) return st;
-  if (p.nchunks == 1) {  // the last adjoint pass and the TV gradient as one kernel
+  if (fused_rows_grad_pays(p)) {  // the last adjoint pass and the TV gradient as one kernel
     p.rows_of = nullptr;  // the adjoint passes overwrite the row workspace
     {
       StageScope sc(p, kStSpread, s);

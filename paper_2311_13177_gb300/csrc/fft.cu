@@ -701,8 +701,7 @@ __global__ void __launch_bounds__(kThreadsOf<NFFT, KIND>, kMinCtasOf<NFFT, KIND>
 // rewritten in place (each CTA reads its slice completely before writing it).
 // The arithmetic is that of the separate kernels, so the iterates are the
 // same bit for bit.  With kRowGrad it stops at the gradient of the loss, for
-// callers with an optimiser of their own: 304 -> 238 us against the adjoint
-// row pass and the TV kernel at 192^2 x 16 bins x 32 frames.
+// callers with an optimiser of their own (fused_rows_grad_pays: where).
 struct FusedArgs {
   float2* rows;        // [T][N][n][C] in: adjoint row intermediate, out: next forward row intermediate
   const float* deapod;
@@ -914,6 +913,9 @@ constexpr int fused_min_blocks() {
 // What the fused row kernel does after the inverse FFT of its row.
 enum RowMode { kRowUpdate = 0, kRowUpdateFwd = 1, kRowGrad = 2 };  // Adam; Adam and the next forward FFT; gradient only
 
+// Transform lengths with a kRowGrad kernel.
+constexpr bool row_grad_size(int n) { return n >= 64 && n <= 768; }
+
 template <int NFFT, int MODE>
 __device__ __forceinline__ void fused_rows_body(const FusedArgs& a, int bx, size_t row, unsigned vb, unsigned nblk) {
   constexpr int EV = kValsFused<NFFT>;
@@ -997,7 +999,10 @@ template <int NFFT>
 cudaError_t launch_fused(const FusedArgs& a, int mode, dim3 grid, cudaStream_t s) {
   const size_t smem = fused_smem<NFFT>(a.N);
   const dim3 block(Shape<NFFT, kValsFused<NFFT>>::THREADS);
-  if (mode == kRowGrad) return launch_dep(fused_rows_kernel<NFFT, kRowGrad>, grid, block, smem, s, a);
+  if (mode == kRowGrad) {
+    if constexpr (row_grad_size(NFFT)) return launch_dep(fused_rows_kernel<NFFT, kRowGrad>, grid, block, smem, s, a);
+    return cudaErrorInvalidValue;
+  }
   if (mode == kRowUpdateFwd) return launch_dep(fused_rows_kernel<NFFT, kRowUpdateFwd>, grid, block, smem, s, a);
   return launch_dep(fused_rows_kernel<NFFT, kRowUpdate>, grid, block, smem, s, a);
 }
@@ -1429,8 +1434,8 @@ cudaError_t configure_n() {
     return e;
   if ((e = cudaFuncSetAttribute(fused_rows_kernel<NFFT, kRowUpdate>, cudaFuncAttributeMaxDynamicSharedMemorySize, fsm)))
     return e;
-  if ((e = cudaFuncSetAttribute(fused_rows_kernel<NFFT, kRowGrad>, cudaFuncAttributeMaxDynamicSharedMemorySize, fsm)))
-    return e;
+  if constexpr (row_grad_size(NFFT))
+    if ((e = smem(fused_rows_kernel<NFFT, kRowGrad>, (size_t)fsm))) return e;
   if constexpr (fused_ws_fits<NFFT>()) {
     if (fused_ws_smem<NFFT>() <= (size_t)optin - 1024) {
       const int wsm = (int)fused_ws_smem<NFFT>();
@@ -2029,6 +2034,24 @@ cudaError_t fused_rows_update(const Plan& p, const float2* Vin, float2* m, float
   }
   if (a.units > red->capacity) return cudaErrorInvalidValue;
   return dispatch_fused(p.n, a, fwd_tail ? kRowUpdateFwd : kRowUpdate, dim3(a.nfb, p.T * p.N), s);
+}
+
+// Whether the gradient of the loss is taken by the fused row kernel or by the
+// adjoint row pass and the TV kernel (the same values; whole prop_loss_grad
+// calls, separate -> fused).  Fused saves a launch and the gradient's trip
+// through memory, 3 to 9 % of a call where it pays: one frame (64^2 x 8 bins
+// 71 -> 68 us, 256^2 x 32 bins 1.09x), and rows of whole 16-bin groups (256^2 x
+// 16 bins x 32 frames 1.08x).  The lanes of a missing bin run along, so with few
+// bins it loses (512^2 x 1 bin x 32 frames: 395 us separate, 1520 fused, of
+// these passes; 192^2 x 5 bins x 32 frames 1.09x a call) unless the rows are too
+// few to fill the SMs; at N <= 24 its CTAs are a warp or two (16^2 x 64 bins x 32
+// frames: 108 against 119 us a call), and at 512 one fits an SM.
+bool fused_rows_grad_pays(const Plan& p) {
+  if (p.nchunks != 1 || !row_grad_size(p.n) || p.N > 384) return false;
+  const long groups = (p.Nf + kFftCols - 1) / kFftCols, units = groups * p.T * p.N;
+  const bool whole = 8 * (kFftCols * groups - p.Nf) <= p.Nf;  // under an eighth of the lanes idle
+  if (p.T == 1) return whole || p.N <= 256;
+  return p.N >= 48 && (whole || (p.N <= 128 && 2 * units <= 5L * p.num_sms));
 }
 
 cudaError_t fused_rows_grad(const Plan& p, const float2* V, float2* grad, const AdamArgs& aa, const Reducer* red,

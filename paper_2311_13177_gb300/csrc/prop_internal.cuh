@@ -504,6 +504,7 @@ prop_status batch_step(BatchMember* mb, int count, cudaStream_t s);
 cudaError_t fused_rows_update(const Plan& p, const float2* Vin, float2* m, float2* v, float2* Vout,
                               const AdamArgs& aa, const Reducer* red, const double* data_loss, double* loss_out,
                               bool fwd_tail, cudaStream_t s);
+bool fused_rows_grad_pays(const Plan& p);
 // The same inverse row FFT fused with the TV gradient: grad = gscale (adjoint) + TV grads at V,
 // loss as in tv_adam.
 cudaError_t fused_rows_grad(const Plan& p, const float2* V, float2* grad, const AdamArgs& aa, const Reducer* red,
