@@ -1097,6 +1097,10 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsFused<NFFT>>::THREADS + kUpdT
   // groups add up to the launch's 64 a thread): 80 a thread hold three
   // voxels' loads with time neighbours where 64 spilled at two.  Together
   // with those loads issued at once: dynamic 445 -> 370 us.
+  // A walk that three voxels at a time do not shorten takes two, and a walk of
+  // one voxel (N <= 32) one: the rest of a step would load its last voxel again.
+  constexpr int LEN = (NFFT / 2 + kUpdThreads / kFftCols - 1) / (kUpdThreads / kFftCols);
+  constexpr int UP = LEN < 2 ? LEN : 2, UT = (LEN + 2) / 3 < (LEN + 1) / 2 ? 3 : UP;
   constexpr bool SPLIT = FT == kUpdThreads;
   constexpr int FREG = EV == 12 ? 48 : 56;  // fused_ws_runs checks the launch's registers
   if (threadIdx.x < FT) {
@@ -1160,7 +1164,7 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsFused<NFFT>>::THREADS + kUpdT
       if (!mbar_wait_bounded(&ready[i & 1], (uint32_t)((i >> 1) & 1))) s_abort_u = 1;
       USync::sync();
       if (s_abort_u) break;
-      local = update_row_any<true, 3, 2>(a, gbuf + (size_t)(i & 1) * gsz, i2, t, fbase, ut, kUpdThreads, local);
+      local = update_row_any<true, UT, UP>(a, gbuf + (size_t)(i & 1) * gsz, i2, t, fbase, ut, kUpdThreads, local);
       mbar_arrive(&done[i & 1]);
     }
   }
