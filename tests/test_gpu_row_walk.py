@@ -1,7 +1,9 @@
 """The warp-specialised row kernel's walks of one, two, three, four and six voxels
 (N = 16 to 192; the voxels in flight follow the length) against the per-row
 kernel, whose arithmetic is the same: equal bit for bit, with and without time
-neighbours, a dead lane and a ragged last run."""
+neighbours, a dead lane and a ragged last run.  The loss sums a thread's terms in
+FP32 over its walks, at most 60 of them here (one unit a CTA in the per-row
+kernel, several in the other): 60 roundings of 6e-8 of positive terms, 5e-6."""
 import numpy as np
 import pytest
 import torch
@@ -23,4 +25,4 @@ def test_both_row_kernels_give_the_same_volume(N, Nf, T):
         got.append(plan.reconstruct(y, q))
         plan.destroy()
     assert torch.equal(got[0][0], got[1][0])
-    assert np.max(np.abs(got[0][1] - got[1][1]) / np.abs(got[0][1])) < 1e-12
+    assert np.max(np.abs(got[0][1] - got[1][1]) / np.abs(got[0][1])) < 5e-6
