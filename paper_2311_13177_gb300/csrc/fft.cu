@@ -914,7 +914,7 @@ constexpr int fused_min_blocks() {
 enum RowMode { kRowUpdate = 0, kRowUpdateFwd = 1, kRowGrad = 2 };  // Adam; Adam and the next forward FFT; gradient only
 
 // Transform lengths with a kRowGrad kernel.
-constexpr bool row_grad_size(int n) { return n >= 64 && n <= 768; }
+constexpr bool row_grad_size(int n) { return n >= 48 && n <= 768; }
 
 template <int NFFT, int MODE>
 __device__ __forceinline__ void fused_rows_body(const FusedArgs& a, int bx, size_t row, unsigned vb, unsigned nblk) {
@@ -2043,19 +2043,17 @@ cudaError_t fused_rows_update(const Plan& p, const float2* Vin, float2* m, float
 // Whether the gradient of the loss is taken by the fused row kernel or by the
 // adjoint row pass and the TV kernel (the same values; whole prop_loss_grad
 // calls, separate -> fused).  Fused saves a launch and the gradient's trip
-// through memory, 3 to 9 % of a call where it pays: one frame (64^2 x 8 bins
-// 71 -> 68 us, 256^2 x 32 bins 1.09x), and rows of whole 16-bin groups (256^2 x
-// 16 bins x 32 frames 1.08x).  The lanes of a missing bin run along, so with few
-// bins it loses (512^2 x 1 bin x 32 frames: 395 us separate, 1520 fused, of
-// these passes; 192^2 x 5 bins x 32 frames 1.09x a call) unless the rows are too
-// few to fill the SMs; at N <= 24 its CTAs are a warp or two (16^2 x 64 bins x 32
-// frames: 108 against 119 us a call), and at 512 one fits an SM.
+// through memory: 3 to 10 % of a call (one frame of 64^2 x 32 bins 0.91x, 256^2 x
+// 16 bins x 8 frames 0.90x).  But the lanes of a missing bin run along, so with
+// few bins and several frames it loses (512^2 x 1 bin x 32 frames: 395 us
+// separate, 1520 fused, of these passes; 192^2 x 5 bins x 32 frames 1.09x a
+// call); below N = 32 its CTAs are a warp or two (16^2 x 64 bins x 32 frames 108
+// against 119 us a call), and at 512 one fits an SM.
 bool fused_rows_grad_pays(const Plan& p) {
-  if (p.nchunks != 1 || !row_grad_size(p.n) || p.N > 384) return false;
-  const long groups = (p.Nf + kFftCols - 1) / kFftCols, units = groups * p.T * p.N;
-  const bool whole = 8 * (kFftCols * groups - p.Nf) <= p.Nf;  // under an eighth of the lanes idle
-  if (p.T == 1) return whole || p.N <= 256;
-  return p.N >= 48 && (whole || (p.N <= 128 && 2 * units <= 5L * p.num_sms));
+  if (p.nchunks != 1 || !row_grad_size(p.n)) return false;
+  if (p.T == 1) return p.N <= 256 || p.Nf > 2;
+  if (p.N <= 32) return p.N == 32 && p.Nf >= 5 && p.Nf <= kFftCols;
+  return p.Nf >= (p.N <= 128 ? 5 : 12);
 }
 
 cudaError_t fused_rows_grad(const Plan& p, const float2* V, float2* grad, const AdamArgs& aa, const Reducer* red,

@@ -17,7 +17,8 @@ TOL = 5e-6
 
 
 @pytest.mark.parametrize("N,Nf,B,L,R,T", [
-    (32, 8, 3, 4, 32, 1),      # fused, 2N = 64
+    (24, 5, 3, 4, 24, 1),      # fused, 2N = 48
+    (32, 8, 3, 4, 32, 2),      # fused, 2N = 64
     (384, 16, 2, 1, 16, 1),    # fused, 2N = 768
     (48, 15, 4, 3, 49, 3),     # fused, one dead lane
     (24, 33, 4, 3, 25, 3),     # separate, three groups with 15 dead lanes
