@@ -235,11 +235,12 @@ OptArgs make_args(const Plan& p, const float2* Vin, const float2* g, float2* out
   a.N = p.N;
   a.Nf = p.Nf;
   a.T = p.T;
-  a.fw = std::min(p.Nf, kOptThreads);
-  a.nfg = (p.Nf + a.fw - 1) / a.fw;
-  a.runs = kOptThreads / a.fw;
-  a.len = std::min(kOptLen, (p.N + a.runs - 1) / a.runs);
-  a.nxb = (p.N + a.runs * a.len - 1) / (a.runs * a.len);
+  const WalkShape w = walk_shape(p.Nf, p.N, kOptThreads, kOptLen);
+  a.fw = w.fw;
+  a.nfg = w.nfg;
+  a.runs = w.runs;
+  a.len = w.len;
+  a.nxb = w.nxb;
   a.p = aa;
   return a;
 }

@@ -145,7 +145,7 @@ struct ProjUpdArgs {
   const float2* gimg;  // [N][N] image-space gradient of the data term (U^H of the masked k-space gradient)
   const int4* sh;      // [Nf] shifts of the iteration's blade
   int N, Nf, T, tb;
-  int len;             // voxels of an image row that a thread takes
+  WalkShape w;         // single frame: the walks
   AdamArgs ad;         // gscale 1 (gimg already holds the factor 2 and the weights)
   float tv_f, l1;
   double* partials;
@@ -154,59 +154,50 @@ struct ProjUpdArgs {
   double* loss_out;
 };
 
-// Threads of the update along the bins and, by what is left of a block, along x1.
-__host__ __device__ inline int update_bins(int Nf) { return Nf < kProjThreads ? Nf : kProjThreads; }
-
 // Fused update: data gradient by the transposed projection, TV along x1, x2
 // and t (the same arithmetic as the non-uniform model's update), TV along
 // the spectral axis, L1, Adam, and the FP64 loss of the iterate it reads.
-// Grid: (x1 blocks x bin groups, T N rows).  A thread takes one bin and walks
-// `len` voxels along x1, so the x1 TV term and the two pixels that it shares
-// with the voxel before are handed on (two pixel loads instead of four), the
-// bin's shift and its weights are loaded once, and a voxel is one 32-bit byte
-// offset; the loads of U voxels are issued together.  Every neighbour load is
-// unconditional (a missing neighbour reads the voxel itself and is not used).
-// TT: the volume has time neighbours.  Off: uint32_t while three frames are
-// within 4 GB (64-bit offsets cost a CTA per SM: 98 registers instead of 80,
-// 1196 instead of 1053 us for 16 iterations at 256^2 x 32), else size_t.
-template <bool TT, typename Off>
-__global__ void __launch_bounds__(kProjThreads) proj_update_kernel(ProjUpdArgs a) {
+//
+// One frame: a thread takes one bin and walks along x1 (grid: x1 blocks x bin
+// groups, N rows), so the x1 TV term and the two pixels that it shares with the
+// voxel before are handed on (two pixel loads instead of four), the bin's shift
+// and its weights are loaded once, and a voxel is one 32-bit byte offset; the
+// loads of U voxels are issued together.  Every neighbour load is unconditional
+// (a missing neighbour reads the voxel itself and is not used).  Off: uint32_t
+// while the volume is within 4 GB (64-bit offsets cost a CTA per SM: 98 registers
+// instead of 80, 1196 instead of 1053 us for 16 iterations at 256^2 x 32), else
+// size_t.
+template <typename Off>
+__global__ void __launch_bounds__(kProjThreads) proj_walk_kernel(ProjUpdArgs a) {
   grid_dep_wait();
   grid_dep_release();
   constexpr int U = 2;
-  const int row = blockIdx.y;  // t N + i2
-  const int i2 = row % a.N, t = row / a.N;
-  const int fw = update_bins(a.Nf), nfg = (a.Nf + fw - 1) / fw, runs = kProjThreads / fw;
-  const int fg = blockIdx.x % nfg, run = threadIdx.x / fw;
-  const int f = fg * fw + threadIdx.x - run * fw;
-  const int lo = ((int)(blockIdx.x / nfg) * runs + run) * a.len;
-  const int hi = run < runs && f < a.Nf ? min(a.N, lo + a.len) : 0;
+  const int i2 = blockIdx.y;
+  const int fg = blockIdx.x % a.w.nfg, run = threadIdx.x / a.w.fw;
+  const int f = fg * a.w.fw + threadIdx.x - run * a.w.fw;
+  const int lo = ((int)(blockIdx.x / a.w.nfg) * a.w.runs + run) * a.w.len;
+  const int hi = run < a.w.runs && f < a.Nf ? min(a.N, lo + a.w.len) : 0;
   float local = 0.f;
   if (lo < hi) {
     const float eps2 = a.ad.tv_eps * a.ad.tv_eps;
-    const size_t st = (size_t)a.N * a.N * a.Nf;
     const bool xy = a.ad.tv_xy != 0.f;
     const bool h2p = xy && i2 + 1 < a.N, h2m = xy && i2 > 0;
-    const bool htp = TT && t + 1 < a.T, htm = TT && t > 0;
     const bool hfp = a.tv_f != 0.f && f + 1 < a.Nf, hfm = a.tv_f != 0.f && f > 0;
-    // offsets count from the frame before this one (from this one when t = 0)
-    const size_t first = (size_t)(t > 0 ? t - 1 : 0) * st;
-    const char* V = reinterpret_cast<const char*>(a.Vin + first);
-    char* M1 = reinterpret_cast<char*>(a.m + first);
-    char* M2 = reinterpret_cast<char*>(a.v + first);
-    char* Vo = reinterpret_cast<char*>(a.Vout + first);
+    const char* V = reinterpret_cast<const char*>(a.Vin);
+    char* M1 = reinterpret_cast<char*>(a.m);
+    char* M2 = reinterpret_cast<char*>(a.v);
+    char* Vo = reinterpret_cast<char*>(a.Vout);
     auto at = [](const char* b, Off o) { return __ldg(reinterpret_cast<const float2*>(b + o)); };
     auto ref = [](char* b, Off o) -> float2& { return *reinterpret_cast<float2*>(b + o); };
-    const Off sx = (Off)a.Nf * 8, d2 = (Off)a.N * sx, dt = (Off)st * 8;
-    const Off d2p = h2p ? d2 : 0, d2m = h2m ? d2 : 0, dtp = htp ? dt : 0, dtm = htm ? dt : 0;
+    const Off sx = (Off)a.Nf * 8, d2 = (Off)a.N * sx;
+    const Off d2p = h2p ? d2 : 0, d2m = h2m ? d2 : 0;
     const Off dfp = hfp ? 8 : 0, dfm = hfm ? 8 : 0;
-    Off off = (t > 0 ? dt : 0) + (Off)i2 * d2 + (Off)lo * sx + (Off)f * 8;
+    Off off = (Off)i2 * d2 + (Off)lo * sx + (Off)f * 8;
     // pixel rows i2 - o2 and i2 - o2 - 1 of the transposed projection
-    const bool data = t == a.tb;
     const int4 o = __ldg(&a.sh[f]);
     const float w1 = __int_as_float(o.z), w2 = __int_as_float(o.w);
     const int p0 = i2 - o.y, p1 = p0 - 1;
-    const bool r0 = data && p0 >= 0 && p0 < a.N, r1 = data && p1 >= 0 && p1 < a.N;
+    const bool r0 = p0 >= 0 && p0 < a.N, r1 = p1 >= 0 && p1 < a.N;
     const float2* g0 = a.gimg + (size_t)(r0 ? p0 : 0) * a.N;
     const float2* g1 = a.gimg + (size_t)(r1 ? p1 : 0) * a.N;
     const float w00 = (1.f - w2) * (1.f - w1), w01 = (1.f - w2) * w1, w10 = w2 * (1.f - w1), w11 = w2 * w1;
@@ -221,7 +212,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_update_kernel(ProjUpdArgs a
     float2 t1m = make_float2(0.f, 0.f);
     if (xy && lo > 0) t1m = tv_term(csub_rn(x, at(V, off - sx)), eps2, &mag);
     for (int i0 = lo; i0 < hi; i0 += U, off += U * sx) {
-      float2 xp[U], x2p[U], x2m[U], xtp[U], xtm[U], xfp[U], xfm[U], mm[U], vv[U], n0[U], n1[U];
+      float2 xp[U], x2p[U], x2m[U], xfp[U], xfm[U], mm[U], vv[U], n0[U], n1[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int i1 = min(i0 + u, hi - 1);
@@ -229,10 +220,6 @@ __global__ void __launch_bounds__(kProjThreads) proj_update_kernel(ProjUpdArgs a
         xp[u] = at(V, i1 + 1 < a.N ? c + sx : c);
         x2p[u] = at(V, c + d2p);
         x2m[u] = at(V, c - d2m);
-        if constexpr (TT) {
-          xtp[u] = at(V, c + dtp);
-          xtm[u] = at(V, c - dtm);
-        }
         xfp[u] = at(V, c + dfp);
         xfm[u] = at(V, c - dfm);
         mm[u] = ref(M1, c);
@@ -251,8 +238,8 @@ __global__ void __launch_bounds__(kProjThreads) proj_update_kernel(ProjUpdArgs a
         q0 = n0[u];
         q1 = n1[u];
         // voxel_tv_nb's terms in its order
-        float2 gxy = make_float2(0.f, 0.f), gt = make_float2(0.f, 0.f), t1p = make_float2(0.f, 0.f);
-        float sxy = 0.f, stt = 0.f;
+        float2 gxy = make_float2(0.f, 0.f), t1p = make_float2(0.f, 0.f);
+        float sxy = 0.f;
         if (xy) {
           if (i1 + 1 < a.N) {
             t1p = tv_term(csub_rn(xp[u], x), eps2, &mag);
@@ -266,14 +253,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_update_kernel(ProjUpdArgs a
           }
           if (h2m) gxy = cadd_rn(gxy, tv_term(csub_rn(x, x2m[u]), eps2, &mag));
         }
-        if constexpr (TT) {
-          if (htp) {
-            gt = csub_rn(gt, tv_term(csub_rn(xtp[u], x), eps2, &mag));
-            stt = __fadd_rn(stt, mag);
-          }
-          if (htm) gt = cadd_rn(gt, tv_term(csub_rn(x, xtm[u]), eps2, &mag));
-        }
-        float tv = fmaf(a.ad.tv_xy, sxy, __fmul_rn(TT ? a.ad.tv_t : 0.f, stt));
+        float tv = fmaf(a.ad.tv_xy, sxy, 0.f);
         float2 gf = make_float2(0.f, 0.f);
         if (hfp) {
           gf = csub_rn(gf, tv_term(csub_rn(xfp[u], x), eps2, &mag));
@@ -285,7 +265,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_update_kernel(ProjUpdArgs a
           gl = tv_term(x, eps2, &mag);  // x / sqrt(|x|^2 + eps^2) and the smoothed modulus
           tv = fmaf(a.l1, mag, tv);
         }
-        float2 g = total_grad(make_float2(gx, gy), gxy, gt, a.ad);
+        float2 g = total_grad(make_float2(gx, gy), gxy, make_float2(0.f, 0.f), a.ad);
         g.x = fmaf(a.l1, gl.x, fmaf(a.tv_f, gf.x, g.x));
         g.y = fmaf(a.l1, gl.y, fmaf(a.tv_f, gf.y, g.y));
         local = __fadd_rn(local, tv);
@@ -297,6 +277,83 @@ __global__ void __launch_bounds__(kProjThreads) proj_update_kernel(ProjUpdArgs a
         x = xp[u];
       }
     }
+  }
+  finish_loss(local, a.partials, a.counter, a.data_loss, a.loss_out);
+}
+
+// Several frames: grid (blocks per image row, T N rows), 32-bit index math within
+// a row, a block's threads on consecutive values.  The walk holds two voxels with
+// time neighbours in 91 registers, two CTAs an SM, and its scattered runs miss
+// what the frames no longer have in L2: 384^2 x 40 bins x 4 frames 413 us an
+// iteration here, 608 walking; 256^2 x 12 bins x 4 frames 96 and 133.  With one
+// frame the walk is the faster (256^2 x 32 bins 77 -> 69 us).  TT: the volume has
+// time neighbours; every neighbour load is unconditional as above.
+template <bool TT>
+__global__ void __launch_bounds__(kProjThreads) proj_update_kernel(ProjUpdArgs a) {
+  grid_dep_wait();
+  grid_dep_release();
+  const int row = blockIdx.y;  // t N + i2
+  const int i2 = row % a.N, t = row / a.N;
+  const int rl = a.N * a.Nf;
+  const size_t base = (size_t)row * rl;
+  const size_t sx = (size_t)a.Nf, sy = (size_t)rl, st = (size_t)a.N * rl;
+  const float eps2 = a.ad.tv_eps * a.ad.tv_eps;
+  const bool xy = a.ad.tv_xy != 0.f;
+  const bool h2p = xy && i2 + 1 < a.N, h2m = xy && i2 > 0;
+  const bool htp = TT && t + 1 < a.T, htm = TT && t > 0;
+  const bool data = t == a.tb;
+  const float2* __restrict__ Vin = a.Vin;
+  float local = 0.f;
+#pragma unroll 2
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < rl; e += gridDim.x * blockDim.x) {
+    const int i1 = e / a.Nf;
+    const int f = e - i1 * a.Nf;
+    const size_t idx = base + e;
+    const float2 x = Vin[idx];
+    TvNbrs nb;
+    nb.h1p = xy && i1 + 1 < a.N;
+    nb.h1m = xy && i1 > 0;
+    nb.h2p = h2p;
+    nb.h2m = h2m;
+    nb.htp = htp;
+    nb.htm = htm;
+    nb.x1p = Vin[nb.h1p ? idx + sx : idx];
+    nb.x1m = Vin[nb.h1m ? idx - sx : idx];
+    nb.x2p = Vin[h2p ? idx + sy : idx];
+    nb.x2m = Vin[h2m ? idx - sy : idx];
+    if constexpr (TT) {
+      nb.tp = Vin[htp ? idx + st : idx];
+      nb.tm = Vin[htm ? idx - st : idx];
+    } else {
+      nb.tp = nb.tm = x;
+    }
+    const bool hfp = a.tv_f != 0.f && f + 1 < a.Nf, hfm = a.tv_f != 0.f && f > 0;
+    const float2 xfp = Vin[hfp ? idx + 1 : idx];
+    const float2 xfm = Vin[hfm ? idx - 1 : idx];
+    float2 mm = a.m[idx], vv = a.v[idx];
+    const float2 gd = data ? proj_gather(a.gimg, __ldg(&a.sh[f]), a.N, i1, i2) : make_float2(0.f, 0.f);
+    float2 gxy, gt;
+    float tv = voxel_tv_nb(x, nb, a.ad.tv_xy, TT ? a.ad.tv_t : 0.f, eps2, &gxy, &gt);
+    float2 gf = make_float2(0.f, 0.f);
+    float mag;
+    if (hfp) {
+      gf = csub_rn(gf, tv_term(csub_rn(xfp, x), eps2, &mag));
+      tv = fmaf(a.tv_f, mag, tv);
+    }
+    if (hfm) gf = cadd_rn(gf, tv_term(csub_rn(x, xfm), eps2, &mag));
+    float2 gl = make_float2(0.f, 0.f);
+    if (a.l1 != 0.f) {
+      gl = tv_term(x, eps2, &mag);  // x / sqrt(|x|^2 + eps^2) and the smoothed modulus
+      tv = fmaf(a.l1, mag, tv);
+    }
+    float2 g = total_grad(gd, gxy, gt, a.ad);
+    g.x = fmaf(a.l1, gl.x, fmaf(a.tv_f, gf.x, g.x));
+    g.y = fmaf(a.l1, gl.y, fmaf(a.tv_f, gf.y, g.y));
+    local = __fadd_rn(local, tv);
+    const float2 nx = adam_voxel(x, g, mm, vv, a.ad);
+    a.m[idx] = mm;
+    a.v[idx] = vv;
+    a.Vout[idx] = nx;
   }
   finish_loss(local, a.partials, a.counter, a.data_loss, a.loss_out);
 }
@@ -340,15 +397,18 @@ __global__ void __launch_bounds__(kProjThreads) proj_baseline_kernel(const float
   }
 }
 
-// Voxels of a row that a thread of the update takes (at most 8), and the
-// update's blocks per image row.
-int update_len(const Plan& p) {
-  const int runs = kProjThreads / update_bins(p.Nf);
-  return std::min(8, (p.N + runs - 1) / runs);
-}
+WalkShape update_walk(const Plan& p) { return walk_shape(p.Nf, p.N, kProjThreads, 8); }
+// Blocks per image row of the update.  Several frames: about 8 voxels a thread, at
+// most 4, or as many as give an SM four of them (48^2 x 64 bins x 2 frames: 96
+// blocks of 12 voxels a thread took 36 us an iteration).
 int update_row_blocks(const Plan& p) {
-  const int fw = update_bins(p.Nf), runs = kProjThreads / fw, span = runs * update_len(p);
-  return (p.Nf + fw - 1) / fw * ((p.N + span - 1) / span);
+  if (p.T > 1) {
+    const int row = p.N * p.Nf, rows = p.T * p.N, want = std::max(1, std::min(4, row / (8 * kProjThreads)));
+    const int fill = (4 * p.num_sms + rows - 1) / rows;
+    return std::max(want, std::min(fill, (row + kProjThreads - 1) / kProjThreads));
+  }
+  const WalkShape w = update_walk(p);
+  return w.nfg * w.nxb;
 }
 
 // Allocates *ptr unless a previous, interrupted set-up already did.
@@ -602,7 +662,7 @@ prop_status prop_proj_reconstruct(prop_plan plan, const void* ycart_dev, const v
     u.N = p.N;
     u.Nf = p.Nf;
     u.T = p.T;
-    u.len = update_len(p);
+    u.w = update_walk(p);
     u.tb = p.blade_frame[b];
     const double bc1 = 1.0 - std::pow((double)q.beta1, k);
     const double bc2 = 1.0 - std::pow((double)q.beta2, k);
@@ -621,12 +681,10 @@ prop_status prop_proj_reconstruct(prop_plan plan, const void* ycart_dev, const v
     u.counter = p.red_proj_u.counter;
     u.data_loss = p.scalars + 3;
     u.loss_out = p.loss_dev + (k - 1);
-    if (p.T > 1 && q.tv_t != 0.f)
-      PROP_CUDA(launch_dep(small ? proj_update_kernel<true, uint32_t> : proj_update_kernel<true, size_t>, ugrid,
-                           dim3(kProjThreads), 0, s, u));
-    else
-      PROP_CUDA(launch_dep(small ? proj_update_kernel<false, uint32_t> : proj_update_kernel<false, size_t>, ugrid,
-                           dim3(kProjThreads), 0, s, u));
+    const auto kernel = p.T > 1 ? (q.tv_t != 0.f ? proj_update_kernel<true> : proj_update_kernel<false>)
+                        : small ? proj_walk_kernel<uint32_t>
+                                : proj_walk_kernel<size_t>;
+    PROP_CUDA(launch_dep(kernel, ugrid, dim3(kProjThreads), 0, s, u));
     std::swap(cur, nxt);
   }
   if (cur != (float2*)V_dev) PROP_CUDA(cudaMemcpyAsync(V_dev, cur, vbytes, cudaMemcpyDeviceToDevice, s));
