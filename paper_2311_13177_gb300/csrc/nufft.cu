@@ -1388,9 +1388,15 @@ cudaError_t spread(const Plan& p, int f0, int nbins, const float2* r, bool contr
   if (!contrib_ready) {
     dim3 g(grid_for(p.M, 8L * (32 / lp), 16384));
     cudaError_t e;
+    // Large, it lives on the phase table in L1 where that fits, so not beside its
+    // predecessor then (50 blades x 64 bins, a table of 120 KB: 308 us an adjoint
+    // beside it, 284 after it; at 93 and 134 MB of phased residual no difference,
+    // and with a table of 196 KB in the differentiable program 847 and 851 us).
+    const bool early = (size_t)p.M * p.cs * sizeof(float2) <= (size_t)150 << 20 ||
+                       (size_t)p.R * p.Nf * sizeof(float2) > (size_t)160 << 10;
 #define PE(L)                                                                                              \
-  e = launch_dep(phase_expand_kernel<L>, g, dim3(256), 0, s, r, (const float2*)p.phase, p.contrib, p.M, p.R, p.Nf, p.cs, \
-                 nbins, f0)
+  e = launch_when(early, phase_expand_kernel<L>, g, dim3(256), 0, s, r, (const float2*)p.phase, p.contrib, p.M, p.R,  \
+                  p.Nf, p.cs, nbins, f0)
     switch (lp) {
       case 1: PE(1); break;
       case 2: PE(2); break;
@@ -1435,11 +1441,12 @@ cudaError_t spread(const Plan& p, int f0, int nbins, const float2* r, bool contr
 #undef SS
   } else {
     dim3 g((unsigned)std::max(1, std::min(p.n_sitems, 65535)));
-    // More than two items an SM: not beside the interpolation's tiles (its rows
-    // are re-read from L1; 61 bins at N = 128, an iteration: 362 us beside them,
-    // 331 after them; 20 bins at N = 64: 120 and 102).  Few items gain from the
-    // early launch (5 bins at N = 32: 44.4 us, 45.9 without).
-    const bool early = p.n_sitems <= 2 * p.num_sms;
+    // Not beside the interpolation's tiles, unless what it re-reads is small: the
+    // residual's rows come from L1 (61 bins at N = 128, an iteration: 362 us beside
+    // them, 331 after them; 20 bins at N = 64, 1.3 MB: 120 and 102; 45 bins at N =
+    // 96, 2.1 MB: 159 and 145).  Small ones gain from the early launch (5 bins at N =
+    // 32, 98 KB: 44.4 us, 45.9 without).
+    const bool early = (size_t)p.M * p.cs * sizeof(float2) <= (size_t)256 << 10;
 #define SG(L)                                                                                              \
   return launch_when(early, spread_global_kernel<L>, g, dim3(256), 0, s, p.grid, (const float2*)p.contrib, \
                      (const int4*)p.sitems, (const int2*)p.sblob, p.n_sitems, p.cs, nbins)
