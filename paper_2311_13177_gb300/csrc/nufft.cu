@@ -50,6 +50,8 @@ struct InterpArgs {
   unsigned int* counter;
   double* sumsq_out;
   int* err;  // set to 1 when a bounded wait expires
+  const float4* quads;  // the plan's quads in item order, or null: tiles (kb_idx, kb_w, order)
+  const int* cta_off;   // CTA c takes items [cta_off[c], cta_off[c + 1])
   int n_items, R, n, C, Cv, f0, Nf;
   int TR, TC, nct, tpf, nbuf;  // tile rows, cells per row, tiles per row of tiles and per frame
   float scale;
@@ -296,23 +298,178 @@ __global__ void __launch_bounds__(kInterpThreads, 1) interp_kernel(InterpArgs a)
   if (a.partials) reduce_to((double)sumsq, a.partials, a.counter, a.sumsq_out);
 }
 
-struct QuadArgs {
-  const float2* grid;
-  const float4* quads;
-  const int4* items;
-  const float2* phase;
-  float2* y;
-  const float2* y_meas;
-  float2* contrib;  // non-null: also write conj(P) * final value per bin
-  double* partials;
-  unsigned int* counter;
-  double* sumsq_out;
-  int* err;  // set to 1 when a bounded wait expires
-  const int* cta_off;  // CTA c takes items [cta_off[c], cta_off[c + 1])
-  int n, Cv, f0, Nf;
-  float scale;
-  int accumulate;
-};
+// Interpolation for the bin strides CS in {8, 16, 32, 64}, a sample at a time
+// over staged tiles; NCW compute warps and a producer warp.  The producer's
+// lane 0 streams item k's tile into buffer k % nbuf as soon as every compute
+// warp has released the item that last used that buffer ("empty" barrier, one
+// arrival per compute warp), so no compute warp ever waits for another.
+// Compute warps take CS / 2 lanes per sample, each lane two adjacent bins
+// (16-byte shared loads), and 64 / CS samples per warp and round.  The metadata
+// of an item (sample index, packed first tap, the 2W weights) is fetched before
+// its tile is awaited, one sample per lane, and handed out by shuffles.  Every
+// tap of every sample is a shared-memory read (the bound where the samples are
+// dense: quads_body), but the samples of a tile spread over all the warps, so
+// it has the shorter chain where there are few.
+template <int CS, int W, int NCW>
+__device__ __forceinline__ void tiles_body(const InterpArgs& a, int it_beg, int it_end, unsigned vb, unsigned vg) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  constexpr int LPS = CS / 2;                      // lanes per sample
+  constexpr int SPW = tile_samples_per_warp(CS);   // samples per warp and round
+  constexpr int HR = interp_tile_rows(CS, W) + W - 1;  // staged rows
+  constexpr int HC = interp_tile_cols(CS) + W - 1;     // staged cells per row
+  constexpr int WQ = W / 2;
+  constexpr int MPL = (kInterpItem + NCW * SPW - 1) / (NCW * SPW) * SPW;  // samples per warp per item
+  static_assert(MPL <= 32 && MPL / SPW <= LPS, "one prefetched sample per lane; a lane of a sample's per round");
+  constexpr size_t tile_elems = (size_t)HR * HC * CS;
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  const int sub = lane % LPS;
+  const int slot = lane / LPS;
+  float2* bufs = reinterpret_cast<float2*>(smem_raw);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + a.nbuf * tile_elems * sizeof(float2));
+  uint64_t* empty = full + a.nbuf;
+  __shared__ volatile int s_abort;
+  if (threadIdx.x == 0) {
+    for (int b = 0; b < a.nbuf; ++b) {
+      mbar_init(&full[b], 1);
+      mbar_init(&empty[b], NCW);
+    }
+    fence_mbar_init();
+    s_abort = 0;
+  }
+  __syncthreads();
+  grid_dep_wait();
+  grid_dep_release();
+
+  double sumsq = 0.0;
+  if (warp == NCW) {
+    if (lane == 0) {
+      int k = 0;
+      for (int item = it_beg; item < it_end; ++item, ++k) {
+        const int b = k % a.nbuf;
+        if (k >= a.nbuf && !mbar_wait_bounded(&empty[b], (uint32_t)(((k / a.nbuf) - 1) & 1))) {
+          s_abort = 1;
+          break;
+        }
+        if (s_abort) break;
+        issue_tile<W>(a, item, bufs + b * tile_elems, &full[b]);
+      }
+      // at most one copy per buffer can be in flight: the last one issued
+      for (int kk = k > a.nbuf ? k - a.nbuf : 0; kk < k; ++kk)
+        mbar_wait_bounded(&full[kk % a.nbuf], (uint32_t)((kk / a.nbuf) & 1));
+    }
+  } else {
+    const int f_lo = 2 * sub;
+    const bool b0 = f_lo < a.Cv, b1 = f_lo + 1 < a.Cv;
+    int k = 0;
+    for (int item = it_beg; item < it_end; ++item, ++k) {
+      const int b = k % a.nbuf;
+      const ItemGeom g = item_geom(a, item);
+      // lane L prefetches the warp's sample of round L / SPW, slot L % SPW
+      const int sL = (lane / SPW) * NCW * SPW + warp * SPW + (lane % SPW);
+      int mL = 0, jL = 0;
+      uint32_t pL = 0;
+      float2 yL = make_float2(0.f, 0.f);  // the measurement (or the partial sum so far) of the sample
+      float wL[2 * W];
+#pragma unroll
+      for (int q = 0; q < 2 * W; ++q) wL[q] = 0.f;
+      if (lane < MPL && sL < g.count) {
+        const int si = g.start + sL;
+        mL = __ldg(&a.order[si]);
+        pL = __ldg(&a.kb_idx[si]);
+#pragma unroll
+        for (int q = 0; q < WQ; ++q) {
+          const float4 v = __ldg(&a.kb_w[(size_t)WQ * si + q]);
+          wL[4 * q] = v.x;
+          wL[4 * q + 1] = v.y;
+          wL[4 * q + 2] = v.z;
+          wL[4 * q + 3] = v.w;
+        }
+        jL = mL % a.R;
+        if (a.accumulate)
+          yL = a.y[mL];
+        else if (a.y_meas)
+          yL = __ldg(&a.y_meas[mL]);
+      }
+      if (!mbar_wait_warp(&full[b], (uint32_t)((k / a.nbuf) & 1), &s_abort)) break;
+      const float2* tile = bufs + b * tile_elems;
+
+      float2 mine = make_float2(0.f, 0.f);  // the value of the round whose number is the lane's place in its group
+      for (int rnd = 0; rnd * NCW * SPW + warp * SPW < g.count; ++rnd) {
+        const int s = rnd * NCW * SPW + warp * SPW + slot;
+        const bool valid = s < g.count;
+        const int src = rnd * SPW + slot;
+        const int m = __shfl_sync(0xffffffffu, mL, src);
+        const int j = __shfl_sync(0xffffffffu, jL, src);
+        const uint32_t packed = __shfl_sync(0xffffffffu, pL, src);
+        const float2 yprev = make_float2(__shfl_sync(0xffffffffu, yL.x, src), __shfl_sync(0xffffffffu, yL.y, src));
+        float w[2 * W];
+#pragma unroll
+        for (int q = 0; q < 2 * W; ++q) w[q] = __shfl_sync(0xffffffffu, wL[q], src);
+        const float2* P = a.phase + (size_t)j * a.Nf + a.f0 + f_lo;
+        float2 P0 = make_float2(0.f, 0.f), P1 = make_float2(0.f, 0.f);
+        if (valid && b0) P0 = __ldg(P);
+        if (valid && b1) P1 = __ldg(P + 1);
+        float2 tot = make_float2(0.f, 0.f);
+        if (valid) {
+          const int lc = (int)(packed & 0xffff) - g.c0;
+          const int lr = (int)(packed >> 16) - g.r0;
+          const float4* base = reinterpret_cast<const float4*>(tile + ((size_t)lr * HC + lc) * CS + f_lo);
+          // row sums over the x1 taps, folded into the x2 sum row by row
+          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int q = 0; q < W; ++q) {
+            float4 rs = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int c = 0; c < W; ++c) {
+              const float4 gv = base[(q * HC + c) * (CS / 2)];
+              rs.x = fmaf(w[c], gv.x, rs.x);
+              rs.y = fmaf(w[c], gv.y, rs.y);
+              rs.z = fmaf(w[c], gv.z, rs.z);
+              rs.w = fmaf(w[c], gv.w, rs.w);
+            }
+            acc.x = fmaf(w[W + q], rs.x, acc.x);
+            acc.y = fmaf(w[W + q], rs.y, acc.y);
+            acc.z = fmaf(w[W + q], rs.z, acc.z);
+            acc.w = fmaf(w[W + q], rs.w, acc.w);
+          }
+          const float2 z0 = cmulf(P0, make_float2(acc.x, acc.y));
+          const float2 z1 = cmulf(P1, make_float2(acc.z, acc.w));
+          tot = make_float2(z0.x + z1.x, z0.y + z1.y);
+        }
+#pragma unroll
+        for (int o = LPS / 2; o > 0; o >>= 1) {
+          tot.x += __shfl_xor_sync(0xffffffffu, tot.x, o);
+          tot.y += __shfl_xor_sync(0xffffffffu, tot.y, o);
+        }
+        float2 v = make_float2(__fmul_rn(tot.x, a.scale), __fmul_rn(tot.y, a.scale));
+        if (a.accumulate)
+          v = make_float2(__fadd_rn(v.x, yprev.x), __fadd_rn(v.y, yprev.y));
+        else if (a.y_meas)
+          v = make_float2(__fsub_rn(v.x, yprev.x), __fsub_rn(v.y, yprev.y));
+        if (valid && sub == 0) a.y[m] = v;
+        if (valid && sub == rnd) mine = v;
+        if (a.contrib && valid) {
+          // every lane of the sample holds the same reduced value
+          const float2 c0 = cmulcf(P0, v), c1 = cmulcf(P1, v);
+          reinterpret_cast<float4*>(a.contrib + (size_t)m * CS)[sub] = make_float4(c0.x, c0.y, c1.x, c1.y);
+        }
+      }
+      // (a sum a sample would keep the FP64 units busy for a quarter of the kernel)
+      if (a.partials) sumsq += (double)mine.x * mine.x + (double)mine.y * mine.y;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[b]);
+    }
+  }
+  __syncthreads();
+  if (s_abort && threadIdx.x == 0) atomicExch(a.err, 1);
+  if (a.partials) reduce_to_v(sumsq, a.partials, a.counter, a.sumsq_out, vb, vg);
+}
+
+template <int CS, int W>
+__global__ void __launch_bounds__(32 * (kTileWarps + 1), 1) tiles_kernel(InterpArgs a) {
+  tiles_body<CS, W, kTileWarps>(a, a.cta_off[blockIdx.x], a.cta_off[blockIdx.x + 1], blockIdx.x, gridDim.x);
+}
 
 // Interpolation for the bin strides CS in {8, 16, 32, 64}, four samples of a
 // blade at a time.
@@ -340,7 +497,7 @@ struct QuadArgs {
 // unit (a quad, or 32 / CS of them) of an item, the units going round the
 // warps across item borders; no compute warp waits for another.
 template <int CS, int W>
-__device__ __forceinline__ void quads_body(const QuadArgs& a, int it_beg, int it_end, unsigned vb, unsigned vg) {
+__device__ __forceinline__ void quads_body(const InterpArgs& a, int it_beg, int it_end, unsigned vb, unsigned vg) {
   using S = QuadShape<CS, W>;
   constexpr int NCW = kQuadWarps, NS = kQuadStages, UW = S::UW, NR = S::NR;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -611,31 +768,36 @@ __device__ __forceinline__ void quads_body(const QuadArgs& a, int it_beg, int it
 }
 
 template <int CS, int W>
-__global__ void __launch_bounds__(QuadShape<CS, W>::THREADS, 1) quads_kernel(QuadArgs a) {
+__global__ void __launch_bounds__(QuadShape<CS, W>::THREADS, 1) quads_kernel(InterpArgs a) {
   quads_body<CS, W>(a, a.cta_off[blockIdx.x], a.cta_off[blockIdx.x + 1], blockIdx.x, gridDim.x);
 }
 
 // Kernel parameter of the interpolation over a batch of problems.
-struct MultiQuads {
-  QuadArgs a[kMaxBatch];
+struct MultiInterp {
+  InterpArgs a[kMaxBatch];
   int plan_ctas[kMaxBatch];      // CTAs each problem's items were balanced over
   int nreq;
   int cta_begin[kMaxBatch + 1];  // CTA ranges of the problems
 };
 
 // One launch for several problems with the same bin stride and kernel
-// width: CTA b serves problem r (cta_begin[r] <= b < cta_begin[r + 1]) as
-// its CTA v of c = cta_begin[r + 1] - cta_begin[r] and takes the items the
-// problem's plan balanced over its CTAs v P / c .. (v + 1) P / c - 1, so every
-// sample is computed as in the problem's own launch.
+// width, with quads or tiles as each one's plan has it: CTA b serves problem r
+// (cta_begin[r] <= b < cta_begin[r + 1]) as its CTA v of c = cta_begin[r + 1] -
+// cta_begin[r] and takes the items the problem's plan balanced over its CTAs
+// v P / c .. (v + 1) P / c - 1, so every sample is computed as in the problem's
+// own launch.
 template <int CS, int W>
-__global__ void __launch_bounds__(QuadShape<CS, W>::THREADS, 1) quads_multi_kernel(const __grid_constant__ MultiQuads m) {
+__global__ void __launch_bounds__(QuadShape<CS, W>::THREADS, 1) interp_multi_kernel(const __grid_constant__ MultiInterp m) {
   int r = 0;
   while (r + 1 < m.nreq && (int)blockIdx.x >= m.cta_begin[r + 1]) ++r;
   const int v = (int)blockIdx.x - m.cta_begin[r], c = m.cta_begin[r + 1] - m.cta_begin[r];
   const int P = m.plan_ctas[r];
-  const QuadArgs& a = m.a[r];
-  quads_body<CS, W>(a, a.cta_off[(long)v * P / c], a.cta_off[(long)(v + 1) * P / c], (unsigned)v, (unsigned)c);
+  const InterpArgs& a = m.a[r];
+  const int beg = a.cta_off[(long)v * P / c], end = a.cta_off[(long)(v + 1) * P / c];
+  if (a.quads)
+    quads_body<CS, W>(a, beg, end, (unsigned)v, (unsigned)c);
+  else
+    tiles_body<CS, W, kQuadWarps>(a, beg, end, (unsigned)v, (unsigned)c);
 }
 
 // contrib[m][f] = conj(P[j_m][f0 + f]) r_m, LP lanes per sample.
@@ -944,7 +1106,7 @@ struct MultiSpread {
 
 // One launch for several problems with the same bin stride and list kind,
 // CTAs mapped onto each problem's balanced item ranges as in
-// quads_multi_kernel; every cell sums its own terms in its list's order.
+// interp_multi_kernel; every cell sums its own terms in its list's order.
 template <int CS, bool GROUPED>
 __global__ void __launch_bounds__(kSpreadThreads, kSpreadCtasPerSm)
     spread_stage_multi_kernel(const __grid_constant__ MultiSpread m) {
@@ -1126,28 +1288,32 @@ cudaError_t launch_interp(int lp, const InterpArgs& a, dim3 grid, size_t smem, c
   }
 }
 
-template <int W>
-cudaError_t launch_quads(int cs, const QuadArgs& a, int ctas, cudaStream_t s) {
-  const dim3 grid((unsigned)ctas);
+// f(CS, W) with the bin stride and the kernel width as compile-time constants.
+template <class F>
+cudaError_t with_stride(int cs, int W, const F& f) {
+  auto width = [&](auto c) {
+    return W == 8 ? f(c, std::integral_constant<int, 8>()) : f(c, std::integral_constant<int, 6>());
+  };
   switch (cs) {
-    case 8: return launch_dep(quads_kernel<8, W>, grid, dim3(QuadShape<8, W>::THREADS), QuadShape<8, W>::SMEM, s, a);
-    case 16: return launch_dep(quads_kernel<16, W>, grid, dim3(QuadShape<16, W>::THREADS), QuadShape<16, W>::SMEM, s, a);
-    case 32: return launch_dep(quads_kernel<32, W>, grid, dim3(QuadShape<32, W>::THREADS), QuadShape<32, W>::SMEM, s, a);
-    case 64: return launch_dep(quads_kernel<64, W>, grid, dim3(QuadShape<64, W>::THREADS), QuadShape<64, W>::SMEM, s, a);
+    case 8: return width(std::integral_constant<int, 8>());
+    case 16: return width(std::integral_constant<int, 16>());
+    case 32: return width(std::integral_constant<int, 32>());
+    case 64: return width(std::integral_constant<int, 64>());
     default: return cudaErrorInvalidValue;
   }
 }
 
-template <int W>
-cudaError_t launch_quads_multi(int cs, const MultiQuads& m, int ctas, cudaStream_t s) {
-  const dim3 grid((unsigned)ctas);
-  switch (cs) {
-    case 8: return launch_dep(quads_multi_kernel<8, W>, grid, dim3(QuadShape<8, W>::THREADS), QuadShape<8, W>::SMEM, s, m);
-    case 16: return launch_dep(quads_multi_kernel<16, W>, grid, dim3(QuadShape<16, W>::THREADS), QuadShape<16, W>::SMEM, s, m);
-    case 32: return launch_dep(quads_multi_kernel<32, W>, grid, dim3(QuadShape<32, W>::THREADS), QuadShape<32, W>::SMEM, s, m);
-    case 64: return launch_dep(quads_multi_kernel<64, W>, grid, dim3(QuadShape<64, W>::THREADS), QuadShape<64, W>::SMEM, s, m);
-    default: return cudaErrorInvalidValue;
-  }
+cudaError_t launch_quads(const Plan& p, const InterpArgs& a, cudaStream_t s) {
+  return with_stride(p.cs, p.W, [&](auto cs, auto w) {
+    using S = QuadShape<cs(), w()>;
+    return launch_dep(quads_kernel<cs(), w()>, dim3((unsigned)p.quad_cut.ctas), dim3(S::THREADS), S::SMEM, s, a);
+  });
+}
+
+cudaError_t launch_tiles(const Plan& p, const InterpArgs& a, size_t smem, cudaStream_t s) {
+  return with_stride(p.cs, p.W, [&](auto cs, auto w) {
+    return launch_dep(tiles_kernel<cs(), w()>, dim3((unsigned)p.tile_cut.ctas), dim3(32 * (kTileWarps + 1)), smem, s, a);
+  });
 }
 
 template <class K>
@@ -1159,21 +1325,20 @@ cudaError_t allow_smem(K kernel, int optin) {
 }
 
 template <int CS, int W>
-cudaError_t configure_quads() {
-  const int smem = (int)QuadShape<CS, W>::SMEM;
-  const cudaError_t e =
-      cudaFuncSetAttribute(quads_kernel<CS, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(quads_multi_kernel<CS, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+cudaError_t configure_stride(int optin) {
+  cudaError_t e =
+      cudaFuncSetAttribute(quads_kernel<CS, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)QuadShape<CS, W>::SMEM);
+  if (e == cudaSuccess) e = allow_smem(tiles_kernel<CS, W>, optin);
+  return e == cudaSuccess ? allow_smem(interp_multi_kernel<CS, W>, optin) : e;
 }
 
 template <int W>
 cudaError_t configure_interp(int optin) {
   cudaError_t e;
-  if ((e = configure_quads<8, W>())) return e;
-  if ((e = configure_quads<16, W>())) return e;
-  if ((e = configure_quads<32, W>())) return e;
-  if ((e = configure_quads<64, W>())) return e;
+  if ((e = configure_stride<8, W>(optin))) return e;
+  if ((e = configure_stride<16, W>(optin))) return e;
+  if ((e = configure_stride<32, W>(optin))) return e;
+  if ((e = configure_stride<64, W>(optin))) return e;
   if ((e = allow_smem(interp_kernel<1, W>, optin))) return e;
   if ((e = allow_smem(interp_kernel<2, W>, optin))) return e;
   if ((e = allow_smem(interp_kernel<4, W>, optin))) return e;
@@ -1205,8 +1370,7 @@ cudaError_t nufft_configure(int smem_optin) {
 }
 
 size_t interp_tile_bytes(const Plan& p) {
-  const size_t side = interp_tile(p.cs) + p.W - 1;
-  return side * side * p.cs * sizeof(float2);
+  return (size_t)(interp_tile_rows(p.cs, p.W) + p.W - 1) * (interp_tile_cols(p.cs) + p.W - 1) * p.cs * sizeof(float2);
 }
 
 int interp_buffers(const Plan& p) {
@@ -1215,13 +1379,23 @@ int interp_buffers(const Plan& p) {
   return 2 * tile + 1024 <= (size_t)p.smem_optin ? 2 : 1;
 }
 
-// The fields that both interpolation kernels share.
-template <class A>
-A interp_args(const Plan& p, int f0, int nbins, float2* y, const float2* y_meas, bool accumulate, const Reducer* red,
-              double* sumsq, float2* contrib) {
-  A a{};
+// Dynamic shared memory of the tile kernels: the tiles, then a full and an
+// empty barrier per buffer.
+size_t interp_tiles_smem(const Plan& p) {
+  return (size_t)interp_buffers(p) * (interp_tile_bytes(p) + 2 * sizeof(uint64_t));
+}
+
+InterpArgs interp_args(const Plan& p, bool quads, int f0, int nbins, float2* y, const float2* y_meas, bool accumulate,
+                       const Reducer* red, double* sumsq, float2* contrib) {
+  InterpArgs a{};
   a.grid = p.grid;
-  a.items = p.items;
+  a.kb_idx = p.kb_idx;
+  a.kb_w = p.kb_w;
+  a.order = p.order;
+  const InterpCut& cut = quads ? p.quad_cut : p.tile_cut;
+  a.quads = quads ? p.quads : nullptr;
+  a.items = cut.items;
+  a.cta_off = cut.off;
   a.phase = p.phase;
   a.y = y;
   a.y_meas = y_meas;
@@ -1230,46 +1404,36 @@ A interp_args(const Plan& p, int f0, int nbins, float2* y, const float2* y_meas,
   a.counter = red ? red->counter : nullptr;
   a.sumsq_out = sumsq;
   a.err = p.status_dev;
+  a.n_items = cut.n;
+  a.R = p.R;
   a.n = p.n;
+  a.C = p.cs;
   a.Cv = nbins;
   a.f0 = f0;
   a.Nf = p.Nf;
   a.scale = 1.0f / (float)p.N;
   a.accumulate = accumulate ? 1 : 0;
-  return a;
-}
-
-QuadArgs quad_args(const Plan& p, int f0, int nbins, float2* y, const float2* y_meas, bool accumulate,
-                   const Reducer* red, double* sumsq, float2* contrib) {
-  QuadArgs a = interp_args<QuadArgs>(p, f0, nbins, y, y_meas, accumulate, red, sumsq, contrib);
-  a.quads = p.quads;
-  a.cta_off = p.item_cta_off;
+  a.TR = interp_tile_rows(p.cs, p.W);
+  a.TC = interp_tile_cols(p.cs);
+  a.nct = p.n / a.TC;
+  a.tpf = (p.n + a.TR - 1) / a.TR * a.nct;
+  a.nbuf = interp_buffers(p);
   return a;
 }
 
 cudaError_t interp(const Plan& p, int f0, int nbins, float2* y, const float2* y_meas, bool accumulate,
                    const Reducer* red, double* sumsq, float2* contrib, cudaStream_t s) {
-  if (p.n_items == 0) return cudaSuccess;
-  if (p.quads) {  // exactly the plan's balanced CTAs
-    if (red && red->capacity < p.interp_ctas) return cudaErrorInvalidValue;
-    const QuadArgs a = quad_args(p, f0, nbins, y, y_meas, accumulate, red, sumsq, contrib);
-    return p.W == 8 ? launch_quads<8>(p.cs, a, p.interp_ctas, s) : launch_quads<6>(p.cs, a, p.interp_ctas, s);
-  }
-  InterpArgs a = interp_args<InterpArgs>(p, f0, nbins, y, y_meas, accumulate, red, sumsq, contrib);
-  a.kb_idx = p.kb_idx;
-  a.kb_w = p.kb_w;
-  a.order = p.order;
-  a.n_items = p.n_items;
-  a.R = p.R;
-  a.C = p.cs;
-  a.TR = a.TC = interp_tile(p.cs);
-  a.nct = p.n / a.TC;
-  a.tpf = p.n / a.TR * a.nct;
-  a.nbuf = interp_buffers(p);
-  // tiles, then a barrier per buffer; the kernel strides over the items
-  const size_t smem = (size_t)a.nbuf * interp_tile_bytes(p) + a.nbuf * sizeof(uint64_t);
-  const int blocks = std::min(p.n_items, p.num_sms);
+  const InterpCut& cut = p.lone_quads ? p.quad_cut : p.tile_cut;
+  if (cut.n == 0) return cudaSuccess;
+  const InterpArgs a = interp_args(p, p.lone_quads, f0, nbins, y, y_meas, accumulate, red, sumsq, contrib);
+  // the stride's kernels (tiles: where more than half of the bins are live) run
+  // exactly the plan's balanced CTAs, the run-time-stride kernel strides over the items
+  const bool balanced = p.lone_quads || (quad_stride(p.cs) && 2 * nbins > p.cs);
+  const int blocks = balanced ? cut.ctas : std::min(cut.n, p.num_sms);
   if (red && red->capacity < blocks) return cudaErrorInvalidValue;
+  if (p.lone_quads) return launch_quads(p, a, s);
+  const size_t smem = interp_tiles_smem(p);
+  if (balanced) return launch_tiles(p, a, smem, s);
   const int lp = lanes_for(nbins);
   const dim3 grid((unsigned)blocks);
   return p.W == 8 ? launch_interp<8>(lp, a, grid, smem, s) : launch_interp<6>(lp, a, grid, smem, s);
@@ -1277,34 +1441,45 @@ cudaError_t interp(const Plan& p, int f0, int nbins, float2* y, const float2* y_
 
 cudaError_t interp_residual_batch(Plan* const* ps, const float2* const* y_meas, int count, cudaStream_t s) {
   if (count < 1 || count > kMaxBatch) return cudaErrorInvalidValue;
-  MultiQuads m{};
+  int together = 0;
+  bool multi[kMaxBatch];
+  for (int r = 0; r < count; ++r) {
+    const Plan& p = *ps[r];
+    if (p.nchunks != 1) return cudaErrorInvalidValue;
+    multi[r] = quad_stride(p.cs) && p.cs == ps[0]->cs && p.W == ps[0]->W;
+    together += multi[r] ? 1 : 0;
+  }
+  MultiInterp m{};
   m.nreq = 0;
-  Plan* mp[kMaxBatch];
+  long work[kMaxBatch];
+  int cap[kMaxBatch];
+  size_t smem = 0;
   for (int r = 0; r < count; ++r) {
     Plan& p = *ps[r];
-    if (p.nchunks != 1) return cudaErrorInvalidValue;
-    const bool multi = p.quads && ps[0]->quads && p.cs == ps[0]->cs && p.W == ps[0]->W && p.n_items > 0;
-    if (!multi) {  // its own launch
+    if (!multi[r] || together == 1) {  // its own launch
       const cudaError_t e = interp(p, 0, p.Nf, p.resid, y_meas[r], false, &p.red_interp, p.scalars, p.contrib, s);
       if (e != cudaSuccess) return e;
       continue;
     }
-    mp[m.nreq] = &p;
-    m.a[m.nreq] = quad_args(p, 0, p.Nf, p.resid, y_meas[r], false, &p.red_interp, p.scalars, p.contrib);
-    m.plan_ctas[m.nreq] = p.interp_ctas;
-    ++m.nreq;
+    const bool quads = p.quad_cut.n > 0;  // (a plan holds them where they are better for a batch)
+    const InterpCut& cut = quads ? p.quad_cut : p.tile_cut;
+    const int q = m.nreq++;
+    m.a[q] = interp_args(p, quads, 0, p.Nf, p.resid, y_meas[r], false, &p.red_interp, p.scalars, p.contrib);
+    m.plan_ctas[q] = cut.ctas;
+    work[q] = p.M;
+    cap[q] = cut.ctas;
+    if (p.red_interp.capacity < cap[q]) return cudaErrorInvalidValue;
+    if (!quads) smem = std::max(smem, interp_tiles_smem(p));
   }
   if (m.nreq == 0) return cudaSuccess;
-  long work[kMaxBatch];
-  int cap[kMaxBatch];
-  for (int r = 0; r < m.nreq; ++r) {
-    work[r] = mp[r]->M;
-    cap[r] = mp[r]->interp_ctas;
-    if (mp[r]->red_interp.capacity < cap[r]) return cudaErrorInvalidValue;
-  }
-  const Plan& p0 = *mp[0];
+  const Plan& p0 = *ps[0];
   const int ctas = split_ctas(work, cap, m.nreq, std::max(m.nreq, p0.num_sms), m.cta_begin);
-  return p0.W == 8 ? launch_quads_multi<8>(p0.cs, m, ctas, s) : launch_quads_multi<6>(p0.cs, m, ctas, s);
+  return with_stride(p0.cs, p0.W, [&](auto cs, auto w) {
+    using S = QuadShape<cs(), w()>;
+    for (int r = 0; r < m.nreq; ++r)
+      if (m.a[r].quads) smem = std::max(smem, S::SMEM);
+    return launch_dep(interp_multi_kernel<cs(), w()>, dim3((unsigned)ctas), dim3(S::THREADS), smem, s, m);
+  });
 }
 
 cudaError_t spread_batch(Plan* const* ps, int count, cudaStream_t s) {

@@ -186,6 +186,69 @@ void mark_used_blocks(Plan& p, const std::vector<int>& first_tap) {
   p.grid_sparse = 2 * count < p.grid_used_h.size() * (size_t)(n / kGridBlock);
 }
 
+// Interpolation tiles and their work items: samples sorted by (frame, TR x
+// TC-cell tile of their first tap), ascending m within a tile; every non-empty
+// tile's run is cut into items of at most kInterpItem samples.  One CTA per
+// item stages the tile plus its (W - 1)-cell halo in shared memory.
+// At the bin strides 8 to 64 the items are balanced over `ctas` persistent CTAs:
+// longest first to the least loaded CTA, with an item's cost its shared-memory
+// traffic (W^2 taps of cs bins per sample plus the staged tile); each CTA's items
+// are then stored contiguously, in tile order.  The run-time-stride kernel strides
+// over the items, and they stay in tile order (the balanced order takes longer in
+// it: 43 bins at N = 256 81 -> 94 us, 33 bins at N = 192 82 -> 92 us); cta_off is
+// then one 0.
+void build_tiles(const Plan& p, const std::vector<int>& first_tap, int ctas, std::vector<int>& order,
+                 std::vector<int4>& items, std::vector<int>& cta_off) {
+  const int TR = interp_tile_rows(p.cs, p.W), TC = interp_tile_cols(p.cs);
+  const int nrt = (p.n + TR - 1) / TR, nct = p.n / TC;  // tiles per column / per row of the grid
+  const size_t ntile = (size_t)p.T * nrt * nct, LR = (size_t)p.L * p.R;
+  auto tile_of = [&](size_t m) {
+    const size_t frame = (size_t)p.blade_frame[m / LR];
+    return (frame * nrt + first_tap[2 * m + 1] / TR) * nct + first_tap[2 * m] / TC;
+  };
+  std::vector<int> cnt(ntile + 1, 0);
+  for (size_t m = 0; m < (size_t)p.M; ++m) cnt[tile_of(m) + 1]++;
+  for (size_t t = 0; t < ntile; ++t) cnt[t + 1] += cnt[t];
+  std::vector<int4> by_tile;
+  for (size_t t = 0; t < ntile; ++t) {
+    // a tile's run in ceil(c / kInterpItem) items of nearly equal size
+    const int c = cnt[t + 1] - cnt[t];
+    const int parts = (c + kInterpItem - 1) / kInterpItem;
+    for (int q = 0, s = cnt[t]; q < parts; ++q) {
+      const int sz = c / parts + (q < c % parts ? 1 : 0);
+      by_tile.push_back(make_int4((int)t, s, sz, 0));
+      s += sz;
+    }
+  }
+  order.resize(p.M);
+  for (size_t m = 0; m < (size_t)p.M; ++m) order[cnt[tile_of(m)]++] = (int)m;
+  if (!quad_stride(p.cs)) {
+    items.swap(by_tile);
+    cta_off.assign(1, 0);
+    return;
+  }
+  const int P = std::max(1, std::min(ctas, (int)by_tile.size()));
+  const long tile_cost = (long)(TR + p.W - 1) * (TC + p.W - 1) * p.cs / 16;
+  auto cost = [&](const int4& it) { return (long)it.z * p.W * p.W * p.cs / 16 + tile_cost; };
+  std::vector<int> idx(by_tile.size());
+  for (size_t i = 0; i < idx.size(); ++i) idx[i] = (int)i;
+  std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) { return cost(by_tile[a]) > cost(by_tile[b]); });
+  std::vector<long> load(P, 0);
+  std::vector<std::vector<int>> own(P);
+  for (int i : idx) {
+    const int best = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+    load[best] += cost(by_tile[i]);
+    own[best].push_back(i);
+  }
+  items.clear();
+  cta_off.assign(P + 1, 0);
+  for (int c = 0; c < P; ++c) {
+    std::sort(own[c].begin(), own[c].end());
+    for (int i : own[c]) items.push_back(by_tile[i]);
+    cta_off[c + 1] = (int)items.size();
+  }
+}
+
 // Modelled cost of an interpolation item in clock cycles of an SM, from fits
 // to the CTAs' own clocks at the static (32 bins), dynamic (16) and 64-bin
 // configurations: an item's turn round the warps, its quads, and the copies of
@@ -300,6 +363,68 @@ void build_quads(const Plan& p, const std::vector<int>& first_tap, const std::ve
   }
 }
 
+// What the two interpolations of the bin strides 8 to 64 cost, in ns of a CTA:
+// tiles an item, a round of the warps over an item's samples (width 8; the
+// latency of one), a round's worth of samples (width 8; its shared-memory
+// wavefronts); quads an item, a unit (what a warp takes at once; width 8), a
+// grid row added to the ring (its width in cells as at width 8), and the
+// difference of the launches (the quads' 227 KB of shared memory do not overlap
+// the kernel before).  Fitted to the times of both, forward passes replayed from
+// a graph and iterations of a reconstruction, at 1150 geometries (N = 16 to 512,
+// 1 to 32 frames, 1 to 64 lines, both widths): the plan's longest CTA decides,
+// as every CTA runs alone on its SM.
+struct InterpModel {
+  int t_item, t_round, t_samples, q_item, q_unit, q_row, q_launch;
+};
+constexpr InterpModel interp_model(int cs) {
+  return cs == 8    ? InterpModel{1630, 860, 2700, 780, 234, 160, -850}
+         : cs == 16 ? InterpModel{1420, 750, 1520, 1170, 158, 121, 0}
+         : cs == 32 ? InterpModel{1090, 570, 1710, 540, 170, 122, 450}
+                    : InterpModel{730, 1130, 1070, 1790, 251, 72, 1700};
+}
+// Modelled times of a cut: of its longest CTA and of all of them together.
+struct InterpTime {
+  double longest = 0, total = 0;
+  void add(double t) {
+    longest = std::max(longest, t);
+    total += t;
+  }
+};
+InterpTime tiles_time(const Plan& p, const std::vector<int4>& items, const std::vector<int>& cta_off) {
+  const InterpModel k = interp_model(p.cs);
+  const int round = kTileWarps * tile_samples_per_warp(p.cs);
+  InterpTime time;
+  for (size_t c = 0; c + 1 < cta_off.size(); ++c) {
+    long samples = 0, rounds = 0;
+    for (int i = cta_off[c]; i < cta_off[c + 1]; ++i) {
+      samples += items[i].z;
+      rounds += (items[i].z + round - 1) / round;
+    }
+    time.add((double)k.t_item * (cta_off[c + 1] - cta_off[c]) + k.t_round * p.W / 8.0 * rounds +
+             k.t_samples * (p.W * p.W / 64.0) * samples / round);
+  }
+  return time;
+}
+InterpTime quads_time(const Plan& p, const std::vector<int4>& items, const std::vector<int>& cta_off) {
+  const InterpModel k = interp_model(p.cs);
+  const double unit = k.q_unit * (quad_window(p.W) * quad_window(p.W) / 121.0);
+  const double row = (double)k.q_row * quad_row_bytes(p.cs, p.W) / quad_row_bytes(p.cs, 8);
+  InterpTime time;
+  for (size_t c = 0; c + 1 < cta_off.size(); ++c) {
+    long units = 0, rows = 0;
+    for (int i = cta_off[c]; i < cta_off[c + 1]; ++i) {
+      const int4 it = items[i];
+      const int r0 = it.w & 0xffff, nr = it.w >> 16;
+      units += (it.z + quad_per_warp(p.cs) - 1) / quad_per_warp(p.cs);
+      const bool on = i > cta_off[c] && items[i - 1].x == it.x;  // the strip goes on: only new rows
+      rows += nr - std::min(nr, on ? std::max(0, (items[i - 1].w & 0xffff) + (items[i - 1].w >> 16) - r0) : 0);
+    }
+    time.add((double)k.q_item * (cta_off[c + 1] - cta_off[c]) + unit * units + row * rows);
+  }
+  time.longest += k.q_launch;
+  return time;
+}
+
 struct DevAlloc {
   Plan* p;
   size_t* counter;
@@ -342,7 +467,7 @@ void plan_dev_free(Plan* p, void* ptr) {
 void plan_free(Plan* p) {
   if (!p) return;
   void* ptrs[] = {p->kb_idx, p->kb_w, p->phase, p->deapod, p->twiddle, p->blade_frame_d,
-                  p->order, p->quads, p->items, p->item_cta_off, p->grid_used, p->sitems, p->sitem_cta_off, p->spread_claim, p->sblob, p->contrib, p->grid, p->rows,
+                  p->order, p->quads, p->tile_cut.items, p->tile_cut.off, p->quad_cut.items, p->quad_cut.off, p->grid_used, p->sitems, p->sitem_cta_off, p->spread_claim, p->sblob, p->contrib, p->grid, p->rows,
                   p->resid, p->grad, p->status_dev,
                   p->vol2, p->adam_m, p->adam_v, p->loss_dev, p->scalars,
                   p->red_interp.partials, p->red_interp.counter, p->red_tv.partials,
@@ -518,53 +643,47 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
   for (int q = 0; q < n; ++q)
     tw[q] = make_float2((float)std::cos(2 * M_PI * q / n), (float)-std::sin(2 * M_PI * q / n));
 
-  // Interpolation work items.  Bin strides 8 to 64: quads.  Others: samples
-  // sorted by (frame, TR x TC-cell tile of their first tap), ascending m within
-  // a tile; every non-empty tile's run is cut into items of at most kInterpItem
-  // samples.  One CTA per item stages the tile plus its (W-1)-cell halo in
-  // shared memory.
+  // Interpolation work items.  At the bin strides 8 to 64 the plan takes quads
+  // or tiles, whichever the model has faster (the results are the same bit for
+  // bit).  Quads win where samples are dense (the static benchmark's operator,
+  // 32 bins: a forward pass 92 -> 85 us) or crowd into few tiles (one frame of 48
+  // blades of 4 lines at N = 32, 64 bins: 43.7 -> 14 us); tiles where a frame has
+  // few samples (32 frames of 2 x 4 lines at N = 16, 64 bins: 32.0 -> 26.3 us),
+  // where one line a blade leaves half of a quad empty (192^2 x 64 bins, 32
+  // frames: 104 -> 64 us of interpolation) and with 64 bins at width 8 unless the
+  // samples crowd (one scan of 16 blades, N = 256: 168 -> 123 us).  Over the
+  // fitted geometries the rule's forward pass is 0.2 % slower than that of the
+  // better of the two; quads alone were 3.4 %, tiles 23 %.
+  // A batch shares the CTAs out over its plans, so that a plan's share counts, not
+  // its longest CTA: it takes quads where they cost less in total, and a plan keeps
+  // both where the two differ (four plans of 192^2 x 16 bins, two of them with
+  // tiles of their own: 3218 us with those tiles, 3174 with quads for all).
   const size_t LR = (size_t)p->L * p->R;
-  std::vector<int> order;
-  std::vector<int4> items;
-  std::vector<int> cta_off;
+  std::vector<int> order, tile_off, quad_off;
+  std::vector<int4> tile_items, quad_items;
   std::vector<float4> quads;
+  build_tiles(*p, first_tap, p->num_sms, order, tile_items, tile_off);
   if (quad_stride(p->cs)) {
     mark_used_blocks(*p, first_tap);
-    build_quads(*p, first_tap, wd, p->num_sms, quads, items, cta_off);
-    kb_idx.clear();
-    kb_w.clear();
-    p->n_items = (int)items.size();
-    p->interp_ctas = (int)cta_off.size() - 1;
-  } else {
-  const int TR = interp_tile(p->cs), TC = TR;
-  const int nrt = n / TR, nct = n / TC;  // tiles per column / per row of the grid
-  const size_t ntile = (size_t)p->T * nrt * nct;
-  order.resize(p->M);
-  {
-    auto tile_of = [&](size_t m) {
-      const size_t frame = (size_t)p->blade_frame[m / LR];
-      return (frame * nrt + first_tap[2 * m + 1] / TR) * nct + first_tap[2 * m] / TC;
-    };
-    std::vector<int> cnt(ntile + 1, 0);
-    for (size_t m = 0; m < (size_t)p->M; ++m) cnt[tile_of(m) + 1]++;
-    for (size_t t = 0; t < ntile; ++t) cnt[t + 1] += cnt[t];
-    for (size_t t = 0; t < ntile; ++t) {
-      // a tile's run in ceil(c / kInterpItem) items of nearly equal size
-      const int c = cnt[t + 1] - cnt[t];
-      const int parts = (c + kInterpItem - 1) / kInterpItem;
-      for (int q = 0, s = cnt[t]; q < parts; ++q) {
-        const int sz = c / parts + (q < c % parts ? 1 : 0);
-        items.push_back(make_int4((int)t, s, sz, 0));
-        s += sz;
-      }
+    build_quads(*p, first_tap, wd, p->num_sms, quads, quad_items, quad_off);
+    const InterpTime tt = tiles_time(*p, tile_items, tile_off), qt = quads_time(*p, quad_items, quad_off);
+    p->lone_quads = qt.longest < tt.longest;
+    if (!p->lone_quads && qt.total >= tt.total) {
+      quads.clear();
+      quad_items.clear();
+      quad_off.clear();
     }
-    for (size_t m = 0; m < (size_t)p->M; ++m) order[cnt[tile_of(m)]++] = (int)m;
+    if (p->lone_quads) {
+      kb_idx.clear();
+      kb_w.clear();
+      order.clear();
+      tile_items.clear();
+      tile_off.clear();
+    }
   }
-  p->n_items = (int)items.size();
-  cta_off.assign(1, 0);  // the run-time-stride kernel strides over the items
-  // The interpolation reads the per-sample tables in this sorted order, so that
-  // an item's metadata is one contiguous run.
-  {
+  if (!p->lone_quads) {
+    // The tile kernels read the per-sample tables in item order, so that an
+    // item's metadata is one contiguous run.
     std::vector<uint32_t> idx_s(p->M);
     std::vector<float4> w_s(kb_w.size());
     for (size_t i = 0; i < (size_t)p->M; ++i) {
@@ -574,7 +693,6 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
     }
     kb_idx.swap(idx_s);
     kb_w.swap(w_s);
-  }
   }
 
   // Spread gather lists: for every (frame, cell) the samples whose W x W
@@ -739,19 +857,25 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
       return st;             \
     }                        \
   } while (0)
-  if (quads.empty()) {
+  if (!p->lone_quads) {
     TRY(tab(&p->kb_idx, kb_idx.size(), "sample indices"));
     TRY(tab(&p->kb_w, kb_w.size(), "sample weights"));
     TRY(tab(&p->order, order.size(), "interpolation order"));
-  } else {
-    TRY(tab(&p->quads, quads.size(), "interpolation quads"));
   }
+  if (!quads.empty()) TRY(tab(&p->quads, quads.size(), "interpolation quads"));
   TRY(tab(&p->phase, phase.size(), "phase table"));
   TRY(tab(&p->deapod, deapod.size(), "deapodisation table"));
   TRY(tab(&p->twiddle, tw.size(), "twiddles"));
   TRY(tab(&p->blade_frame_d, p->blade_frame.size(), "blade frames"));
-  TRY(tab(&p->items, std::max<size_t>(items.size(), 1), "interpolation items"));
-  TRY(tab(&p->item_cta_off, cta_off.size(), "interpolation item ranges"));
+  const auto cut = [&](InterpCut& c, const std::vector<int4>& items, const std::vector<int>& off) {
+    c.n = (int)items.size();
+    c.ctas = std::max(1, (int)off.size() - 1);
+    if (items.empty()) return PROP_OK;
+    const prop_status s = tab(&c.items, items.size(), "interpolation items");
+    return s == PROP_OK ? tab(&c.off, off.size(), "interpolation item ranges") : s;
+  };
+  TRY(cut(p->tile_cut, tile_items, tile_off));
+  TRY(cut(p->quad_cut, quad_items, quad_off));
   TRY(tab(&p->sitems, std::max<size_t>(sitems.size(), 1), "spread items"));
   TRY(tab(&p->sitem_cta_off, scta_off.size(), "spread item ranges"));
   TRY(tab(&p->sblob, blob.size(), "spread lists"));
@@ -766,12 +890,17 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
     plan_free(p);
     return cuda_fail(e, "grid workspace");
   }
-  if (quads.empty()) {
+  if (!p->lone_quads) {
     TRY(upload(p->kb_idx, kb_idx));
     TRY(upload(p->kb_w, kb_w));
     TRY(upload(p->order, order));
-  } else {
+    TRY(upload(p->tile_cut.items, tile_items));
+    TRY(upload(p->tile_cut.off, tile_off));
+  }
+  if (!quads.empty()) {
     TRY(upload(p->quads, quads));
+    TRY(upload(p->quad_cut.items, quad_items));
+    TRY(upload(p->quad_cut.off, quad_off));
   }
   TRY(upload(p->phase, phase));
   TRY(upload(p->deapod, deapod));
@@ -781,8 +910,6 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
   TRY(upload(p->sitem_cta_off, scta_off));
   TRY(upload(p->sblob, blob));
   if (p->grid_used) TRY(upload(p->grid_used, p->grid_used_h));
-  if (!items.empty()) TRY(upload(p->items, items));
-  TRY(upload(p->item_cta_off, cta_off));
   p->row_kernel = d->row_kernel;
   fft_make_maps(*p);
   if (p->row_kernel == 2 && !p->fused_ws) {
@@ -827,7 +954,7 @@ prop_status plan_ensure_recon(Plan* p, int iters) {
   if (!p->recon_ready) {
     const size_t nv = p->vol_elems();
     const int fused_blocks = (p->Nf + kFftCols - 1) / kFftCols * p->T * p->N;  // fused row kernel's CTAs
-    const int red_cap = std::max(std::max(1 << 15, p->n_items), fused_blocks);
+    const int red_cap = std::max(1 << 15, fused_blocks);
     if ((st = rec(&p->resid, (size_t)p->M, "residual")) != PROP_OK) return st;
     if ((st = rec(&p->grad, nv, "gradient")) != PROP_OK) return st;
     if ((st = rec(&p->vol2, nv, "volume buffer")) != PROP_OK) return st;
@@ -870,15 +997,15 @@ size_t plan_estimate_bytes(const prop_plan_desc* d, int iters) {
   const size_t W = d->kb_width == 8 ? 8 : 6;
   const size_t chunk = d->bin_chunk == 0 ? std::min<size_t>(Nf, kMaxChunk) : std::min<size_t>(d->bin_chunk, Nf);
   const size_t cs = chunk + (chunk & 1);
-  const size_t tile = (size_t)interp_tile((int)cs);
+  const size_t TR = (size_t)interp_tile_rows((int)cs, (int)W), TC = (size_t)interp_tile_cols((int)cs);
   const size_t nquads = B * (((size_t)d->lines + 1) / 2) * (((size_t)d->readout + 1) / 2);
   const size_t ncell = T * n * n;
   const size_t vol = T * N * N * Nf;
-  const bool quads = quad_stride((int)cs);
-  const size_t interp_items = quads ? nquads : M / kInterpItem + T * (n / tile) * (n / tile) + 1;
+  const size_t quads = quad_stride((int)cs) ? nquads : 0;  // the plan may take these, tiles or both
+  const size_t interp_items = quads + M / kInterpItem + T * ((n + TR - 1) / TR) * (n / TC) + 1;
   const size_t spread_items = (M * W * W + kSpreadCellCost * ncell) / kSpreadItemCost + 1;
   size_t b = 0;
-  b += quads ? nquads * quad_record((int)W) * 16 : 8 * M + M * (W / 2) * 16;                    // sample tables
+  b += quads * quad_record((int)W) * 16 + 8 * M + M * (W / 2) * 16;                             // sample tables
   b += (size_t)d->readout * Nf * 8 + 4 * N + 8 * n + 4 * B;
   const size_t cell_lists = 8 * (ncell + spread_items) + 8 * (M * W * W + (kSpreadListPad - 1) * std::min(ncell, M * W * W));
   const size_t group_lists = 8 * (ncell / 4) + 8 + (4 + 16) * 2 * 16 * M + 16 * (ncell / 4);  // items <= groups

@@ -38,12 +38,21 @@ constexpr int kFftCols = 16;       // columns (complex lines) per FFT tile
 // 4-line tiles still read whole 32-byte sectors along a column).
 constexpr int kCartCols = 4;
 
-// Interpolation tile (rows and cells per row) of the run-time bin strides:
-// 16 x 16 up to 32 bins, 8 x 8 above.
-constexpr int interp_tile(int cs) { return cs > 32 ? 8 : 16; }
+// Interpolation tile (rows x cells per row) for bin stride cs and kernel
+// width W: 16 x 16 up to 32 bins, 8 x 8 above.  At width 8 with 32 bins a
+// 16 x 16 tile plus its 7-cell halo (23 x 23 cells, 135 KB) leaves room for
+// one buffer only, so its copy could not overlap the previous tile's work;
+// 12 rows of 16 (19 x 23 staged cells, 112 KB) double-buffer and stage 2.3x
+// the cells they own (16 x 16: 2.1x; 8 x 8: 3.5x, which measured slower).
+// Rows of tiles need not divide the grid: the last one wraps past row n - 1.
+constexpr int interp_tile_rows(int cs, int W) { return cs > 32 ? 8 : (W == 8 && cs == 32 ? 12 : 16); }
+constexpr int interp_tile_cols(int cs) { return cs > 32 ? 8 : 16; }
+constexpr int kTileWarps = 16;  // compute warps of the tile kernels at the bin strides 8 to 64
+constexpr int tile_samples_per_warp(int cs) { return 64 / cs; }  // and round: a lane takes two bins
 
-// Quads: the interpolation of the bin strides 8, 16, 32 and 64 takes the
-// samples of a blade 2 lines x 2 readout positions at a time.  They lie on a
+// Quads: at the bin strides 8, 16, 32 and 64 the interpolation may take the
+// samples of a blade 2 lines x 2 readout positions at a time (interp_model in
+// plan.cu: when).  They lie on a
 // rotated square lattice 2 grid cells apart, so along each axis their first
 // taps differ by at most floor(2 sqrt 2) + 1 = 3 cells whatever the angle, and
 // one window of (W + 3)^2 cells holds the four W x W footprints.
@@ -181,6 +190,14 @@ struct DeviceAllocator {
   virtual void release(void* ptr) = 0;
 };
 
+// Interpolation work items, grouped by the persistent CTAs they are balanced over
+// (run-time bin strides: in tile order, off unused); n = 0: none.
+struct InterpCut {
+  int4* items = nullptr;   // [n]
+  int* off = nullptr;      // [ctas + 1] CTA c takes items [off[c], off[c + 1])
+  int n = 0, ctas = 1;
+};
+
 struct Plan {
   DeviceAllocator* alloc = nullptr;
   // geometry
@@ -201,19 +218,19 @@ struct Plan {
   std::vector<int> blade_frame;
 
   // device tables
-  uint32_t* kb_idx = nullptr;    // [M] packed (i1 | i2 << 16) first tap, mod n, in interpolation order
+  uint32_t* kb_idx = nullptr;    // [M] packed (i1 | i2 << 16) first tap, mod n, in tile item order
   float4* kb_w = nullptr;        // [M][W/2] -> 2W floats: w1[W] (x1 taps) then w2[W] (x2 taps), same order
   float2* phase = nullptr;       // [R][Nf] exp(-2 pi i k_r Delta_f)
   float* deapod = nullptr;       // [N]
   float2* twiddle = nullptr;     // [n] exp(-2 pi i k / n)
   int* blade_frame_d = nullptr;  // [B]
-  int* order = nullptr;          // [M] samples sorted by grid tile (interpolation order)
-  float4* quads = nullptr;       // [quads][quad_record(W)] in item order (bin strides 8 to 64; instead of the three above)
-  int4* items = nullptr;         // [n_items] grouped by CTA: (tile of its frame, first sample, count, 0), or with quads
-                                 // (frame * strips + strip, first quad, count, first grid row | grid rows << 16)
-  int* item_cta_off = nullptr;   // [interp_ctas + 1] CTA c interpolates items [off[c], off[c + 1])
-  int n_items = 0;
-  int interp_ctas = 1;           // persistent interpolation CTAs the items are balanced over
+  int* order = nullptr;          // [M] samples sorted by grid tile (tile item order)
+  float4* quads = nullptr;       // [quads][quad_record(W)] in item order
+  // Interpolation by tiles (the three tables above) and by quads, either or both:
+  // what the plan's own launch takes, and quads where a batch is better off with them
+  InterpCut tile_cut;            // items (frame * tiles + tile, first sample, count, 0)
+  InterpCut quad_cut;            // items (frame * strips + strip, first quad, count, first grid row | grid rows << 16)
+  bool lone_quads = false;       // the plan's own launch takes quads
   // Spread gather: cells in patch-major order (frame, 8x8-cell patch,
   // row-major in the patch), cut into items; each item is one blob of
   // (cell, list end) pairs followed by its cells' (offset m * cs, weight
