@@ -189,14 +189,11 @@ void mark_used_blocks(Plan& p, const std::vector<int>& first_tap) {
 // Interpolation tiles and their work items: samples sorted by (frame, TR x
 // TC-cell tile of their first tap), ascending m within a tile; every non-empty
 // tile's run is cut into items of at most kInterpItem samples.  One CTA per
-// item stages the tile plus its (W - 1)-cell halo in shared memory.
-// At the bin strides 8 to 64 the items are balanced over `ctas` persistent CTAs:
-// longest first to the least loaded CTA, with an item's cost its shared-memory
-// traffic (W^2 taps of cs bins per sample plus the staged tile); each CTA's items
-// are then stored contiguously, in tile order.  The run-time-stride kernel strides
-// over the items, and they stay in tile order (the balanced order takes longer in
-// it: 43 bins at N = 256 81 -> 94 us, 33 bins at N = 192 82 -> 92 us); cta_off is
-// then one 0.
+// item stages the tile plus its (W - 1)-cell halo in shared memory.  Static
+// balance over `ctas` persistent CTAs: longest item first to the least loaded
+// CTA, with an item's cost its shared-memory traffic (W^2 taps of cs bins per
+// sample plus the staged tile); each CTA's items are then stored contiguously,
+// in tile order.
 void build_tiles(const Plan& p, const std::vector<int>& first_tap, int ctas, std::vector<int>& order,
                  std::vector<int4>& items, std::vector<int>& cta_off) {
   const int TR = interp_tile_rows(p.cs, p.W), TC = interp_tile_cols(p.cs);
@@ -222,11 +219,6 @@ void build_tiles(const Plan& p, const std::vector<int>& first_tap, int ctas, std
   }
   order.resize(p.M);
   for (size_t m = 0; m < (size_t)p.M; ++m) order[cnt[tile_of(m)]++] = (int)m;
-  if (!quad_stride(p.cs)) {
-    items.swap(by_tile);
-    cta_off.assign(1, 0);
-    return;
-  }
   const int P = std::max(1, std::min(ctas, (int)by_tile.size()));
   const long tile_cost = (long)(TR + p.W - 1) * (TC + p.W - 1) * p.cs / 16;
   auto cost = [&](const int4& it) { return (long)it.z * p.W * p.W * p.cs / 16 + tile_cost; };

@@ -190,8 +190,8 @@ struct DeviceAllocator {
   virtual void release(void* ptr) = 0;
 };
 
-// Interpolation work items, grouped by the persistent CTAs they are balanced over
-// (run-time bin strides: in tile order, off unused); n = 0: none.
+// Interpolation work items, grouped by the persistent CTAs they are balanced over;
+// n = 0: none.
 struct InterpCut {
   int4* items = nullptr;   // [n]
   int* off = nullptr;      // [ctas + 1] CTA c takes items [off[c], off[c + 1])

@@ -36,10 +36,7 @@ static bool takes_quads(int N, int Nf, int B, int L, int R, int T, int W) {
   const int TR = interp_tile_rows(p.cs, W), TC = interp_tile_cols(p.cs);
   const int nct = p.n / TC, tpf = (p.n + TR - 1) / TR * nct;
   std::vector<int> seen(p.M, 0);
-  if (quad_stride(p.cs))
-    CHECK((int)off.size() - 1 <= 152 && off[0] == 0 && off.back() == (int)items.size());
-  else
-    CHECK(off.size() == 1 && off[0] == 0);
+  CHECK((int)off.size() - 1 <= 152 && off[0] == 0 && off.back() == (int)items.size());
   for (size_t c = 0; c + 1 < off.size(); ++c) CHECK(off[c] < off[c + 1]);
   for (const int4& it : items) {
     CHECK(it.z >= 1 && it.z <= kInterpItem);
