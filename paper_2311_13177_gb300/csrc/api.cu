@@ -76,22 +76,22 @@ prop_status check_device_status(Plan& p) {
   return PROP_OK;
 }
 
-// Copies `count` doubles of a call's result to the host, synchronises and
-// reports an expired bounded wait.  A single value and the status word go
-// through the plan's pinned words, so that the call waits for the device once.
-prop_status finish_call(Plan& p, double* host, const double* dev, int count, cudaStream_t s) {
-  if (count == 1 && p.host_words) {
-    PROP_CUDA(cudaMemcpyAsync(p.host_words, dev, sizeof(double), cudaMemcpyDeviceToHost, s));
-    PROP_CUDA(cudaMemcpyAsync(p.host_words + 1, p.status_dev, sizeof(int), cudaMemcpyDeviceToHost, s));
+// Copies a call's result to the host, synchronises and reports an expired bounded
+// wait.  The value and the status word go through the plan's pinned words, so
+// that the call waits for the device once.
+prop_status finish_call(Plan& p, double* host, const double* dev, cudaStream_t s) {
+  if (!p.host_words) {
+    PROP_CUDA(cudaMemcpyAsync(host, dev, sizeof(double), cudaMemcpyDeviceToHost, s));
     PROP_CUDA(cudaStreamSynchronize(s));
-    int st = 0;
-    std::memcpy(&st, p.host_words + 1, sizeof(int));
-    *host = p.host_words[0];
-    return st ? check_device_status(p) : PROP_OK;
+    return check_device_status(p);
   }
-  PROP_CUDA(cudaMemcpyAsync(host, dev, sizeof(double) * count, cudaMemcpyDeviceToHost, s));
+  PROP_CUDA(cudaMemcpyAsync(p.host_words, dev, sizeof(double), cudaMemcpyDeviceToHost, s));
+  PROP_CUDA(cudaMemcpyAsync(p.host_words + 1, p.status_dev, sizeof(int), cudaMemcpyDeviceToHost, s));
   PROP_CUDA(cudaStreamSynchronize(s));
-  return check_device_status(p);
+  int st = 0;
+  std::memcpy(&st, p.host_words + 1, sizeof(int));
+  *host = p.host_words[0];
+  return st ? check_device_status(p) : PROP_OK;
 }
 
 // y = A V, or r = A V - y_meas with |r|^2 reduced into *sumsq.  rows_ready:
@@ -572,7 +572,7 @@ prop_status prop_loss_grad(prop_plan plan, const void* y_dev, const prop_recon_p
   float2* out = grad_dev ? (float2*)grad_dev : p.grad;
   if ((st = loss_grad_device(p, (const float2*)y_dev, a, (const float2*)V_dev, out, p.scalars + 1, s)) != PROP_OK)
     return st;
-  return finish_call(p, loss_host, p.scalars + 1, 1, s);
+  return finish_call(p, loss_host, p.scalars + 1, s);
 }
 
 prop_status prop_render(prop_plan plan, const void* V_dev, int f_lo, int f_hi, void* image_dev, void* stream) {

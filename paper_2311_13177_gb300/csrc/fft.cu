@@ -529,7 +529,7 @@ struct FftArgs {
   float2* dst;
   const float* deapod;
   const float2* twiddle;
-  int N, n, Nf;
+  int Nf;
   int C;   // bin stride of the workspace (the plan's chunk)
   int Cv;  // valid bins in this chunk (<= C)
   int f0;
@@ -714,7 +714,7 @@ struct FusedArgs {
   unsigned int* counter;
   const double* data_loss;
   double* loss_out;
-  int N, n, Nf, C, T;
+  int N, Nf, C, T;
   float scale;         // adjoint scale (1/N)
   AdamArgs ad;
   // warp-specialised kernel only
@@ -1204,7 +1204,7 @@ struct ColArgs {
   const float2* twiddle;
   int* err;
   size_t nq;
-  int N, n, qtiles, ntiles, bh, nbox;
+  int qtiles, ntiles, bh, nbox;
   const uint64_t* used;  // grid blocks in use [frame][u1 / 2], or null
   int ushift;            // log2 of the 16-line tiles in two grid columns
   uint64_t box_mask;     // adjoint: the grid blocks in one box, at bit 0
@@ -1569,8 +1569,6 @@ ColArgs col_args(const Plan& p, int kind) {
   a.twiddle = p.twiddle;
   a.err = p.status_dev;
   a.nq = (size_t)p.n * p.cs;
-  a.N = p.N;
-  a.n = p.n;
   a.qtiles = (int)(a.nq / kFftCols);
   a.ntiles = a.qtiles * p.T;
   a.bh = col_box_rows(p, kind);
@@ -1819,8 +1817,6 @@ FftArgs base_args(const Plan& p) {
   FftArgs a{};
   a.deapod = p.deapod;
   a.twiddle = p.twiddle;
-  a.N = p.N;
-  a.n = p.n;
   a.Nf = p.Nf;
   a.C = p.cs;
   a.Cv = p.chunk;
@@ -1949,7 +1945,6 @@ FusedArgs fused_args(const Plan& p, const float2* Vin, float2* m, float2* v, flo
   a.data_loss = data_loss;
   a.loss_out = loss_out;
   a.N = p.N;
-  a.n = p.n;
   a.Nf = p.Nf;
   a.C = p.cs;
   a.T = p.T;

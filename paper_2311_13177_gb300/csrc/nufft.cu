@@ -8,20 +8,20 @@
 // displaced along the readout picks up a phase linear in k_r), summed over
 // the bins.  A persistent CTA per SM streams the grid rows it needs into shared
 // memory with TMA bulk copies (completion on mbarriers) ahead of its compute
-// warps, which take a blade's samples four at a time (quads_kernel; a sample
-// at a time over staged tiles for other bin strides).  Bins are the fastest
-// axis, so the lanes that serve a sample read consecutive bins of a cell
-// (conflict-free).
+// warps, which take a blade's samples four at a time (quads_kernel) or one at a
+// time over staged tiles (tiles_kernel, whichever the plan's model has faster;
+// interp_kernel for run-time bin strides).  Bins are the fastest axis, so the
+// lanes that serve a sample read consecutive bins of a cell (conflict-free).
 //
 // Adjoint: G'_{t,f}[cell] = sum_m w(m, cell) conj(P[j_m][f]) r_m.  The
 // phased residual contrib[m][f] = conj(P[j_m][f]) r_m is formed once per
 // sample (fused into the interpolation when the grid holds every bin), then
 // the grid is gathered from plan-time lists in a fixed order: every group
-// of kSpreadGroupRows x kSpreadGroupCols cells reads each covering sample's
-// phased residual once and adds it with that sample's weight on each of its
-// cells (per-cell lists where the stride or a list's length rules the
-// groups out).  No atomics,
-// every cell written exactly once, bitwise reproducible.
+// of kSpreadGroup x kSpreadGroup cells reads each covering sample's phased
+// residual once and adds it with that sample's weight on each of its cells
+// (per-cell lists where the stride or a list's length rules the groups out).
+// No atomics, every cell of the grid blocks that samples reach written exactly
+// once (with per-cell lists: of the grid), bitwise reproducible.
 #include "prop_internal.cuh"
 #include "tma.cuh"
 

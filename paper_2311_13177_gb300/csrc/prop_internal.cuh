@@ -407,7 +407,8 @@ void fft_make_maps(Plan& p);
 cudaError_t interp(const Plan& p, int f0, int nbins, float2* y, const float2* y_meas,
                    bool accumulate, const Reducer* red, double* sumsq, float2* contrib, cudaStream_t s);
 // Adjoint spread of r into the grid chunk: contrib[m][f] = conj(P[j_m][f0+f]) r_m,
-// then every cell gathers sum_{(m, w) in its list} w contrib[m][f] (every cell written).
+// then every cell of the blocks in use (Plan::grid_used) gathers
+// sum_{(m, w) in its list} w contrib[m][f].
 cudaError_t nufft_configure(int smem_optin);
 int interp_buffers(const Plan& p);
 // contrib_ready: p.contrib already holds this chunk's phased residual (fused by interp).
