@@ -648,8 +648,9 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
   // better of the two; quads alone were 3.4 %, tiles 23 %.
   // A batch shares the CTAs out over its plans, so that a plan's share counts, not
   // its longest CTA: it takes quads where they cost less in total, and a plan keeps
-  // both where the two differ (four plans of 192^2 x 16 bins, two of them with
-  // tiles of their own: 3218 us with those tiles, 3174 with quads for all).
+  // both where the two differ.  At 8 and 16 bins, where a batch of both kinds was 5
+  // to 8 % slower than one of quads (four plans of 96^2 x 16 bins: 884 and 814 us),
+  // tiles have to cost half as much in total (24^2 x 16 bins: 245 and 267 us).
   const size_t LR = (size_t)p->L * p->R;
   std::vector<int> order, tile_off, quad_off;
   std::vector<int4> tile_items, quad_items;
@@ -660,7 +661,7 @@ prop_status plan_build(const prop_plan_desc* d, Plan** out, DeviceAllocator* all
     build_quads(*p, first_tap, wd, p->num_sms, quads, quad_items, quad_off);
     const InterpTime tt = tiles_time(*p, tile_items, tile_off), qt = quads_time(*p, quad_items, quad_off);
     p->lone_quads = qt.longest < tt.longest;
-    if (!p->lone_quads && qt.total >= tt.total) {
+    if (!p->lone_quads && tt.total < (p->cs <= 16 ? 0.5 : 1.0) * qt.total) {
       quads.clear();
       quad_items.clear();
       quad_off.clear();
