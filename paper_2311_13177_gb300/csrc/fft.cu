@@ -1385,15 +1385,17 @@ __global__ void __launch_bounds__(Shape<NFFT, kValsCols<NFFT>>::THREADS, col_cta
 // to four an SM, a launch asks for so much shared memory that no SM takes more
 // than its share (forward passes one after the other: 64^2 x 16 bins 14.2 ->
 // 11.4 us, 8 frames of 32^2 x 32 bins 14.8 -> 12.4; adjoint of 96^2 x 64 bins
-// 38.1 -> 31.2).
+// 38.1 -> 31.2).  Fewer CTAs than a quarter of the SMs spread by themselves, and
+// start later if they have to wait for an empty SM (32^2 x 8 bins 7.9 us, 7.5
+// without; from 48 CTAs on, 48^2 x 8 bins 8.4 and 10.0).
 constexpr size_t kEvenShare = (size_t)228 * 1024 / 2;  // the most that is asked for: one CTA an SM
 
 template <int NFFT>
 cudaError_t launch(int kind, const FftArgs& a, dim3 grid, int sms, cudaStream_t s) {
   auto go = [&](auto kern, int lines, int threads, size_t smem) {
     const dim3 g((grid.x + lines - 1) / lines, grid.y);
-    const size_t share = ((size_t)g.x * g.y + sms - 1) / sms;
-    if (share <= 4) smem = std::max(smem, (size_t)228 * 1024 / (share + 1));
+    const size_t ctas = (size_t)g.x * g.y, share = (ctas + sms - 1) / sms;
+    if (4 * ctas > (size_t)sms && share <= 4) smem = std::max(smem, (size_t)228 * 1024 / (share + 1));
     return launch_dep(kern, g, dim3(threads), smem, s, a);
   };
 #define PROP_GO(K) go(fft_kernel<NFFT, K>, kColsOf<NFFT, K>, kThreadsOf<NFFT, K>, kSmemOf<NFFT, K>)
